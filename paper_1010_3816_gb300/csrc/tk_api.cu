@@ -47,7 +47,7 @@ void release(tk_solver *S)
     void *ptrs[] = {S->u[0], S->u[1], S->half, S->node, S->b_node, S->w_row,
                     S->x_node, S->x_half, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
                     S->adj[0], S->adj[1], S->u_init, S->dhalf, S->dnode, S->db_node, S->pflags,
-                    S->obs_scr, S->xbuf, S->cmp, S->gpm};
+                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (int k = 0; k < 2; ++k)
@@ -131,6 +131,7 @@ void fill_launch(const tk_solver *S, tk::StepLaunch &L)
     L.node = S->node;
     L.cmp = S->cmp;
     L.gpm = S->gpm;
+    L.step = S->step;
     L.wave_cap = S->wave_cap;
     L.wave = S->wave;
     L.w_row = S->w_row;
@@ -169,8 +170,8 @@ constexpr double kAutoGrowthPerStep = 2.5e-5;
 // waits only for the warps it depends on, so that no launch boundary or block
 // barrier separates the steps.  Measured: FP32 25601 x 64, 15.7 us per step in
 // sweeps of four, 16.6 in pairs, 18.3 with a launch per pair; FP64 1601 x 32,
-// 6.5 against 14.5 us with a launch per step; FP64 25601 x 32 / 64 / 128, 73.3
-// / 146.9 / 287.0 against 79.0 / 150.3 / 297.4 us.  A grid whose blocks cannot
+// 6.2 against 8.6 us with a launch per step; FP64 25601 x 32 / 64 / 128, 44.3
+// / 89.3 / 185.2 against 49.4 / 93.9 / 189.9 us.  A grid whose blocks cannot
 // all be resident at once falls back to one launch per step (2 for FP32).
 static void set_launch_mode(tk_solver *S, int mode)
 {
@@ -234,7 +235,7 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     // two-step (ring) kernel's, both one wave of resident blocks
     S->persist_blocks = (precision == TK_PREC_F32)
                             ? S->fused_blocks
-                            : tk::persistent_grid_blocks(precision, S->K, Nr, S->num_sms, S->warps);
+                            : tk::persistent_grid_blocks(S->K, Nr, S->num_sms, S->warps);
     S->multi_blocks = tk::multi_grid_shape(precision, S->K, Nr, S->num_sms, &S->multi_warps);
     set_launch_mode(S, 0);
 
@@ -244,6 +245,8 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     if (st == TK_OK) st = alloc(S, &S->u[1], se * S->esz);
     if (st == TK_OK) st = alloc(S, &S->half, (size_t)Nr * tk::kNCH * S->NP * S->esz);
     if (st == TK_OK) st = alloc(S, &S->node, (size_t)Nr * tk::kNCN * S->NP * S->esz);
+    if (st == TK_OK && precision == TK_PREC_F64)
+        st = alloc(S, (void **)&S->step, (size_t)Nr * S->K * tk::kStepBytes);
     if (st == TK_OK && precision == TK_PREC_F32)
         st = alloc(S, (void **)&S->cmp, (size_t)Nr * tk::kNCC * S->NP * sizeof(float));
     if (st == TK_OK && precision == TK_PREC_F32)
@@ -293,7 +296,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
     TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                        S->dt / S->substeps, S->x_node, S->x_half, S->ang,
                                        S->precision, S->half, S->node, S->b_node, S->w_row,
-                                       S->cmp, S->gpm, S->stream));
+                                       S->cmp, S->gpm, S->stream, nullptr, nullptr, false, S->step));
     S->have_coeffs = true;
     S->have_state = false;
     S->epoch++;   // the tables' time step may have changed: recapture graphs
@@ -312,7 +315,8 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
             TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                                S->dt / S->substeps, S->x_node, S->x_half, S->ang,
                                                S->precision, S->half, S->node, S->b_node,
-                                               S->w_row, S->cmp, S->gpm, S->stream));
+                                               S->w_row, S->cmp, S->gpm, S->stream, nullptr, nullptr,
+                                               false, S->step));
         }
     }
     return TK_OK;
@@ -365,7 +369,7 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
     if (e == cudaSuccess)
         e = tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs, S->dt / S->substeps,
                                     S->x_node, S->x_half, S->ang, S->precision, S->half, S->node, S->b_node,
-                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, ang_given);
+                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, ang_given, S->step);
     if (e == cudaSuccess && dev) e = cudaStreamSynchronize(S->stream);
     if (dev) cudaFree(dev);
     if (e != cudaSuccess) return fail(S, TK_ERR_CUDA, "tk_set_coefficients: %s", cudaGetErrorString(e));
@@ -620,8 +624,9 @@ tk_status tk_step(tk_solver *S, int n)
     if (S->persist && (long long)n * S->substeps >= 2) {
         // every inner step of the call in one cooperative launch; its waits
         // are bounded, and a wait that timed out is reported here
-        // the one-step sweep keeps two flags per block (its first and last warp)
-        const int nflags = 2 * S->persist_blocks > S->multi_blocks ? 2 * S->persist_blocks : S->multi_blocks;
+        // the one-step sweep keeps two flags per block and 32 rows (its first and last team)
+        const int pf = (S->precision == TK_PREC_F64 ? 2 * S->K : 1) * S->persist_blocks;
+        const int nflags = pf > S->multi_blocks ? pf : S->multi_blocks;
         const size_t fbytes = (size_t)nflags * sizeof(unsigned int) + sizeof(int);
         if (!S->pflags) {
             st = alloc(S, (void **)&S->pflags, fbytes);

@@ -7,12 +7,13 @@
 // share the outer step dt.  One outer step is kmax = lcm(k_i) ticks; member i
 // steps on ticks t with (t + 1) % (kmax / k_i) == 0 and writes its waveform
 // sample on the last tick.  Each tick is one launch of a persistent kernel:
-// warps take work items (member, column range) from a queue in device memory
-// until it is empty; items are ordered by decreasing cost (columns x rows),
-// so the longest ones start first.  A warp recomputes the half-step value at
-// the left edge of its item, so items are independent; the arithmetic of
-// every half node and node is the same code as the single-solver kernel, and
-// the results are bit-identical to stepping each solver alone.
+// its warps (FP64: its blocks, whose teams share an item's columns) take work
+// items (member, column range) from a queue in device memory until it is empty;
+// items are ordered by decreasing cost (columns x rows), so the longest ones
+// start first.  The half-step value at the left edge of a range is recomputed,
+// so items are independent; the arithmetic of every half node and node is the
+// same code as the single-solver kernel, and the results are bit-identical to
+// stepping each solver alone.
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -22,6 +23,7 @@
 #include <vector>
 
 #include "tk_solver_impl.h"
+#include "tk_split.cuh"
 #include "tk_stencil.cuh"
 
 namespace tk {
@@ -32,6 +34,7 @@ constexpr int kBatchThreads = 128;
 struct BatchMember {
     void *u0, *u1;            // the member's two time levels
     const void *half, *node;  // folded coefficient tables
+    const unsigned char *step;   // FP64: the step's tables
     int Nr, K;
     int substeps, ratio;      // k_i and kmax / k_i
     int level0;               // level holding the state when the call started
@@ -92,22 +95,58 @@ __device__ void sweep(const BatchMember &m, const T *__restrict__ u_in, T *__res
     }
 }
 
+// The block's share of an FP64 item: its teams take equal parts of the columns.
+template <int K>
+__device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long long *bar, SplitRows *rows,
+                            SplitRingState &st, const double *__restrict__ u_in, double *__restrict__ u_out,
+                            int i0, int i1, bool observe_now)
+{
+    constexpr int TEAMS = kBatchThreads / 32 / K, NP = 32 * K;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
+    SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
+    const SplitSweep<K> sw{ring + wib, bar, m.step + team.h * kStepBytes, (const double *)m.half,
+                           (const double *)m.node, m.Nr, m.en, nullptr};
+    const int a = i0 + t * (i1 - i0) / TEAMS, b = i0 + (t + 1) * (i1 - i0) / TEAMS;
+    if (b <= a) return;
+    sw.run(st, team, u_in, a, b, false, [] {}, [&](int i, const double (&o)[4]) {
+        double *p = u_out + (size_t)i * (4 * NP) + 32 * team.h + lane;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[k * NP] = o[k];
+        if (observe_now) observe_team<K>(i, o, team, m.obs, m.wave, m.cap, m.sample, m.w_row, 0);
+    });
+}
+
 // One tick for every participating member.  ctr[0]: next work item, ctr[1]:
 // blocks finished.  The last block to finish empties the queue for the next
 // launch and, after the last tick of an outer step, moves every member's
 // sample counter on (every block has read them by then).
 template <typename T>
-__global__ void __launch_bounds__(kBatchThreads)
+__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 4 : 1)
 batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem *__restrict__ items,
                   int nitems, int tick, int kmax, int outer, unsigned int *ctr)
 {
     chain_start();   // the queue counters and the members' levels are the previous tick's
     const int lane = threadIdx.x & 31;
     const bool last_tick = (tick == kmax - 1);
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int WARPS = F64 ? kBatchThreads / 32 : 1;
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    __shared__ unsigned long long bars[WARPS][2];
+    __shared__ SplitRows rows[WARPS];
+    __shared__ int next;
+    SplitRingState st;
+    if constexpr (F64) split_ring_init(bars[threadIdx.x >> 5], lane);
     for (;;) {
         int it = 0;
-        if (lane == 0) it = (int)atomicAdd(&ctr[0], 1u);
-        it = __shfl_sync(kFull, it, 0);
+        if constexpr (F64) {   // one item per block
+            __syncthreads();
+            if (threadIdx.x == 0) next = (int)atomicAdd(&ctr[0], 1u);
+            __syncthreads();
+            it = next;
+        } else {
+            if (lane == 0) it = (int)atomicAdd(&ctr[0], 1u);
+            it = __shfl_sync(kFull, it, 0);
+        }
         if (it >= nitems) break;
         const BatchItem w = items[it];
         const BatchMember &m = mem[w.member];
@@ -116,10 +155,20 @@ batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem
         const T *u_in = (const T *)(lev ? m.u1 : m.u0);
         T *u_out = (T *)(lev ? m.u0 : m.u1);
         const bool obs_now = last_tick && m.obs.n > 0;
-        switch (m.K) {
-        case 1: sweep<T, 1>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
-        case 2: sweep<T, 2>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
-        default: sweep<T, 4>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
+        if constexpr (F64) {
+            SplitRing *ring = reinterpret_cast<SplitRing *>(sh_raw);
+            unsigned long long *bar = bars[threadIdx.x >> 5];
+            switch (m.K) {
+            case 1: sweep_teams<1>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
+            case 2: sweep_teams<2>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
+            default: sweep_teams<4>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
+            }
+        } else {
+            switch (m.K) {
+            case 1: sweep<T, 1>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
+            case 2: sweep<T, 2>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
+            default: sweep<T, 4>(m, u_in, u_out, w.i0, w.i1, obs_now, lane); break;
+            }
         }
     }
     __syncthreads();
@@ -139,12 +188,22 @@ batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem
 
 }  // namespace
 
+// Shared memory of the FP64 kernel's table rings.
+constexpr size_t kBatchSmem = kBatchThreads / 32 * sizeof(SplitRing);
+
 static int batch_resident_blocks(int precision)
 {
     int n = 0;
-    cudaError_t e = precision == 0
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<double>, kBatchThreads, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<float>, kBatchThreads, 0);
+    cudaError_t e = cudaSuccess;
+    if (precision == 0) {
+        e = cudaFuncSetAttribute(batch_step_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kBatchSmem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<double>, kBatchThreads,
+                                                              kBatchSmem);
+    } else {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<float>, kBatchThreads, 0);
+    }
     return (e != cudaSuccess || n < 1) ? 1 : n;
 }
 
@@ -153,7 +212,7 @@ static cudaError_t launch_batch_tick(int precision, int blocks, const BatchMembe
                                      int outer, unsigned int *ctr, cudaStream_t st)
 {
     if (precision == 0)
-        return launch_chained(batch_step_kernel<double>, (unsigned)blocks, kBatchThreads, 0, st, mem,
+        return launch_chained(batch_step_kernel<double>, (unsigned)blocks, kBatchThreads, kBatchSmem, st, mem,
                               nmem, items, nitems, tick, kmax, outer, ctr);
     return launch_chained(batch_step_kernel<float>, (unsigned)blocks, kBatchThreads, 0, st, mem, nmem,
                           items, nitems, tick, kmax, outer, ctr);
@@ -277,6 +336,7 @@ tk_status upload_members(tk_batch *B)
         tk::StepLaunch L;
         tkh::fill_launch(S, L);
         m.obs = L.obs;
+        m.step = L.step;
     }
     TKB_CUDA(B, cudaMemcpyAsync(B->d_mem, h.data(), B->n * sizeof(tk::BatchMember),
                                 cudaMemcpyHostToDevice, B->stream));
@@ -377,9 +437,11 @@ tk_status tk_batch_create(tk_batch **out, tk_solver *const *members, int n)
         B->blocks = S0->num_sms * tk::batch_resident_blocks(B->precision);
         long long cols = 0;
         for (tk_solver *S : B->mem) cols += S->Nr;
-        // default: about four items per warp of the resident grid
-        const long long warps = (long long)B->blocks * (tk::kBatchThreads / 32);
-        int seg = (int)std::max(8LL, cols / std::max(1LL, 4 * warps));
+        // default: about four items per taker (FP64: a block, FP32: a warp) of
+        // the resident grid, but at least four columns per warp (FP32: eight),
+        // since every range's left half node is formed twice
+        const long long takers = (long long)B->blocks * (B->precision == 0 ? 1 : tk::kBatchThreads / 32);
+        int seg = (int)std::max(B->precision == 0 ? 16LL : 8LL, cols / std::max(1LL, 4 * takers));
         st = build_items(B, seg);
     }
     if (st != TK_OK) {

@@ -210,8 +210,41 @@ __device__ Raw raw_from(const double *__restrict__ r, int Nth, int Nr, int jp, i
     return c;
 }
 
+// The exponent of a class sum s: s < 2^result, kSplitAbsent for 0; sets *cold
+// for a sum that is not finite or too large for the split form.
+__device__ int class_exponent(double s, int *cold)
+{
+    if (s == 0.0) return kSplitAbsent;
+    const int e = ((__double2hiint(s) >> 20) & 0x7ff) - 1022;
+    if (!(e <= kSplitMaxClass)) {
+        *cold = 1;
+        return kSplitMaxClass;
+    }
+    return e;
+}
+
+// c 2^(62 - C) rounded to the nearest integer, as limbs; |c| < 2^C.
+__device__ int2 split_entry(double c, int C)
+{
+    const long long b = __double_as_longlong(c);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0) return make_int2(0, 0);
+    long long v = (b & 0xfffffffffffffll) | (1ll << 52);
+    const int up = e - 1075 + 62 - C;    // <= 9
+    if (up >= 0) v <<= up;
+    else v = up < -54 ? 0 : (v + (1ll << (-up - 1))) >> -up;
+    v |= 1;   // odd, so that the limbs of -c are those of c with the other sign
+    if (b < 0) v = -v;
+    const int l = (int)v;
+    return make_int2((int)((v - l) >> 32), l);
+}
+
+// One thread per point, a block holding all NP rows of its columns (blockDim.x
+// = NP): a column's flags in the step tables are over its rows.
+constexpr int kTableThreads = 256;
+
 template <typename T>
-__global__ void coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs,
+__global__ void __launch_bounds__(kTableThreads) coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs,
                                     double dt, const double *__restrict__ x_node,
                                     const double *__restrict__ x_half,
                                     const double *__restrict__ ang, T *__restrict__ half,
@@ -219,11 +252,17 @@ __global__ void coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int 
                                     double *__restrict__ w_row, float *__restrict__ cmp,
                                     float *__restrict__ gpm, F32Derive fd,
                                     const double *__restrict__ raw_node,
-                                    const double *__restrict__ raw_half)
+                                    const double *__restrict__ raw_half,
+                                    unsigned char *__restrict__ step)
 {
-    const int jp = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (jp >= NP || i >= Nr) return;
+    __shared__ int flags[kTableThreads / 32][2];   // per column: cold, has imaginary coefficients
+    const int jp = threadIdx.x;
+    const int i = blockIdx.x * blockDim.y + threadIdx.y;
+    if (step) {
+        const int k = threadIdx.y * blockDim.x + threadIdx.x;
+        if (k < kTableThreads / 32 * 2) (&flags[0][0])[k] = 0;
+        __syncthreads();
+    }
     const Geo P = geometry(KP);
     T *hcol = half + (size_t)i * kNCH * NP + jp;
     T *ncol = node + (size_t)i * kNCN * NP + jp;
@@ -236,7 +275,7 @@ __global__ void coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int 
     const double dth = M_PI / Nth;
     const double ith2 = 1.0 / (dth * dth), i2th = 1.0 / (2.0 * dth);
     const double p = (variable == 0 && (abs(P.m) & 1)) ? -1.0 : 1.0;   // ghost parity
-    if (jp < Nth) {
+    if (jp < Nth && i < Nr) {
         const double th = (jp + 0.5) * dth;
         if (i == 0 && w_row) w_row[jp] = (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
         // angular stencil A+ (row j+1), A- (row j-1); the centre gets -(A+ + A-)
@@ -325,6 +364,42 @@ __global__ void coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int 
     } else if (i == 0 && w_row) {
         w_row[jp] = 0.0;
     }
+    if (step) {
+        const double hd[kStepHalfF64] = {hv[H_HP], hv[H_HQ], hv[H_PAR], hv[H_PCR], hv[H_PI]};
+        const double hs[kSplitEntries] = {hv[H_FAR], hv[H_FCR], hv[H_KP], hv[H_KM], hv[H_FAI], hv[H_FCI]};
+        const double nd[kStepNodeF64] = {nv[N_B], nv[N_PPR], nv[N_PMR], nv[N_C2I]};
+        const double ns[kSplitEntries] = {nv[N_FMR], nv[N_FPR], nv[N_KP], nv[N_KM], nv[N_FMI], nv[N_FPI]};
+        int ex[2][2];
+        int cold = 0;
+        for (int w = 0; w < 2; ++w) {
+            const double *v = w ? ns : hs;
+            ex[w][0] = class_exponent((fabs(v[S_FA]) + fabs(v[S_FC])) + 2.0 * (fabs(v[S_KP]) + fabs(v[S_KM])), &cold);
+            ex[w][1] = class_exponent(fabs(v[S_GA]) + fabs(v[S_GC]), &cold);
+        }
+        // plain stores of the same value
+        if (cold) flags[threadIdx.y][0] = 1;
+        if (ex[0][1] != kSplitAbsent || ex[1][1] != kSplitAbsent || hv[H_PI] != 0.0 || nv[N_C2I] != 0.0)
+            flags[threadIdx.y][1] = 1;
+        __syncthreads();
+        if (i < Nr) {
+            const int lane = jp & 31;
+            unsigned char *block = step + ((size_t)i * (NP / 32) + jp / 32) * kStepBytes;
+            double *d = reinterpret_cast<double *>(block) + lane;
+            auto entries = [&](const double *v, const int (&e)[2]) {
+                for (int q = 0; q < kSplitEntries; ++q, d += 32)
+                    *reinterpret_cast<int2 *>(d) = flags[threadIdx.y][0] ? make_int2(0, 0)
+                                                                         : split_entry(v[q], e[q >= S_GA]);
+            };
+            for (int q = 0; q < kStepHalfF64; ++q, d += 32) *d = hd[q];
+            entries(hs, ex[0]);
+            for (int q = 0; q < kStepNodeF64; ++q, d += 32) *d = nd[q];
+            entries(ns, ex[1]);
+            int *x = reinterpret_cast<int *>(block + kStepExps);
+            for (int w = 0; w < 2; ++w) x[32 * w + lane] = (ex[w][0] & 0xffff) | (ex[w][1] << 16);
+            if (lane < 4) x[64 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
+        }
+    }
+    if (i >= Nr) return;
     if constexpr (sizeof(T) == 4) {
         // FP32: sixteen entries rounded from FP64, the other five derived from
         // them in FP32 exactly as the compact-table kernel derives them
@@ -475,7 +550,7 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
                                 const double *x_half, double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node, const double *raw_half,
-                                bool ang_given)
+                                bool ang_given, unsigned char *step)
 {
     const F32Derive fd = f32_derive(dt_inner);
     if (variable != 0 && !ang_given) {
@@ -483,18 +558,18 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    dim3 block(32, 8);
-    dim3 grid((NP + 31) / 32, (Nr + 7) / 8);
+    dim3 block(NP, kTableThreads / NP);
+    dim3 grid((Nr + block.y - 1) / block.y);
     if (precision == 0)
         coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
                                                              x_node, x_half, ang, (double *)half,
                                                              (double *)node, b_node, w_row, nullptr,
-                                                             nullptr, fd, raw_node, raw_half);
+                                                             nullptr, fd, raw_node, raw_half, step);
     else
         coeff_tables_kernel<float><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
                                                             x_node, x_half, ang, (float *)half,
                                                             (float *)node, b_node, w_row, cmp, gpm, fd,
-                                                            raw_node, raw_half);
+                                                            raw_node, raw_half, nullptr);
     return cudaGetLastError();
 }
 

@@ -72,6 +72,28 @@ inline F32Derive f32_derive(double dt_inner)
     return F32Derive{(float)(1.0 / e2), (float)(2.0 * e2), (float)(2.0 / e2)};
 }
 
+// The FP64 step's tables (tk_split.cuh), filled from the entries above: those
+// that stay FP64,
+//   half node: HP, HQ, PAR, PCR, PI      node: B, PPR, PMR, C2I
+// and the coupling of Phi to Pi as integers, six limb pairs,
+//   half node: FAR, FCR, KP, KM, FAI, FCI    node: FMR, FPR, KP, KM, FMI, FPI
+// One contiguous block of kStepBytes per column and 32 rows, step[i][row /
+// 32]: the half node's FP64 entries and limb pairs, then the node's, each
+// [entry][32] (8 bytes); [2][32] ints with the row's exponents of the two
+// integer classes of the half node and of the node (the low half bounds |FA| +
+// |FC| + 2 |KP| + 2 |KM|, the high half |GA| + |GC|); then two ints, cold and
+// has imaginary coefficients (over the whole column), and eight bytes of padding.
+enum { D_HP = 0, D_HQ, D_PAR, D_PCR, D_PI };
+enum { D_B = 0, D_PPR, D_PMR, D_C2I };
+constexpr int kStepHalfF64 = 5, kStepNodeF64 = 4;
+constexpr int kSplitEntries = 6;
+enum { S_FA = 0, S_FC, S_KP, S_KM, S_GA, S_GC };
+constexpr int kStepExps = (kStepHalfF64 + kStepNodeF64 + 2 * kSplitEntries) * 256;   // offset of the exponents
+constexpr int kStepBytes = kStepExps + 256 + 16;
+constexpr int kSplitAbsent = -20000;    // exponent of a class whose entries are all zero
+constexpr int kSplitMaxClass = 20;      // largest class exponent; larger tables are cold
+constexpr int kSplitMaxExp = 1900;      // columns with this exponent field or more are cold
+
 struct Kerr {
     double M, a;  // black-hole mass and spin
     int s, m;     // spin weight, azimuthal mode
@@ -109,13 +131,15 @@ cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int
 // factors gpm[2][NP] (gp, then gm); both may be NULL for FP64.  raw_node,
 // raw_half (device, [9][Ntheta][Nr], half node i at r*_{i+1/2}): coefficients
 // supplied by the caller instead of computed (x_node, x_half then unused);
-// ang_given: ang already holds the regularised stencil.
+// ang_given: ang already holds the regularised stencil.  step: the FP64
+// step's tables (NULL: not wanted).
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
                                 double drs, double dt_inner, const double *x_node,
                                 const double *x_half, double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node = nullptr,
-                                const double *raw_half = nullptr, bool ang_given = false);
+                                const double *raw_half = nullptr, bool ang_given = false,
+                                unsigned char *step = nullptr);
 
 // The raw coefficients of the precompute, [9][Ntheta][Nr] at nodes and half
 // nodes (device output buffers).
@@ -158,6 +182,7 @@ struct StepLaunch {
     const void *node;
     const float *cmp;     // FP32: compact tables [i][kNCC][jp] (the four-step sweep)
     const float *gpm;     // FP32: theta factors gp[NP], gm[NP]
+    const unsigned char *step;   // FP64: the step's tables
     // waveform (only on the last inner step of an outer step)
     int write_wave;
     const long long *sample_ctr;  // device: index of the sample the outer step writes
@@ -171,11 +196,11 @@ cudaError_t launch_lw_step(const StepLaunch &L, cudaStream_t st);
 // Launch shape of the step kernel for a grid: returns the number of blocks
 // and sets *warps to the warps per block.
 int step_grid_shape(int precision, int K, int Nr, int num_sms, int *warps);
-// Many steps in one cooperative launch (small grids): the grid size for it,
-// 0 if it cannot run; the launch itself (L.u_in holds u^n, u_other is the
+// Many FP64 steps in one cooperative launch: the grid size for it, 0 if it
+// cannot run; the launch itself (L.u_in holds u^n, u_other is the
 // second level; flags: one zeroed unsigned int per block; *err set on a wait
 // that timed out).
-int persistent_grid_blocks(int precision, int K, int Nr, int num_sms, int warps);
+int persistent_grid_blocks(int K, int Nr, int num_sms, int warps);
 // Diagnostic of the persistent launches' bounded neighbour wait (one-warp
 // blocks; flags: n_blocks zeroed unsigned ints).
 cudaError_t launch_wait_check(int n_blocks, int silent, long long max_spins, unsigned int *flags,

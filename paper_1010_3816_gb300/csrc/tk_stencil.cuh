@@ -115,6 +115,45 @@ __device__ __forceinline__ void load_col(const T *__restrict__ p, T (&u)[4][K])
     for (int c = 0; c < 4; ++c) ldk<T, K>(p + c * NP, u[c]);
 }
 
+// State loads of the one-step sweep: through L1 when the state is read-only
+// for the launch, from L2 (ld.global.cg) when other blocks of the same launch
+// have written it (the persistent kernel), so that no stale L1 line is read.
+template <typename T, int K, bool CG>
+__device__ __forceinline__ void load_state(const T *p, T (&u)[4][K])
+{
+    if constexpr (!CG) {
+        load_col<T, K>(p, u);
+    } else {
+        constexpr int NP = 32 * K;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const T *q = p + c * NP;
+            if constexpr (sizeof(T) == 8 && K == 1) {
+                u[c][0] = __ldcg(q);
+            } else if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                for (int t = 0; t < K; t += 2) {
+                    const double2 x = __ldcg(reinterpret_cast<const double2 *>(q + t));
+                    u[c][t] = x.x;
+                    u[c][t + 1] = x.y;
+                }
+            } else if constexpr (K == 1) {
+                u[c][0] = __ldcg(q);
+            } else if constexpr (K == 2) {
+                const float2 x = __ldcg(reinterpret_cast<const float2 *>(q));
+                u[c][0] = x.x;
+                u[c][1] = x.y;
+            } else {
+                const float4 x = __ldcg(reinterpret_cast<const float4 *>(q));
+                u[c][0] = x.x;
+                u[c][1] = x.y;
+                u[c][2] = x.z;
+                u[c][3] = x.w;
+            }
+        }
+    }
+}
+
 template <typename T, int K>
 __device__ __forceinline__ void store_col(T *__restrict__ p, const T (&u)[4][K])
 {
@@ -548,6 +587,57 @@ __device__ __forceinline__ void observe(int i, int lane, const T (&o)[4][K], con
         if (lane == 0) sample = *(volatile const long long *)sample_ctr + sample_offset;
         observe_one_at<T, K>(lane, k, slot, o[0], o[1], obs, wave, cap, w_row, sample);
     }
+}
+
+// Bulk copies (the TMA unit's cp.async.bulk) of a column's tables into a
+// warp's shared-memory ring: one thread issues the two copies of a column
+// (half-node and node tables, contiguous in global memory), which complete on
+// the mbarrier of their ring slot; the warp waits on that mbarrier's phase
+// before reading the slot.
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(unsigned long long *bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+
+__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+
+__device__ __forceinline__ void mbar_expect(unsigned long long *bar, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_fetch(void *dst, const void *src, unsigned bytes, unsigned long long *bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+__device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned parity)
+{
+    unsigned ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Polls of a ring slot's mbarrier before the wait gives up (each try_wait
+// itself suspends the warp for a while); a copy of valid memory completes
+// long before.
+constexpr long long kMaxMbarPolls = 1ll << 22;
+
+__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity)
+{
+    for (long long i = 0; i < kMaxMbarPolls; ++i)
+        if (mbar_test(bar, parity)) return true;
+    return false;
 }
 
 // Bounded waits of the persistent kernels.  A wait gives up after kMaxSpins

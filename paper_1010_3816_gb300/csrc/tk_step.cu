@@ -1,21 +1,23 @@
 // tk_step.cu -- the fused two-step Lax-Wendroff time step, Eqs. (lw1) and (lw2).
 //
-// One warp owns all theta rows of a range of r* columns ("segment") and walks
-// it from left to right.  Per column i it
+// One warp (FP64: a team of one to four warps, 32 theta rows each) owns all
+// theta rows of a range of r* columns ("segment") and walks it from left to
+// right.  Per column i it
 //   1. loads u^n_{i+1} (one coalesced vector load per plane),
 //   2. forms the half-step value u^{n+1/2}_{i+1/2} (Eq. lw1: the averaging of
 //      the paper's kernel_average1 plus the bracketed right-hand side), with
 //      the theta neighbours of the averaged Phi taken from the adjacent lanes
-//      by warp shuffles,
+//      (FP32: by warp shuffles, FP64: through shared memory),
 //   3. forms u^{n+1}_i from u^{n+1/2}_{i-1/2} (kept in registers from the
 //      previous column), u^{n+1/2}_{i+1/2} and u^n_i (Eq. lw2),
 //   4. stores u^{n+1}_i, zero on the two radial edges (Sec. 3.2), and
 //   5. on the last inner step of an outer step, writes the observer's partial
 //      bilinear sample when i is one of its two interpolation columns.
 // The half-step planes of the paper's OpenCL code never exist in memory.  The
-// theta-pole boundary conditions are folded into the coefficient tables, so
-// the arithmetic is branch-free: 28 FP64 (or FP32) operations per half node
-// and 28 per node.
+// theta-pole boundary conditions are folded into the coefficient tables.  FP32
+// takes 28 operations per half node and 28 per node; FP64 does part of them in
+// integers (tk_split.cuh).
+#include "tk_split.cuh"
 #include "tk_stencil.cuh"
 
 namespace tk {
@@ -56,56 +58,18 @@ __device__ __forceinline__ void advance_sample(const WaveArgs &wa, int samples =
 
 // Warps per block.  A "wide" launch runs one block per SM with the most warps
 // (a multiple of four) whose registers fit in the SM's register file at the
-// register count the kernel compiles to for that element type and K; a
-// "narrow" launch runs blocks of four warps, several per SM, for grids too
-// small to give every warp of a wide launch a column.
+// register count the kernel compiles to for that element type and K (FP64: 16
+// at 128 registers whatever K, whose rows are a team's); a "narrow" launch runs
+// blocks of four warps, several per SM, for grids too small to give every warp
+// (team) of a wide launch a column.
 template <typename T, int K>
 constexpr int wide_warps()
 {
-    return sizeof(T) == 8 ? (K == 1 ? 24 : K == 2 ? 16 : 8) : (K == 1 ? 32 : K == 2 ? 24 : 16);
+    return sizeof(T) == 8 ? 16 : (K == 1 ? 32 : K == 2 ? 24 : 16);
 }
 
-// State loads of the one-step sweep: through L1 when the state is read-only
-// for the launch, from L2 (ld.global.cg) when other blocks of the same launch
-// have written it (the persistent kernel), so that no stale L1 line is read.
-template <typename T, int K, bool CG>
-__device__ __forceinline__ void load_state(const T *p, T (&u)[4][K])
-{
-    if constexpr (!CG) {
-        load_col<T, K>(p, u);
-    } else {
-        constexpr int NP = 32 * K;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const T *q = p + c * NP;
-            if constexpr (sizeof(T) == 8 && K == 1) {
-                u[c][0] = __ldcg(q);
-            } else if constexpr (sizeof(T) == 8) {
-#pragma unroll
-                for (int t = 0; t < K; t += 2) {
-                    const double2 x = __ldcg(reinterpret_cast<const double2 *>(q + t));
-                    u[c][t] = x.x;
-                    u[c][t + 1] = x.y;
-                }
-            } else if constexpr (K == 1) {
-                u[c][0] = __ldcg(q);
-            } else if constexpr (K == 2) {
-                const float2 x = __ldcg(reinterpret_cast<const float2 *>(q));
-                u[c][0] = x.x;
-                u[c][1] = x.y;
-            } else {
-                const float4 x = __ldcg(reinterpret_cast<const float4 *>(q));
-                u[c][0] = x.x;
-                u[c][1] = x.y;
-                u[c][2] = x.z;
-                u[c][3] = x.w;
-            }
-        }
-    }
-}
-
-// One Lax-Wendroff step over the block's columns (the body of lw_step_kernel):
-// every warp walks its range, the first warp of the block recomputes its left
+// One FP32 Lax-Wendroff step over the block's columns (lw_step_kernel's body;
+// FP64's is SplitSweep): every warp walks its range, the first warp of the block recomputes its left
 // half node, the others receive it through shared memory after a block
 // barrier.  write: observe this step; sample_offset: samples after the
 // counter's value.
@@ -199,11 +163,34 @@ __device__ __forceinline__ void step_sweep(unsigned char *sh_raw, const T *__res
 template <typename T, int K, int W>
 __global__ void __launch_bounds__(W * 32, wide_warps<T, K>() / W)
 lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__restrict__ half,
-               const T *__restrict__ node, int Nr, T eh, T en, const WaveArgs wa)
+               const T *__restrict__ node, const unsigned char *__restrict__ step, int Nr, T eh, T en,
+               const WaveArgs wa)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     if (kUsePDL) chain_start();
-    step_sweep<T, K, W>(sh_raw, u_in, u_out, half, node, Nr, eh, en, wa, wa.write, 0);
+    if constexpr (sizeof(T) == 8) {
+        __shared__ unsigned long long bars[W][2];
+        __shared__ SplitRows rows[W];
+        const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
+        split_ring_init(bars[wib], lane);
+        SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
+        const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib],
+                               step + (wib % K) * kStepBytes, half, node, Nr, en, nullptr};
+        int i0, i1;
+        team_range<W, K>(Nr, t, &i0, &i1);
+        SplitRingState st;
+        if (i1 > i0)
+            sw.run(st, team, u_in, i0, i1, false, [] {}, [&](int i, const double (&o)[4]) {
+                double *p = u_out + (size_t)i * (4 * 32 * K) + 32 * team.h + lane;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) p[k * 32 * K] = o[k];
+                if (wa.write)
+                    observe_team<K>(i, o, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, 0);
+            });
+        sw.drain(st);
+    } else {
+        step_sweep<T, K, W>(sh_raw, u_in, u_out, half, node, Nr, eh, en, wa, wa.write, 0);
+    }
     if (wa.write) advance_sample(wa);
 }
 
@@ -239,186 +226,73 @@ __device__ __forceinline__ bool neighbour_barrier(unsigned int *flags, unsigned 
 }
 
 
-// One step of the persistent sweep with no block barrier: every warp waits
-// only for what it uses.  Counters (number of finished steps, or of steps
-// whose first phase is finished) per warp in shared memory, and per block
-// for its first and last warp in global memory (flags[b] and
-// flags[blocks + b]).  Step s of warp w:
-//   - first phase (every half node and node that involves only the block's
-//     columns, as in step_sweep): it reads the right sibling's first column
-//     and overwrites its own last half node, which the right sibling read in
-//     the last step, so it waits until that sibling has finished step s - 1;
-//     then it publishes that its first phase of step s is done;
-//   - the block's last warp waits until the right neighbouring block's first
-//     warp has finished step s - 1 (it reads that warp's column, and
-//     overwrites its own last column, which that warp read), then forms it;
-//   - the deferred first node: the block's first warp waits until the left
-//     neighbouring block's last warp has finished step s - 1 and forms its
-//     left half node from that warp's column; every other warp waits until
-//     its left sibling's first phase of step s is done and takes that
-//     sibling's last half node;
-//   - it publishes that it has finished step s.
-// Every wait is bounded; after one ran out every later wait returns at once.
-// Same arithmetic on the same operands as step_sweep.
-template <typename T, int K, int W>
-__device__ __forceinline__ void step_sweep_async(unsigned char *sh_raw, const T *__restrict__ u_in,
-                                                 T *__restrict__ u_out, const T *__restrict__ half,
-                                                 const T *__restrict__ node, int Nr, T en,
-                                                 const WaveArgs &wa, int write, int sample_offset,
-                                                 unsigned int *flags, unsigned int *first_done,
-                                                 unsigned int *step_done, unsigned int s, int *err)
-{
-    constexpr int NP = 32 * K;
-    constexpr size_t SP = 4 * NP, HP = (size_t)kNCH * NP, NQ = (size_t)kNCN * NP;
-    T(*sh)[3][4][NP] = reinterpret_cast<T(*)[3][4][NP]>(sh_raw);
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    int i0, i1, left;
-    warp_range<W>(Nr, wib, &i0, &i1, &left);
-    // The launch has at most Nr / W blocks, so every block has at least W
-    // columns and warp_range gives every warp at least one; a warp without
-    // one would never publish, and its left sibling's wait would run out.
-    if (i1 <= i0) return;
-    const int row = lane * K;
-    const bool lead = (left < 0);
-    const int b1 = (int)(((long long)(blockIdx.x + 1) * Nr) / gridDim.x);
-    const bool last = (i1 == b1);
-    const int iend = last ? i1 - 1 : i1;
-    const unsigned int nb = gridDim.x;
-    if (s > 0 && !last) warp_wait_cta(&step_done[wib + 1], s, err);
-    T ua[4][K], hm[4][K];
-    zero_col<T, K>(hm);
-    load_state<T, K, true>(u_in + (size_t)i0 * SP + row, ua);
-    for (int i = i0; i < iend; ++i) {
-        T uc[4][K], hp[4][K], o[4][K];
-        if (i + 1 < Nr) {
-            load_state<T, K, true>(u_in + (size_t)(i + 1) * SP + row, uc);
-            half_node<T, K>(ua, uc, half + (size_t)i * HP + row, hp);
-        } else {
-            zero_col<T, K>(uc);
-            zero_col<T, K>(hp);
-        }
-        if (i == i0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int t = 0; t < K; ++t) {
-                    sh[wib][1][c][row + t] = ua[c][t];
-                    sh[wib][2][c][row + t] = hp[c][t];
-                }
-        } else {
-            full_node<T, K>(hm, hp, ua, node + (size_t)i * NQ + row, en, o);
-            if (i == 0 || i == Nr - 1) zero_col<T, K>(o);
-            store_col<T, K>(u_out + (size_t)i * SP + row, o);
-            if (write) observe<T, K>(i, lane, o, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, sample_offset);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int t = 0; t < K; ++t) {
-                hm[c][t] = hp[c][t];
-                ua[c][t] = uc[c][t];
-            }
-    }
-    if (!last)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int t = 0; t < K; ++t) sh[wib][0][c][row + t] = hm[c][t];
-    warp_publish_cta(&first_done[wib], s + 1);
-    if (last) {
-        if (s > 0 && blockIdx.x + 1 < nb) warp_wait_flag(flags + blockIdx.x + 1, s, err);
-        const int i = i1 - 1;
-        T uc[4][K], hp[4][K];
-        if (i + 1 < Nr) {
-            load_state<T, K, true>(u_in + (size_t)(i + 1) * SP + row, uc);
-            half_node<T, K>(ua, uc, half + (size_t)i * HP + row, hp);
-        } else {
-            zero_col<T, K>(uc);
-            zero_col<T, K>(hp);
-        }
-        if (i == i0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int t = 0; t < K; ++t) {
-                    sh[wib][1][c][row + t] = ua[c][t];
-                    sh[wib][2][c][row + t] = hp[c][t];
-                }
-        } else {
-            T o[4][K];
-            full_node<T, K>(hm, hp, ua, node + (size_t)i * NQ + row, en, o);
-            if (i == 0 || i == Nr - 1) zero_col<T, K>(o);
-            store_col<T, K>(u_out + (size_t)i * SP + row, o);
-            if (write) observe<T, K>(i, lane, o, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, sample_offset);
-        }
-        __syncwarp();
-    }
-    {
-        T hl[4][K], uf[4][K], hf[4][K], o[4][K];
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int t = 0; t < K; ++t) {
-                uf[c][t] = sh[wib][1][c][row + t];
-                hf[c][t] = sh[wib][2][c][row + t];
-            }
-        if (lead) {
-            if (s > 0 && blockIdx.x > 0) warp_wait_flag(flags + nb + blockIdx.x - 1, s, err);
-            if (i0 > 0) {
-                T ul[4][K];
-                load_state<T, K, true>(u_in + (size_t)(i0 - 1) * SP + row, ul);
-                half_node<T, K>(ul, uf, half + (size_t)(i0 - 1) * HP + row, hl);
-            } else {
-                zero_col<T, K>(hl);
-            }
-        } else {
-            warp_wait_cta(&first_done[left], s + 1, err);
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int t = 0; t < K; ++t) hl[c][t] = sh[left][0][c][row + t];
-        }
-        full_node<T, K>(hl, hf, uf, node + (size_t)i0 * NQ + row, en, o);
-        if (i0 == 0 || i0 == Nr - 1) zero_col<T, K>(o);
-        store_col<T, K>(u_out + (size_t)i0 * SP + row, o);
-        if (write) observe<T, K>(i0, lane, o, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, sample_offset);
-    }
-    if (lead) warp_publish_gpu(flags + blockIdx.x, s + 1);
-    if (last) warp_publish_gpu(flags + nb + blockIdx.x, s + 1);
-    warp_publish_cta(&step_done[wib], s + 1);
-}
-
 // Every Lax-Wendroff step of a call in one launch (the FP64 default).  All
-// blocks are resident at once (cooperative launch).  There is no barrier between steps:
-// each warp waits only for the warps whose data it reads or overwrites -- its
-// two siblings in the block, and for a block's first and last warp the edge
-// warp of the neighbouring block -- through counters of finished steps
-// (step_sweep_async).  Every wait is bounded: after kMaxSpins polls the warp
-// sets *err, and from then on every wait returns at once, so this kernel runs
-// its remaining steps without waiting and the persistent kernels below leave
-// their loops (the state is then invalid and the host reports the error).
-// State loads go through L2 (other blocks write them).  u0 holds u^n at the start; the result
-// is in u0 or u1 by the parity of n_inner.
-template <typename T, int K, int W>
-__global__ void __launch_bounds__(W * 32, wide_warps<T, K>() / W)
-lw_persistent_kernel(T *u0, T *u1, const T *__restrict__ half, const T *__restrict__ node, int Nr,
-                     T en, const WaveArgs wa, int n_inner, int substeps, unsigned int *flags, int *err)
+// blocks are resident at once (cooperative launch).  There is no barrier between
+// steps: before step s a warp waits until the warps that hold its rows in the
+// two neighbouring teams (in the block, or across its edge) have finished step
+// s - 1, because it reads one column of each and overwrites the columns that
+// they read: for the left one before it starts, for the right one before it
+// reads that column.  The progress counters are in shared memory, for a block's
+// first and last team also in global memory (flags[b K + h] and flags[(blocks +
+// b) K + h] for the rows from 32 h).  Every wait is bounded: after kMaxSpins
+// polls the warp sets *err, and from then on every wait returns at once, so this
+// kernel runs its remaining steps without waiting and the persistent kernels
+// below leave their loops (the state is then invalid and the host reports the
+// error); the barriers of a team are outside this, all its warps run the same
+// loop.  State loads go through L2 (other blocks write them).  u0 holds u^n at
+// the start; the result is in u0 or u1 by the parity of n_inner.
+template <int K, int W>
+__global__ void __launch_bounds__(W * 32, wide_warps<double, K>() / W)
+lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, const double *__restrict__ node,
+                     const unsigned char *__restrict__ step, int Nr, double en, const WaveArgs wa, int n_inner,
+                     int substeps, unsigned int *flags, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
-    __shared__ unsigned int first_done[W], step_done[W];
-    if (threadIdx.x < W) {
-        first_done[threadIdx.x] = 0;
-        step_done[threadIdx.x] = 0;
-    }
+    __shared__ unsigned int step_done[W];
+    __shared__ unsigned long long bars[W][2];
+    __shared__ SplitRows rows[W];
+    constexpr int TEAMS = W / K;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K;
+    if (threadIdx.x < W) step_done[threadIdx.x] = 0;
+    split_ring_init(bars[wib], lane);
     __syncthreads();
+    const int nb = (int)gridDim.x, b = (int)blockIdx.x;
+    SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
+    const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib], step + h * kStepBytes, half,
+                           node, Nr, en, err};
+    // The launch has at most Nr / TEAMS blocks, so every team has a column; one
+    // without would never publish, and its neighbours' waits would run out.
+    int i0, i1;
+    team_range<W, K>(Nr, t, &i0, &i1);
+    SplitRingState st;
     for (int s = 0; s < n_inner; ++s) {
-        const T *in = (s & 1) ? u1 : u0;
-        T *out = (s & 1) ? u0 : u1;
+        const double *in = (s & 1) ? u1 : u0;
+        double *out = (s & 1) ? u0 : u1;
         const int write = wa.write && ((s + 1) % substeps == 0);
-        step_sweep_async<T, K, W>(sh_raw, in, out, half, node, Nr, en, wa, write, (s + 1) / substeps - 1, flags,
-                                  first_done, step_done, (unsigned)s, err);
+        if (s > 0) {
+            if (t > 0) warp_wait_cta(&step_done[wib - K], s, err);
+            else if (b > 0) warp_wait_flag(flags + (nb + b - 1) * K + h, s, err);
+        }
+        sw.run(
+            st, team, in, i0, i1, s + 1 < n_inner,
+            [&] {
+                if (s == 0) return;
+                if (t + 1 < TEAMS) warp_wait_cta(&step_done[wib + K], s, err);
+                else if (b + 1 < nb) warp_wait_flag(flags + (b + 1) * K + h, s, err);
+            },
+            [&](int i, const double (&o)[4]) {
+                double *p = out + (size_t)i * (4 * 32 * K) + 32 * h + lane;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) p[k * 32 * K] = o[k];
+                if (write)
+                    observe_team<K>(i, o, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row,
+                                    (s + 1) / substeps - 1);
+            });
+        if (t == 0) warp_publish_gpu(flags + b * K + h, s + 1);
+        if (t == TEAMS - 1) warp_publish_gpu(flags + (nb + b) * K + h, s + 1);
+        warp_publish_cta(&step_done[wib], s + 1);
     }
+    sw.drain(st);
     if (wa.write) advance_sample(wa, n_inner / substeps);
 }
 
@@ -445,10 +319,11 @@ __global__ void wait_check_kernel(unsigned int *flags, int *err, int silent, lon
 }
 
 // Two Lax-Wendroff steps per launch, u^n -> u^{n+2}, for the HBM-bound
-// precision: state and tables cross DRAM once per two steps.  A warp owns the
-// output columns [i0, i1) of the same split as the one-step kernel and
+// precision (lw_step2_ring_kernel below; this FP64 form, a team of warps per
+// column as in the one-step kernel, runs on request): state and tables cross
+// DRAM once per two steps.  A team owns the output columns [i0, i1) of the same split as the one-step kernel and
 // recomputes the intermediate level u^{n+1} on [i0 - 1, i1], one column
-// beyond each end, so warps need nothing from each other.  It loads u^n_p for
+// beyond each end, so teams need nothing from each other.  It loads u^n_p for
 // p = i0 - 2 .. i1 + 1 and runs four lagged stages per p: the level-1 half
 // node p - 1/2, the level-1 node p - 1, the level-2 half node p - 3/2 and the
 // level-2 node p - 2.  The tables of a column are read twice, one column
@@ -459,71 +334,93 @@ __global__ void wait_check_kernel(unsigned int *flags, int *err, int silent, lon
 template <typename T, int K>
 constexpr int fused_warps()
 {
-    return sizeof(T) == 8 ? (K == 1 ? 20 : K == 2 ? 8 : 4) : (K == 1 ? 32 : K == 2 ? 16 : 8);
+    return sizeof(T) == 8 ? 12 : (K == 1 ? 32 : K == 2 ? 16 : 8);
 }
 
-template <typename T, int K, int W>
-__global__ void __launch_bounds__(W * 32, fused_warps<T, K>() / W)
-lw_step2_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__restrict__ half,
-                const T *__restrict__ node, int Nr, T eh, T en, const WaveArgs wa, int obs_mask)
+template <int K, int W>
+__global__ void __launch_bounds__(W * 32, fused_warps<double, K>() / W)
+lw_step2_kernel(const double *__restrict__ u_in, double *__restrict__ u_out, const double *__restrict__ half,
+                const double *__restrict__ node, const unsigned char *__restrict__ step, int Nr, double en,
+                const WaveArgs wa, int obs_mask)
 {
     constexpr int NP = 32 * K;
-    constexpr size_t SP = 4 * NP, HP = (size_t)kNCH * NP, NQ = (size_t)kNCN * NP;
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    int i0, i1, left;
-    warp_range<W>(Nr, wib, &i0, &i1, &left);
-    const int row = lane * K;
+    __shared__ SplitRows rows[W];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
+    SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
+    const int row = 32 * team.h + lane;
+    int i0, i1;
+    team_range<W, K>(Nr, t, &i0, &i1);
     const int second = obs_mask & 1;   // sample offset of the level-2 observation
+    const FmaK<double> k1 = fma_k<double>();
+    auto clear = [](double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = 0.0;
+    };
+    // the half node between columns i and i + 1, the node i, their tables read from global memory
+    auto block = [&](int i) { return step + ((size_t)i * K + team.h) * kStepBytes; };
+    auto half_at = [&](int i, const double (&x)[4], const SplitPhi &px, const double (&y)[4], const SplitPhi &py,
+                       double (&o)[4]) {
+        split_half_node<K>(x, px, y, py, block(i), team, half + (size_t)i * (kNCH * NP) + row, k1, o);
+    };
+    auto node_at = [&](int i, const double (&m)[4], const double (&p)[4], const double (&u)[4], double (&o)[4]) {
+        SplitPhi pm, pp;
+        split_phi(m, pm);
+        split_phi(p, pp);
+        split_full_node<K>(m, pm, p, pp, u, block(i), team, node + (size_t)i * (kNCN * NP) + row, en, k1, o);
+    };
     if (i1 > i0) {
-        T a0[4][K], h1m[4][K], u1m[4][K], h2m[4][K];
-        zero_col<T, K>(a0);
-        zero_col<T, K>(h1m);
-        zero_col<T, K>(u1m);
-        zero_col<T, K>(h2m);
+        double a0[4], h1m[4], u1m[4], h2m[4];
+        SplitPhi pa, p1;    // the integers of a0 and u1m
+        clear(a0);
+        clear(h1m);
+        clear(u1m);
+        clear(h2m);
+        split_phi(a0, pa);
+        p1 = pa;
+#pragma unroll 1
         for (int p = i0 - 2; p <= i1 + 1; ++p) {
-            T c0[4][K], h1p[4][K], u1c[4][K], h2p[4][K];
-            if (p >= 0 && p < Nr) load_col<T, K>(u_in + (size_t)p * SP + row, c0);
-            else zero_col<T, K>(c0);
+            double c0[4], h1p[4], u1c[4], h2p[4];
+            SplitPhi pc, pc1;
+            if (p >= 0 && p < Nr) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) c0[k] = u_in[(size_t)p * (4 * NP) + k * NP + row];
+            } else {
+                clear(c0);
+            }
+            split_phi(c0, pc);
             // level 1, half node between p - 1 and p
-            if (p >= i0 - 1 && p >= 1 && p < Nr)
-                half_node<T, K>(a0, c0, half + (size_t)(p - 1) * HP + row, h1p);
-            else
-                zero_col<T, K>(h1p);
+            if (p >= i0 - 1 && p >= 1 && p < Nr) half_at(p - 1, a0, pa, c0, pc, h1p);
+            else clear(h1p);
             // level 1, node q = p - 1 (zero on the radial edges and outside the grid)
             const int q = p - 1;
-            if (p >= i0 && q >= 1 && q <= Nr - 2)
-                full_node<T, K>(h1m, h1p, a0, node + (size_t)q * NQ + row, en, u1c);
-            else
-                zero_col<T, K>(u1c);
+            if (p >= i0 && q >= 1 && q <= Nr - 2) node_at(q, h1m, h1p, a0, u1c);
+            else clear(u1c);
             if ((obs_mask & 1) && q >= i0 && q < i1)
-                observe<T, K>(q, lane, u1c, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, 0);
+                observe_team<K>(q, u1c, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, 0);
             // level 2, half node between r = p - 2 and p - 1
             const int r = p - 2;
-            if (p >= i0 + 1 && r >= 0 && r + 1 < Nr)
-                half_node<T, K>(u1m, u1c, half + (size_t)r * HP + row, h2p);
-            else
-                zero_col<T, K>(h2p);
+            split_phi(u1c, pc1);
+            if (p >= i0 + 1 && r >= 0 && r + 1 < Nr) half_at(r, u1m, p1, u1c, pc1, h2p);
+            else clear(h2p);
             // level 2, node r
             if (p >= i0 + 2) {
-                T o[4][K];
-                if (r >= 1 && r <= Nr - 2)
-                    full_node<T, K>(h2m, h2p, u1m, node + (size_t)r * NQ + row, en, o);
-                else
-                    zero_col<T, K>(o);
-                store_col<T, K>(u_out + (size_t)r * SP + row, o);
+                double o[4];
+                if (r >= 1 && r <= Nr - 2) node_at(r, h2m, h2p, u1m, o);
+                else clear(o);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) u_out[(size_t)r * (4 * NP) + k * NP + row] = o[k];
                 if (obs_mask & 2)
-                    observe<T, K>(r, lane, o, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, second);
+                    observe_team<K>(r, o, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, second);
             }
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int t = 0; t < K; ++t) {
-                    a0[c][t] = c0[c][t];
-                    h1m[c][t] = h1p[c][t];
-                    u1m[c][t] = u1c[c][t];
-                    h2m[c][t] = h2p[c][t];
-                }
+            for (int c = 0; c < 4; ++c) {
+                a0[c] = c0[c];
+                h1m[c] = h1p[c];
+                u1m[c] = u1c[c];
+                h2m[c] = h2p[c];
+            }
+            pa = pc;
+            p1 = pc1;
         }
     }
     if (obs_mask) advance_sample(wa, (obs_mask & 1) + ((obs_mask >> 1) & 1));
@@ -568,57 +465,6 @@ __device__ __forceinline__ void cp_async(void *smem, const void *gmem)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
-// Bulk copies (the TMA unit's cp.async.bulk) of a column's tables into a
-// warp's shared-memory ring: one thread issues the two copies of a column
-// (half-node and node tables, contiguous in global memory), which complete on
-// the mbarrier of their ring slot; the warp waits on that mbarrier's phase
-// before reading the slot.
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_expect(unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_fetch(void *dst, const void *src, unsigned bytes, unsigned long long *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned parity)
-{
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Polls of a ring slot's mbarrier before the wait gives up (each try_wait
-// itself suspends the warp for a while); a copy of valid memory completes
-// long before.
-constexpr long long kMaxMbarPolls = 1ll << 22;
-
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity)
-{
-    for (long long i = 0; i < kMaxMbarPolls; ++i)
-        if (mbar_test(bar, parity)) return true;
-    return false;
-}
 
 // The ring's per-warp state across sweeps: the slot of the next copy (also
 // the slot the next wait is for), and per slot the parity of the next phase
@@ -1084,7 +930,7 @@ lw_multi_persistent_kernel(T *u0, T *u1, const float *__restrict__ cmp, const fl
 template <typename T, int K, int W>
 constexpr size_t step_smem_bytes()
 {
-    return (size_t)W * 3 * 4 * 32 * K * sizeof(T);
+    return sizeof(T) == 8 ? (size_t)W * sizeof(SplitRing) : (size_t)W * 3 * 4 * 32 * K * sizeof(T);
 }
 
 // Opt the kernel in to its dynamic shared memory once (above 48 KB).
@@ -1104,13 +950,13 @@ cudaError_t launch_shape(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
     if (e != cudaSuccess) return e;
     if (!kUsePDL) {
         lw_step_kernel<T, K, W><<<L.blocks, W * 32, step_smem_bytes<T, K, W>(), st>>>(
-            (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.Nr,
+            (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr,
             (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
         return cudaGetLastError();
     }
     return launch_chained(lw_step_kernel<T, K, W>, (unsigned)L.blocks, W * 32, step_smem_bytes<T, K, W>(),
                           st, (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node,
-                          L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
+                          L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
 }
 
 template <typename T, int K, int W>
@@ -1138,23 +984,23 @@ cudaError_t launch_ring(const StepLaunch &L, const WaveArgs &wa, T eh, T en, int
 template <typename T, int K>
 cudaError_t launch_fused(const StepLaunch &L, const WaveArgs &wa, cudaStream_t st)
 {
-    const T eh = (T)(0.25 * L.dt_inner), en = (T)(0.5 * L.dt_inner);
+    const T en = (T)(0.5 * L.dt_inner);
     const int mask = L.write_wave ? L.obs_mask : 0;
     if constexpr (sizeof(T) == 4) {
         constexpr int WR = ring_warps<T, K>();
-        if (L.warps == WR) return launch_ring<T, K, WR>(L, wa, eh, en, mask, st);
-        if (L.warps == kNarrowWarps) return launch_ring<T, K, kNarrowWarps>(L, wa, eh, en, mask, st);
+        if (L.warps == WR) return launch_ring<T, K, WR>(L, wa, (T)(0.25 * L.dt_inner), en, mask, st);
+        if (L.warps == kNarrowWarps) return launch_ring<T, K, kNarrowWarps>(L, wa, (T)(0.25 * L.dt_inner), en, mask, st);
         return cudaErrorInvalidValue;
     } else {
         constexpr int WF = fused_warps<T, K>();
         if (L.warps == WF)
-            lw_step2_kernel<T, K, WF><<<L.blocks, WF * 32, 0, st>>>(
-                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.Nr, eh, en,
-                wa, mask);
+            lw_step2_kernel<K, WF><<<L.blocks, WF * 32, 0, st>>>(
+                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr, en, wa,
+                mask);
         else if (L.warps == kNarrowWarps)
-            lw_step2_kernel<T, K, kNarrowWarps><<<L.blocks, kNarrowWarps * 32, 0, st>>>(
-                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.Nr, eh, en,
-                wa, mask);
+            lw_step2_kernel<K, kNarrowWarps><<<L.blocks, kNarrowWarps * 32, 0, st>>>(
+                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr, en, wa,
+                mask);
         else
             return cudaErrorInvalidValue;
         return cudaGetLastError();
@@ -1197,7 +1043,8 @@ int grid_shape(int Nr, int num_sms, int *warps)
     // one column per warp (on a small grid every warp's sweep is
     // latency-bound, and shorter sweeps finish sooner).
     constexpr int WW = wide_warps<T, K>();
-    if ((long long)Nr >= (long long)num_sms * WW && resident_blocks<T, K, WW>() >= 1) {
+    constexpr int KT = sizeof(T) == 8 ? K : 1;   // warps that share a column (FP64: a team)
+    if ((long long)Nr >= (long long)num_sms * (WW / KT) && resident_blocks<T, K, WW>() >= 1) {
         *warps = WW;
         return num_sms;
     }
@@ -1205,7 +1052,7 @@ int grid_shape(int Nr, int num_sms, int *warps)
     int per_sm = resident_blocks<T, K, kNarrowWarps>();
     if (per_sm < 1) per_sm = 1;
     int blocks = num_sms * per_sm;
-    if (blocks > Nr / kNarrowWarps) blocks = Nr / kNarrowWarps;
+    if (blocks > Nr / (kNarrowWarps / KT)) blocks = Nr / (kNarrowWarps / KT);
     return blocks < 1 ? 1 : blocks;
 }
 
@@ -1227,7 +1074,7 @@ int fused_shape(int Nr, int num_sms, int *warps)
                 &n, lw_step2_ring_kernel<T, K, kNarrowWarps>, kNarrowWarps * 32,
                 ring_smem_bytes<T, K>() / ring_warps<T, K>() * kNarrowWarps);
     } else {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_step2_kernel<T, K, kNarrowWarps>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_step2_kernel<K, kNarrowWarps>,
                                                           kNarrowWarps * 32, 0);
     }
     if (e != cudaSuccess || n < 1) n = 1;
@@ -1236,34 +1083,33 @@ int fused_shape(int Nr, int num_sms, int *warps)
     return blocks < 1 ? 1 : blocks;
 }
 
-template <typename T, int K, int W>
+template <int K, int W>
 int persistent_blocks_w(int Nr, int num_sms)
 {
     int n = 0;
-    if (step_smem_setup<T, K, W>() != cudaSuccess) return 0;
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_persistent_kernel<T, K, W>,
+    static cudaError_t e0 = cudaFuncSetAttribute(lw_persistent_kernel<K, W>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)step_smem_bytes<T, K, W>());
+                                                 (int)step_smem_bytes<double, K, W>());
     if (e0 != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_persistent_kernel<T, K, W>, W * 32,
-                                                      step_smem_bytes<T, K, W>()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_persistent_kernel<K, W>, W * 32,
+                                                      step_smem_bytes<double, K, W>()) != cudaSuccess ||
         n < 1)
         return 0;
     int blocks = num_sms * n;
-    if (blocks > Nr / W) blocks = Nr / W;
+    if (blocks > Nr / (W / K)) blocks = Nr / (W / K);
     return blocks < 1 ? 0 : blocks;
 }
 
-template <typename T, int K>
+template <int K>
 int persistent_blocks(int Nr, int num_sms, int warps)
 {
-    constexpr int WW = wide_warps<T, K>();
-    if (warps == WW) return persistent_blocks_w<T, K, WW>(Nr, num_sms);
-    if (warps == kNarrowWarps) return persistent_blocks_w<T, K, kNarrowWarps>(Nr, num_sms);
+    constexpr int WW = wide_warps<double, K>();
+    if (warps == WW) return persistent_blocks_w<K, WW>(Nr, num_sms);
+    if (warps == kNarrowWarps) return persistent_blocks_w<K, kNarrowWarps>(Nr, num_sms);
     return 0;
 }
 
-template <typename T, int K, int W>
+template <int K, int W>
 cudaError_t launch_persistent_w(const StepLaunch &L, void *u_other, int n_inner, int substeps,
                                 unsigned int *flags, int *err, cudaStream_t st)
 {
@@ -1275,24 +1121,24 @@ cudaError_t launch_persistent_w(const StepLaunch &L, void *u_other, int n_inner,
     wa.wave = L.wave;
     wa.w_row = L.w_row;
     wa.obs = L.obs;
-    T *u0 = (T *)L.u_in, *u1 = (T *)u_other;
-    const T *half = (const T *)L.half, *node = (const T *)L.node;
+    double *u0 = (double *)L.u_in, *u1 = (double *)u_other;
+    const double *half = (const double *)L.half, *node = (const double *)L.node;
+    const unsigned char *step = L.step;
     int Nr = L.Nr;
-    T en = (T)(0.5 * L.dt_inner);
-    void *args[] = {&u0, &u1, &half, &node, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err};
-    return cudaLaunchCooperativeKernel((const void *)lw_persistent_kernel<T, K, W>, dim3(L.blocks),
-                                       dim3(W * 32), args, step_smem_bytes<T, K, W>(), st);
+    double en = 0.5 * L.dt_inner;
+    void *args[] = {&u0, &u1, &half, &node, &step, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err};
+    return cudaLaunchCooperativeKernel((const void *)lw_persistent_kernel<K, W>, dim3(L.blocks), dim3(W * 32),
+                                       args, step_smem_bytes<double, K, W>(), st);
 }
 
-template <typename T, int K>
+template <int K>
 cudaError_t launch_persistent_typed(const StepLaunch &L, void *u_other, int n_inner, int substeps,
                                     unsigned int *flags, int *err, cudaStream_t st)
 {
-    constexpr int WW = wide_warps<T, K>();
-    if (L.warps == WW)
-        return launch_persistent_w<T, K, WW>(L, u_other, n_inner, substeps, flags, err, st);
+    constexpr int WW = wide_warps<double, K>();
+    if (L.warps == WW) return launch_persistent_w<K, WW>(L, u_other, n_inner, substeps, flags, err, st);
     if (L.warps == kNarrowWarps)
-        return launch_persistent_w<T, K, kNarrowWarps>(L, u_other, n_inner, substeps, flags, err, st);
+        return launch_persistent_w<K, kNarrowWarps>(L, u_other, n_inner, substeps, flags, err, st);
     return cudaErrorInvalidValue;
 }
 
@@ -1439,15 +1285,11 @@ cudaError_t launch_multi_persistent(const StepLaunch &L, void *u_other, int n_gr
     return cudaErrorInvalidValue;
 }
 
-int persistent_grid_blocks(int precision, int K, int Nr, int num_sms, int warps)
+int persistent_grid_blocks(int K, int Nr, int num_sms, int warps)
 {
-    if (precision == 0)
-        return K == 1 ? persistent_blocks<double, 1>(Nr, num_sms, warps)
-             : K == 2 ? persistent_blocks<double, 2>(Nr, num_sms, warps)
-                      : persistent_blocks<double, 4>(Nr, num_sms, warps);
-    return K == 1 ? persistent_blocks<float, 1>(Nr, num_sms, warps)
-         : K == 2 ? persistent_blocks<float, 2>(Nr, num_sms, warps)
-                  : persistent_blocks<float, 4>(Nr, num_sms, warps);
+    return K == 1 ? persistent_blocks<1>(Nr, num_sms, warps)
+         : K == 2 ? persistent_blocks<2>(Nr, num_sms, warps)
+                  : persistent_blocks<4>(Nr, num_sms, warps);
 }
 
 cudaError_t launch_wait_check(int n_blocks, int silent, long long max_spins, unsigned int *flags,
@@ -1461,14 +1303,10 @@ cudaError_t launch_wait_check(int n_blocks, int silent, long long max_spins, uns
 cudaError_t launch_lw_persistent(const StepLaunch &L, void *u_other, int n_inner, int substeps,
                                  unsigned int *flags, int *err, cudaStream_t st)
 {
-    if (L.precision == 0) {
-        if (L.K == 1) return launch_persistent_typed<double, 1>(L, u_other, n_inner, substeps, flags, err, st);
-        if (L.K == 2) return launch_persistent_typed<double, 2>(L, u_other, n_inner, substeps, flags, err, st);
-        return launch_persistent_typed<double, 4>(L, u_other, n_inner, substeps, flags, err, st);
-    }
-    if (L.K == 1) return launch_persistent_typed<float, 1>(L, u_other, n_inner, substeps, flags, err, st);
-    if (L.K == 2) return launch_persistent_typed<float, 2>(L, u_other, n_inner, substeps, flags, err, st);
-    return launch_persistent_typed<float, 4>(L, u_other, n_inner, substeps, flags, err, st);
+    if (L.precision != 0) return cudaErrorInvalidValue;
+    if (L.K == 1) return launch_persistent_typed<1>(L, u_other, n_inner, substeps, flags, err, st);
+    if (L.K == 2) return launch_persistent_typed<2>(L, u_other, n_inner, substeps, flags, err, st);
+    return launch_persistent_typed<4>(L, u_other, n_inner, substeps, flags, err, st);
 }
 
 int fused_grid_shape(int precision, int K, int Nr, int num_sms, int *warps)
