@@ -15,15 +15,17 @@
 // waveform sample of an outer step is linear in the state, so its loss
 // gradient enters as a source on the adjoint state of that step.
 //
-// A warp owns all theta rows of a range of output columns and walks it left
-// to right; the work split and the hand-off of the left-edge eta between the
-// warps of a block are those of the forward step kernel.
+// FP32: a warp owns all theta rows of a range of output columns and walks it
+// left to right; the left-edge eta is handed over between the warps of a block.
+// FP64: a team of warps does, as in the forward step, with the coupling of Pi
+// to Phi in integers (tk_split_adjoint.cuh).
 #include <math.h>
 #include <string.h>
 
 #include <vector>
 
 #include "tk_solver_impl.h"
+#include "tk_split_adjoint.cuh"
 #include "tk_stencil.cuh"
 
 namespace tk {
@@ -205,11 +207,11 @@ __device__ __forceinline__ void mu_node(const T (&l)[4][K], const T (&ep)[4][K],
 
 // Warps per block of the wide launch (one block per SM): the most warps, in
 // multiples of four, whose registers fit in the register file at the count
-// the kernel compiles to for this element type and K.
+// the kernel compiles to for this element type and K (FP64: 128 whatever K).
 template <typename T, int K>
 constexpr int adj_wide_warps()
 {
-    return sizeof(T) == 8 ? (K == 1 ? 24 : K == 2 ? 16 : 8) : (K == 1 ? 32 : K == 2 ? 24 : 12);
+    return sizeof(T) == 8 ? 16 : (K == 1 ? 32 : K == 2 ? 24 : 12);
 }
 
 // Shared memory per warp, in theta-columns of NP values: [0, 6) eta at the
@@ -328,10 +330,9 @@ lw_adjoint_kernel(const T *__restrict__ lam, T *__restrict__ mu_out, const T *__
     }
 }
 
-// Every adjoint step of a tk_adjoint call in one cooperative launch, with the
-// dataflow of the forward persistent sweep (step_sweep_async): no barrier
-// between steps; each warp waits (bounded) only for its two siblings and, at
-// a block's edges, the neighbouring block's edge warp.  Step s:
+// FP32: every adjoint step of a tk_adjoint call in one cooperative launch, no
+// barrier between steps; each warp waits (bounded) only for its two siblings and,
+// at a block's edges, the neighbouring block's edge warp.  Step s:
 //   - first phase (every half node and node that involves only the block's
 //     columns): it reads the right sibling's first column and overwrites its
 //     own last half node, which that sibling read in the last step, so it
@@ -483,7 +484,7 @@ __device__ __forceinline__ void adj_sweep_async(unsigned char *sh_raw, const T *
     warp_publish_cta(&step_done[wib], s + 1);
 }
 
-// Launch step s is the transpose of inner step n_inner - 1 - s: the gradient
+// (FP32) Launch step s is the transpose of inner step n_inner - 1 - s: the gradient
 // of sample count - 1 - s / substeps is injected at its first sub-step.  The
 // adjoint state starts in a0; the result is in a0 or a1 by the parity of
 // n_inner.
@@ -506,6 +507,124 @@ lw_adjoint_persistent_kernel(T *a0, T *a1, const T *__restrict__ half, const T *
         adj_sweep_async<T, K, W>(sh_raw, lam, mu, half, node, Nr, en, inj, inject && (s % substeps == 0),
                                  inj.count - 1 - s / substeps, flags, first_done, step_done, (unsigned)s, err);
     }
+}
+
+// ---- FP64: teams of warps and integer coupling (tk_split_adjoint.cuh) ----
+
+// load_lam for one row per lane.
+template <int K>
+__device__ __forceinline__ void load_lam_row(const double *__restrict__ lam, int i, int Nr, int row,
+                                             const InjectArgs &inj, int on, long long sample, double (&l)[4])
+{
+    constexpr int NP = 32 * K;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) l[c] = __ldcg(lam + (size_t)i * (4 * NP) + c * NP + row);
+    if (on) {
+        for (int k = 0; k < inj.obs.n; ++k) {
+            const int slot = (i == inj.obs.i0[k]) ? 0 : ((i == inj.obs.i0[k] + 1) ? 1 : -1);
+            if (slot < 0) continue;
+            const int j0 = inj.obs.j0[k];
+            const double wr = slot ? inj.obs.wr1[k] : inj.obs.wr0[k];
+            const double *g = inj.dwave + ((size_t)k * inj.count + sample) * 2;
+            double wt = 0.0;
+            if (row == j0) wt = wr * (1.0 - inj.obs.ft[k]) * inj.w_row[j0];
+            else if (row == j0 + 1) wt = wr * inj.obs.ft[k] * inj.w_row[j0 + 1];
+            if (wt != 0.0) {
+                l[0] += wt * g[0];
+                l[1] += wt * g[1];
+            }
+        }
+    }
+    if (i == 0 || i == Nr - 1)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) l[c] = 0.0;
+}
+
+template <int K>
+__device__ __forceinline__ void store_row(double *__restrict__ u, int i, int row, const double (&o)[4])
+{
+    constexpr int NP = 32 * K;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) u[(size_t)i * (4 * NP) + c * NP + row] = o[c];
+}
+
+template <int K, int W>
+__global__ void __launch_bounds__(W * 32, adj_wide_warps<double, K>() / W)
+lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_out, const double *__restrict__ half,
+                       const double *__restrict__ node, const unsigned char *__restrict__ tab, int Nr, double en,
+                       const InjectArgs inj)
+{
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    __shared__ unsigned long long bars[W][2];
+    __shared__ SplitRows rows[W];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
+    chain_start();   // lam is the previous launch's output
+    split_ring_init(bars[wib], lane);
+    SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
+    const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
+                         en, nullptr};
+    int i0, i1;
+    team_range<W, K>(Nr, t, &i0, &i1);
+    SplitRingState st;
+    if (i1 > i0)
+        sw.run(
+            st, team,
+            [&](int i, double (&l)[4]) { load_lam_row<K>(lam, i, Nr, row, inj, inj.on, inj.sample, l); }, i0, i1,
+            false, [] {}, [&](int i, const double (&o)[4]) { store_row<K>(mu_out, i, row, o); });
+    sw.drain(st);
+}
+
+// Every adjoint step of a tk_adjoint call in one cooperative launch, with the
+// waits of the forward persistent sweep (lw_persistent_kernel).  Launch step s
+// is the transpose of inner step n_inner - 1 - s, as in
+// lw_adjoint_persistent_kernel.
+template <int K, int W>
+__global__ void __launch_bounds__(W * 32, adj_wide_warps<double, K>() / W)
+lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restrict__ half,
+                                  const double *__restrict__ node, const unsigned char *__restrict__ tab, int Nr,
+                                  double en, const InjectArgs inj, int inject, long long n_inner, int substeps,
+                                  unsigned int *flags, int *err)
+{
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    __shared__ unsigned int step_done[W];
+    __shared__ unsigned long long bars[W][2];
+    __shared__ SplitRows rows[W];
+    constexpr int TEAMS = W / K;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
+    if (threadIdx.x < W) step_done[threadIdx.x] = 0;
+    split_ring_init(bars[wib], lane);
+    __syncthreads();
+    const int nb = (int)gridDim.x, b = (int)blockIdx.x;
+    SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
+    const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
+                         en, err};
+    int i0, i1;
+    team_range<W, K>(Nr, t, &i0, &i1);   // at most Nr / TEAMS blocks: every team has a column
+    SplitRingState st;
+    for (long long s = 0; s < n_inner; ++s) {
+        const double *lam = (s & 1) ? a1 : a0;
+        double *mu = (s & 1) ? a0 : a1;
+        const int on = inject && (s % substeps == 0);
+        const long long sample = inj.count - 1 - s / substeps;
+        const unsigned int e = (unsigned int)s;
+        if (s > 0) {
+            if (t > 0) warp_wait_cta(&step_done[wib - K], e, err);
+            else if (b > 0) warp_wait_flag(flags + (nb + b - 1) * K + h, e, err);
+        }
+        sw.run(
+            st, team, [&](int i, double (&l)[4]) { load_lam_row<K>(lam, i, Nr, row, inj, on, sample, l); }, i0, i1,
+            s + 1 < n_inner,
+            [&] {
+                if (s == 0) return;
+                if (t + 1 < TEAMS) warp_wait_cta(&step_done[wib + K], e, err);
+                else if (b + 1 < nb) warp_wait_flag(flags + (b + 1) * K + h, e, err);
+            },
+            [&](int i, const double (&o)[4]) { store_row<K>(mu, i, row, o); });
+        if (t == 0) warp_publish_gpu(flags + b * K + h, e + 1);
+        if (t == TEAMS - 1) warp_publish_gpu(flags + (nb + b) * K + h, e + 1);
+        warp_publish_cta(&step_done[wib], e + 1);
+    }
+    sw.drain(st);
 }
 
 // Transpose of the initial-data map of tk_set_initial_data: the adjoint state
@@ -680,70 +799,89 @@ cudaError_t launch_param_tangent(int K, int blocks, const double *u, const doubl
 template <typename T, int K, int W>
 constexpr size_t adj_smem_bytes()
 {
-    return (size_t)W * kAdjShared * 32 * K * sizeof(T);
+    return sizeof(T) == 8 ? (size_t)W * sizeof(AdjRing) : (size_t)W * kAdjShared * 32 * K * sizeof(T);
+}
+
+// The kernels of a precision: one launch per step, and every step in one.
+template <typename T, int K, int W>
+const void *adj_kernel()
+{
+    if constexpr (sizeof(T) == 8) return (const void *)lw_adjoint_team_kernel<K, W>;
+    else return (const void *)lw_adjoint_kernel<T, K, W>;
+}
+
+template <typename T, int K, int W>
+const void *adj_persistent_kernel()
+{
+    if constexpr (sizeof(T) == 8) return (const void *)lw_adjoint_team_persistent_kernel<K, W>;
+    else return (const void *)lw_adjoint_persistent_kernel<T, K, W>;
 }
 
 template <typename T, int K, int W>
 cudaError_t adj_smem_setup()
 {
-    static cudaError_t e = cudaFuncSetAttribute(lw_adjoint_kernel<T, K, W>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+    static cudaError_t e = cudaFuncSetAttribute(adj_kernel<T, K, W>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)adj_smem_bytes<T, K, W>());
     return e;
 }
 
 template <typename T, int K, int W>
-cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const void *node,
+cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab,
                              int Nr, int blocks, double dt_in, const InjectArgs &inj,
                              cudaStream_t st)
 {
     cudaError_t e = adj_smem_setup<T, K, W>();
     if (e != cudaSuccess) return e;
-    return launch_chained(lw_adjoint_kernel<T, K, W>, (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(),
-                          st, (const T *)lam, (T *)mu, (const T *)half, (const T *)node, Nr,
-                          (T)(0.25 * dt_in), (T)(0.5 * dt_in), inj);
+    if constexpr (sizeof(T) == 8)
+        return launch_chained(lw_adjoint_team_kernel<K, W>, (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st,
+                              (const double *)lam, (double *)mu, (const double *)half, (const double *)node, tab, Nr,
+                              0.5 * dt_in, inj);
+    else
+        return launch_chained(lw_adjoint_kernel<T, K, W>, (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(),
+                              st, (const T *)lam, (T *)mu, (const T *)half, (const T *)node, Nr,
+                              (T)(0.25 * dt_in), (T)(0.5 * dt_in), inj);
 }
 
 template <typename T, int K>
-cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *node, int Nr,
+cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab, int Nr,
                        int blocks, int warps, double dt_in, const InjectArgs &inj, cudaStream_t st)
 {
     constexpr int WW = adj_wide_warps<T, K>();
     if (warps == WW)
-        return launch_adj_shape<T, K, WW>(lam, mu, half, node, Nr, blocks, dt_in, inj, st);
+        return launch_adj_shape<T, K, WW>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, st);
     if (warps == kNarrowWarps)
-        return launch_adj_shape<T, K, kNarrowWarps>(lam, mu, half, node, Nr, blocks, dt_in, inj, st);
+        return launch_adj_shape<T, K, kNarrowWarps>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, st);
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_adjoint_step(int precision, int K, const void *lam, void *mu, const void *half,
-                                const void *node, int Nr, int blocks, int warps, double dt_in,
+                                const void *node, const unsigned char *tab, int Nr, int blocks, int warps, double dt_in,
                                 const InjectArgs &inj, cudaStream_t st)
 {
     if (precision == 0) {
-        if (K == 1) return launch_adj<double, 1>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
-        if (K == 2) return launch_adj<double, 2>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
-        return launch_adj<double, 4>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
+        if (K == 1) return launch_adj<double, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+        if (K == 2) return launch_adj<double, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+        return launch_adj<double, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
     }
-    if (K == 1) return launch_adj<float, 1>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
-    if (K == 2) return launch_adj<float, 2>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
-    return launch_adj<float, 4>(lam, mu, half, node, Nr, blocks, warps, dt_in, inj, st);
+    if (K == 1) return launch_adj<float, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+    if (K == 2) return launch_adj<float, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+    return launch_adj<float, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
 }
 
 template <typename T, int K, int W>
 int adj_persistent_blocks_w(int Nr, int num_sms)
 {
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_adjoint_persistent_kernel<T, K, W>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const void *kern = adj_persistent_kernel<T, K, W>();
+    static cudaError_t e0 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)adj_smem_bytes<T, K, W>());
     int n = 0;
     if (e0 != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_adjoint_persistent_kernel<T, K, W>, W * 32,
-                                                      adj_smem_bytes<T, K, W>()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, W * 32, adj_smem_bytes<T, K, W>()) != cudaSuccess ||
         n < 1)
         return 0;
+    constexpr int C = W / (sizeof(T) == 8 ? K : 1);   // columns at a time (FP64: teams)
     long long blocks = (long long)num_sms * n;
-    if (blocks > Nr / W) blocks = Nr / W;
+    if (blocks > Nr / C) blocks = Nr / C;
     return blocks < 1 ? 0 : (int)blocks;
 }
 
@@ -757,7 +895,8 @@ int adj_persistent_blocks_t(int Nr, int num_sms, int warps)
 }
 
 template <typename T, int K, int W>
-cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const void *node, int Nr, int blocks,
+cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const void *node,
+                                    const unsigned char *tab, int Nr, int blocks,
                                     double dt_in, const InjectArgs &inj, int inject, long long n_inner,
                                     int substeps, unsigned int *flags, int *err, cudaStream_t st)
 {
@@ -765,23 +904,25 @@ cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const 
     const T *h = (const T *)half, *nd = (const T *)node;
     T en = (T)(0.5 * dt_in);
     InjectArgs in = inj;
-    void *args[] = {&p0, &p1, &h, &nd, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
-    return cudaLaunchCooperativeKernel((const void *)lw_adjoint_persistent_kernel<T, K, W>, dim3(blocks),
-                                       dim3(W * 32), args, adj_smem_bytes<T, K, W>(), st);
+    void *args64[] = {&p0, &p1, &h, &nd, &tab, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
+    void *args32[] = {&p0, &p1, &h, &nd, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
+    return cudaLaunchCooperativeKernel(adj_persistent_kernel<T, K, W>(), dim3(blocks), dim3(W * 32),
+                                       sizeof(T) == 8 ? args64 : args32, adj_smem_bytes<T, K, W>(), st);
 }
 
 template <typename T, int K>
-cudaError_t launch_adj_persistent_t(void *a0, void *a1, const void *half, const void *node, int Nr, int blocks,
+cudaError_t launch_adj_persistent_t(void *a0, void *a1, const void *half, const void *node,
+                                    const unsigned char *tab, int Nr, int blocks,
                                     int warps, double dt_in, const InjectArgs &inj, int inject,
                                     long long n_inner, int substeps, unsigned int *flags, int *err,
                                     cudaStream_t st)
 {
     constexpr int WW = adj_wide_warps<T, K>();
     if (warps == WW)
-        return launch_adj_persistent_w<T, K, WW>(a0, a1, half, node, Nr, blocks, dt_in, inj, inject, n_inner,
+        return launch_adj_persistent_w<T, K, WW>(a0, a1, half, node, tab, Nr, blocks, dt_in, inj, inject, n_inner,
                                                  substeps, flags, err, st);
     if (warps == kNarrowWarps)
-        return launch_adj_persistent_w<T, K, kNarrowWarps>(a0, a1, half, node, Nr, blocks, dt_in, inj, inject,
+        return launch_adj_persistent_w<T, K, kNarrowWarps>(a0, a1, half, node, tab, Nr, blocks, dt_in, inj, inject,
                                                            n_inner, substeps, flags, err, st);
     return cudaErrorInvalidValue;
 }
@@ -800,27 +941,27 @@ int adjoint_persistent_blocks(int precision, int K, int Nr, int num_sms, int war
 }
 
 cudaError_t launch_adjoint_persistent(int precision, int K, void *a0, void *a1, const void *half,
-                                      const void *node, int Nr, int blocks, int warps, double dt_in,
+                                      const void *node, const unsigned char *tab, int Nr, int blocks, int warps, double dt_in,
                                       const InjectArgs &inj, int inject, long long n_inner, int substeps,
                                       unsigned int *flags, int *err, cudaStream_t st)
 {
     if (precision == 0) {
         if (K == 1)
-            return launch_adj_persistent_t<double, 1>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+            return launch_adj_persistent_t<double, 1>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                                       n_inner, substeps, flags, err, st);
         if (K == 2)
-            return launch_adj_persistent_t<double, 2>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+            return launch_adj_persistent_t<double, 2>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                                       n_inner, substeps, flags, err, st);
-        return launch_adj_persistent_t<double, 4>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+        return launch_adj_persistent_t<double, 4>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                                   n_inner, substeps, flags, err, st);
     }
     if (K == 1)
-        return launch_adj_persistent_t<float, 1>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+        return launch_adj_persistent_t<float, 1>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                                  n_inner, substeps, flags, err, st);
     if (K == 2)
-        return launch_adj_persistent_t<float, 2>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+        return launch_adj_persistent_t<float, 2>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                                  n_inner, substeps, flags, err, st);
-    return launch_adj_persistent_t<float, 4>(a0, a1, half, node, Nr, blocks, warps, dt_in, inj, inject,
+    return launch_adj_persistent_t<float, 4>(a0, a1, half, node, tab, Nr, blocks, warps, dt_in, inj, inject,
                                              n_inner, substeps, flags, err, st);
 }
 
@@ -829,7 +970,7 @@ int adj_resident()
 {
     int n = 0;
     if (adj_smem_setup<T, K, W>() != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_adjoint_kernel<T, K, W>, W * 32,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, adj_kernel<T, K, W>(), W * 32,
                                                       adj_smem_bytes<T, K, W>()) != cudaSuccess)
         n = 0;
     return n;
@@ -839,7 +980,8 @@ template <typename T, int K>
 int adj_shape(int Nr, int num_sms, int *warps)
 {
     constexpr int WW = adj_wide_warps<T, K>();
-    if ((long long)Nr >= (long long)num_sms * WW && adj_resident<T, K, WW>() >= 1) {
+    constexpr int KT = sizeof(T) == 8 ? K : 1;   // warps that share a column (FP64: a team)
+    if ((long long)Nr >= (long long)num_sms * (WW / KT) && adj_resident<T, K, WW>() >= 1) {
         *warps = WW;
         return num_sms;
     }
@@ -847,7 +989,7 @@ int adj_shape(int Nr, int num_sms, int *warps)
     int per_sm = adj_resident<T, K, kNarrowWarps>();
     if (per_sm < 1) per_sm = 1;
     int blocks = num_sms * per_sm;
-    if (blocks > Nr / kNarrowWarps) blocks = Nr / kNarrowWarps;
+    if (blocks > Nr / (kNarrowWarps / KT)) blocks = Nr / (kNarrowWarps / KT);
     return blocks < 1 ? 1 : blocks;
 }
 
@@ -865,6 +1007,22 @@ int adjoint_grid_shape(int precision, int K, int Nr, int num_sms, int *warps)
 }
 
 }  // namespace tk
+
+// The FP64 adjoint's tables, formed from the step's when these have changed.
+static tk_status adjoint_tables(tk_solver *S)
+{
+    if (S->precision != TK_PREC_F64 || S->adj_tab_of == S->coeffs_id) return TK_OK;
+    if (!S->adj_tab) {
+        tk_status st = tkh::alloc(S, (void **)&S->adj_tab, (size_t)S->Nr * S->K * tk::kAdjBytes);
+        if (st != TK_OK) return st;
+    }
+    const dim3 block(S->NP, tk::kAdjTableThreads / S->NP), grid((S->Nr + block.y - 1) / block.y);
+    tk::adj_tables_kernel<<<grid, block, 0, S->stream>>>(S->Nr, S->NP, (const double *)S->half,
+                                                         (const double *)S->node, S->adj_tab);
+    TK_CUDA(S, cudaGetLastError());
+    S->adj_tab_of = S->coeffs_id;
+    return TK_OK;
+}
 
 extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfinal,
                                 int on_device, double *grad, int grad_on_device, int independent_pi)
@@ -885,6 +1043,8 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
             st = tkh::alloc(S, &S->adj[k], se * S->esz);
             if (st != TK_OK) return st;
         }
+    st = adjoint_tables(S);
+    if (st != TK_OK) return st;
     const long long count = S->count;
     double *dwave = nullptr;
     double *dfin = nullptr;
@@ -947,17 +1107,18 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
                             : 0;
     if (pblocks > 0 && e == cudaSuccess) {
         unsigned int *flags = nullptr;
-        const size_t fbytes = (size_t)2 * pblocks * sizeof(unsigned int) + sizeof(int);
+        const int nflags = 2 * pblocks * (S->precision == TK_PREC_F64 ? S->K : 1);
+        const size_t fbytes = (size_t)nflags * sizeof(unsigned int) + sizeof(int);
         st = tkh::alloc(S, (void **)&flags, fbytes);
         if (st != TK_OK) {
             cleanup();
             return st;
         }
-        int *derr = (int *)(flags + 2 * pblocks);
+        int *derr = (int *)(flags + nflags);
         int herr = 0;
         e = cudaMemsetAsync(flags, 0, fbytes, S->stream);
         if (e == cudaSuccess)
-            e = tk::launch_adjoint_persistent(S->precision, S->K, S->adj[0], S->adj[1], S->half, S->node, S->Nr,
+            e = tk::launch_adjoint_persistent(S->precision, S->K, S->adj[0], S->adj[1], S->half, S->node, S->adj_tab, S->Nr,
                                               pblocks, S->adj_warps, dt_in, inj, dwave != nullptr, n_inner,
                                               S->substeps, flags, derr, S->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, S->stream);
@@ -975,7 +1136,8 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
                 inj.on = (k == 0) && dwave != nullptr;
                 inj.sample = t;
                 e = tk::launch_adjoint_step(S->precision, S->K, S->adj[cur], S->adj[cur ^ 1], S->half,
-                                            S->node, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
+                                            S->node, S->adj_tab, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj,
+                                            S->stream);
                 cur ^= 1;
             }
     }
@@ -1052,6 +1214,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         cleanup();
         return s2;
     };
+    if ((st = adjoint_tables(S)) != TK_OK) return st;
     for (int q = 0; q < 2; ++q)
         if (!S->adj[q] && (st = tkh::alloc(S, &S->adj[q], sb)) != TK_OK) return bail(st);
     if (!S->dhalf && (st = tkh::alloc(S, (void **)&S->dhalf, nh * sizeof(double))) != TK_OK) return bail(st);
@@ -1166,7 +1329,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
                                              S->dnode, S->Nr, dt_in, inj, acc, S->stream);
                 if (e == cudaSuccess)
                     e = tk::launch_adjoint_step(0, S->K, S->adj[cur], S->adj[cur ^ 1], S->half, S->node,
-                                                S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
+                                                S->adj_tab, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
                 cur ^= 1;
             }
     }

@@ -47,7 +47,7 @@ void release(tk_solver *S)
     void *ptrs[] = {S->u[0], S->u[1], S->half, S->node, S->b_node, S->w_row,
                     S->x_node, S->x_half, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
                     S->adj[0], S->adj[1], S->u_init, S->dhalf, S->dnode, S->db_node, S->pflags,
-                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step};
+                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step, S->adj_tab};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (int k = 0; k < 2; ++k)
@@ -299,6 +299,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
                                        S->cmp, S->gpm, S->stream, nullptr, nullptr, false, S->step));
     S->have_coeffs = true;
     S->have_state = false;
+    S->coeffs_id++;
     S->epoch++;   // the tables' time step may have changed: recapture graphs
     if (S->auto_k) {
         // substeps from the stability bound at the default growth per step,
@@ -375,6 +376,7 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
     if (e != cudaSuccess) return fail(S, TK_ERR_CUDA, "tk_set_coefficients: %s", cudaGetErrorString(e));
     S->have_coeffs = true;
     S->have_state = false;
+    S->coeffs_id++;
     S->epoch++;
     return TK_OK;
 }

@@ -27,6 +27,8 @@ struct tk_solver {
     int *flag = nullptr;
     unsigned long long *stiff = nullptr;  // [max omega^2, max b] as double bit patterns
     long long *ctr = nullptr;   // [0]: sample index of the next outer step, [1]: blocks done
+    unsigned char *adj_tab = nullptr;   // FP64 adjoint: its tables, allocated and formed on use
+    long long coeffs_id = 0, adj_tab_of = -1;   // which coefficients are set, which adj_tab was formed from
     void *adj[2] = {nullptr, nullptr};  // adjoint state levels (tk_adjoint), allocated on use
     // parameter gradients (tk_param_gradient): u^0 and the derivative tables
     void *u_init = nullptr;             // copy of u^0 (FP64 solvers)

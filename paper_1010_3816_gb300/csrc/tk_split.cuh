@@ -52,6 +52,7 @@
 // propagate as IEEE arithmetic has them.
 #pragma once
 
+#include "tk_split_tables.cuh"
 #include "tk_stencil.cuh"
 
 namespace tk {
@@ -59,10 +60,10 @@ namespace {
 
 // ---- integers ----
 
-// Phi_R, Phi_I of a lane's row as integers: the magnitude, all its bits
+// Two components of a lane's row as integers: the magnitude, all its bits
 // inverted where the value is negative (so that a right shift cuts both signs
 // alike), the exponent field, and 1 unless the value is zero (or subnormal).
-struct SplitPhi {
+struct SplitInts {
     long long x[2];
     int e[2];
     int j[2];
@@ -100,22 +101,24 @@ __device__ __forceinline__ int2 limbs(long long x)
     return make_int2((int)(x >> 32) + (int)((unsigned)x >> 31), (int)x);
 }
 
-__device__ __forceinline__ void split_phi(const double (&u)[4], SplitPhi &o)
+// Of components C0 and C0 + 1.
+template <int C0>
+__device__ __forceinline__ void split_ints(const double (&u)[4], SplitInts &o)
 {
     unsigned top = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const unsigned hi = (unsigned)__double2hiint(u[k]);
         top = max(top, hi & 0x7fffffffu);
-        if (k >= 2) continue;
+        if (k < C0 || k >= C0 + 2) continue;
         const unsigned lo = (unsigned)__double2loint(u[k]);
         const int e = (int)((hi >> 20) & 0x7ffu), j = min(e, 1);
         const unsigned m = (hi & 0xfffffu) | 0x100000u;
         const unsigned s = (unsigned)((int)hi >> 31), mask = (unsigned)-j;
         const unsigned xh = (__funnelshift_l(lo, m, 7) ^ s) & mask, xl = ((lo << 7) ^ s) & mask;
-        o.x[k] = ((long long)(int)xh << 32) | xl;
-        o.e[k] = e;
-        o.j[k] = j;
+        o.x[k - C0] = ((long long)(int)xh << 32) | xl;
+        o.e[k - C0] = e;
+        o.j[k - C0] = j;
     }
     o.top = top;
 }
@@ -252,7 +255,7 @@ struct StepTab {
 // Pi_I, as integers T 2^(O - 1080).  False (the same in the whole team) where
 // a value or the table (cold) calls for the FP64 instructions.
 template <int K, bool NODE>
-__device__ __forceinline__ bool split_coupling(const SplitPhi &a, const SplitPhi &c, const StepTab<NODE> &tab,
+__device__ __forceinline__ bool split_coupling(const SplitInts &a, const SplitInts &c, const StepTab<NODE> &tab,
                                                bool cold, bool imag, SplitTeam<K> &team, long long (&T)[2],
                                                int (&O)[2])
 {
@@ -382,8 +385,8 @@ __device__ __forceinline__ Row4 row4(const double (&x)[4]) { return {x[0], x[1],
 // Eq. (lw1) between columns a and c (half_node's result: Phi divided by e);
 // half64: the lane's row of the unsplit table.
 template <int K>
-__device__ __forceinline__ void split_half_node(const double (&a)[4], const SplitPhi &pa, const double (&c)[4],
-                                                const SplitPhi &pc, const unsigned char *block, SplitTeam<K> &team,
+__device__ __forceinline__ void split_half_node(const double (&a)[4], const SplitInts &pa, const double (&c)[4],
+                                                const SplitInts &pc, const unsigned char *block, SplitTeam<K> &team,
                                                 const double *half64, const FmaK<double> &k1, double (&h)[4])
 {
     const StepTab<false> tab{block, team.lane};
@@ -418,8 +421,8 @@ __device__ __forceinline__ void split_half_node(const double (&a)[4], const Spli
 
 // Eq. (lw2) (full_node's result) from the half nodes left (m) and right (p).
 template <int K>
-__device__ __forceinline__ void split_full_node(const double (&m)[4], const SplitPhi &pm, const double (&p)[4],
-                                                const SplitPhi &pp, const double (&u)[4], const unsigned char *block,
+__device__ __forceinline__ void split_full_node(const double (&m)[4], const SplitInts &pm, const double (&p)[4],
+                                                const SplitInts &pp, const double (&u)[4], const unsigned char *block,
                                                 SplitTeam<K> &team, const double *node64, double en,
                                                 const FmaK<double> &k1, double (&out)[4])
 {
@@ -554,21 +557,21 @@ struct SplitSweep {
             for (int k = 0; k < 4; ++k) u[k] = __ldcg(p + k * NP);
         };
         double a[4], hm[4], un[4];
-        SplitPhi pa, pm;
+        SplitInts pa, pm;
 #pragma unroll
         for (int k = 0; k < 4; ++k) hm[k] = 0.0;
-        split_phi(hm, pm);
+        split_ints<0>(hm, pm);
         load(pu, a);
         if (ib + 1 == i1) before_right();
         pu += 4 * NP;
         if (ib + 1 < Nr) load(pu, un);
-        split_phi(a, pa);
+        split_ints<0>(a, pa);
 #pragma unroll 1
         for (int i = ib; i < i1; ++i) {
             double o[4];
             if (i + 1 < Nr) {
                 double c[4], hp[4];
-                SplitPhi pc, pp;
+                SplitInts pc, pp;
                 const int nx = i + 1 < ie ? i + 1 : again ? ib : -1;
                 if (nx >= 0) fetch(st, st.cur ^ 1, nx, team.lane);
 #pragma unroll
@@ -578,12 +581,12 @@ struct SplitSweep {
                     pu += 4 * NP;
                     if (i + 2 < Nr) load(pu, un);
                 }
-                split_phi(c, pc);
+                split_ints<0>(c, pc);
                 await(st, st.cur);
                 const unsigned char *block = ring->tab[st.cur];
                 st.cur ^= 1;
                 split_half_node<K>(a, pa, c, pc, block, team, half64 + (size_t)i * (kNCH * NP) + row, k1, hp);
-                split_phi(hp, pp);
+                split_ints<0>(hp, pp);
                 if (i >= i0) {
                     if (i > 0) {
                         split_full_node<K>(hm, pm, hp, pp, a, block, team, node64 + (size_t)i * (kNCN * NP) + row,

@@ -358,36 +358,36 @@ lw_step2_kernel(const double *__restrict__ u_in, double *__restrict__ u_out, con
     };
     // the half node between columns i and i + 1, the node i, their tables read from global memory
     auto block = [&](int i) { return step + ((size_t)i * K + team.h) * kStepBytes; };
-    auto half_at = [&](int i, const double (&x)[4], const SplitPhi &px, const double (&y)[4], const SplitPhi &py,
+    auto half_at = [&](int i, const double (&x)[4], const SplitInts &px, const double (&y)[4], const SplitInts &py,
                        double (&o)[4]) {
         split_half_node<K>(x, px, y, py, block(i), team, half + (size_t)i * (kNCH * NP) + row, k1, o);
     };
     auto node_at = [&](int i, const double (&m)[4], const double (&p)[4], const double (&u)[4], double (&o)[4]) {
-        SplitPhi pm, pp;
-        split_phi(m, pm);
-        split_phi(p, pp);
+        SplitInts pm, pp;
+        split_ints<0>(m, pm);
+        split_ints<0>(p, pp);
         split_full_node<K>(m, pm, p, pp, u, block(i), team, node + (size_t)i * (kNCN * NP) + row, en, k1, o);
     };
     if (i1 > i0) {
         double a0[4], h1m[4], u1m[4], h2m[4];
-        SplitPhi pa, p1;    // the integers of a0 and u1m
+        SplitInts pa, p1;    // the integers of a0 and u1m
         clear(a0);
         clear(h1m);
         clear(u1m);
         clear(h2m);
-        split_phi(a0, pa);
+        split_ints<0>(a0, pa);
         p1 = pa;
 #pragma unroll 1
         for (int p = i0 - 2; p <= i1 + 1; ++p) {
             double c0[4], h1p[4], u1c[4], h2p[4];
-            SplitPhi pc, pc1;
+            SplitInts pc, pc1;
             if (p >= 0 && p < Nr) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) c0[k] = u_in[(size_t)p * (4 * NP) + k * NP + row];
             } else {
                 clear(c0);
             }
-            split_phi(c0, pc);
+            split_ints<0>(c0, pc);
             // level 1, half node between p - 1 and p
             if (p >= i0 - 1 && p >= 1 && p < Nr) half_at(p - 1, a0, pa, c0, pc, h1p);
             else clear(h1p);
@@ -399,7 +399,7 @@ lw_step2_kernel(const double *__restrict__ u_in, double *__restrict__ u_out, con
                 observe_team<K>(q, u1c, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, 0);
             // level 2, half node between r = p - 2 and p - 1
             const int r = p - 2;
-            split_phi(u1c, pc1);
+            split_ints<0>(u1c, pc1);
             if (p >= i0 + 1 && r >= 0 && r + 1 < Nr) half_at(r, u1m, p1, u1c, pc1, h2p);
             else clear(h2p);
             // level 2, node r

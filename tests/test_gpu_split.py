@@ -1,7 +1,8 @@
-"""The FP64 step's integer coupling (csrc/tk_split.cuh): teams of warps at the
-edges of their 32-row pieces and of the radial split, all launch structures on
-the same bits, powers of two of the data, and the columns that take the FP64
-instructions (huge values, infinities).
+"""The FP64 step's integer coupling (csrc/tk_split.cuh) and its transpose
+(csrc/tk_split_adjoint.cuh): teams of warps at the edges of their 32-row pieces
+and of the radial split, all launch structures on the same bits, powers of two
+of the data, and the columns that take the FP64 instructions (huge values,
+infinities).
 
 Tolerances.  With the oracle's own coefficients a run differs from the oracle
 by roundings only: per Lax-Wendroff step a value takes at most 16 of them
@@ -176,3 +177,74 @@ def test_a_non_finite_value_stays_in_its_stencil(bad, Nth, j, comp):
     with pytest.raises(tk.TkError):
         g.check_finite()
     g.close()
+
+
+# ---- the transposed step (csrc/tk_split_adjoint.cuh) ----
+
+def _adjoint(w, mode=0, scale=1.0, n=3):
+    """(initial planes, final state, its loss gradient, dL/d(initial planes))."""
+    g = _solver(w, mode)
+    rng = np.random.default_rng(5)
+    u0 = rng.standard_normal((4, w.Ntheta, w.Nr))
+    u0[:, :, [0, -1]] = 0.0
+    g.set_initial(*u0)
+    g.step(n)
+    dL = rng.standard_normal(u0.shape)
+    dL[:, :, [0, -1]] = 0.0
+    grad = np.empty_like(u0)
+    g.adjoint(grad, dL_dfinal=dL * scale, independent_pi=True)
+    uN = g.state()
+    g.close()
+    return u0, uN, dL * scale, grad
+
+
+@pytest.mark.parametrize("Nr,Nth", SIZES)
+@pytest.mark.parametrize("a", [0.9, 0.0])
+def test_adjoint_is_the_transpose_at_the_edges(Nr, Nth, a):
+    """<dL, u_N> = <dL/du_0, u_0>: each side is off by the roundings of three
+    steps, 16 of 2^-53 each, times the growth allowed above."""
+    u0, uN, dL, grad = _adjoint(_work(Nr, Nth, a=a))
+    norm = np.linalg.norm
+    assert abs(np.vdot(dL, uN) - np.vdot(grad, u0)) <= TOL * (norm(dL) * norm(uN) + norm(grad) * norm(u0))
+
+
+@pytest.mark.parametrize("Nr,Nth,scale", [(700, 64, 1.0), (333, 97, 1.0), (90, 40, 2.0 ** 877), (153, 20, 2.0 ** 890)])
+def test_adjoint_launch_structures_agree(Nr, Nth, scale):
+    """One persistent launch and one launch per step: the same bits, also where
+    columns are cold, and there the others' result but for its roundings."""
+    w = _work(Nr, Nth, substeps=2)
+    ref = _adjoint(w, -1, scale)[3]
+    assert np.isfinite(ref).all()
+    assert np.array_equal(_adjoint(w, 1, scale)[3], ref)
+    plain = _adjoint(w)[3]
+    assert np.linalg.norm(ref / scale - plain) <= TOL * np.linalg.norm(plain)
+
+
+@pytest.mark.parametrize("p", [-700, 500])
+def test_adjoint_powers_of_two_scale_exactly(p):
+    w = _work(200, 64)
+    assert np.array_equal(_adjoint(w, scale=2.0 ** p)[3], _adjoint(w)[3] * 2.0 ** p)
+
+
+def test_adjoint_tables_follow_the_coefficients():
+    """A solver precomputed again uses the new black hole's tables."""
+    w = _work(90, 40)
+    g = _solver(w)
+    rng = np.random.default_rng(6)
+    u0 = rng.standard_normal((4, w.Ntheta, w.Nr))
+    dL = rng.standard_normal(u0.shape)
+    grads = []
+    for a in (0.9, 0.3):
+        g.precompute(a, w.M, w.s, w.m)
+        g.set_initial(*u0)
+        g.step(2)
+        grads.append(np.empty_like(u0))
+        g.adjoint(grads[-1], dL_dfinal=dL, independent_pi=True)
+    g.close()
+    h = _solver(w.with_(a=0.3))
+    h.set_initial(*u0)
+    h.step(2)
+    want = np.empty_like(u0)
+    h.adjoint(want, dL_dfinal=dL, independent_pi=True)
+    h.close()
+    assert np.array_equal(grads[1], want) and not np.array_equal(grads[0], want)
