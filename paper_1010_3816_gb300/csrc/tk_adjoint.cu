@@ -1224,7 +1224,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         (st = tkh::alloc(S, (void **)&tnode, nn * sizeof(double))) != TK_OK ||
         (st = tkh::alloc(S, (void **)&tb, nb * sizeof(double))) != TK_OK ||
         (st = tkh::alloc(S, (void **)&tw, (size_t)S->NP * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tx, (size_t)2 * S->Nr * sizeof(double))) != TK_OK ||
+        (st = tkh::alloc(S, (void **)&tx, (size_t)2 * S->Nr * tk::kRadial * sizeof(double))) != TK_OK ||
         (st = tkh::alloc(S, (void **)&tang, (size_t)2 * S->NP * sizeof(double))) != TK_OK)
         return bail(st);
     if (on_device) {
@@ -1253,11 +1253,11 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
             tk::Kerr P = S->kerr;
             if (param == 0) P.a += off[q];
             else P.M += off[q];
-            e = tk::launch_invert_tortoise(P, S->rs_min, S->drs, S->Nr, tx, tx + S->Nr, S->stream);
+            e = tk::launch_invert_tortoise(P, S->rs_min, S->drs, S->Nr, tx, S->stream);
             if (e == cudaSuccess)
-                e = tk::launch_coeff_tables(P, S->variable, S->Nr, S->Nth, S->NP, S->drs, dt_in, tx,
-                                            tx + S->Nr, tang, 0, thalf, tnode, tb, tw, nullptr,
-                                            nullptr, S->stream);
+                // the angular stencil depends on s and m only: formed with the first
+                e = tk::launch_coeff_tables(P, S->variable, S->Nr, S->Nth, S->NP, S->drs, dt_in, tx, tang, 0, thalf,
+                                            tnode, tb, tw, nullptr, nullptr, S->stream, nullptr, nullptr, q > 0);
             if (e == cudaSuccess) e = tk::launch_axpy(nh, wgt[q], thalf, S->dhalf, S->stream);
             if (e == cudaSuccess) e = tk::launch_axpy(nn, wgt[q], tnode, S->dnode, S->stream);
             if (e == cudaSuccess) e = tk::launch_axpy(nb, wgt[q], tb, S->db_node, S->stream);

@@ -45,7 +45,7 @@ tk_status alloc(tk_solver *S, void **p, size_t bytes)
 void release(tk_solver *S)
 {
     void *ptrs[] = {S->u[0], S->u[1], S->half, S->node, S->b_node, S->w_row,
-                    S->x_node, S->x_half, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
+                    S->rad, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
                     S->adj[0], S->adj[1], S->u_init, S->dhalf, S->dnode, S->db_node, S->pflags,
                     S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step, S->adj_tab};
     for (void *p : ptrs)
@@ -253,8 +253,7 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
         st = alloc(S, (void **)&S->gpm, (size_t)2 * S->NP * sizeof(float));
     if (st == TK_OK) st = alloc(S, (void **)&S->b_node, (size_t)Nr * S->NP * sizeof(double));
     if (st == TK_OK) st = alloc(S, (void **)&S->w_row, (size_t)S->NP * sizeof(double));
-    if (st == TK_OK) st = alloc(S, (void **)&S->x_node, (size_t)Nr * sizeof(double));
-    if (st == TK_OK) st = alloc(S, (void **)&S->x_half, (size_t)Nr * sizeof(double));
+    if (st == TK_OK) st = alloc(S, (void **)&S->rad, (size_t)2 * Nr * tk::kRadial * sizeof(double));
     if (st == TK_OK) st = alloc(S, (void **)&S->ang, (size_t)2 * S->NP * sizeof(double));
     if (st == TK_OK) st = alloc(S, (void **)&S->flag, sizeof(int));
     if (st == TK_OK) st = alloc(S, (void **)&S->stiff, 2 * sizeof(unsigned long long));
@@ -291,10 +290,10 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
     S->kerr.s = s;
     S->kerr.m = m;
     if (S->auto_k) S->substeps = 1;
-    TK_CUDA(S, tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->x_node, S->x_half,
+    TK_CUDA(S, tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->rad,
                                           S->stream));
     TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
-                                       S->dt / S->substeps, S->x_node, S->x_half, S->ang,
+                                       S->dt / S->substeps, S->rad, S->ang,
                                        S->precision, S->half, S->node, S->b_node, S->w_row,
                                        S->cmp, S->gpm, S->stream, nullptr, nullptr, false, S->step));
     S->have_coeffs = true;
@@ -314,7 +313,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
         if (k != 1) {
             S->substeps = k;
             TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
-                                               S->dt / S->substeps, S->x_node, S->x_half, S->ang,
+                                               S->dt / S->substeps, S->rad, S->ang,
                                                S->precision, S->half, S->node, S->b_node,
                                                S->w_row, S->cmp, S->gpm, S->stream, nullptr, nullptr,
                                                false, S->step));
@@ -366,10 +365,10 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, S->stream);
     }
     if (e == cudaSuccess)
-        e = tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->x_node, S->x_half, S->stream);
+        e = tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->rad, S->stream);
     if (e == cudaSuccess)
         e = tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs, S->dt / S->substeps,
-                                    S->x_node, S->x_half, S->ang, S->precision, S->half, S->node, S->b_node,
+                                    S->rad, S->ang, S->precision, S->half, S->node, S->b_node,
                                     S->w_row, S->cmp, S->gpm, S->stream, dn, dh, ang_given, S->step);
     if (e == cudaSuccess && dev) e = cudaStreamSynchronize(S->stream);
     if (dev) cudaFree(dev);
@@ -389,14 +388,14 @@ tk_status tk_get_coefficients(tk_solver *S, double *node9, double *half9, int on
     if (!node9 || !half9) return fail(S, TK_ERR_ARG, "tk_get_coefficients: node9/half9 are NULL");
     const size_t n9 = (size_t)9 * S->Nth * S->Nr;
     if (on_device) {
-        TK_CUDA(S, tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->x_node, S->x_half, node9,
+        TK_CUDA(S, tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->rad, node9,
                                          half9, S->stream));
         return TK_OK;
     }
     double *dev = nullptr;
     st = alloc(S, (void **)&dev, 2 * n9 * sizeof(double));
     if (st != TK_OK) return st;
-    cudaError_t e = tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->x_node, S->x_half, dev,
+    cudaError_t e = tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->rad, dev,
                                           dev + n9, S->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(node9, dev, n9 * sizeof(double), cudaMemcpyDeviceToHost, S->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(half9, dev + n9, n9 * sizeof(double), cudaMemcpyDeviceToHost, S->stream);
@@ -856,7 +855,7 @@ tk_status tk_stability_bound(tk_solver *S, double growth_per_step, double *dt_ma
     if (!(growth_per_step > 0.0) || !(growth_per_step < 1.0))
         return fail(S, TK_ERR_ARG, "tk_stability_bound: growth_per_step must be in (0, 1)");
     unsigned long long h[2] = {0, 0};
-    TK_CUDA(S, tk::launch_stiffness(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->x_node, S->ang,
+    TK_CUDA(S, tk::launch_stiffness(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->rad, S->ang,
                                     S->stiff, S->stream));
     TK_CUDA(S, cudaMemcpyAsync(h, S->stiff, sizeof h, cudaMemcpyDeviceToHost, S->stream));
     TK_CUDA(S, cudaStreamSynchronize(S->stream));

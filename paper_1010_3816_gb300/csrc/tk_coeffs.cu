@@ -14,6 +14,7 @@
 
 #include "tk_internal.h"
 #include "tk_split_tables.cuh"
+#include "tk_stencil.cuh"
 
 namespace tk {
 namespace {
@@ -49,14 +50,23 @@ __device__ double rstar_of_x(const Geo &P, double x)
 
 __device__ double x_of_rstar(const Geo &P, double target)
 {
-    // r*(e^y) is increasing in y with slope (r^2 + a^2)/(r - r-): keep a
-    // bracket [ylo, yhi] around the root and take Newton steps inside it,
-    // falling back to bisection when a step leaves the bracket.
-    double ylo = -700.0, yhi = 1.0;
-    for (int g = 0; g < 64 && rstar_of_x(P, exp(yhi)) < target; ++g) yhi += 1.0;
-    double y = (target > P.rp + 4.0 * P.M) ? log(target)
-                                           : (target - P.rp) / P.Ap + log(2.0 * P.M);
-    if (!(y > ylo && y < yhi)) y = 0.5 * (ylo + yhi);
+    // r*(e^y) is increasing in y with slope (r^2 + a^2)/(r - r-): Newton steps
+    // inside a bracket [ylo, yhi] of the root, bisection when a step leaves it.
+    // x >= max(r*, 2M) has r*(x) >= r* (the logarithms then add at least -M and
+    // r+ >= M), which bounds the root from above.  Far out Newton starts from
+    // there (r*(e^y) is convex, so it comes down monotonically), further in from
+    // the horizon's asymptotics.  It ends when a step no longer changes y, or
+    // only goes back to the value before: seven evaluations or fewer, each a
+    // serial chain of some 100 FP64 instructions of 64 cycles (with the bracket
+    // tested before the end, as once, a converged step fell out of it and up to
+    // 52 bisections followed: 307 us for any grid, now 57 at 1601
+    // radii and 75 at 4001).
+    const double top = log(fmax(target, 2.0 * P.M));
+    double ylo = -700.0, yhi = nextafter(top, 1e3);
+    double y = (target > P.rp + 4.0 * P.M) ? top : (target - P.rp) / P.Ap + log(2.0 * P.M);
+    y = fmin(y, top);
+    if (!(y > ylo)) y = 0.5 * (ylo + yhi);
+    double before = y;
     for (int it = 0; it < 200; ++it) {
         const double x = exp(y);
         const double r = P.rp + x;
@@ -64,24 +74,57 @@ __device__ double x_of_rstar(const Geo &P, double target)
         if (f == 0.0) break;
         if (f < 0.0) ylo = y; else yhi = y;
         double yn = y - f * (r - P.rm) / (r * r + P.a * P.a);
-        if (!(yn > ylo && yn < yhi)) yn = 0.5 * (ylo + yhi);
-        if (yn == y) break;
+        if (yn == y || yn == before) break;
+        if (!(yn > ylo && yn < yhi)) {
+            yn = 0.5 * (ylo + yhi);
+            if (yn == ylo || yn == yhi) break;
+        }
+        before = y;
         y = yn;
     }
     return exp(y);
 }
 
-__global__ void invert_tortoise_kernel(Kerr KP, double rs_min, double drs, int Nr,
-                                       double *x_node, double *x_half)
+// What the coefficients need of a radius (x = r - r+), kRadial doubles.
+struct Radial {
+    double r, vp, Dl, dDl;       // r, varpi = r^2 + a^2, Delta = x (r - r-), d Delta / dr
+    double tor;                  // dr/dr* = Delta / varpi
+    double fs, fss;              // (d_* r^3)/r^3, (d_*^2 r^3)/r^3
+    double ctr, cti0, cti1;      // Sigma^2 Re C_t, Sigma^2 Im C_t = cti0 + cti1 cos
+    double e0, c3i;              // Sigma^2 E0, Sigma^2 Im c3
+};
+static_assert(sizeof(Radial) == kRadial * sizeof(double), "kRadial");
+
+__device__ Radial radial_part(const Geo &P, double x)
 {
+    const double M = P.M, a = P.a, s = P.s, m = P.m;
+    const double r = P.rp + x, r2 = r * r, a2 = a * a;
+    Radial R;
+    R.r = r;
+    R.vp = r2 + a2;
+    R.Dl = x * (r - P.rm);
+    R.dDl = 2.0 * (r - M);
+    R.tor = R.Dl / R.vp;
+    R.fs = 3.0 * R.Dl / (r * R.vp);
+    R.fss = R.tor * ((6.0 * r * R.Dl + 3.0 * r2 * R.dDl) / R.vp - 6.0 * r2 * r * R.Dl / (R.vp * R.vp)) / (r2 * r);
+    R.ctr = 2.0 * s * (r * R.Dl - M * (r2 - a2));
+    R.cti0 = 4.0 * M * a * m * r;
+    R.cti1 = 2.0 * s * a * R.Dl;
+    R.e0 = 2.0 * r * R.Dl + s * R.dDl * R.vp;
+    R.c3i = 2.0 * m * s * a * (r - M);
+    return R;
+}
+
+// The tortoise inversion and the radial parts: nodes i in rad[i], half nodes
+// i + 1/2 in rad[Nr + i].
+__global__ void invert_tortoise_kernel(Kerr KP, double rs_min, double drs, int Nr, double *rad)
+{
+    asm volatile("griddepcontrol.launch_dependents;");   // the angular stencil may run beside it
     const Geo P = geometry(KP);
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < Nr) {
-        x_node[k] = x_of_rstar(P, rs_min + k * drs);
-    } else if (k < 2 * Nr - 1) {
-        const int i = k - Nr;                       // half node i + 1/2
-        x_half[i] = x_of_rstar(P, rs_min + (i + 0.5) * drs);
-    }
+    if (k >= 2 * Nr - 1) return;
+    const double rs = k < Nr ? rs_min + k * drs : rs_min + (k - Nr + 0.5) * drs;
+    *reinterpret_cast<Radial *>(rad + (size_t)k * kRadial) = radial_part(P, x_of_rstar(P, rs));
 }
 
 // Coefficients of   d_t Phi + b d_* Phi = Pi,
@@ -94,48 +137,52 @@ struct Raw {
     double b, c1r, c1i, c2r, c2i, c3r, c3i, c4, c5;
 };
 
-__device__ Raw raw_coefficients(const Geo &P, int variable, double x, double th)
+// What they need of a polar angle.
+struct Angular {
+    double sn, cs, g, V;
+};
+
+__device__ Angular angular_part(const Geo &P, int variable, double th)
 {
-    const double M = P.M, a = P.a, s = P.s, m = P.m;
-    const double r = P.rp + x, r2 = r * r, a2 = a * a;
-    const double vp = r2 + a2;                 // varpi
-    const double Dl = x * (r - P.rm);          // Delta
-    const double dDl = 2.0 * (r - M);          // d Delta / dr
-    double sn, cs;
-    sincos(th, &sn, &cs);
-    const double sn2 = sn * sn;
-    const double S2 = vp * vp - a2 * Dl * sn2; // Sigma^2
-    const double Sg = sqrt(S2);
-    const double b = vp / Sg;
-    const double tor = Dl / vp;                // dr/dr*
-    const double db = tor * (2.0 * r / Sg - vp * (4.0 * r * vp - a2 * dDl * sn2) / (2.0 * S2 * Sg));
-    const double fs = 3.0 * Dl / (r * vp);     // (d_* r^3)/r^3
-    const double fss = tor * ((6.0 * r * Dl + 3.0 * r2 * dDl) / vp - 6.0 * r2 * r * Dl / (vp * vp)) / (r2 * r);
-    const double Ctr = 2.0 * s * (r * Dl - M * (r2 - a2)) / S2;
-    const double Cti = (4.0 * M * a * m * r + 2.0 * s * a * Dl * cs) / S2;
-    const double E0 = (2.0 * r * Dl + s * dDl * vp) / S2;
-    const double c4 = Dl / S2;
-    double g, V;
+    const double s = P.s, m = P.m;
+    Angular A;
+    sincos(th, &A.sn, &A.cs);
     if (variable == 0) {
-        g = cs / sn;
-        V = -(m + s * cs) * (m + s * cs) / sn2 + s;
+        A.g = A.cs / A.sn;
+        A.V = -(m + s * A.cs) * (m + s * A.cs) / (A.sn * A.sn) + s;
     } else {
         const double al = 0.5 * fabs(m + s), be = 0.5 * fabs(m - s);
         const int l0 = max(abs(P.m), abs(P.s));
         const double t2 = tan(0.5 * th);
-        g = cs / sn + 2.0 * (al / t2 - be * t2);
-        V = -(double)(l0 - P.s) * (double)(l0 + P.s + 1);
+        A.g = A.cs / A.sn + 2.0 * (al / t2 - be * t2);
+        A.V = -(double)(l0 - P.s) * (double)(l0 + P.s + 1);
     }
+    return A;
+}
+
+__device__ Raw raw_coefficients(const Geo &P, const double *__restrict__ rad, const Angular &A)
+{
+    const Radial R = *reinterpret_cast<const Radial *>(rad);
+    const double a2 = P.a * P.a, m = P.m;
+    const double sn2 = A.sn * A.sn;
+    const double S2 = R.vp * R.vp - a2 * R.Dl * sn2; // Sigma^2
+    const double Sg = sqrt(S2);
+    const double b = R.vp / Sg;
+    const double db = R.tor * (2.0 * R.r / Sg - R.vp * (4.0 * R.r * R.vp - a2 * R.dDl * sn2) / (2.0 * S2 * Sg));
+    const double Ctr = R.ctr / S2;
+    const double Cti = (R.cti0 + R.cti1 * A.cs) / S2;
+    const double E0 = R.e0 / S2;
+    const double c4 = R.Dl / S2;
     Raw o;
     o.b = b;
-    o.c1r = b * Ctr + (2.0 * b * b * fs + E0) - b * db;
+    o.c1r = b * Ctr + (2.0 * b * b * R.fs + E0) - b * db;
     o.c1i = b * Cti;
     o.c2r = -Ctr;
     o.c2i = -Cti;
-    o.c3r = b * b * fss + E0 * fs + m * m * a2 / S2 + c4 * V;
-    o.c3i = 2.0 * m * s * a * (r - M) / S2;
+    o.c3r = b * b * R.fss + E0 * R.fs + m * m * a2 / S2 + c4 * A.V;
+    o.c3i = R.c3i / S2;
     o.c4 = c4;
-    o.c5 = c4 * g;
+    o.c5 = c4 * A.g;
     return o;
 }
 
@@ -158,17 +205,22 @@ __device__ double sl_weight(int s, int m, double th)
 // P = sin(theta) w^2 at the faces theta = f dth (zero on both poles), Q_j the
 // mean of P over the cell by 4-point Gauss-Legendre on 64 sub-panels.
 // ang[j] = P_{j+1}/(Q_j dth^2), ang[NP + j] = P_j/(Q_j dth^2); zero on padding rows.
-// One warp per row j: lane l integrates sub-panels l and l + 32, then the
-// warp sums the 32 partial sums in a fixed tree order.
+// One block per row j, one thread per Gauss point (each evaluation is a serial
+// chain of two powers, a sine and a cosine: ~10 us, so all of them at once);
+// then the first warp adds them, lane l those of sub-panels l and l + 32, and
+// the 32 partial sums in a fixed tree order: 32 us, with a warp per row that
+// took two panels a lane in turn 88.  Each block ends only after the kernel it
+// is chained to (the next kernel reads what both wrote).
 constexpr int kStencilPanels = 64;
 
-__global__ void regular_stencil_kernel(int s, int m, int Nth, int NP, double *__restrict__ ang)
+__global__ void __launch_bounds__(4 * kStencilPanels)
+regular_stencil_kernel(int s, int m, int Nth, int NP, double *__restrict__ ang)
 {
-    const int j = blockIdx.x;
-    const int lane = threadIdx.x;
-    if (j >= NP) return;
+    __shared__ double val[kStencilPanels][4], face[2];
+    const int j = blockIdx.x, tid = threadIdx.x;
     if (j >= Nth) {
-        if (lane == 0) {
+        if (tid == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             ang[j] = 0.0;
             ang[NP + j] = 0.0;
         }
@@ -178,19 +230,23 @@ __global__ void regular_stencil_kernel(int s, int m, int Nth, int NP, double *__
     const double xg[2] = {0.3399810435848563, 0.8611363115940526};
     const double wg[2] = {0.6521451548625461, 0.3478548451374538};
     const double h = dth / kStencilPanels;
-    double acc = 0.0;
-    for (int k = lane; k < kStencilPanels; k += 32) {
+    {
+        const int k = tid >> 2, g = (tid >> 1) & 1;
         const double c = j * dth + (k + 0.5) * h;
-        for (int g = 0; g < 2; ++g)
-            acc += wg[g] * (sl_weight(s, m, c - 0.5 * h * xg[g]) + sl_weight(s, m, c + 0.5 * h * xg[g]));
+        val[k][tid & 3] = sl_weight(s, m, (tid & 1) ? c + 0.5 * h * xg[g] : c - 0.5 * h * xg[g]);
     }
+    if (tid < 2) face[tid] = (j + tid == 0 || j + tid == Nth) ? 0.0 : sl_weight(s, m, (j + tid) * dth);
+    __syncthreads();
+    if (tid >= 32) return;
+    double acc = 0.0;
+    for (int k = tid; k < kStencilPanels; k += 32)
+        for (int g = 0; g < 2; ++g) acc += wg[g] * (val[k][2 * g] + val[k][2 * g + 1]);
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane != 0) return;
+    if (tid != 0) return;
     const double Q = 0.5 * h * acc / dth;
-    const double Plo = (j == 0) ? 0.0 : sl_weight(s, m, j * dth);
-    const double Phi = (j == Nth - 1) ? 0.0 : sl_weight(s, m, (j + 1) * dth);
-    ang[j] = Phi / (Q * dth * dth);
-    ang[NP + j] = Plo / (Q * dth * dth);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ang[j] = face[1] / (Q * dth * dth);
+    ang[NP + j] = face[0] / (Q * dth * dth);
 }
 
 // Raw coefficients supplied by the caller: [9][Nth][Nr] in the order of Raw
@@ -212,232 +268,239 @@ __device__ Raw raw_from(const double *__restrict__ r, int Nth, int Nr, int jp, i
 }
 
 // One thread per point, a block holding all NP rows of its columns (blockDim.x
-// = NP): a column's flags in the step tables are over its rows.
+// = NP): a column's flags in the step tables are over its rows.  Bound by the
+// FP64 pipe: what depends on the radius alone comes from the inversion kernel,
+// what depends on the angle alone is formed once per thread, which takes
+// columns in turns (with both formed at every point 372 us at 4001 x 64, now
+// 217).
 constexpr int kTableThreads = 256;
 
 template <typename T>
-__global__ void __launch_bounds__(kTableThreads) coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs,
-                                    double dt, const double *__restrict__ x_node,
-                                    const double *__restrict__ x_half,
-                                    const double *__restrict__ ang, T *__restrict__ half,
-                                    T *__restrict__ node, double *__restrict__ b_node,
-                                    double *__restrict__ w_row, float *__restrict__ cmp,
-                                    float *__restrict__ gpm, F32Derive fd,
-                                    const double *__restrict__ raw_node,
-                                    const double *__restrict__ raw_half,
-                                    unsigned char *__restrict__ step)
+__global__ void __launch_bounds__(kTableThreads)
+coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, double dt,
+                    const double *__restrict__ rad, const double *__restrict__ ang, T *__restrict__ half,
+                    T *__restrict__ node, double *__restrict__ b_node, double *__restrict__ w_row,
+                    float *__restrict__ cmp, float *__restrict__ gpm, F32Derive fd,
+                    const double *__restrict__ raw_node, const double *__restrict__ raw_half,
+                    unsigned char *__restrict__ step)
 {
     __shared__ int flags[kTableThreads / 32][2];   // per column: cold, has imaginary coefficients
     const int jp = threadIdx.x;
-    const int i = blockIdx.x * blockDim.y + threadIdx.y;
-    if (step) {
-        const int k = threadIdx.y * blockDim.x + threadIdx.x;
-        if (k < kTableThreads / 32 * 2) (&flags[0][0])[k] = 0;
-        __syncthreads();
-    }
     const Geo P = geometry(KP);
-    T *hcol = half + (size_t)i * kNCH * NP + jp;
-    T *ncol = node + (size_t)i * kNCN * NP + jp;
-    double hv[kNCH], nv[kNCN];
-    for (int q = 0; q < kNCH; ++q) hv[q] = 0.0;
-    for (int q = 0; q < kNCN; ++q) nv[q] = 0.0;
-    double bn = 0.0;
-    double c4n = 0.0, c4h = 0.0;   // c4 at the node and at the half node
-    double gpv = 0.0, gmv = 0.0;   // theta-only stencil factors of the row
     const double dth = M_PI / Nth;
-    const double ith2 = 1.0 / (dth * dth), i2th = 1.0 / (2.0 * dth);
-    const double p = (variable == 0 && (abs(P.m) & 1)) ? -1.0 : 1.0;   // ghost parity
-    if (jp < Nth && i < Nr) {
-        const double th = (jp + 0.5) * dth;
-        if (i == 0 && w_row) w_row[jp] = (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
-        // angular stencil A+ (row j+1), A- (row j-1); the centre gets -(A+ + A-)
-        //   literal:     A+- = 1/dth^2 +- cot(theta)/(2 dth) times c4, i.e. c4/dth^2 +- c5/(2 dth)
-        //   regularised: A+- = c4 ang[.]  (self-adjoint form, no ghosts)
-        const double Ap = (variable != 0) ? ang[jp] : 0.0;
-        const double Am = (variable != 0) ? ang[NP + jp] : 0.0;
-        if (variable != 0) {
-            gpv = Ap;
-            gmv = Am;
-        } else {
-            double sn, cs;
-            sincos(th, &sn, &cs);
-            gpv = (jp == Nth - 1) ? 0.0 : ith2 + (cs / sn) * i2th;   // ghosts folded on the edge rows
-            gmv = (jp == 0) ? 0.0 : ith2 - (cs / sn) * i2th;
+    const double th = (jp + 0.5) * dth;
+    const Angular A = (jp < Nth && !raw_node) ? angular_part(P, variable, th) : Angular{};
+    // the columns of the grid in turns (the row's angular part is formed once)
+    for (int c0 = blockIdx.x * blockDim.y; c0 < Nr; c0 += gridDim.x * blockDim.y) {
+        const int i = c0 + threadIdx.y;
+        if (step) {
+            const int k = threadIdx.y * blockDim.x + threadIdx.x;
+            __syncthreads();
+            if (k < kTableThreads / 32 * 2) (&flags[0][0])[k] = 0;
+            __syncthreads();
         }
-        {   // node r*_i, Eq. (lw2), step dt
-            const Raw c = raw_node ? raw_from(raw_node, Nth, Nr, jp, i)
-                                   : raw_coefficients(P, variable, x_node[i], th);
-            bn = c.b;
-            if (i > 0 && i < Nr - 1) {
-                c4n = c.c4;
-                const double h2 = 0.5 * dt;
-                const double B = dt * c.b / drs;
-                const double g1r = dt * c.c1r / drs, g1i = dt * c.c1i / drs;
+        T *hcol = half + (size_t)i * kNCH * NP + jp;
+        T *ncol = node + (size_t)i * kNCN * NP + jp;
+        double hv[kNCH], nv[kNCN];
+        for (int q = 0; q < kNCH; ++q) hv[q] = 0.0;
+        for (int q = 0; q < kNCN; ++q) nv[q] = 0.0;
+        double bn = 0.0;
+        double c4n = 0.0, c4h = 0.0;   // c4 at the node and at the half node
+        double gpv = 0.0, gmv = 0.0;   // theta-only stencil factors of the row
+        const double ith2 = 1.0 / (dth * dth), i2th = 1.0 / (2.0 * dth);
+        const double p = (variable == 0 && (abs(P.m) & 1)) ? -1.0 : 1.0;   // ghost parity
+        if (jp < Nth && i < Nr) {
+            if (i == 0 && w_row) w_row[jp] = (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
+            // angular stencil A+ (row j+1), A- (row j-1); the centre gets -(A+ + A-)
+            //   literal:     A+- = 1/dth^2 +- cot(theta)/(2 dth) times c4, i.e. c4/dth^2 +- c5/(2 dth)
+            //   regularised: A+- = c4 ang[.]  (self-adjoint form, no ghosts)
+            const double Ap = (variable != 0) ? ang[jp] : 0.0;
+            const double Am = (variable != 0) ? ang[NP + jp] : 0.0;
+            if (variable != 0) {
+                gpv = Ap;
+                gmv = Am;
+            } else {
+                double sn, cs;
+                sincos(th, &sn, &cs);
+                gpv = (jp == Nth - 1) ? 0.0 : ith2 + (cs / sn) * i2th;   // ghosts folded on the edge rows
+                gmv = (jp == 0) ? 0.0 : ith2 - (cs / sn) * i2th;
+            }
+            {   // node r*_i, Eq. (lw2), step dt
+                const Raw c = raw_node ? raw_from(raw_node, Nth, Nr, jp, i)
+                                       : raw_coefficients(P, rad + (size_t)i * kRadial, A);
+                bn = c.b;
+                if (i > 0 && i < Nr - 1) {
+                    c4n = c.c4;
+                    const double h2 = 0.5 * dt;
+                    const double B = dt * c.b / drs;
+                    const double g1r = dt * c.c1r / drs, g1i = dt * c.c1i / drs;
+                    double kp, km;
+                    if (variable == 0) {
+                        kp = h2 * (c.c4 * ith2 + c.c5 * i2th);
+                        km = h2 * (c.c4 * ith2 - c.c5 * i2th);
+                    } else {
+                        kp = h2 * c.c4 * Ap;
+                        km = h2 * c.c4 * Am;
+                    }
+                    const double dg = kp + km;
+                    double fpr = g1r + h2 * c.c3r - dg, fmr = -g1r + h2 * c.c3r - dg;
+                    if (variable == 0 && jp == 0) { fpr += p * km; fmr += p * km; km = 0.0; }
+                    if (variable == 0 && jp == Nth - 1) { fpr += p * kp; fmr += p * kp; kp = 0.0; }
+                    // entries that multiply half-node Phi values carry the factor eh
+                    // (the half node returns Phi / eh, see the half-node tables)
+                    const double eh = 0.25 * dt;
+                    nv[N_B] = eh * B;
+                    nv[N_PPR] = B + h2 * c.c2r;
+                    nv[N_PMR] = -B + h2 * c.c2r;
+                    nv[N_C2I] = h2 * c.c2i;
+                    nv[N_FPR] = eh * fpr;
+                    nv[N_FPI] = eh * (g1i + h2 * c.c3i);
+                    nv[N_FMR] = eh * fmr;
+                    nv[N_FMI] = eh * (-g1i + h2 * c.c3i);
+                    nv[N_KP] = eh * kp;
+                    nv[N_KM] = eh * km;
+                }
+            }
+            if (i < Nr - 1) {   // half node r*_{i+1/2}, Eq. (lw1), step dt/2
+                const Raw c = raw_half ? raw_from(raw_half, Nth, Nr, jp, i)
+                                       : raw_coefficients(P, rad + (size_t)(Nr + i) * kRadial, A);
+                c4h = c.c4;
+                const double dtau = 0.5 * dt, e2 = 0.5 * dtau;
+                const double B = dtau * c.b / drs;
+                const double g1r = dtau * c.c1r / drs, g1i = dtau * c.c1i / drs;
                 double kp, km;
                 if (variable == 0) {
-                    kp = h2 * (c.c4 * ith2 + c.c5 * i2th);
-                    km = h2 * (c.c4 * ith2 - c.c5 * i2th);
+                    kp = e2 * (c.c4 * ith2 + c.c5 * i2th);
+                    km = e2 * (c.c4 * ith2 - c.c5 * i2th);
                 } else {
-                    kp = h2 * c.c4 * Ap;
-                    km = h2 * c.c4 * Am;
+                    kp = e2 * c.c4 * Ap;
+                    km = e2 * c.c4 * Am;
                 }
                 const double dg = kp + km;
-                double fpr = g1r + h2 * c.c3r - dg, fmr = -g1r + h2 * c.c3r - dg;
-                if (variable == 0 && jp == 0) { fpr += p * km; fmr += p * km; km = 0.0; }
-                if (variable == 0 && jp == Nth - 1) { fpr += p * kp; fmr += p * kp; kp = 0.0; }
-                // entries that multiply half-node Phi values carry the factor eh
-                // (the half node returns Phi / eh, see the half-node tables)
-                const double eh = 0.25 * dt;
-                nv[N_B] = eh * B;
-                nv[N_PPR] = B + h2 * c.c2r;
-                nv[N_PMR] = -B + h2 * c.c2r;
-                nv[N_C2I] = h2 * c.c2i;
-                nv[N_FPR] = eh * fpr;
-                nv[N_FPI] = eh * (g1i + h2 * c.c3i);
-                nv[N_FMR] = eh * fmr;
-                nv[N_FMI] = eh * (-g1i + h2 * c.c3i);
-                nv[N_KP] = eh * kp;
-                nv[N_KM] = eh * km;
+                double far = -g1r + e2 * c.c3r - dg, fcr = g1r + e2 * c.c3r - dg;
+                if (variable == 0 && jp == 0) { far += p * km; fcr += p * km; km = 0.0; }
+                if (variable == 0 && jp == Nth - 1) { far += p * kp; fcr += p * kp; kp = 0.0; }
+                // the Phi half-node value is returned divided by e2 (= eh): its
+                // Pi term e2 (Pi_a + Pi_c) then needs no multiplication
+                hv[H_HP] = (0.5 + B) / e2;
+                hv[H_HQ] = (0.5 - B) / e2;
+                hv[H_PAR] = 0.5 - B + e2 * c.c2r;
+                hv[H_PCR] = 0.5 + B + e2 * c.c2r;
+                hv[H_PI] = e2 * c.c2i;
+                hv[H_FAR] = far;
+                hv[H_FAI] = -g1i + e2 * c.c3i;
+                hv[H_FCR] = fcr;
+                hv[H_FCI] = g1i + e2 * c.c3i;
+                hv[H_KP] = kp;
+                hv[H_KM] = km;
+            }
+        } else if (i == 0 && w_row) {
+            w_row[jp] = 0.0;
+        }
+        if (step) {
+            const double hd[kStepHalfF64] = {hv[H_HP], hv[H_HQ], hv[H_PAR], hv[H_PCR], hv[H_PI]};
+            const double hs[kSplitEntries] = {hv[H_FAR], hv[H_FCR], hv[H_KP], hv[H_KM], hv[H_FAI], hv[H_FCI]};
+            const double nd[kStepNodeF64] = {nv[N_B], nv[N_PPR], nv[N_PMR], nv[N_C2I]};
+            const double ns[kSplitEntries] = {nv[N_FMR], nv[N_FPR], nv[N_KP], nv[N_KM], nv[N_FMI], nv[N_FPI]};
+            int ex[2][2];
+            int cold = 0;
+            for (int w = 0; w < 2; ++w) {
+                const double *v = w ? ns : hs;
+                ex[w][0] = class_exponent((fabs(v[S_FA]) + fabs(v[S_FC])) + 2.0 * (fabs(v[S_KP]) + fabs(v[S_KM])),
+                                          &cold);
+                ex[w][1] = class_exponent(fabs(v[S_GA]) + fabs(v[S_GC]), &cold);
+            }
+            // plain stores of the same value
+            if (cold) flags[threadIdx.y][0] = 1;
+            if (ex[0][1] != kSplitAbsent || ex[1][1] != kSplitAbsent || hv[H_PI] != 0.0 || nv[N_C2I] != 0.0)
+                flags[threadIdx.y][1] = 1;
+            __syncthreads();
+            if (i < Nr) {
+                const int lane = jp & 31;
+                unsigned char *block = step + ((size_t)i * (NP / 32) + jp / 32) * kStepBytes;
+                double *d = reinterpret_cast<double *>(block) + lane;
+                auto entries = [&](const double *v, const int (&e)[2]) {
+                    for (int q = 0; q < kSplitEntries; ++q, d += 32)
+                        *reinterpret_cast<int2 *>(d) = flags[threadIdx.y][0] ? make_int2(0, 0)
+                                                                             : split_entry(v[q], e[q >= S_GA]);
+                };
+                for (int q = 0; q < kStepHalfF64; ++q, d += 32) *d = hd[q];
+                entries(hs, ex[0]);
+                for (int q = 0; q < kStepNodeF64; ++q, d += 32) *d = nd[q];
+                entries(ns, ex[1]);
+                int *x = reinterpret_cast<int *>(block + kStepExps);
+                for (int w = 0; w < 2; ++w) x[32 * w + lane] = (ex[w][0] & 0xffff) | (ex[w][1] << 16);
+                if (lane < 4) x[64 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
             }
         }
-        if (i < Nr - 1) {   // half node r*_{i+1/2}, Eq. (lw1), step dt/2
-            const Raw c = raw_half ? raw_from(raw_half, Nth, Nr, jp, i)
-                                   : raw_coefficients(P, variable, x_half[i], th);
-            c4h = c.c4;
-            const double dtau = 0.5 * dt, e2 = 0.5 * dtau;
-            const double B = dtau * c.b / drs;
-            const double g1r = dtau * c.c1r / drs, g1i = dtau * c.c1i / drs;
-            double kp, km;
-            if (variable == 0) {
-                kp = e2 * (c.c4 * ith2 + c.c5 * i2th);
-                km = e2 * (c.c4 * ith2 - c.c5 * i2th);
-            } else {
-                kp = e2 * c.c4 * Ap;
-                km = e2 * c.c4 * Am;
+        if (i >= Nr) continue;
+        if constexpr (sizeof(T) == 4) {
+            // FP32: sixteen entries rounded from FP64, the other five derived from
+            // them in FP32 exactly as the compact-table kernel derives them
+            float cv[kNCC];
+            cv[C_HP] = (float)hv[H_HP];
+            cv[C_PAR] = (float)hv[H_PAR];
+            cv[C_PI] = (float)hv[H_PI];
+            cv[C_FAR] = (float)hv[H_FAR];
+            cv[C_FAI] = (float)hv[H_FAI];
+            cv[C_FCR] = (float)hv[H_FCR];
+            cv[C_FCI] = (float)hv[H_FCI];
+            cv[C_C4H] = (jp < Nth && i < Nr - 1) ? (float)(0.25 * dt * c4h) : 0.0f;
+            cv[C_B] = (float)nv[N_B];
+            cv[C_PMR] = (float)nv[N_PMR];
+            cv[C_C2I] = (float)nv[N_C2I];
+            cv[C_FPR] = (float)nv[N_FPR];
+            cv[C_FPI] = (float)nv[N_FPI];
+            cv[C_FMR] = (float)nv[N_FMR];
+            cv[C_FMI] = (float)nv[N_FMI];
+            cv[C_C4N] = (jp < Nth && i > 0 && i < Nr - 1) ? (float)(0.25 * dt * 0.5 * dt * c4n) : 0.0f;
+            const float gp = (float)gpv, gm = (float)gmv;
+            if (i == 0 && gpm) {
+                gpm[jp] = gp;
+                gpm[NP + jp] = gm;
             }
-            const double dg = kp + km;
-            double far = -g1r + e2 * c.c3r - dg, fcr = g1r + e2 * c.c3r - dg;
-            if (variable == 0 && jp == 0) { far += p * km; fcr += p * km; km = 0.0; }
-            if (variable == 0 && jp == Nth - 1) { far += p * kp; fcr += p * kp; kp = 0.0; }
-            // the Phi half-node value is returned divided by e2 (= eh): its
-            // Pi term e2 (Pi_a + Pi_c) then needs no multiplication
-            hv[H_HP] = (0.5 + B) / e2;
-            hv[H_HQ] = (0.5 - B) / e2;
-            hv[H_PAR] = 0.5 - B + e2 * c.c2r;
-            hv[H_PCR] = 0.5 + B + e2 * c.c2r;
-            hv[H_PI] = e2 * c.c2i;
-            hv[H_FAR] = far;
-            hv[H_FAI] = -g1i + e2 * c.c3i;
-            hv[H_FCR] = fcr;
-            hv[H_FCI] = g1i + e2 * c.c3i;
-            hv[H_KP] = kp;
-            hv[H_KM] = km;
+            float h32[kNCH], n32[kNCN];
+            h32[H_HP] = cv[C_HP];
+            h32[H_HQ] = __fadd_rn(fd.ih, -cv[C_HP]);
+            h32[H_PAR] = cv[C_PAR];
+            h32[H_PCR] = __fadd_rn(cv[C_PAR], __fmaf_rn(fd.t2, cv[C_HP], -1.0f));
+            h32[H_PI] = cv[C_PI];
+            h32[H_FAR] = cv[C_FAR];
+            h32[H_FAI] = cv[C_FAI];
+            h32[H_FCR] = cv[C_FCR];
+            h32[H_FCI] = cv[C_FCI];
+            h32[H_KP] = __fmul_rn(cv[C_C4H], gp);
+            h32[H_KM] = __fmul_rn(cv[C_C4H], gm);
+            n32[N_B] = cv[C_B];
+            n32[N_PPR] = __fmaf_rn(fd.bn2, cv[C_B], cv[C_PMR]);
+            n32[N_PMR] = cv[C_PMR];
+            n32[N_C2I] = cv[C_C2I];
+            n32[N_FPR] = cv[C_FPR];
+            n32[N_FPI] = cv[C_FPI];
+            n32[N_FMR] = cv[C_FMR];
+            n32[N_FMI] = cv[C_FMI];
+            n32[N_KP] = __fmul_rn(cv[C_C4N], gp);
+            n32[N_KM] = __fmul_rn(cv[C_C4N], gm);
+            for (int q = 0; q < kNCH; ++q) hcol[(size_t)q * NP] = h32[q];
+            for (int q = 0; q < kNCN; ++q) ncol[(size_t)q * NP] = n32[q];
+            if (cmp) {
+                float *ccol = cmp + (size_t)i * kNCC * NP + jp;
+                for (int q = 0; q < kNCC; ++q) ccol[(size_t)q * NP] = cv[q];
+            }
+        } else {
+            for (int q = 0; q < kNCH; ++q) hcol[(size_t)q * NP] = (T)hv[q];
+            for (int q = 0; q < kNCN; ++q) ncol[(size_t)q * NP] = (T)nv[q];
         }
-    } else if (i == 0 && w_row) {
-        w_row[jp] = 0.0;
+        b_node[(size_t)i * NP + jp] = bn;
     }
-    if (step) {
-        const double hd[kStepHalfF64] = {hv[H_HP], hv[H_HQ], hv[H_PAR], hv[H_PCR], hv[H_PI]};
-        const double hs[kSplitEntries] = {hv[H_FAR], hv[H_FCR], hv[H_KP], hv[H_KM], hv[H_FAI], hv[H_FCI]};
-        const double nd[kStepNodeF64] = {nv[N_B], nv[N_PPR], nv[N_PMR], nv[N_C2I]};
-        const double ns[kSplitEntries] = {nv[N_FMR], nv[N_FPR], nv[N_KP], nv[N_KM], nv[N_FMI], nv[N_FPI]};
-        int ex[2][2];
-        int cold = 0;
-        for (int w = 0; w < 2; ++w) {
-            const double *v = w ? ns : hs;
-            ex[w][0] = class_exponent((fabs(v[S_FA]) + fabs(v[S_FC])) + 2.0 * (fabs(v[S_KP]) + fabs(v[S_KM])), &cold);
-            ex[w][1] = class_exponent(fabs(v[S_GA]) + fabs(v[S_GC]), &cold);
-        }
-        // plain stores of the same value
-        if (cold) flags[threadIdx.y][0] = 1;
-        if (ex[0][1] != kSplitAbsent || ex[1][1] != kSplitAbsent || hv[H_PI] != 0.0 || nv[N_C2I] != 0.0)
-            flags[threadIdx.y][1] = 1;
-        __syncthreads();
-        if (i < Nr) {
-            const int lane = jp & 31;
-            unsigned char *block = step + ((size_t)i * (NP / 32) + jp / 32) * kStepBytes;
-            double *d = reinterpret_cast<double *>(block) + lane;
-            auto entries = [&](const double *v, const int (&e)[2]) {
-                for (int q = 0; q < kSplitEntries; ++q, d += 32)
-                    *reinterpret_cast<int2 *>(d) = flags[threadIdx.y][0] ? make_int2(0, 0)
-                                                                         : split_entry(v[q], e[q >= S_GA]);
-            };
-            for (int q = 0; q < kStepHalfF64; ++q, d += 32) *d = hd[q];
-            entries(hs, ex[0]);
-            for (int q = 0; q < kStepNodeF64; ++q, d += 32) *d = nd[q];
-            entries(ns, ex[1]);
-            int *x = reinterpret_cast<int *>(block + kStepExps);
-            for (int w = 0; w < 2; ++w) x[32 * w + lane] = (ex[w][0] & 0xffff) | (ex[w][1] << 16);
-            if (lane < 4) x[64 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
-        }
-    }
-    if (i >= Nr) return;
-    if constexpr (sizeof(T) == 4) {
-        // FP32: sixteen entries rounded from FP64, the other five derived from
-        // them in FP32 exactly as the compact-table kernel derives them
-        float cv[kNCC];
-        cv[C_HP] = (float)hv[H_HP];
-        cv[C_PAR] = (float)hv[H_PAR];
-        cv[C_PI] = (float)hv[H_PI];
-        cv[C_FAR] = (float)hv[H_FAR];
-        cv[C_FAI] = (float)hv[H_FAI];
-        cv[C_FCR] = (float)hv[H_FCR];
-        cv[C_FCI] = (float)hv[H_FCI];
-        cv[C_C4H] = (jp < Nth && i < Nr - 1) ? (float)(0.25 * dt * c4h) : 0.0f;
-        cv[C_B] = (float)nv[N_B];
-        cv[C_PMR] = (float)nv[N_PMR];
-        cv[C_C2I] = (float)nv[N_C2I];
-        cv[C_FPR] = (float)nv[N_FPR];
-        cv[C_FPI] = (float)nv[N_FPI];
-        cv[C_FMR] = (float)nv[N_FMR];
-        cv[C_FMI] = (float)nv[N_FMI];
-        cv[C_C4N] = (jp < Nth && i > 0 && i < Nr - 1) ? (float)(0.25 * dt * 0.5 * dt * c4n) : 0.0f;
-        const float gp = (float)gpv, gm = (float)gmv;
-        if (i == 0 && gpm) {
-            gpm[jp] = gp;
-            gpm[NP + jp] = gm;
-        }
-        float h32[kNCH], n32[kNCN];
-        h32[H_HP] = cv[C_HP];
-        h32[H_HQ] = __fadd_rn(fd.ih, -cv[C_HP]);
-        h32[H_PAR] = cv[C_PAR];
-        h32[H_PCR] = __fadd_rn(cv[C_PAR], __fmaf_rn(fd.t2, cv[C_HP], -1.0f));
-        h32[H_PI] = cv[C_PI];
-        h32[H_FAR] = cv[C_FAR];
-        h32[H_FAI] = cv[C_FAI];
-        h32[H_FCR] = cv[C_FCR];
-        h32[H_FCI] = cv[C_FCI];
-        h32[H_KP] = __fmul_rn(cv[C_C4H], gp);
-        h32[H_KM] = __fmul_rn(cv[C_C4H], gm);
-        n32[N_B] = cv[C_B];
-        n32[N_PPR] = __fmaf_rn(fd.bn2, cv[C_B], cv[C_PMR]);
-        n32[N_PMR] = cv[C_PMR];
-        n32[N_C2I] = cv[C_C2I];
-        n32[N_FPR] = cv[C_FPR];
-        n32[N_FPI] = cv[C_FPI];
-        n32[N_FMR] = cv[C_FMR];
-        n32[N_FMI] = cv[C_FMI];
-        n32[N_KP] = __fmul_rn(cv[C_C4N], gp);
-        n32[N_KM] = __fmul_rn(cv[C_C4N], gm);
-        for (int q = 0; q < kNCH; ++q) hcol[(size_t)q * NP] = h32[q];
-        for (int q = 0; q < kNCN; ++q) ncol[(size_t)q * NP] = n32[q];
-        if (cmp) {
-            float *ccol = cmp + (size_t)i * kNCC * NP + jp;
-            for (int q = 0; q < kNCC; ++q) ccol[(size_t)q * NP] = cv[q];
-        }
-    } else {
-        for (int q = 0; q < kNCH; ++q) hcol[(size_t)q * NP] = (T)hv[q];
-        for (int q = 0; q < kNCN; ++q) ncol[(size_t)q * NP] = (T)nv[q];
-    }
-    b_node[(size_t)i * NP + jp] = bn;
 }
 
 // The raw coefficients the precompute forms, [9][Nth][Nr] in the order of Raw,
 // at the nodes and (column i < Nr - 1) the half nodes r*_{i+1/2}; column
 // Nr - 1 of the half table is zero.  Grid-stride over the Nth * Nr points.
 __global__ void raw_export_kernel(Kerr KP, int variable, int Nr, int Nth,
-                                  const double *__restrict__ x_node, const double *__restrict__ x_half,
-                                  double *__restrict__ out_node, double *__restrict__ out_half)
+                                  const double *__restrict__ rad, double *__restrict__ out_node,
+                                  double *__restrict__ out_half)
 {
     const Geo P = geometry(KP);
     const size_t plane = (size_t)Nth * Nr;
@@ -445,11 +508,12 @@ __global__ void raw_export_kernel(Kerr KP, int variable, int Nr, int Nth,
          k += (size_t)gridDim.x * blockDim.x) {
         const int jp = (int)(k / Nr), i = (int)(k % Nr);
         const double th = (jp + 0.5) * (M_PI / Nth);
-        const Raw c = raw_coefficients(P, variable, x_node[i], th);
+        const Angular A = angular_part(P, variable, th);
+        const Raw c = raw_coefficients(P, rad + (size_t)i * kRadial, A);
         const double v[9] = {c.b, c.c1r, c.c1i, c.c2r, c.c2i, c.c3r, c.c3i, c.c4, c.c5};
         for (int q = 0; q < 9; ++q) out_node[q * plane + k] = v[q];
         Raw h = {};
-        if (i < Nr - 1) h = raw_coefficients(P, variable, x_half[i], th);
+        if (i < Nr - 1) h = raw_coefficients(P, rad + (size_t)(Nr + i) * kRadial, A);
         const double w[9] = {h.b, h.c1r, h.c1i, h.c2r, h.c2i, h.c3r, h.c3i, h.c4, h.c5};
         for (int q = 0; q < 9; ++q) out_half[q * plane + k] = w[q];
     }
@@ -461,7 +525,7 @@ __global__ void raw_export_kernel(Kerr KP, int variable, int Nr, int Nth,
 // maxima are written as the bit patterns of non-negative doubles, which order
 // like unsigned integers: out[0] = max omega^2, out[1] = max b.
 __global__ void stiffness_kernel(Kerr KP, int variable, int Nr, int Nth, int NP,
-                                 const double *__restrict__ x_node, const double *__restrict__ ang,
+                                 const double *__restrict__ rad, const double *__restrict__ ang,
                                  unsigned long long *__restrict__ out)
 {
     const int jp = blockIdx.x * blockDim.x + threadIdx.x;
@@ -471,7 +535,7 @@ __global__ void stiffness_kernel(Kerr KP, int variable, int Nr, int Nth, int NP,
         const Geo P = geometry(KP);
         const double dth = M_PI / Nth;
         const double th = (jp + 0.5) * dth;
-        const Raw c = raw_coefficients(P, variable, x_node[i], th);
+        const Raw c = raw_coefficients(P, rad + (size_t)i * kRadial, angular_part(P, variable, th));
         const double asum = (variable != 0) ? ang[jp] + ang[NP + jp] : 2.0 / (dth * dth);
         w2 = sqrt(c.c3r * c.c3r + c.c3i * c.c3i) + 2.0 * c.c4 * asum;
         bb = c.b;
@@ -490,56 +554,57 @@ __global__ void stiffness_kernel(Kerr KP, int variable, int Nr, int Nth, int NP,
 }  // namespace
 
 cudaError_t launch_stiffness(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                             const double *x_node, const double *ang, unsigned long long *out,
+                             const double *rad, const double *ang, unsigned long long *out,
                              cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     dim3 block(32, 8), grid((NP + 31) / 32, (Nr + 7) / 8);
-    stiffness_kernel<<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, x_node, ang, out);
+    stiffness_kernel<<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, rad, ang, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *x_node,
-                              const double *x_half, double *out_node, double *out_half, cudaStream_t st)
+cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *rad, double *out_node,
+                              double *out_half, cudaStream_t st)
 {
     const size_t n = (size_t)Ntheta * Nr;
     const int blocks = (int)std::min<size_t>((n + 255) / 256, 152 * 8);
-    raw_export_kernel<<<blocks, 256, 0, st>>>(P, variable, Nr, Ntheta, x_node, x_half, out_node, out_half);
+    raw_export_kernel<<<blocks, 256, 0, st>>>(P, variable, Nr, Ntheta, rad, out_node, out_half);
     return cudaGetLastError();
 }
 
-cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr,
-                                   double *x_node, double *x_half, cudaStream_t st)
+cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr, double *rad, cudaStream_t st)
 {
+    // one warp per block: few warps, each a serial chain, over all the SMs
     const int n = 2 * Nr - 1;
-    invert_tortoise_kernel<<<(n + 127) / 128, 128, 0, st>>>(P, rs_min, drs, Nr, x_node, x_half);
+    invert_tortoise_kernel<<<(n + 31) / 32, 32, 0, st>>>(P, rs_min, drs, Nr, rad);
     return cudaGetLastError();
 }
 
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                                double drs, double dt_inner, const double *x_node,
-                                const double *x_half, double *ang, int precision, void *half,
+                                double drs, double dt_inner, const double *rad, double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node, const double *raw_half,
                                 bool ang_given, unsigned char *step)
 {
     const F32Derive fd = f32_derive(dt_inner);
     if (variable != 0 && !ang_given) {
-        regular_stencil_kernel<<<NP, 32, 0, st>>>(P.s, P.m, Ntheta, NP, ang);
-        cudaError_t e = cudaGetLastError();
+        // chained to the tortoise inversion, of which it needs nothing (and which
+        // started after every earlier use of ang): the two run side by side
+        cudaError_t e = launch_chained(regular_stencil_kernel, (unsigned)NP, 4 * kStencilPanels, 0, st, P.s, P.m, Ntheta,
+                                       NP, ang);
         if (e != cudaSuccess) return e;
     }
     dim3 block(NP, kTableThreads / NP);
-    dim3 grid((Nr + block.y - 1) / block.y);
+    dim3 grid(std::min<unsigned>((Nr + block.y - 1) / block.y, 152 * 4));
     if (precision == 0)
         coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
-                                                             x_node, x_half, ang, (double *)half,
+                                                             rad, ang, (double *)half,
                                                              (double *)node, b_node, w_row, nullptr,
                                                              nullptr, fd, raw_node, raw_half, step);
     else
         coeff_tables_kernel<float><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
-                                                            x_node, x_half, ang, (float *)half,
+                                                            rad, ang, (float *)half,
                                                             (float *)node, b_node, w_row, cmp, gpm, fd,
                                                             raw_node, raw_half, nullptr);
     return cudaGetLastError();

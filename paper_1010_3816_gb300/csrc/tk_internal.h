@@ -125,17 +125,18 @@ struct WaveRead {
 };
 
 // ---- coefficient precompute (tk_coeffs.cu) ----
-cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr,
-                                   double *x_node, double *x_half, cudaStream_t st);
+// rad: the radial parts of the coefficients, kRadial doubles per radius, nodes
+// r*_i in rad[i], half nodes r*_{i+1/2} (i < Nr - 1) in rad[Nr + i].
+constexpr int kRadial = 12;
+cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr, double *rad, cudaStream_t st);
 // FP32 (precision 1) also writes the compact tables cmp and the theta
 // factors gpm[2][NP] (gp, then gm); both may be NULL for FP64.  raw_node,
 // raw_half (device, [9][Ntheta][Nr], half node i at r*_{i+1/2}): coefficients
-// supplied by the caller instead of computed (x_node, x_half then unused);
+// supplied by the caller instead of computed (rad then unused);
 // ang_given: ang already holds the regularised stencil.  step: the FP64
 // step's tables (NULL: not wanted).
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                                double drs, double dt_inner, const double *x_node,
-                                const double *x_half, double *ang, int precision, void *half,
+                                double drs, double dt_inner, const double *rad, double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node = nullptr,
                                 const double *raw_half = nullptr, bool ang_given = false,
@@ -143,11 +144,11 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
 
 // The raw coefficients of the precompute, [9][Ntheta][Nr] at nodes and half
 // nodes (device output buffers).
-cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *x_node,
-                              const double *x_half, double *out_node, double *out_half, cudaStream_t st);
+cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *rad,
+                              double *out_node, double *out_half, cudaStream_t st);
 
 cudaError_t launch_stiffness(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                             const double *x_node, const double *ang, unsigned long long *out,
+                             const double *rad, const double *ang, unsigned long long *out,
                              cudaStream_t st);
 
 // ---- state import / export (tk_layout.cu) ----

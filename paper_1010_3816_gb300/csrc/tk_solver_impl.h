@@ -21,7 +21,8 @@ struct tk_solver {
     void *half = nullptr, *node = nullptr;
     float *cmp = nullptr, *gpm = nullptr;   // FP32: compact tables, theta factors (tk_internal.h)
     unsigned char *step = nullptr;   // FP64: the step's tables (tk_internal.h)
-    double *b_node = nullptr, *w_row = nullptr, *x_node = nullptr, *x_half = nullptr;
+    double *b_node = nullptr, *w_row = nullptr;
+    double *rad = nullptr;      // radial parts of the coefficients (tk_internal.h)
     double *ang = nullptr;      // regularised angular stencil [2][NP]
     double *staging = nullptr;  // 4 * Nth * Nr doubles, for host transfers
     int *flag = nullptr;
