@@ -47,9 +47,10 @@
 // 20 warps (96 registers, spills): 120 us.
 //
 // Subnormal values count as zero in the coupling, and a coupling below 2^-1022
-// is dropped.  Columns with a value above 1e263, an infinity or a NaN, and columns whose tables are not
-// finite or too large, take the FP64 instructions alone, so that such values
-// propagate as IEEE arithmetic has them.
+// is dropped.  Columns with a Phi above 1e263, infinite or NaN, and columns whose
+// tables are not finite or too large, take the FP64 instructions alone, so that
+// such values propagate as IEEE arithmetic has them; Pi only ever meets FP64
+// instructions (testing it too took 89.6 instead of 88.8 us on 25601 x 64).
 #pragma once
 
 #include "tk_split_tables.cuh"
@@ -67,7 +68,6 @@ struct SplitInts {
     long long x[2];
     int e[2];
     int j[2];
-    unsigned top;   // largest high word of the row's four magnitudes
 };
 
 __device__ __forceinline__ int nonzero(int hi, int lo) { return (int)min((unsigned)(hi | lo), 1u); }
@@ -105,12 +105,9 @@ __device__ __forceinline__ int2 limbs(long long x)
 template <int C0>
 __device__ __forceinline__ void split_ints(const double (&u)[4], SplitInts &o)
 {
-    unsigned top = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = C0; k < C0 + 2; ++k) {
         const unsigned hi = (unsigned)__double2hiint(u[k]);
-        top = max(top, hi & 0x7fffffffu);
-        if (k < C0 || k >= C0 + 2) continue;
         const unsigned lo = (unsigned)__double2loint(u[k]);
         const int e = (int)((hi >> 20) & 0x7ffu), j = min(e, 1);
         const unsigned m = (hi & 0xfffffu) | 0x100000u;
@@ -120,7 +117,6 @@ __device__ __forceinline__ void split_ints(const double (&u)[4], SplitInts &o)
         o.e[k - C0] = e;
         o.j[k - C0] = j;
     }
-    o.top = top;
 }
 
 // The accumulators of a class's sum.
@@ -271,7 +267,7 @@ __device__ __forceinline__ bool split_coupling(const SplitInts &a, const SplitIn
     int2 eu2, ed2;
     const bool over =
         team.exchange(make_int4(sh[0], sl[0], sh[1], sl[1]), make_int2(e1[0], e1[1]),
-                      cold || max(a.top, c.top) >= ((unsigned)kSplitMaxExp << 20), su, eu2, sd, ed2);
+                      cold || max(e1[0], e1[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
     if (over) return false;
     const int rx = tab.row_exp();
     long long G[2];   // the other part's share

@@ -167,7 +167,7 @@ __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF
     int2 eu2, ed2;
     const bool hot = team.exchange(
         make_int4((int)(p.x[0] >> 32), (int)p.x[0], (int)(p.x[1] >> 32), (int)p.x[1]), make_int2(p.e[0], p.e[1]),
-        p.top >= ((unsigned)kSplitMaxExp << 20), su, eu2, sd, ed2);
+        max(p.e[0], p.e[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
     const int rx = tab.row_exp();
     AdjSums g1, g2;
 #pragma unroll
