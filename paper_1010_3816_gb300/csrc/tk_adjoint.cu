@@ -22,6 +22,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "tk_solver_impl.h"
@@ -666,14 +667,30 @@ __global__ void initial_transpose_kernel(int Nr, int Nth, int NP, double drs,
 // where N' is the node update with the derivative tables and no constant
 // terms, h' = H' u the half nodes with the derivative tables, and N applies
 // the ordinary node tables to h'.  One warp per column range, recomputing
-// its left edge; every block adds its partial sum to its own slot of acc, so
-// the sum is in a fixed order.
+// its left edge.
+//
+// One launch contracts up to kLamSteps successive steps, blockIdx.y = q the
+// transpose's steps first + q of a segment (counted from its end, whose last
+// sample is t_last): u^j at u_last - q * (one state), lam~ in lams.p[q].  Every
+// block writes its partial sum to its own slot, [q][block], and
+// tangent_sum_kernel adds them to acc in the order of the steps, so that the
+// sum does not depend on how the steps are grouped (nor the split into blocks,
+// a function of Nr alone).  Bound by the FP64 pipe: with a launch per step a
+// 1601 x 32 grid had one column per warp, which forms two half nodes to use
+// one, 20.8 us a step; with several steps a launch a warp can take more
+// columns (four from 1536 radii on; fewer below, where the shortest checkpoint
+// interval would leave the chip idle), 11.7 us.
+constexpr int kLamSteps = 8;
+struct LamSet {
+    const double *p[kLamSteps];
+};
+
 template <int K>
 __global__ void __launch_bounds__(128)
-param_tangent_kernel(const double *__restrict__ u, const double *__restrict__ lam,
-                     const double *__restrict__ half, const double *__restrict__ node,
+param_tangent_kernel(const double *__restrict__ u_last, const __grid_constant__ LamSet lams, long long first, long long t_last,
+                     int substeps, const double *__restrict__ half, const double *__restrict__ node,
                      const double *__restrict__ dhalf, const double *__restrict__ dnode, int Nr,
-                     double eh, double en, const InjectArgs inj, double *__restrict__ acc)
+                     double eh, double en, const InjectArgs inj, double *__restrict__ part_sums)
 {
     constexpr int NP = 32 * K;
     constexpr size_t SP = 4 * NP, HP = (size_t)kNCH * NP, NQ = (size_t)kNCN * NP;
@@ -683,6 +700,10 @@ param_tangent_kernel(const double *__restrict__ u, const double *__restrict__ la
     int i0, i1, left;
     warp_range<4>(Nr, wib, &i0, &i1, &left);
     const int row = lane * K;
+    const int q = blockIdx.y;
+    const double *__restrict__ u = u_last - (size_t)q * Nr * SP, *__restrict__ lam = lams.p[q];
+    const int on = (first + q) % substeps == 0;
+    const long long sample = t_last - (first + q) / substeps;
     double sum = 0.0;
     if (i1 > i0) {
         double ua[4][K], hm[4][K], dm[4][K], zero[4][K];
@@ -712,7 +733,7 @@ param_tangent_kernel(const double *__restrict__ u, const double *__restrict__ la
                 double d1[4][K], d2[4][K], l[4][K];
                 full_node<double, K>(hm, hp, zero, dnode + (size_t)i * NQ + row, 0.0, d1);
                 full_node<double, K>(dm, dp, zero, node + (size_t)i * NQ + row, en, d2);
-                load_lam<double, K>(lam, i, Nr, lane, inj, inj.on, inj.sample, l);
+                load_lam<double, K>(lam, i, Nr, lane, inj, on, sample, l);
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -732,7 +753,18 @@ param_tangent_kernel(const double *__restrict__ u, const double *__restrict__ la
     for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     if (lane == 0) part[wib] = sum;
     __syncthreads();
-    if (threadIdx.x == 0) acc[blockIdx.x] += (part[0] + part[1]) + (part[2] + part[3]);
+    if (threadIdx.x == 0)
+        part_sums[(size_t)q * gridDim.x + blockIdx.x] = (part[0] + part[1]) + (part[2] + part[3]);
+}
+
+__global__ void tangent_sum_kernel(const double *__restrict__ part_sums, int blocks, int steps,
+                                   double *__restrict__ acc)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= blocks) return;
+    double s = acc[k];
+    for (int q = 0; q < steps; ++q) s += part_sums[(size_t)q * blocks + k];
+    acc[k] = s;
 }
 
 // Initial-data term for a momentum derived from Phi^0: Pi^0 = b d_* Phi^0
@@ -766,33 +798,23 @@ __global__ void param_initial_kernel(int Nr, int Nth, int NP, const double *__re
     }
 }
 
-// dst += w * src over n doubles.
-__global__ void axpy_kernel(size_t n, double w, const double *__restrict__ src, double *__restrict__ dst)
-{
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x)
-        dst[k] = fma(w, src[k], dst[k]);
-}
-
-cudaError_t launch_axpy(size_t n, double w, const double *src, double *dst, cudaStream_t st)
-{
-    size_t blocks = (n + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    axpy_kernel<<<(unsigned)blocks, 256, 0, st>>>(n, w, src, dst);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_param_tangent(int K, int blocks, const double *u, const double *lam,
-                                 const double *half, const double *node, const double *dhalf,
-                                 const double *dnode, int Nr, double dt_in, const InjectArgs &inj,
-                                 double *acc, cudaStream_t st)
+cudaError_t launch_param_tangent(int K, int blocks, int steps, const double *u_last, const LamSet &lams, long long first,
+                                 long long t_last, int substeps, const double *half, const double *node,
+                                 const double *dhalf, const double *dnode, int Nr, double dt_in,
+                                 const InjectArgs &inj, double *part_sums, double *acc, cudaStream_t st)
 {
     const double eh = 0.25 * dt_in, en = 0.5 * dt_in;
+    const dim3 grid(blocks, steps);
     if (K == 1)
-        param_tangent_kernel<1><<<blocks, 128, 0, st>>>(u, lam, half, node, dhalf, dnode, Nr, eh, en, inj, acc);
+        param_tangent_kernel<1><<<grid, 128, 0, st>>>(u_last, lams, first, t_last, substeps, half, node, dhalf, dnode,
+                                                      Nr, eh, en, inj, part_sums);
     else if (K == 2)
-        param_tangent_kernel<2><<<blocks, 128, 0, st>>>(u, lam, half, node, dhalf, dnode, Nr, eh, en, inj, acc);
+        param_tangent_kernel<2><<<grid, 128, 0, st>>>(u_last, lams, first, t_last, substeps, half, node, dhalf, dnode,
+                                                      Nr, eh, en, inj, part_sums);
     else
-        param_tangent_kernel<4><<<blocks, 128, 0, st>>>(u, lam, half, node, dhalf, dnode, Nr, eh, en, inj, acc);
+        param_tangent_kernel<4><<<grid, 128, 0, st>>>(u_last, lams, first, t_last, substeps, half, node, dhalf, dnode,
+                                                      Nr, eh, en, inj, part_sums);
+    tangent_sum_kernel<<<(blocks + 127) / 128, 128, 0, st>>>(part_sums, blocks, steps, acc);
     return cudaGetLastError();
 }
 
@@ -1201,13 +1223,17 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     const size_t nh = (size_t)S->Nr * tk::kNCH * S->NP, nn = (size_t)S->Nr * tk::kNCN * S->NP;
     const size_t nb = (size_t)S->Nr * S->NP;
 
-    // scratch, freed on every exit
-    double *dwave = nullptr, *thalf = nullptr, *tnode = nullptr, *tb = nullptr, *tw = nullptr;
-    double *tx = nullptr, *tang = nullptr, *ck = nullptr, *seg = nullptr, *acc = nullptr;
+    // the steps contracted per launch: their adjoint states are kept, two in the
+    // solver's own buffers, the others in the scratch (256 MB at most)
+    int Q = (int)std::min<long long>(std::min<long long>(C * k, tk::kLamSteps), 1 + (long long)((256ull << 20) / sb));
+    const int blocks = std::max(1, S->Nr / (4 * std::min(4, 1 + S->Nr / 512))), pblocks = 1024;
+
+    // scratch in one allocation, freed on every exit
+    double *dwave = nullptr, *scratch = nullptr;
+    double *tx = nullptr, *tang = nullptr, *ck = nullptr, *seg = nullptr, *acc = nullptr, *parts = nullptr;
+    double *lam_more = nullptr;
     auto cleanup = [&]() {
-        void *p[] = {thalf, tnode, tb, tw, tx, tang, ck, seg, acc};
-        for (void *q : p)
-            if (q) cudaFree(q);
+        if (scratch) cudaFree(scratch);
         if (dwave && !on_device) cudaFree(dwave);
     };
     auto bail = [&](tk_status s2) {
@@ -1220,13 +1246,28 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     if (!S->dhalf && (st = tkh::alloc(S, (void **)&S->dhalf, nh * sizeof(double))) != TK_OK) return bail(st);
     if (!S->dnode && (st = tkh::alloc(S, (void **)&S->dnode, nn * sizeof(double))) != TK_OK) return bail(st);
     if (!S->db_node && (st = tkh::alloc(S, (void **)&S->db_node, nb * sizeof(double))) != TK_OK) return bail(st);
-    if ((st = tkh::alloc(S, (void **)&thalf, nh * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tnode, nn * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tb, nb * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tw, (size_t)S->NP * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tx, (size_t)2 * S->Nr * tk::kRadial * sizeof(double))) != TK_OK ||
-        (st = tkh::alloc(S, (void **)&tang, (size_t)2 * S->NP * sizeof(double))) != TK_OK)
-        return bail(st);
+    // (one allocation: each costs some 70 us with its release); without the
+    // further adjoint states where the memory does not reach
+    for (;; Q = 1) {
+        struct { double **p; size_t n; } piece[] = {
+            {&ck, (size_t)nck * se}, {&seg, (size_t)(C * k) * se}, {&lam_more, (size_t)(Q - 1) * se},
+            {&tx, (size_t)tk::kShifts * 2 * S->Nr * tk::kRadial}, {&tang, (size_t)2 * S->NP},
+            {&acc, (size_t)(blocks + pblocks)}, {&parts, (size_t)Q * blocks}};
+        size_t total = 0;
+        for (auto &x : piece) total += (x.n + 31) / 32 * 32;
+        st = tkh::alloc(S, (void **)&scratch, total * sizeof(double));
+        if (st == TK_OK) {
+            double *at = scratch;
+            for (auto &x : piece) {
+                *x.p = at;
+                at += (x.n + 31) / 32 * 32;
+            }
+            break;
+        }
+        if (Q == 1) return bail(st);
+    }
+    double *lam[tk::kLamSteps + 1];   // a ring of Q + 1 adjoint states
+    for (int q = 0; q <= Q; ++q) lam[q] = q < 2 ? (double *)S->adj[q] : lam_more + (size_t)(q - 2) * se;
     if (on_device) {
         dwave = const_cast<double *>(dL_dwave);
     } else {
@@ -1244,29 +1285,18 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         const double M = S->kerr.M, a = S->kerr.a;
         double d = 1e-3 * M;
         if (d > 0.25 * (M - fabs(a))) d = 0.25 * (M - fabs(a));
-        const double off[4] = {d, -d, 2 * d, -2 * d};
-        const double wgt[4] = {8.0 / (12 * d), -8.0 / (12 * d), -1.0 / (12 * d), 1.0 / (12 * d)};
-        e = cudaMemsetAsync(S->dhalf, 0, nh * sizeof(double), S->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(S->dnode, 0, nn * sizeof(double), S->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(S->db_node, 0, nb * sizeof(double), S->stream);
-        for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
-            tk::Kerr P = S->kerr;
-            if (param == 0) P.a += off[q];
-            else P.M += off[q];
-            e = tk::launch_invert_tortoise(P, S->rs_min, S->drs, S->Nr, tx, S->stream);
-            if (e == cudaSuccess)
-                // the angular stencil depends on s and m only: formed with the first
-                e = tk::launch_coeff_tables(P, S->variable, S->Nr, S->Nth, S->NP, S->drs, dt_in, tx, tang, 0, thalf,
-                                            tnode, tb, tw, nullptr, nullptr, S->stream, nullptr, nullptr, q > 0);
-            if (e == cudaSuccess) e = tk::launch_axpy(nh, wgt[q], thalf, S->dhalf, S->stream);
-            if (e == cudaSuccess) e = tk::launch_axpy(nn, wgt[q], tnode, S->dnode, S->stream);
-            if (e == cudaSuccess) e = tk::launch_axpy(nb, wgt[q], tb, S->db_node, S->stream);
+        const double off[tk::kShifts] = {d, -d, 2 * d, -2 * d};
+        tk::KerrSet kp = {{}, {8.0 / (12 * d), -8.0 / (12 * d), -1.0 / (12 * d), 1.0 / (12 * d)}};
+        for (int q = 0; q < tk::kShifts; ++q) {
+            kp.k[q] = S->kerr;
+            if (param == 0) kp.k[q].a += off[q];
+            else kp.k[q].M += off[q];
         }
+        e = tk::launch_table_derivative(kp, S->variable, S->rs_min, S->Nr, S->Nth, S->NP, S->drs, dt_in, tx, tang,
+                                        S->dhalf, S->dnode, S->db_node, S->stream);
     }
     if (e != cudaSuccess) return bail(tkh::fail(S, TK_ERR_CUDA, "tk_param_gradient: %s", cudaGetErrorString(e)));
     // 2. checkpoints of the trajectory every C outer steps, from u^0
-    if ((st = tkh::alloc(S, (void **)&ck, (size_t)nck * sb)) != TK_OK) return bail(st);
-    if ((st = tkh::alloc(S, (void **)&seg, (size_t)(C * k) * sb)) != TK_OK) return bail(st);
     tk::StepLaunch L;
     tkh::fill_launch(S, L);
     L.write_wave = 0;
@@ -1285,24 +1315,9 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         }
     }
     // 3. backward over the segments: recompute the segment's inner states,
-    //    then the tangent contraction and the adjoint step for each of them
-    int blocks = 0;
-    if (e == cudaSuccess) {
-        const int K = S->K;
-        int per = 0;
-        if (K == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tk::param_tangent_kernel<1>, 128, 0);
-        else if (K == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tk::param_tangent_kernel<2>, 128, 0);
-        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tk::param_tangent_kernel<4>, 128, 0);
-        if (per < 1) per = 1;
-        blocks = S->num_sms * per;
-        if (blocks > S->Nr / 4) blocks = S->Nr / 4;
-        if (blocks < 1) blocks = 1;
-    }
-    const int pblocks = 1024;
-    if (e == cudaSuccess && (st = tkh::alloc(S, (void **)&acc, (size_t)(blocks + pblocks) * sizeof(double))) != TK_OK)
-        return bail(st);
+    //    then, Q steps at a time, the adjoint steps and their tangent contraction
     if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, (size_t)(blocks + pblocks) * sizeof(double), S->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(S->adj[0], 0, sb, S->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(lam[0], 0, sb, S->stream);
     tk::InjectArgs inj;
     memset(&inj, 0, sizeof inj);
     inj.count = count;
@@ -1319,25 +1334,30 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
             L.u_out = seg + (size_t)(j + 1) * se;
             e = tk::launch_lw_step(L, S->stream);
         }
-        for (long long t = t0 + len - 1; t >= t0 && e == cudaSuccess; --t)
-            for (int kk = 0; kk < k && e == cudaSuccess; ++kk) {
-                inj.on = (kk == 0);
-                inj.sample = t;
-                const long long j = (t - t0) * k + (k - 1 - kk);     // u^j is the step's input
-                e = tk::launch_param_tangent(S->K, blocks, seg + (size_t)j * se, (const double *)S->adj[cur],
-                                             (const double *)S->half, (const double *)S->node, S->dhalf,
-                                             S->dnode, S->Nr, dt_in, inj, acc, S->stream);
-                if (e == cudaSuccess)
-                    e = tk::launch_adjoint_step(0, S->K, S->adj[cur], S->adj[cur ^ 1], S->half, S->node,
-                                                S->adj_tab, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
-                cur ^= 1;
+        for (long long g = 0; g < len * k && e == cudaSuccess;) {   // transposed steps from the segment's end
+            const int n = (int)std::min<long long>(Q, len * k - g);
+            tk::LamSet set = {};
+            for (int q = 0; q < n && e == cudaSuccess; ++q) {
+                const int nxt = cur == Q ? 0 : cur + 1;
+                set.p[q] = lam[cur];
+                inj.on = (g + q) % k == 0;
+                inj.sample = t0 + len - 1 - (g + q) / k;
+                e = tk::launch_adjoint_step(0, S->K, lam[cur], lam[nxt], S->half, S->node, S->adj_tab, S->Nr,
+                                            S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
+                cur = nxt;
             }
+            if (e == cudaSuccess)
+                e = tk::launch_param_tangent(S->K, blocks, n, seg + (size_t)(len * k - 1 - g) * se, set, g,
+                                             t0 + len - 1, k, (const double *)S->half, (const double *)S->node,
+                                             S->dhalf, S->dnode, S->Nr, dt_in, inj, parts, acc, S->stream);
+            g += n;
+        }
     }
     // 4. the initial-data term (momentum derived from Phi^0 through b)
     if (e == cudaSuccess && S->init_pi_derived) {
         tk::param_initial_kernel<<<pblocks, 256, 0, S->stream>>>(S->Nr, S->Nth, S->NP,
                                                                   (const double *)S->u_init,
-                                                                  (const double *)S->adj[cur], S->b_node,
+                                                                  lam[cur], S->b_node,
                                                                   S->db_node, acc + blocks);
         e = cudaGetLastError();
     }

@@ -117,10 +117,12 @@ __device__ Radial radial_part(const Geo &P, double x)
 
 // The tortoise inversion and the radial parts: nodes i in rad[i], half nodes
 // i + 1/2 in rad[Nr + i].
-__global__ void invert_tortoise_kernel(Kerr KP, double rs_min, double drs, int Nr, double *rad)
+// Black hole blockIdx.y of the set goes to rad + blockIdx.y 2 Nr kRadial.
+__global__ void invert_tortoise_kernel(const __grid_constant__ KerrSet kp, double rs_min, double drs, int Nr, double *rad)
 {
     asm volatile("griddepcontrol.launch_dependents;");   // the angular stencil may run beside it
-    const Geo P = geometry(KP);
+    const Geo P = geometry(kp.k[blockIdx.y]);
+    rad += (size_t)blockIdx.y * 2 * Nr * kRadial;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= 2 * Nr - 1) return;
     const double rs = k < Nr ? rs_min + k * drs : rs_min + (k - Nr + 0.5) * drs;
@@ -267,6 +269,114 @@ __device__ Raw raw_from(const double *__restrict__ r, int Nth, int Nr, int jp, i
     return c;
 }
 
+// What the tables hold of one point.
+struct Entries {
+    double hv[kNCH], nv[kNCN];   // half node i + 1/2, node i
+    double bn;                   // b at the node
+    double c4n, c4h;             // c4 at the node and at the half node
+    double gpv, gmv;             // theta-only stencil factors of the row
+};
+
+// Of row jp < NP (polar angle th) and column i; all zero outside the grid.
+__device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr, int Nth, int NP, double drs, double dt,
+                                              double dth, double th, int i, int jp, const double *__restrict__ rad,
+                                              const double *__restrict__ ang, const Angular &A,
+                                              const double *__restrict__ raw_node,
+                                              const double *__restrict__ raw_half, Entries &E)
+{
+    double (&hv)[kNCH] = E.hv, (&nv)[kNCN] = E.nv;
+    for (int q = 0; q < kNCH; ++q) hv[q] = 0.0;
+    for (int q = 0; q < kNCN; ++q) nv[q] = 0.0;
+    E.bn = E.c4n = E.c4h = E.gpv = E.gmv = 0.0;
+    const double ith2 = 1.0 / (dth * dth), i2th = 1.0 / (2.0 * dth);
+    const double p = (variable == 0 && (abs(P.m) & 1)) ? -1.0 : 1.0;   // ghost parity
+    if (jp < Nth && i < Nr) {
+        // angular stencil A+ (row j+1), A- (row j-1); the centre gets -(A+ + A-)
+        //   literal:     A+- = 1/dth^2 +- cot(theta)/(2 dth) times c4, i.e. c4/dth^2 +- c5/(2 dth)
+        //   regularised: A+- = c4 ang[.]  (self-adjoint form, no ghosts)
+        const double Ap = (variable != 0) ? ang[jp] : 0.0;
+        const double Am = (variable != 0) ? ang[NP + jp] : 0.0;
+        if (variable != 0) {
+            E.gpv = Ap;
+            E.gmv = Am;
+        } else {
+            double sn, cs;
+            sincos(th, &sn, &cs);
+            E.gpv = (jp == Nth - 1) ? 0.0 : ith2 + (cs / sn) * i2th;   // ghosts folded on the edge rows
+            E.gmv = (jp == 0) ? 0.0 : ith2 - (cs / sn) * i2th;
+        }
+        {   // node r*_i, Eq. (lw2), step dt
+            const Raw c = raw_node ? raw_from(raw_node, Nth, Nr, jp, i)
+                                   : raw_coefficients(P, rad + (size_t)i * kRadial, A);
+            E.bn = c.b;
+            if (i > 0 && i < Nr - 1) {
+                E.c4n = c.c4;
+                const double h2 = 0.5 * dt;
+                const double B = dt * c.b / drs;
+                const double g1r = dt * c.c1r / drs, g1i = dt * c.c1i / drs;
+                double kp, km;
+                if (variable == 0) {
+                    kp = h2 * (c.c4 * ith2 + c.c5 * i2th);
+                    km = h2 * (c.c4 * ith2 - c.c5 * i2th);
+                } else {
+                    kp = h2 * c.c4 * Ap;
+                    km = h2 * c.c4 * Am;
+                }
+                const double dg = kp + km;
+                double fpr = g1r + h2 * c.c3r - dg, fmr = -g1r + h2 * c.c3r - dg;
+                if (variable == 0 && jp == 0) { fpr += p * km; fmr += p * km; km = 0.0; }
+                if (variable == 0 && jp == Nth - 1) { fpr += p * kp; fmr += p * kp; kp = 0.0; }
+                // entries that multiply half-node Phi values carry the factor eh
+                // (the half node returns Phi / eh, see the half-node tables)
+                const double eh = 0.25 * dt;
+                nv[N_B] = eh * B;
+                nv[N_PPR] = B + h2 * c.c2r;
+                nv[N_PMR] = -B + h2 * c.c2r;
+                nv[N_C2I] = h2 * c.c2i;
+                nv[N_FPR] = eh * fpr;
+                nv[N_FPI] = eh * (g1i + h2 * c.c3i);
+                nv[N_FMR] = eh * fmr;
+                nv[N_FMI] = eh * (-g1i + h2 * c.c3i);
+                nv[N_KP] = eh * kp;
+                nv[N_KM] = eh * km;
+            }
+        }
+        if (i < Nr - 1) {   // half node r*_{i+1/2}, Eq. (lw1), step dt/2
+            const Raw c = raw_half ? raw_from(raw_half, Nth, Nr, jp, i)
+                                   : raw_coefficients(P, rad + (size_t)(Nr + i) * kRadial, A);
+            E.c4h = c.c4;
+            const double dtau = 0.5 * dt, e2 = 0.5 * dtau;
+            const double B = dtau * c.b / drs;
+            const double g1r = dtau * c.c1r / drs, g1i = dtau * c.c1i / drs;
+            double kp, km;
+            if (variable == 0) {
+                kp = e2 * (c.c4 * ith2 + c.c5 * i2th);
+                km = e2 * (c.c4 * ith2 - c.c5 * i2th);
+            } else {
+                kp = e2 * c.c4 * Ap;
+                km = e2 * c.c4 * Am;
+            }
+            const double dg = kp + km;
+            double far = -g1r + e2 * c.c3r - dg, fcr = g1r + e2 * c.c3r - dg;
+            if (variable == 0 && jp == 0) { far += p * km; fcr += p * km; km = 0.0; }
+            if (variable == 0 && jp == Nth - 1) { far += p * kp; fcr += p * kp; kp = 0.0; }
+            // the Phi half-node value is returned divided by e2 (= eh): its
+            // Pi term e2 (Pi_a + Pi_c) then needs no multiplication
+            hv[H_HP] = (0.5 + B) / e2;
+            hv[H_HQ] = (0.5 - B) / e2;
+            hv[H_PAR] = 0.5 - B + e2 * c.c2r;
+            hv[H_PCR] = 0.5 + B + e2 * c.c2r;
+            hv[H_PI] = e2 * c.c2i;
+            hv[H_FAR] = far;
+            hv[H_FAI] = -g1i + e2 * c.c3i;
+            hv[H_FCR] = fcr;
+            hv[H_FCI] = g1i + e2 * c.c3i;
+            hv[H_KP] = kp;
+            hv[H_KM] = km;
+        }
+    }
+}
+
 // One thread per point, a block holding all NP rows of its columns (blockDim.x
 // = NP): a column's flags in the step tables are over its rows.  Bound by the
 // FP64 pipe: what depends on the radius alone comes from the inversion kernel,
@@ -301,102 +411,11 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
         }
         T *hcol = half + (size_t)i * kNCH * NP + jp;
         T *ncol = node + (size_t)i * kNCN * NP + jp;
-        double hv[kNCH], nv[kNCN];
-        for (int q = 0; q < kNCH; ++q) hv[q] = 0.0;
-        for (int q = 0; q < kNCN; ++q) nv[q] = 0.0;
-        double bn = 0.0;
-        double c4n = 0.0, c4h = 0.0;   // c4 at the node and at the half node
-        double gpv = 0.0, gmv = 0.0;   // theta-only stencil factors of the row
-        const double ith2 = 1.0 / (dth * dth), i2th = 1.0 / (2.0 * dth);
-        const double p = (variable == 0 && (abs(P.m) & 1)) ? -1.0 : 1.0;   // ghost parity
-        if (jp < Nth && i < Nr) {
-            if (i == 0 && w_row) w_row[jp] = (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
-            // angular stencil A+ (row j+1), A- (row j-1); the centre gets -(A+ + A-)
-            //   literal:     A+- = 1/dth^2 +- cot(theta)/(2 dth) times c4, i.e. c4/dth^2 +- c5/(2 dth)
-            //   regularised: A+- = c4 ang[.]  (self-adjoint form, no ghosts)
-            const double Ap = (variable != 0) ? ang[jp] : 0.0;
-            const double Am = (variable != 0) ? ang[NP + jp] : 0.0;
-            if (variable != 0) {
-                gpv = Ap;
-                gmv = Am;
-            } else {
-                double sn, cs;
-                sincos(th, &sn, &cs);
-                gpv = (jp == Nth - 1) ? 0.0 : ith2 + (cs / sn) * i2th;   // ghosts folded on the edge rows
-                gmv = (jp == 0) ? 0.0 : ith2 - (cs / sn) * i2th;
-            }
-            {   // node r*_i, Eq. (lw2), step dt
-                const Raw c = raw_node ? raw_from(raw_node, Nth, Nr, jp, i)
-                                       : raw_coefficients(P, rad + (size_t)i * kRadial, A);
-                bn = c.b;
-                if (i > 0 && i < Nr - 1) {
-                    c4n = c.c4;
-                    const double h2 = 0.5 * dt;
-                    const double B = dt * c.b / drs;
-                    const double g1r = dt * c.c1r / drs, g1i = dt * c.c1i / drs;
-                    double kp, km;
-                    if (variable == 0) {
-                        kp = h2 * (c.c4 * ith2 + c.c5 * i2th);
-                        km = h2 * (c.c4 * ith2 - c.c5 * i2th);
-                    } else {
-                        kp = h2 * c.c4 * Ap;
-                        km = h2 * c.c4 * Am;
-                    }
-                    const double dg = kp + km;
-                    double fpr = g1r + h2 * c.c3r - dg, fmr = -g1r + h2 * c.c3r - dg;
-                    if (variable == 0 && jp == 0) { fpr += p * km; fmr += p * km; km = 0.0; }
-                    if (variable == 0 && jp == Nth - 1) { fpr += p * kp; fmr += p * kp; kp = 0.0; }
-                    // entries that multiply half-node Phi values carry the factor eh
-                    // (the half node returns Phi / eh, see the half-node tables)
-                    const double eh = 0.25 * dt;
-                    nv[N_B] = eh * B;
-                    nv[N_PPR] = B + h2 * c.c2r;
-                    nv[N_PMR] = -B + h2 * c.c2r;
-                    nv[N_C2I] = h2 * c.c2i;
-                    nv[N_FPR] = eh * fpr;
-                    nv[N_FPI] = eh * (g1i + h2 * c.c3i);
-                    nv[N_FMR] = eh * fmr;
-                    nv[N_FMI] = eh * (-g1i + h2 * c.c3i);
-                    nv[N_KP] = eh * kp;
-                    nv[N_KM] = eh * km;
-                }
-            }
-            if (i < Nr - 1) {   // half node r*_{i+1/2}, Eq. (lw1), step dt/2
-                const Raw c = raw_half ? raw_from(raw_half, Nth, Nr, jp, i)
-                                       : raw_coefficients(P, rad + (size_t)(Nr + i) * kRadial, A);
-                c4h = c.c4;
-                const double dtau = 0.5 * dt, e2 = 0.5 * dtau;
-                const double B = dtau * c.b / drs;
-                const double g1r = dtau * c.c1r / drs, g1i = dtau * c.c1i / drs;
-                double kp, km;
-                if (variable == 0) {
-                    kp = e2 * (c.c4 * ith2 + c.c5 * i2th);
-                    km = e2 * (c.c4 * ith2 - c.c5 * i2th);
-                } else {
-                    kp = e2 * c.c4 * Ap;
-                    km = e2 * c.c4 * Am;
-                }
-                const double dg = kp + km;
-                double far = -g1r + e2 * c.c3r - dg, fcr = g1r + e2 * c.c3r - dg;
-                if (variable == 0 && jp == 0) { far += p * km; fcr += p * km; km = 0.0; }
-                if (variable == 0 && jp == Nth - 1) { far += p * kp; fcr += p * kp; kp = 0.0; }
-                // the Phi half-node value is returned divided by e2 (= eh): its
-                // Pi term e2 (Pi_a + Pi_c) then needs no multiplication
-                hv[H_HP] = (0.5 + B) / e2;
-                hv[H_HQ] = (0.5 - B) / e2;
-                hv[H_PAR] = 0.5 - B + e2 * c.c2r;
-                hv[H_PCR] = 0.5 + B + e2 * c.c2r;
-                hv[H_PI] = e2 * c.c2i;
-                hv[H_FAR] = far;
-                hv[H_FAI] = -g1i + e2 * c.c3i;
-                hv[H_FCR] = fcr;
-                hv[H_FCI] = g1i + e2 * c.c3i;
-                hv[H_KP] = kp;
-                hv[H_KM] = km;
-            }
-        } else if (i == 0 && w_row) {
-            w_row[jp] = 0.0;
-        }
+        Entries E;
+        table_entries(P, variable, Nr, Nth, NP, drs, dt, dth, th, i, jp, rad, ang, A, raw_node, raw_half, E);
+        const double (&hv)[kNCH] = E.hv, (&nv)[kNCN] = E.nv;
+        if (i == 0 && w_row)
+            w_row[jp] = jp >= Nth ? 0.0 : (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
         if (step) {
             const double hd[kStepHalfF64] = {hv[H_HP], hv[H_HQ], hv[H_PAR], hv[H_PCR], hv[H_PI]};
             const double hs[kSplitEntries] = {hv[H_FAR], hv[H_FCR], hv[H_KP], hv[H_KM], hv[H_FAI], hv[H_FCI]};
@@ -445,7 +464,7 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
             cv[C_FAI] = (float)hv[H_FAI];
             cv[C_FCR] = (float)hv[H_FCR];
             cv[C_FCI] = (float)hv[H_FCI];
-            cv[C_C4H] = (jp < Nth && i < Nr - 1) ? (float)(0.25 * dt * c4h) : 0.0f;
+            cv[C_C4H] = (jp < Nth && i < Nr - 1) ? (float)(0.25 * dt * E.c4h) : 0.0f;
             cv[C_B] = (float)nv[N_B];
             cv[C_PMR] = (float)nv[N_PMR];
             cv[C_C2I] = (float)nv[N_C2I];
@@ -453,8 +472,8 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
             cv[C_FPI] = (float)nv[N_FPI];
             cv[C_FMR] = (float)nv[N_FMR];
             cv[C_FMI] = (float)nv[N_FMI];
-            cv[C_C4N] = (jp < Nth && i > 0 && i < Nr - 1) ? (float)(0.25 * dt * 0.5 * dt * c4n) : 0.0f;
-            const float gp = (float)gpv, gm = (float)gmv;
+            cv[C_C4N] = (jp < Nth && i > 0 && i < Nr - 1) ? (float)(0.25 * dt * 0.5 * dt * E.c4n) : 0.0f;
+            const float gp = (float)E.gpv, gm = (float)E.gmv;
             if (i == 0 && gpm) {
                 gpm[jp] = gp;
                 gpm[NP + jp] = gm;
@@ -491,7 +510,45 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
             for (int q = 0; q < kNCH; ++q) hcol[(size_t)q * NP] = (T)hv[q];
             for (int q = 0; q < kNCN; ++q) ncol[(size_t)q * NP] = (T)nv[q];
         }
-        b_node[(size_t)i * NP + jp] = bn;
+        b_node[(size_t)i * NP + jp] = E.bn;
+    }
+}
+
+// The tables' derivative in a parameter of the black hole: the sum over q of
+// w[q] times the tables of kp.k[q], whose radial parts are rad[q].  One pass:
+// the tables of the shifted parameters stay in registers.  Bound by the FP64
+// pipe: 214 us at 1601 x 32; with each shifted table written out and added by
+// kernels of their own the four took 350 us and twice the table memory.
+__global__ void __launch_bounds__(kTableThreads)
+table_derivative_kernel(const __grid_constant__ KerrSet kp, int variable, int Nr, int Nth, int NP, double drs, double dt,
+                        const double *__restrict__ rad, const double *__restrict__ ang, double *__restrict__ half,
+                        double *__restrict__ node, double *__restrict__ b_node)
+{
+    const int jp = threadIdx.x;
+    const double dth = M_PI / Nth;
+    const double th = (jp + 0.5) * dth;
+    const Angular A = jp < Nth ? angular_part(geometry(kp.k[0]), variable, th) : Angular{};
+    for (int i = blockIdx.x * blockDim.y + threadIdx.y; i < Nr; i += gridDim.x * blockDim.y) {
+        double v[kNCH + kNCN + 1];
+#pragma unroll
+        for (int k = 0; k < kNCH + kNCN + 1; ++k) v[k] = 0.0;
+#pragma unroll 1
+        for (int q = 0; q < kShifts; ++q) {
+            Entries E;
+            table_entries(geometry(kp.k[q]), variable, Nr, Nth, NP, drs, dt, dth, th, i, jp,
+                          rad + (size_t)q * 2 * Nr * kRadial, ang, A, nullptr, nullptr, E);
+            const double w = kp.w[q];
+#pragma unroll
+            for (int k = 0; k < kNCH; ++k) v[k] = fma(w, E.hv[k], v[k]);
+#pragma unroll
+            for (int k = 0; k < kNCN; ++k) v[kNCH + k] = fma(w, E.nv[k], v[kNCH + k]);
+            v[kNCH + kNCN] = fma(w, E.bn, v[kNCH + kNCN]);
+        }
+#pragma unroll
+        for (int k = 0; k < kNCH; ++k) half[((size_t)i * kNCH + k) * NP + jp] = v[k];
+#pragma unroll
+        for (int k = 0; k < kNCN; ++k) node[((size_t)i * kNCN + k) * NP + jp] = v[kNCH + k];
+        b_node[(size_t)i * NP + jp] = v[kNCH + kNCN];
     }
 }
 
@@ -573,11 +630,43 @@ cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, c
     return cudaGetLastError();
 }
 
+// The angular stencil, chained to the tortoise inversion: it needs nothing of
+// it, and that started after every earlier use of ang, so the two run side by side.
+static cudaError_t launch_stencil(int s, int m, int Ntheta, int NP, double *ang, cudaStream_t st)
+{
+    return launch_chained(regular_stencil_kernel, (unsigned)NP, 4 * kStencilPanels, 0, st, s, m, Ntheta, NP, ang);
+}
+
+// one warp per block: few warps, each a serial chain, over all the SMs
+static cudaError_t launch_inversion(const KerrSet &kp, int n, double rs_min, double drs, int Nr, double *rad,
+                                    cudaStream_t st)
+{
+    invert_tortoise_kernel<<<dim3((2 * Nr + 30) / 32, n), 32, 0, st>>>(kp, rs_min, drs, Nr, rad);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr, double *rad, cudaStream_t st)
 {
-    // one warp per block: few warps, each a serial chain, over all the SMs
-    const int n = 2 * Nr - 1;
-    invert_tortoise_kernel<<<(n + 31) / 32, 32, 0, st>>>(P, rs_min, drs, Nr, rad);
+    KerrSet kp = {};
+    kp.k[0] = P;
+    return launch_inversion(kp, 1, rs_min, drs, Nr, rad, st);
+}
+
+static dim3 table_grid(int Nr, const dim3 &block)
+{
+    return dim3(std::min<unsigned>((Nr + block.y - 1) / block.y, 152 * 4));
+}
+
+cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_min, int Nr, int Ntheta, int NP,
+                                    double drs, double dt_inner, double *rad, double *ang, double *half,
+                                    double *node, double *b_node, cudaStream_t st)
+{
+    cudaError_t e = launch_inversion(kp, kShifts, rs_min, drs, Nr, rad, st);
+    if (e == cudaSuccess && variable != 0) e = launch_stencil(kp.k[0].s, kp.k[0].m, Ntheta, NP, ang, st);
+    if (e != cudaSuccess) return e;
+    const dim3 block(NP, kTableThreads / NP);
+    table_derivative_kernel<<<table_grid(Nr, block), block, 0, st>>>(kp, variable, Nr, Ntheta, NP, drs, dt_inner, rad,
+                                                                     ang, half, node, b_node);
     return cudaGetLastError();
 }
 
@@ -589,14 +678,11 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
 {
     const F32Derive fd = f32_derive(dt_inner);
     if (variable != 0 && !ang_given) {
-        // chained to the tortoise inversion, of which it needs nothing (and which
-        // started after every earlier use of ang): the two run side by side
-        cudaError_t e = launch_chained(regular_stencil_kernel, (unsigned)NP, 4 * kStencilPanels, 0, st, P.s, P.m, Ntheta,
-                                       NP, ang);
+        cudaError_t e = launch_stencil(P.s, P.m, Ntheta, NP, ang, st);
         if (e != cudaSuccess) return e;
     }
     dim3 block(NP, kTableThreads / NP);
-    dim3 grid(std::min<unsigned>((Nr + block.y - 1) / block.y, 152 * 4));
+    const dim3 grid = table_grid(Nr, block);
     if (precision == 0)
         coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
                                                              rad, ang, (double *)half,

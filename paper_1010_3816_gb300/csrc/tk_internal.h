@@ -99,6 +99,13 @@ struct Kerr {
     int s, m;     // spin weight, azimuthal mode
 };
 
+// Shifted black holes and the weights of a finite difference in a parameter.
+constexpr int kShifts = 4;
+struct KerrSet {
+    Kerr k[kShifts];
+    double w[kShifts];
+};
+
 struct ObsDev {
     int n;                          // number of observers
     int i0[kMaxObservers];          // lower r* column of the interpolation cell
@@ -141,6 +148,13 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
                                 cudaStream_t st, const double *raw_node = nullptr,
                                 const double *raw_half = nullptr, bool ang_given = false,
                                 unsigned char *step = nullptr);
+
+// The derivative of the FP64 tables in a parameter of the black hole, sum_q w[q]
+// tables(k[q]); rad: kShifts times the radial parts, ang: the angular stencil,
+// both scratch.
+cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_min, int Nr, int Ntheta, int NP,
+                                    double drs, double dt_inner, double *rad, double *ang, double *half,
+                                    double *node, double *b_node, cudaStream_t st);
 
 // The raw coefficients of the precompute, [9][Ntheta][Nr] at nodes and half
 // nodes (device output buffers).

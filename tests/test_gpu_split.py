@@ -248,3 +248,21 @@ def test_adjoint_tables_follow_the_coefficients():
     h.adjoint(want, dL_dfinal=dL, independent_pi=True)
     h.close()
     assert np.array_equal(grads[1], want) and not np.array_equal(grads[0], want)
+
+
+@pytest.mark.parametrize("Nr,Nth", [(9, 20), (130, 45), (333, 97), (1700, 32)])
+def test_param_gradient_does_not_depend_on_the_grouping(Nr, Nth):
+    """The transposed steps are contracted up to eight at a time, at most those
+    of a checkpoint interval: every grouping gives the same bits, and one step
+    at a time (C = substeps = 1) is the plain order."""
+    for k in (1, 3):
+        w = _work(Nr, Nth, substeps=k)
+        g = _solver(w)
+        g.set_initial(*initial_planes(w))
+        g.add_observer(w.rs_min + 0.6 * (Nr - 1) * w.drs, 1.1)
+        g.step(11)
+        dL = np.random.default_rng(7).standard_normal((1, 11, 2))
+        grads = [g.param_gradient("a", dL, C) for C in (1, 0, 4, 11)]
+        g.close()
+        assert np.isfinite(grads[0]) and grads[0] != 0.0
+        assert grads == [grads[0]] * 4
