@@ -1228,10 +1228,15 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     int Q = (int)std::min<long long>(std::min<long long>(C * k, tk::kLamSteps), 1 + (long long)((256ull << 20) / sb));
     const int blocks = std::max(1, S->Nr / (4 * std::min(4, 1 + S->Nr / 512))), pblocks = 1024;
 
+    // small grids: a segment's levels in one launch (lw_column_kernel writing a
+    // trajectory), 4.3 us a step at 1601 x 32 where a launch per step takes 8.6
+    const bool columns = S->persist && S->persist_columns && C * k <= 0x7fffffff;
+    const size_t nflags = columns ? (size_t)2 * S->K * S->persist_blocks : 0;
+
     // scratch in one allocation, freed on every exit
     double *dwave = nullptr, *scratch = nullptr;
     double *tx = nullptr, *tang = nullptr, *ck = nullptr, *seg = nullptr, *acc = nullptr, *parts = nullptr;
-    double *lam_more = nullptr;
+    double *lam_more = nullptr, *pflags = nullptr;
     auto cleanup = [&]() {
         if (scratch) cudaFree(scratch);
         if (dwave && !on_device) cudaFree(dwave);
@@ -1252,7 +1257,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         struct { double **p; size_t n; } piece[] = {
             {&ck, (size_t)nck * se}, {&seg, (size_t)(C * k) * se}, {&lam_more, (size_t)(Q - 1) * se},
             {&tx, (size_t)tk::kShifts * 2 * S->Nr * tk::kRadial}, {&tang, (size_t)2 * S->NP},
-            {&acc, (size_t)(blocks + pblocks)}, {&parts, (size_t)Q * blocks}};
+            {&acc, (size_t)(blocks + pblocks)}, {&parts, (size_t)Q * blocks}, {&pflags, 1 + (nflags + 1) / 2}};
         size_t total = 0;
         for (auto &x : piece) total += (x.n + 31) / 32 * 32;
         st = tkh::alloc(S, (void **)&scratch, total * sizeof(double));
@@ -1300,10 +1305,38 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     tk::StepLaunch L;
     tkh::fill_launch(S, L);
     L.write_wave = 0;
-    e = cudaMemcpyAsync(ck, S->u_init, sb, cudaMemcpyDeviceToDevice, S->stream);
+    unsigned int *flags = (unsigned int *)pflags;
+    int *perr = (int *)(flags + nflags);
+    if (e == cudaSuccess) e = cudaMemsetAsync(perr, 0, sizeof(int), S->stream);
+    // n >= 1 levels after src, to dst, dst + se, ..
+    auto levels = [&](const double *src, double *dst, long long n) {
+        tk::StepLaunch P = L;
+        P.u_in = src;
+        if (columns && n >= 2) {
+            P.blocks = S->persist_blocks;
+            P.columns = S->persist_columns;
+            P.stride = se;
+            cudaError_t r = cudaMemsetAsync(flags, 0, nflags * sizeof(unsigned int), S->stream);
+            return r != cudaSuccess ? r : tk::launch_lw_persistent(P, dst, (int)n, k, flags, perr, S->stream);
+        }
+        cudaError_t r = cudaSuccess;
+        for (long long j = 0; j < n && r == cudaSuccess; ++j, dst += se) {
+            P.u_out = dst;
+            r = tk::launch_lw_step(P, S->stream);
+            P.u_in = dst;
+        }
+        return r;
+    };
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ck, S->u_init, sb, cudaMemcpyDeviceToDevice, S->stream);
     for (long long c = 0; c + 1 < nck && e == cudaSuccess; ++c) {
         const double *src = ck + (size_t)c * se;
         double *dst = ck + (size_t)(c + 1) * se;
+        if (columns && C * k >= 2) {
+            e = levels(src, seg, C * k);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(dst, seg + (size_t)(C * k - 1) * se, sb, cudaMemcpyDeviceToDevice, S->stream);
+            continue;
+        }
         // C outer steps: ping-pong through the first two segment slots
         const void *in = src;
         for (long long j = 0; j < C * k && e == cudaSuccess; ++j) {
@@ -1329,11 +1362,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         const long long t0 = c * C, len = (c == nck - 1) ? count - t0 : C;
         // seg[j] = u^{t0 k + j}, j < len k
         e = cudaMemcpyAsync(seg, ck + (size_t)c * se, sb, cudaMemcpyDeviceToDevice, S->stream);
-        for (long long j = 0; j + 1 < len * k && e == cudaSuccess; ++j) {
-            L.u_in = seg + (size_t)j * se;
-            L.u_out = seg + (size_t)(j + 1) * se;
-            e = tk::launch_lw_step(L, S->stream);
-        }
+        if (e == cudaSuccess && len * k > 1) e = levels(seg, seg + se, len * k - 1);
         for (long long g = 0; g < len * k && e == cudaSuccess;) {   // transposed steps from the segment's end
             const int n = (int)std::min<long long>(Q, len * k - g);
             tk::LamSet set = {};
@@ -1364,7 +1393,12 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     std::vector<double> h((size_t)blocks + pblocks, 0.0);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(double), cudaMemcpyDeviceToHost, S->stream);
+    int herr = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, perr, sizeof(int), cudaMemcpyDeviceToHost, S->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(S->stream);
+    if (e == cudaSuccess && herr)
+        return bail(tkh::fail(S, TK_ERR_INTERNAL, "tk_param_gradient: a block of the persistent launch waited too long "
+                                                  "for a neighbour; the gradient is not valid"));
     if (e != cudaSuccess)
         return bail(tkh::fail(S, e == cudaErrorMemoryAllocation ? TK_ERR_OOM : TK_ERR_CUDA,
                               "tk_param_gradient: %s", cudaGetErrorString(e)));

@@ -124,6 +124,8 @@ void fill_launch(const tk_solver *S, tk::StepLaunch &L)
     L.NP = S->NP;
     L.blocks = S->blocks;
     L.warps = S->warps;
+    L.columns = 0;
+    L.stride = 0;
     L.fused = 0;
     L.obs_mask = 0;
     L.dt_inner = S->dt / S->substeps;
@@ -235,7 +237,7 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     // two-step (ring) kernel's, both one wave of resident blocks
     S->persist_blocks = (precision == TK_PREC_F32)
                             ? S->fused_blocks
-                            : tk::persistent_grid_blocks(S->K, Nr, S->num_sms, S->warps);
+                            : tk::persistent_grid_blocks(S->K, Nr, S->num_sms, S->warps, &S->persist_columns);
     S->multi_blocks = tk::multi_grid_shape(precision, S->K, Nr, S->num_sms, &S->multi_warps);
     set_launch_mode(S, 0);
 
@@ -638,6 +640,7 @@ tk_status tk_step(tk_solver *S, int n)
         tk::StepLaunch L;
         tkh::fill_launch(S, L);
         L.blocks = S->persist_blocks;
+        L.columns = S->persist_columns;
         L.warps = S->precision == TK_PREC_F32 ? S->fused_warps : S->warps;
         L.u_in = S->u[S->cur];
         L.write_wave = S->nobs > 0;

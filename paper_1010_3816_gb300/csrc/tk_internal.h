@@ -188,6 +188,8 @@ struct StepLaunch {
     int Nr, NP;
     int blocks;           // grid size (columns are split evenly over its warps)
     int warps;            // warps per block (from step_grid_shape or fused_grid_shape)
+    int columns;          // persistent FP64 launch: columns per block of lw_column_kernel, 0: the other kernel
+    size_t stride;        // with columns: write every step's level, u_other + s stride
     int fused;            // 1: two Lax-Wendroff steps in this launch (lw_step2_kernel)
     int obs_mask;         // fused: bit 0, an outer step ends after the first step; bit 1, after the second
     double dt_inner;      // Lax-Wendroff step
@@ -215,7 +217,8 @@ int step_grid_shape(int precision, int K, int Nr, int num_sms, int *warps);
 // cannot run; the launch itself (L.u_in holds u^n, u_other is the
 // second level; flags: one zeroed unsigned int per block; *err set on a wait
 // that timed out).
-int persistent_grid_blocks(int K, int Nr, int num_sms, int warps);
+// *columns: what L.columns has to be.
+int persistent_grid_blocks(int K, int Nr, int num_sms, int warps, int *columns);
 // Diagnostic of the persistent launches' bounded neighbour wait (one-warp
 // blocks; flags: n_blocks zeroed unsigned ints).
 cudaError_t launch_wait_check(int n_blocks, int silent, long long max_spins, unsigned int *flags,

@@ -296,6 +296,138 @@ lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, co
     if (wa.write) advance_sample(wa, n_inner / substeps);
 }
 
+// The same steps on grids with no more columns than the chip holds teams: one
+// column per team, everything a team needs stays in the SM.  A block has
+// T columns and one team more; team j forms the half node to the right of
+// column T b - 1 + j, and for j > 0 then the node of that column from its own
+// half node and that of team j - 1, so that only a block's
+// left half node is formed twice (in lw_persistent_kernel every team's is, and
+// on these grids a team has one column: 40 FP64 instructions an update instead
+// of 31) and a step's chain is one half node and one node, not two and one.
+// The tables are fetched once, a team's column stays in its registers, its
+// neighbours in the block read it in shared memory; only a block's first and
+// last column go through global memory (and all of them after the last step),
+// under the flags of lw_persistent_kernel and its bounded waits.  A block's own
+// teams meet at two block barriers a step.  The arithmetic, and so every bit,
+// is that of the other launch structures.
+//
+// T = 3 (16 / K / 4 blocks per SM: 1824 columns at 32 rows) where the grid fits,
+// else T = 7 (2128 columns; not at 128 rows, 32 warps a block).  us per step, this
+// launch (lw_persistent_kernel): 401 x 32 3.2 (5.1), 1601 x 32 4.3 (6.1), 912 x 64
+// 4.6 (6.4), 456 x 128 4.9 (7.9); 1825 x 32 with T = 7 4.6 (6.2).  Where T = 3 fits
+// T = 7 is slower (1601 x 32: 4.6), T = 5 too (6.2, one block per SM at a time).
+//
+// stride != 0: step s writes the whole level to u1 + s stride instead (a
+// trajectory), u0 stays.
+template <int K, int T>
+constexpr int column_warps()
+{
+    return (T + 1) * K;
+}
+
+template <int K, int T>
+constexpr size_t column_smem_bytes()
+{
+    return (size_t)column_warps<K, T>() * (kStepBytes + 2 * 4 * 32 * sizeof(double));
+}
+
+template <int K, int T>
+__global__ void __launch_bounds__(column_warps<K, T>() * 32, 16 / column_warps<K, T>())
+lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const double *__restrict__ node,
+                 const unsigned char *__restrict__ step, int Nr, double en, const WaveArgs wa, int n_inner,
+                 int substeps, unsigned int *flags, int *err, size_t stride)
+{
+    constexpr int W = (T + 1) * K, NP = 32 * K;
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    __shared__ unsigned long long bars[W];
+    __shared__ SplitRows rows[W];
+    double *hn = reinterpret_cast<double *>(sh_raw + W * kStepBytes);   // half nodes, [team][4][NP]
+    double *uc = hn + W * 4 * 32;                                       // columns, [team][4][NP]
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, j = wib / K, h = wib % K, row = 32 * h + lane;
+    const int nb = (int)gridDim.x, b = (int)blockIdx.x, col = b * T - 1 + j;
+    const bool owner = j > 0 && col < Nr;              // of a column
+    const bool halves = col >= 0 && col + 1 < Nr;      // there is a half node right of it
+    const unsigned char *tab = sh_raw + wib * kStepBytes;
+    const FmaK<double> k1 = fma_k<double>();
+    SplitTeam<K> team{rows + j * K, h, lane, 1 + j};
+    auto load = [&](const double *u, int i, double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = __ldcg(u + (size_t)i * (4 * NP) + k * NP + row);
+    };
+    auto put = [&](double *p, int t, const double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[(t * 4 + k) * NP + row] = x[k];
+    };
+    auto get = [&](const double *p, int t, double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = p[(t * 4 + k) * NP + row];
+    };
+    if (halves) {
+        if (lane == 0) {
+            mbar_init(&bars[wib]);
+            mbar_init_fence();
+            mbar_expect(&bars[wib], kStepBytes);
+            bulk_fetch(sh_raw + wib * kStepBytes, step + ((size_t)col * K + h) * kStepBytes, kStepBytes, &bars[wib]);
+        }
+        __syncwarp();
+        if (!mbar_wait(&bars[wib], 0)) atomicExch(err, 1);
+    }
+    double a[4];   // column col
+    if (owner) {
+        load(u0, col, a);
+        put(uc, j, a);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int s = 0; s < n_inner; ++s) {
+        const double *in = stride ? (s > 0 ? u1 + (s - 1) * stride : u0) : (s & 1) ? u1 : u0;
+        double *out = stride ? u1 + s * stride : (s & 1) ? u0 : u1;
+        const int write = wa.write && ((s + 1) % substeps == 0);
+        double hp[4];
+        if (halves) {
+            double c[4];
+            SplitInts pa, pc;
+            if (s > 0 && j == 0) warp_wait_flag(flags + (nb + b - 1) * K + h, s, err);
+            if (s > 0 && j == T) warp_wait_flag(flags + (b + 1) * K + h, s, err);
+            if (j == 0) load(in, col, a);
+            if (j == T) load(in, col + 1, c);
+            else get(uc, j + 1, c);
+            split_ints<0>(a, pa);
+            split_ints<0>(c, pc);
+            split_half_node<K>(a, pa, c, pc, tab, team, half + (size_t)col * (kNCH * NP) + row, k1, hp);
+            put(hn, j, hp);
+        }
+        __syncthreads();
+        if (owner) {
+            if (col > 0 && halves) {
+                double hm[4], o[4];
+                SplitInts pm, pp;
+                get(hn, j - 1, hm);
+                split_ints<0>(hm, pm);
+                split_ints<0>(hp, pp);
+                split_full_node<K>(hm, pm, hp, pp, a, tab, team, node + (size_t)col * (kNCN * NP) + row, en, k1, o);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[k] = o[k];
+            } else {   // a radial edge
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[k] = 0.0;
+            }
+            put(uc, j, a);
+            if (j == 1 || j == T || s + 1 == n_inner || stride) {
+                double *p = out + (size_t)col * (4 * NP) + row;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) p[k * NP] = a[k];
+            }
+            if (j == 1) warp_publish_gpu(flags + b * K + h, s + 1);
+            if (j == T) warp_publish_gpu(flags + (nb + b) * K + h, s + 1);
+            if (write)
+                observe_team<K>(col, a, team, wa.obs, wa.wave, wa.cap, wa.sample, wa.w_row, (s + 1) / substeps - 1);
+        }
+        __syncthreads();
+    }
+    if (wa.write) advance_sample(wa, n_inner / substeps);
+}
+
 // Diagnostic of the bounded waits: every block but `silent` publishes epoch 1
 // and waits for its neighbours as the persistent kernels do between steps
 // (the block-level wait, error word err[0]), then waits for each neighbour
@@ -1109,6 +1241,34 @@ int persistent_blocks(int Nr, int num_sms, int warps)
     return 0;
 }
 
+// Blocks of the one-column-per-team launch, 0 where the grid has too many columns.
+template <int K, int T>
+int column_blocks_t(int Nr, int num_sms)
+{
+    int n = 0;
+    static cudaError_t e0 = cudaFuncSetAttribute(lw_column_kernel<K, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)column_smem_bytes<K, T>());
+    if (e0 != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_column_kernel<K, T>, column_warps<K, T>() * 32,
+                                                      column_smem_bytes<K, T>()) != cudaSuccess)
+        return 0;
+    const int blocks = (Nr + T - 1) / T;
+    return blocks <= num_sms * n ? blocks : 0;
+}
+
+template <int K>
+int column_blocks(int Nr, int num_sms, int *columns)
+{
+    int blocks = column_blocks_t<K, 3>(Nr, num_sms);
+    *columns = blocks > 0 ? 3 : 0;
+    if constexpr (K < 4)
+        if (blocks == 0) {
+            blocks = column_blocks_t<K, 7>(Nr, num_sms);
+            if (blocks > 0) *columns = 7;
+        }
+    return blocks;
+}
+
 template <int K, int W>
 cudaError_t launch_persistent_w(const StepLaunch &L, void *u_other, int n_inner, int substeps,
                                 unsigned int *flags, int *err, cudaStream_t st)
@@ -1126,7 +1286,16 @@ cudaError_t launch_persistent_w(const StepLaunch &L, void *u_other, int n_inner,
     const unsigned char *step = L.step;
     int Nr = L.Nr;
     double en = 0.5 * L.dt_inner;
-    void *args[] = {&u0, &u1, &half, &node, &step, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err};
+    size_t stride = L.stride;
+    void *args[] = {&u0, &u1, &half, &node, &step, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err, &stride};
+    if (L.columns == 3)
+        return cudaLaunchCooperativeKernel((const void *)lw_column_kernel<K, 3>, dim3(L.blocks),
+                                           dim3(column_warps<K, 3>() * 32), args, column_smem_bytes<K, 3>(), st);
+    if constexpr (K < 4)
+        if (L.columns == 7)
+            return cudaLaunchCooperativeKernel((const void *)lw_column_kernel<K, 7>, dim3(L.blocks),
+                                               dim3(column_warps<K, 7>() * 32), args, column_smem_bytes<K, 7>(), st);
+    if (stride) return cudaErrorInvalidValue;
     return cudaLaunchCooperativeKernel((const void *)lw_persistent_kernel<K, W>, dim3(L.blocks), dim3(W * 32),
                                        args, step_smem_bytes<double, K, W>(), st);
 }
@@ -1285,11 +1454,17 @@ cudaError_t launch_multi_persistent(const StepLaunch &L, void *u_other, int n_gr
     return cudaErrorInvalidValue;
 }
 
-int persistent_grid_blocks(int K, int Nr, int num_sms, int warps)
+int persistent_grid_blocks(int K, int Nr, int num_sms, int warps, int *columns)
 {
-    return K == 1 ? persistent_blocks<1>(Nr, num_sms, warps)
-         : K == 2 ? persistent_blocks<2>(Nr, num_sms, warps)
-                  : persistent_blocks<4>(Nr, num_sms, warps);
+    const int blocks = K == 1 ? persistent_blocks<1>(Nr, num_sms, warps)
+                     : K == 2 ? persistent_blocks<2>(Nr, num_sms, warps)
+                              : persistent_blocks<4>(Nr, num_sms, warps);
+    const int cols = blocks == 0 ? 0
+                   : K == 1 ? column_blocks<1>(Nr, num_sms, columns)
+                   : K == 2 ? column_blocks<2>(Nr, num_sms, columns)
+                            : column_blocks<4>(Nr, num_sms, columns);
+    if (cols == 0) *columns = 0;
+    return cols > 0 ? cols : blocks;
 }
 
 cudaError_t launch_wait_check(int n_blocks, int silent, long long max_spins, unsigned int *flags,

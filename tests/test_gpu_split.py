@@ -266,3 +266,16 @@ def test_param_gradient_does_not_depend_on_the_grouping(Nr, Nth):
         g.close()
         assert np.isfinite(grads[0]) and grads[0] != 0.0
         assert grads == [grads[0]] * 4
+
+
+@pytest.mark.parametrize("Nr,Nth", [(4, 32), (1824, 20), (1825, 32), (2128, 32), (2129, 32), (912, 64), (913, 50),
+                                    (1064, 64), (1065, 64), (456, 128), (457, 97)])
+def test_small_grid_launch_at_its_edges(Nr, Nth):
+    """One column per team, at the ends of its range and of its blocks of three
+    or seven columns: the bits of one launch per step, state and samples, for an
+    odd number of steps too."""
+    w = _work(Nr, Nth, substeps=1)
+    for n in (2, 5):
+        ref, wref = _run(w, 1, n=n)
+        s, wv = _run(w, 0, n=n)
+        assert np.array_equal(s, ref) and all(np.array_equal(a, b) for a, b in zip(wv, wref))
