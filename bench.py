@@ -42,19 +42,24 @@ from inputs import (ADJOINT_16001x128, KERR_25601x64, SCHWARZSCHILD_1601x32,  # 
 WORKLOADS = {"kerr": KERR_25601x64, "schwarzschild": SCHWARZSCHILD_1601x32,
              "batched": None, "adjoint": ADJOINT_16001x128}
 
-# FP64 work of the step kernel per grid-point update, counted from its source:
-# half node (Eq. lw1) 4 adds + 2 multiplies + 20 FMAs, node (Eq. lw2) 4 adds +
-# 24 FMAs; an FMA counts 2 flops.  The adds and multiplies are issued as FMAs
-# with 1 and -0 (54 DFMA instructions), so at most 98 of the 108 flops a full
-# pipe would do are useful.
-FP64_FLOP_PER_UPDATE = (4 + 2 + 2 * 20) + (4 + 2 * 24)          # = 98
-FP64_INSTR_PER_UPDATE = 26 + 28
-# adjoint step per update: 46 FMAs + 6 multiplies + 10 adds (transposed blocks
-# and transposed theta couplings at the node and the half node)
-ADJ_FLOP_PER_UPDATE = 2 * 46 + 6 + 10                            # = 108
-ADJ_INSTR_PER_UPDATE = 62
+# Work of the FP64 step per grid-point update.  The scheme has 98 flops (half
+# node, Eq. lw1: 4 adds, 2 multiplies, 20 FMAs; node, Eq. lw2: 4 adds, 24 FMAs;
+# an FMA counts 2).  The 48 of the coupling of Phi to Pi are done on the integer
+# units; on the FP64 pipe are left, counted from the source, 2 adds + 10 FMAs and
+# 4 adds + 12 FMAs, the adds issued as FMAs with 1 (28 DFMA instructions).  The
+# roofline below counts only what the FP64 pipe does.
+SCHEME_FLOP_PER_UPDATE = 98
+FP64_FLOP_PER_UPDATE = (2 + 2 * 10) + (4 + 2 * 12)               # = 50
+FP64_INSTR_PER_UPDATE = 12 + 16
+# adjoint step per update: 108 flops, on the FP64 pipe eta 2 multiplies + 14
+# FMAs, mu 6 adds + 12 FMAs (34 DFMA instructions)
+ADJ_SCHEME_FLOP_PER_UPDATE = 108
+ADJ_FLOP_PER_UPDATE = (2 + 2 * 14) + (6 + 2 * 12)                # = 60
+ADJ_INSTR_PER_UPDATE = 16 + 18
 STATE_BYTES_PER_UPDATE = {0: 64, 1: 32}                         # read u^n, write u^{n+1}
-TABLE_BYTES_PER_UPDATE = {0: 21 * 8, 1: 21 * 4}                 # 11 + 10 table entries
+# FP64: 9 doubles, 12 limb pairs, two exponents and the block's flags per point
+# (5648 bytes per column and 32 rows); FP32: 11 + 10 table entries
+TABLE_BYTES_PER_UPDATE = {0: 5648 / 32, 1: 21 * 4}
 # the four-step FP32 sweep reads the compact FP32 tables: 16 of the 21 entries
 # per point (the other five are derived in the kernel)
 FP32_SWEEP_TABLE_BYTES = 16 * 4
@@ -69,8 +74,8 @@ FP32_FMA_PER_CLK_PER_SM = 128
 # keyed by (workload name, precision); the capture's command and figures are in the
 # named summary under profiles/.
 MEASURED_TRAFFIC = {
-    # one persistent launch of 200 steps: 65.775047 + 10.831660 GB, per step
-    ("kerr_a0.9_25601x64_38400steps", 0): ((65.775047e9 + 10.831660e9) / 200,
+    # one persistent launch of 100 steps: 34.491594 + 5.232270 GB, per step
+    ("kerr_a0.9_25601x64_38400steps", 0): ((34.491594e9 + 5.232270e9) / 100,
                                            "profiles/lw_persistent_f64_kerr_25601x64.md"),
     # one launch of 50 sweeps of four steps: 6.726055 + 1.280336 GB
     ("kerr_a0.9_25601x64_38400steps", 1): ((6.726055e9 + 1.280336e9) / 50,
@@ -377,7 +382,11 @@ def run_batched(args, tk, torch, rank, world, local, steps=None, warmup=None, em
                        "l2": L2_NOTE},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "lw_persistent_kernel<double>" if seg == 0 else "batch_step_kernel<double>",
+                         "kernel": "lw_persistent_kernel" if seg == 0 else "batch_step_kernel<double>",
+                         "flop_per_update": FP64_FLOP_PER_UPDATE,
+                         "scheme_flop_per_update": SCHEME_FLOP_PER_UPDATE,
+                         "fp64_issue_frac": FP64_INSTR_PER_UPDATE * updates / kern_s /
+                         (NUM_SMS * FP64_FMA_PER_CLK_PER_SM * f_clk),
                          "peak_source": "152 SMs x 2 DFMA/clk (measured) x 2 flop x median SM clock"},
             "plain_tk_step": {"value": plain, "unit": "updates/s",
                               "what": "the same instances through tk_step one after another"},
@@ -468,11 +477,12 @@ def run_adjoint(args, tk, torch, rank, world, local):
     n_inner = n_outer * w.substeps
     fwd_persistent = tk.tk_get_steps_per_launch(g.h) == -1
 
-    def fp64_roof(kernel, flop, instr, seconds):
+    def fp64_roof(kernel, flop, scheme, instr, seconds):
         launch_s = seconds / n_inner
         ach = flop * w.points / launch_s / 1e12
         return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": None, "kernel": kernel, "flop_per_update": flop,
+                "scheme_flop_per_update": scheme,
                 "fp64_issue_frac": instr * w.points / launch_s /
                 (NUM_SMS * FP64_FMA_PER_CLK_PER_SM * f_clk),
                 "launch_us": launch_s * 1e6,
@@ -503,12 +513,12 @@ def run_adjoint(args, tk, torch, rank, world, local):
                        "gradient_wrt": ["amplitude", "centre", "width", "initial planes"],
                        "parallelism": "single GPU", "l2": L2_NOTE},
             "forward_updates_per_s": inner / fwd, "adjoint_updates_per_s": inner / bwd,
-            "roofline_adjoint": fp64_roof("lw_adjoint_persistent_kernel<double>" if fwd_persistent
-                                          else "lw_adjoint_kernel<double>", ADJ_FLOP_PER_UPDATE,
-                                          ADJ_INSTR_PER_UPDATE, bwd),
+            "roofline_adjoint": fp64_roof("lw_adjoint_team_persistent_kernel" if fwd_persistent
+                                          else "lw_adjoint_team_kernel", ADJ_FLOP_PER_UPDATE,
+                                          ADJ_SCHEME_FLOP_PER_UPDATE, ADJ_INSTR_PER_UPDATE, bwd),
             "grad": [float(x) for x in grads], "param_gradient": pgrad,
-            "roofline": fp64_roof("lw_persistent_kernel<double>" if fwd_persistent else "lw_step_kernel<double>",
-                                  FP64_FLOP_PER_UPDATE, FP64_INSTR_PER_UPDATE, fwd),
+            "roofline": fp64_roof("lw_persistent_kernel" if fwd_persistent else "lw_step_kernel<double>",
+                                  FP64_FLOP_PER_UPDATE, SCHEME_FLOP_PER_UPDATE, FP64_INSTR_PER_UPDATE, fwd),
             "cpu_baseline": None, "e2e": None, "clocks": clk,
             # per timed step: the forward solve and the adjoint sweep, each one
             # persistent launch, or one launch per inner step
@@ -746,7 +756,9 @@ def measure_solve(args, tk, torch, w, precision, steps, warmup, rank, world, loc
         probe = fp64_probe(tk, f_clk)
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": "lw_persistent_kernel<double>" if fp64_persistent else "lw_step_kernel<double>",
+                "kernel": ("lw_step_kernel<double>" if not fp64_persistent else "lw_column_kernel"
+                           if w.Nr * (1 if w.Ntheta <= 32 else 2 if w.Ntheta <= 64 else 4) <= 1824
+                           else "lw_persistent_kernel"),
                 "peak_source": "152 SMs x 2 DFMA/clk x 2 flop x median SM clock "
                                f"{f_clk / 1e6:.0f} MHz (GB300 FP64 FMA issue rate; "
                                "profiles/fp64_pipe_peak.md)",
@@ -754,6 +766,7 @@ def measure_solve(args, tk, torch, w, precision, steps, warmup, rank, world, loc
                 "frac_of_measured": achieved / probe["tflops"],
                 "peak_measured_source": "tk_probe_fp64_fma in this run: " + probe["how"],
                 "traffic_source": traffic_src, "flop_per_update": FP64_FLOP_PER_UPDATE,
+                "scheme_flop_per_update": SCHEME_FLOP_PER_UPDATE,
                 "fp64_issue_frac": FP64_INSTR_PER_UPDATE * pts / kern_s /
                 (NUM_SMS * FP64_FMA_PER_CLK_PER_SM * f_clk),
                 "step_us": kern_s * 1e6,

@@ -231,7 +231,8 @@ tk_status tk_extract_noalloc(tk_solver *S, int obs_id, int first, int count, dou
  *              independent_pi = 1, planes4 including dL/d(pi planes)
  *   grad_on_device location of grad
  * The solver's state is not touched.  Allocates two adjoint state levels on
- * first use (kept until tk_destroy) and temporary buffers for host inputs.
+ * first use and, in FP64, the transposed tables (6416 bytes per column and 32
+ * rows), all kept until tk_destroy, and temporary buffers for host inputs.
  * Synchronizes the stream when an input or the output is in host memory. */
 tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfinal, int on_device,
                      double *grad, int grad_on_device, int independent_pi);
@@ -328,7 +329,7 @@ tk_status tk_synchronize(tk_solver *S);
  * Lax-Wendroff tick advances all of them.  Members may differ in every other
  * parameter; with k_i inner steps per outer step each, an outer step is
  * lcm(k_i) <= 64 ticks and member i steps on every (lcm/k_i)-th tick.  The
- * batch kernel is persistent: its warps take (member, column range) items,
+ * batch kernel is persistent: its warps (FP64: blocks) take (member, column range) items,
  * longest first, from a queue in device memory.  Whole chunks of outer steps
  * are replayed from a captured CUDA graph.  Results are bit-identical to
  * stepping each member alone with tk_step.  Everything runs on the first

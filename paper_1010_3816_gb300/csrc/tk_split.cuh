@@ -14,10 +14,12 @@
 //
 // Measured, 25601 x 64, per step of the persistent launch: 147.0 us with the 54
 // instructions, 100.2 with this coupling converted by the FP64 conversion
-// instruction (which costs as much as a DFMA), 89.3 with the conversion in
+// instruction (which costs as much as a DFMA), 88.8 with the conversion in
 // integers too; the FP64 pipe is then 83 % busy, the rest is latency of the
 // integer chains with four warps per sub-partition.  25601 x 32: 73.2 -> 44.3,
-// x 128: 287 -> 185 us.  All of the step in integers (8 FP64 instructions left)
+// x 128: 287 -> 184 us.  More of the node in integers does not pay: with Pi + T
+// rounded once there (26 FP64 instructions) 90.0, with B (m - p) + Phi too (22)
+// 92.0 us: 37 integer instructions cost what a DFMA does.  All of the step in integers (8 FP64 instructions left)
 // took 147 us: its 1235 integer instructions per update are then the bound.
 //
 // Numbers.  A value is an integer X, 2^59 <= |X| < 2^60, with its own exponent
