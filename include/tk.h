@@ -252,7 +252,7 @@ tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfin
  * (<= 0: about sqrt(samples / substeps), the choice that minimises memory),
  * then, segment by segment from the last, the segment's inner states from its
  * checkpoint, against which the adjoint sweep runs.  Device memory:
- * (samples / C + C * substeps) states, up to seven adjoint states (256 MB at
+ * (samples / C + C * substeps) states, up to nine adjoint states (256 MB at
  * most, none where the memory does not reach) and one set of tables; the cost
  * is about two forward runs plus one adjoint run plus the tangent
  * contractions.  Writes the gradient to *grad (host).  Synchronizes. */

@@ -512,14 +512,11 @@ lw_adjoint_persistent_kernel(T *a0, T *a1, const T *__restrict__ half, const T *
 
 // ---- FP64: teams of warps and integer coupling (tk_split_adjoint.cuh) ----
 
-// load_lam for one row per lane.
-template <int K>
-__device__ __forceinline__ void load_lam_row(const double *__restrict__ lam, int i, int Nr, int row,
-                                             const InjectArgs &inj, int on, long long sample, double (&l)[4])
+// load_lam for one row per lane: the waveform gradient and the radial edges on a
+// loaded column.
+__device__ __forceinline__ void inject_row(int i, int Nr, int row, const InjectArgs &inj, int on, long long sample,
+                                           double (&l)[4])
 {
-    constexpr int NP = 32 * K;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) l[c] = __ldcg(lam + (size_t)i * (4 * NP) + c * NP + row);
     if (on) {
         for (int k = 0; k < inj.obs.n; ++k) {
             const int slot = (i == inj.obs.i0[k]) ? 0 : ((i == inj.obs.i0[k] + 1) ? 1 : -1);
@@ -539,6 +536,16 @@ __device__ __forceinline__ void load_lam_row(const double *__restrict__ lam, int
     if (i == 0 || i == Nr - 1)
 #pragma unroll
         for (int c = 0; c < 4; ++c) l[c] = 0.0;
+}
+
+template <int K>
+__device__ __forceinline__ void load_lam_row(const double *__restrict__ lam, int i, int Nr, int row,
+                                             const InjectArgs &inj, int on, long long sample, double (&l)[4])
+{
+    constexpr int NP = 32 * K;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) l[c] = __ldcg(lam + (size_t)i * (4 * NP) + c * NP + row);
+    inject_row(i, Nr, row, inj, on, sample, l);
 }
 
 template <int K>
@@ -626,6 +633,170 @@ lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restri
         warp_publish_cta(&step_done[wib], e + 1);
     }
     sw.drain(st);
+}
+
+// The same on grids with no more columns than the chip holds teams: lw_column_kernel
+// transposed.  A block has T columns and T + 1 teams; team j owns column T b - 1 +
+// j (j > 0) and forms eta at the half node to its right.  A column's sums are
+// formed once, by its owner (the block's outer neighbours' by the teams at its
+// ends), and the one to the left goes to the left team through shared memory with
+// lam~; eta and its sum to the right go to the right team for mu.  Two block
+// barriers a step; tables and columns stay in the SM.  us per step, this launch
+// (lw_adjoint_team_persistent_kernel, one or two columns per team): 1601 x 32 6.5
+// (10.0), 1824 x 32 7.2 (10.0 at 1825), 912 x 64 7.6 (9.6), 456 x 128 8.3 (10.9).
+// Bound by the chain pair - barrier - eta - pair - barrier - mu and by the FP64
+// pipe of the SMs with four blocks.  first: launch step s is the transposed step
+// first + s of the call; stride != 0: step s writes the whole level to a1 + s
+// stride, a0 stays.
+constexpr int kAdjColumns = 3;
+
+template <int K>
+struct AdjColumnShared {
+    static constexpr int T = kAdjColumns, NP = 32 * K;
+    alignas(16) unsigned char tab[T + 2][K][kAdjBytes];   // of columns T b - 2 ..
+    double lam[T + 1][4][NP], eta[T + 1][4][NP];
+    long long sum[2][T + 1][2][NP];                       // of lam~ to the left, of eta to the right
+    int exp[2][T + 1][2][NP];
+    int hot[2][T + 1];
+    SplitRows rows[(T + 1) * K];
+    unsigned long long bars[(T + 1) * K];
+};
+
+template <int K>
+__global__ void __launch_bounds__((kAdjColumns + 1) * K * 32, 4 / K)
+lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half, const double *__restrict__ node,
+                         const unsigned char *__restrict__ tab, int Nr, double en, const InjectArgs inj, int inject,
+                         long long n_inner, int substeps, unsigned int *flags, int *err, long long first,
+                         size_t stride)
+{
+    constexpr int T = kAdjColumns, NP = 32 * K;
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    AdjColumnShared<K> &sh = *reinterpret_cast<AdjColumnShared<K> *>(sh_raw);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, j = wib / K, h = wib % K, row = 32 * h + lane;
+    const int nb = (int)gridDim.x, b = (int)blockIdx.x, col = b * T - 1 + j;
+    const bool owner = j > 0 && col < Nr;              // of a column
+    const bool halves = col >= 0 && col + 1 < Nr;      // there is a half node right of it
+    const bool before = col > 0 && col < Nr;           // and one left of it
+    const FmaK<double> k1 = fma_k<double>();
+    SplitTeam<K> team{sh.rows + j * K, h, lane, 1 + j};
+    const unsigned char *left = sh.tab[j][h], *own = sh.tab[j + 1][h];   // of columns col - 1 and col
+    auto put = [&](double (*p)[NP], const double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[k][row] = x[k];
+    };
+    auto get = [&](const double (*p)[NP], double (&x)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = p[k][row];
+    };
+    auto put_sums = [&](int w, const AdjSums &s, bool hot) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            sh.sum[w][j][g][row] = s.T[g];
+            sh.exp[w][j][g][row] = s.O[g];
+        }
+        if (row == 0) sh.hot[w][j] = hot;
+    };
+    auto get_sums = [&](int w, int t, AdjSums &s) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            s.T[g] = sh.sum[w][t][g][row];
+            s.O[g] = sh.exp[w][t][g][row];
+        }
+        return sh.hot[w][t] != 0;
+    };
+    const bool extra = j == 0 && before;               // the block left of the first
+    if (halves || extra) {
+        if (lane == 0) {
+            unsigned long long *bar = &sh.bars[wib];
+            mbar_init(bar);
+            mbar_init_fence();
+            mbar_expect(bar, ((halves ? 1 : 0) + (extra ? 1 : 0)) * kAdjBytes);
+            if (halves) bulk_fetch(sh.tab[j + 1][h], tab + ((size_t)col * K + h) * kAdjBytes, kAdjBytes, bar);
+            if (extra) bulk_fetch(sh.tab[0][h], tab + ((size_t)(col - 1) * K + h) * kAdjBytes, kAdjBytes, bar);
+        }
+        __syncwarp();
+        if (!mbar_wait(&sh.bars[wib], 0)) atomicExch(err, 1);
+    }
+    double a[4];   // the column's adjoint state
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = owner ? __ldcg(a0 + (size_t)col * (4 * NP) + k * NP + row) : 0.0;
+    __syncthreads();
+#pragma unroll 1
+    for (long long s = 0; s < n_inner; ++s) {
+        const double *in = stride ? (s > 0 ? a1 + (s - 1) * stride : a0) : (s & 1) ? a1 : a0;
+        double *out = stride ? a1 + s * stride : (s & 1) ? a0 : a1;
+        const int on = inject && ((first + s) % substeps == 0);
+        const long long sample = inj.count - 1 - (first + s) / substeps;
+        const unsigned int e = (unsigned int)s;
+        // lam~ and its sums
+        AdjSums sa, sl;
+        adj_zero(sa);
+        adj_zero(sl);
+        bool hot_a = false;
+        if (j == 0 && halves) {
+            if (s > 0) warp_wait_flag(flags + (nb + b - 1) * K + h, e, err);
+            load_lam_row<K>(in, col, Nr, row, inj, on, sample, a);
+        } else if (owner) {
+            inject_row(col, Nr, row, inj, on, sample, a);
+        }
+        if (before && (owner || halves)) {
+            const int2 head = *reinterpret_cast<const int2 *>(left + kAdjExps + 256);
+            hot_a = adj_pair<K, false>(a, AdjTab<false>{left, lane}, head.y != 0, team, sa, sl);
+        }
+        put(sh.lam[j], a);
+        put_sums(0, sl, hot_a);
+        double c[4];
+        AdjSums sr;
+        bool hot_c = false;
+        const int2 head = halves ? *reinterpret_cast<const int2 *>(own + kAdjExps + 256) : make_int2(0, 0);
+        const bool imag = head.y != 0;
+        if (j == T && halves) {
+            if (s > 0) warp_wait_flag(flags + (b + 1) * K + h, e, err);
+            load_lam_row<K>(in, col + 1, Nr, row, inj, on, sample, c);
+            AdjSums unused;
+            hot_c = adj_pair<K, false>(c, AdjTab<false>{own, lane}, imag, team, unused, sr);
+        }
+        __syncthreads();
+        // eta
+        double ep[4];
+        AdjSums s1, s2;
+        bool hot_p = false;
+        if (halves) {
+            if (j < T) {
+                get(sh.lam[j + 1], c);
+                hot_c = get_sums(0, j + 1, sr);
+            }
+            if (hot_a || hot_c || head.x)
+                eta_row_cold<K>(a, c, node + (size_t)col * (kNCN * NP) + row, en, team, ep);
+            else
+                eta_row(a, c, sa, sr, imag, own, lane, en, k1, ep);
+            hot_p = adj_pair<K, true>(ep, AdjTab<true>{own, lane}, imag, team, s1, s2);
+            put(sh.eta[j], ep);
+            put_sums(1, s2, hot_p);
+        }
+        __syncthreads();
+        // mu
+        if (owner) {
+            if (col > 0 && halves) {
+                double em[4], o[4];
+                AdjSums sm;
+                get(sh.eta[j - 1], em);
+                const bool hot_m = get_sums(1, j - 1, sm);
+                if (hot_p || hot_m || head.x)
+                    mu_row_cold<K>(a, ep, em, half + (size_t)col * (kNCH * NP) + row, team, o);
+                else
+                    mu_row(a, ep, em, s1, sm, imag, own, lane, k1, o);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[k] = o[k];
+            } else {   // a radial edge
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[k] = 0.0;
+            }
+            if (j == 1 || j == T || s + 1 == n_inner || stride) store_row<K>(out, col, row, a);
+            if (j == 1) warp_publish_gpu(flags + b * K + h, e + 1);
+            if (j == T) warp_publish_gpu(flags + (nb + b) * K + h, e + 1);
+        }
+    }
 }
 
 // Transpose of the initial-data map of tk_set_initial_data: the adjoint state
@@ -949,6 +1120,57 @@ cudaError_t launch_adj_persistent_t(void *a0, void *a1, const void *half, const 
     return cudaErrorInvalidValue;
 }
 
+// Blocks of the one-column-per-team launch (FP64), 0 where the grid has too many
+// columns.
+template <int K>
+int adj_column_blocks(int Nr, int num_sms)
+{
+    int n = 0;
+    static cudaError_t e0 = cudaFuncSetAttribute(lw_adjoint_column_kernel<K>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)sizeof(AdjColumnShared<K>));
+    if (e0 != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_adjoint_column_kernel<K>, (kAdjColumns + 1) * K * 32,
+                                                      sizeof(AdjColumnShared<K>)) != cudaSuccess)
+        return 0;
+    const int blocks = (Nr + kAdjColumns - 1) / kAdjColumns;
+    return blocks <= num_sms * n ? blocks : 0;
+}
+
+int adjoint_column_blocks(int precision, int K, int Nr, int num_sms)
+{
+    if (precision != 0) return 0;
+    return K == 1 ? adj_column_blocks<1>(Nr, num_sms)
+         : K == 2 ? adj_column_blocks<2>(Nr, num_sms)
+                  : adj_column_blocks<4>(Nr, num_sms);
+}
+
+template <int K>
+cudaError_t launch_adj_columns(double *a0, double *a1, const void *half, const void *node, const unsigned char *tab,
+                               int Nr, int blocks, double dt_in, const InjectArgs &inj, int inject, long long n_inner,
+                               int substeps, unsigned int *flags, int *err, long long first, size_t stride,
+                               cudaStream_t st)
+{
+    const double *h = (const double *)half, *nd = (const double *)node;
+    double en = 0.5 * dt_in;
+    InjectArgs in = inj;
+    void *args[] = {&a0, &a1, &h, &nd, &tab, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err, &first, &stride};
+    return cudaLaunchCooperativeKernel((const void *)lw_adjoint_column_kernel<K>, dim3(blocks),
+                                       dim3((kAdjColumns + 1) * K * 32), args, sizeof(AdjColumnShared<K>), st);
+}
+
+cudaError_t launch_adjoint_columns(int K, double *a0, double *a1, const void *half, const void *node,
+                                   const unsigned char *tab, int Nr, int blocks, double dt_in, const InjectArgs &inj,
+                                   int inject, long long n_inner, int substeps, unsigned int *flags, int *err,
+                                   long long first, size_t stride, cudaStream_t st)
+{
+    auto go = [&](auto launch) {
+        return launch(a0, a1, half, node, tab, Nr, blocks, dt_in, inj, inject, n_inner, substeps, flags, err, first,
+                      stride, st);
+    };
+    return K == 1 ? go(launch_adj_columns<1>) : K == 2 ? go(launch_adj_columns<2>) : go(launch_adj_columns<4>);
+}
+
 // Blocks of the persistent adjoint launch for this grid (all resident at
 // once, at most Nr / warps), or 0 if it cannot run.
 int adjoint_persistent_blocks(int precision, int K, int Nr, int num_sms, int warps)
@@ -1129,7 +1351,8 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
                             : 0;
     if (pblocks > 0 && e == cudaSuccess) {
         unsigned int *flags = nullptr;
-        const int nflags = 2 * pblocks * (S->precision == TK_PREC_F64 ? S->K : 1);
+        const int cblocks = tk::adjoint_column_blocks(S->precision, S->K, S->Nr, S->num_sms);
+        const int nflags = 2 * std::max(pblocks, cblocks) * (S->precision == TK_PREC_F64 ? S->K : 1);
         const size_t fbytes = (size_t)nflags * sizeof(unsigned int) + sizeof(int);
         st = tkh::alloc(S, (void **)&flags, fbytes);
         if (st != TK_OK) {
@@ -1139,7 +1362,11 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
         int *derr = (int *)(flags + nflags);
         int herr = 0;
         e = cudaMemsetAsync(flags, 0, fbytes, S->stream);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && cblocks > 0)
+            e = tk::launch_adjoint_columns(S->K, (double *)S->adj[0], (double *)S->adj[1], S->half, S->node, S->adj_tab,
+                                           S->Nr, cblocks, dt_in, inj, dwave != nullptr, n_inner, S->substeps, flags,
+                                           derr, 0, 0, S->stream);
+        else if (e == cudaSuccess)
             e = tk::launch_adjoint_persistent(S->precision, S->K, S->adj[0], S->adj[1], S->half, S->node, S->adj_tab, S->Nr,
                                               pblocks, S->adj_warps, dt_in, inj, dwave != nullptr, n_inner,
                                               S->substeps, flags, derr, S->stream);
@@ -1224,14 +1451,18 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     const size_t nb = (size_t)S->Nr * S->NP;
 
     // the steps contracted per launch: their adjoint states are kept, two in the
-    // solver's own buffers, the others in the scratch (256 MB at most)
+    // solver's own buffers (small grids: in the scratch, in a row), the others in
+    // the scratch (256 MB at most)
     int Q = (int)std::min<long long>(std::min<long long>(C * k, tk::kLamSteps), 1 + (long long)((256ull << 20) / sb));
     const int blocks = std::max(1, S->Nr / (4 * std::min(4, 1 + S->Nr / 512))), pblocks = 1024;
 
     // small grids: a segment's levels in one launch (lw_column_kernel writing a
     // trajectory), 4.3 us a step at 1601 x 32 where a launch per step takes 8.6
     const bool columns = S->persist && S->persist_columns && C * k <= 0x7fffffff;
-    const size_t nflags = columns ? (size_t)2 * S->K * S->persist_blocks : 0;
+    // and the transposed steps that one tangent launch contracts (6.5 us a step
+    // there, 11 with a launch each; for fewer than four the launch costs more)
+    int cblocks = S->persist && Q >= 4 ? tk::adjoint_column_blocks(0, S->K, S->Nr, S->num_sms) : 0;
+    const size_t nflags = (size_t)2 * S->K * std::max(columns ? S->persist_blocks : 0, cblocks);
 
     // scratch in one allocation, freed on every exit
     double *dwave = nullptr, *scratch = nullptr;
@@ -1253,9 +1484,9 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     if (!S->db_node && (st = tkh::alloc(S, (void **)&S->db_node, nb * sizeof(double))) != TK_OK) return bail(st);
     // (one allocation: each costs some 70 us with its release); without the
     // further adjoint states where the memory does not reach
-    for (;; Q = 1) {
+    for (;; Q = 1, cblocks = 0) {
         struct { double **p; size_t n; } piece[] = {
-            {&ck, (size_t)nck * se}, {&seg, (size_t)(C * k) * se}, {&lam_more, (size_t)(Q - 1) * se},
+            {&ck, (size_t)nck * se}, {&seg, (size_t)(C * k) * se}, {&lam_more, (size_t)(cblocks ? Q + 1 : Q - 1) * se},
             {&tx, (size_t)tk::kShifts * 2 * S->Nr * tk::kRadial}, {&tang, (size_t)2 * S->NP},
             {&acc, (size_t)(blocks + pblocks)}, {&parts, (size_t)Q * blocks}, {&pflags, 1 + (nflags + 1) / 2}};
         size_t total = 0;
@@ -1269,10 +1500,11 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
             }
             break;
         }
-        if (Q == 1) return bail(st);
+        if (Q == 1 && !cblocks) return bail(st);
     }
     double *lam[tk::kLamSteps + 1];   // a ring of Q + 1 adjoint states
-    for (int q = 0; q <= Q; ++q) lam[q] = q < 2 ? (double *)S->adj[q] : lam_more + (size_t)(q - 2) * se;
+    for (int q = 0; q <= Q; ++q)
+        lam[q] = cblocks ? lam_more + (size_t)q * se : q < 2 ? (double *)S->adj[q] : lam_more + (size_t)(q - 2) * se;
     if (on_device) {
         dwave = const_cast<double *>(dL_dwave);
     } else {
@@ -1366,7 +1598,15 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
         for (long long g = 0; g < len * k && e == cudaSuccess;) {   // transposed steps from the segment's end
             const int n = (int)std::min<long long>(Q, len * k - g);
             tk::LamSet set = {};
-            for (int q = 0; q < n && e == cudaSuccess; ++q) {
+            if (cblocks) {   // lam[0] to lam[1], .., lam[n]
+                for (int q = 0; q < n; ++q) set.p[q] = lam[q];
+                e = cudaMemsetAsync(flags, 0, nflags * sizeof(unsigned int), S->stream);
+                if (e == cudaSuccess)
+                    e = tk::launch_adjoint_columns(S->K, lam[0], lam[1], S->half, S->node, S->adj_tab, S->Nr, cblocks,
+                                                   dt_in, inj, 1, n, k, flags, perr,
+                                                   (count - t0 - len) * k + g, se, S->stream);
+            }
+            for (int q = 0; !cblocks && q < n && e == cudaSuccess; ++q) {
                 const int nxt = cur == Q ? 0 : cur + 1;
                 set.p[q] = lam[cur];
                 inj.on = (g + q) % k == 0;
@@ -1379,6 +1619,8 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
                 e = tk::launch_param_tangent(S->K, blocks, n, seg + (size_t)(len * k - 1 - g) * se, set, g,
                                              t0 + len - 1, k, (const double *)S->half, (const double *)S->node,
                                              S->dhalf, S->dnode, S->Nr, dt_in, inj, parts, acc, S->stream);
+            if (e == cudaSuccess && cblocks)
+                e = cudaMemcpyAsync(lam[0], lam[n], sb, cudaMemcpyDeviceToDevice, S->stream);
             g += n;
         }
     }

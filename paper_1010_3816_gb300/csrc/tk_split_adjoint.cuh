@@ -264,6 +264,85 @@ __device__ __noinline__ Row4 cold_mu(Row4 l, Row4 p, Row4 m, double ypR, double 
     return o;
 }
 
+// ---- eta and mu on a lane's row, for lw_adjoint_column_kernel ----
+// (the sweep below has the same operations in place: called from there, these
+// cost it four bytes of spills and 1 % of its time)
+
+// eta at the half node between columns with lam~ a and c, from their sums sa and
+// sr; p: the table block of the left column.
+__device__ __forceinline__ void eta_row(const double (&a)[4], const double (&c)[4], const AdjSums &sa, const AdjSums &sr,
+                                        bool imag, const unsigned char *p, int lane, double E, const FmaK<double> &k1,
+                                        double (&ep)[4])
+{
+    const AdjSums s = adj_add(sa, sr);
+    const double BA = adj_f64(p, A_BA, lane), BC = adj_f64(p, A_BC, lane);
+    const double PP = adj_f64(p, A_PP, lane), PM = adj_f64(p, A_PM, lane);
+    ep[0] = fma(BC, c[0], fma(-BA, a[0], split_value(s.T[0], s.O[0])));
+    ep[1] = fma(BC, c[1], fma(-BA, a[1], split_value(s.T[1], s.O[1])));
+    double x = fma(E, c[0], fma(PP, a[2], fma(E, a[0], k1.nz)));
+    double y = fma(E, c[1], fma(PP, a[3], fma(E, a[1], k1.nz)));
+    if (imag) {
+        const double CA = adj_f64(p, A_CA, lane), CC = adj_f64(p, A_CC, lane);
+        x = fma(CC, c[3], fma(CA, a[3], x));
+        y = fma(-CC, c[2], fma(-CA, a[2], y));
+    }
+    ep[2] = fma(PM, c[2], x);
+    ep[3] = fma(PM, c[3], y);
+}
+
+// The same with the FP64 instructions alone; ta: the left column's row of the
+// unsplit node table.
+template <int K>
+__device__ __forceinline__ void eta_row_cold(const double (&a)[4], const double (&c)[4], const double *ta, double E,
+                                             SplitTeam<K> &team, double (&ep)[4])
+{
+    constexpr int NP = 32 * K;
+    double za[2], zc[2];
+    const double *tc = ta + kNCN * NP;
+    cold_sources<K>(a, ta + N_KP * NP, ta + N_KM * NP, team, za);
+    cold_sources<K>(c, tc + N_KP * NP, tc + N_KM * NP, team, zc);
+    const Row4 r = cold_eta<NP>(row4(a), row4(c), za[0], za[1], zc[0], zc[1], ta, tc, E);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ep[k] = r.v[k];
+}
+
+// mu at a node from its lam~ a and eta right (ep) and left (em) of it with their
+// sums s1 and sm.
+__device__ __forceinline__ void mu_row(const double (&a)[4], const double (&ep)[4], const double (&em)[4],
+                                       const AdjSums &s1, const AdjSums &sm, bool imag, const unsigned char *p, int lane,
+                                       const FmaK<double> &k1, double (&o)[4])
+{
+    const AdjSums s = adj_add(s1, sm);
+    const double HP = adj_f64(p, A_HP, lane), HQ = adj_f64(p, A_HQ, lane);
+    const double PA = adj_f64(p, A_PA, lane), PC = adj_f64(p, A_PC, lane);
+    o[0] = fma(HQ, em[0], fma(HP, ep[0], fma(a[0], k1.one, split_value(s.T[0], s.O[0]))));
+    o[1] = fma(HQ, em[1], fma(HP, ep[1], fma(a[1], k1.one, split_value(s.T[1], s.O[1]))));
+    double x = fma(em[0], k1.one, fma(PA, ep[2], fma(ep[0], k1.one, a[2])));
+    double y = fma(em[1], k1.one, fma(PA, ep[3], fma(ep[1], k1.one, a[3])));
+    if (imag) {
+        const double PI = adj_f64(p, A_PI, lane), PJ = adj_f64(p, A_PJ, lane);
+        x = fma(PJ, em[3], fma(PI, ep[3], x));
+        y = fma(-PJ, em[2], fma(-PI, ep[2], y));
+    }
+    o[2] = fma(PC, em[2], x);
+    o[3] = fma(PC, em[3], y);
+}
+
+// tp: the node's row of the unsplit half-node table.
+template <int K>
+__device__ __forceinline__ void mu_row_cold(const double (&a)[4], const double (&ep)[4], const double (&em)[4],
+                                            const double *tp, SplitTeam<K> &team, double (&o)[4])
+{
+    constexpr int NP = 32 * K;
+    double yp[2], ym[2];
+    const double *tm = tp - kNCH * NP;
+    cold_sources<K>(ep, tp + H_KP * NP, tp + H_KM * NP, team, yp);
+    cold_sources<K>(em, tm + H_KP * NP, tm + H_KM * NP, team, ym);
+    const Row4 r = cold_mu<NP>(row4(a), row4(ep), row4(em), yp[0], yp[1], ym[0], ym[1], tp, tm);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[k] = r.v[k];
+}
+
 // ---- the sweep of one transposed step over a team's columns ----
 
 struct AdjRing {

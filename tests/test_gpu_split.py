@@ -279,3 +279,12 @@ def test_small_grid_launch_at_its_edges(Nr, Nth):
         ref, wref = _run(w, 1, n=n)
         s, wv = _run(w, 0, n=n)
         assert np.array_equal(s, ref) and all(np.array_equal(a, b) for a, b in zip(wv, wref))
+
+
+@pytest.mark.parametrize("Nr,Nth,k", [(4, 32, 1), (5, 20, 2), (1824, 32, 1), (1825, 32, 1), (911, 50, 3), (912, 64, 1),
+                                      (913, 64, 1), (455, 128, 2), (456, 97, 1), (457, 128, 1)])
+def test_small_grid_adjoint_at_its_edges(Nr, Nth, k):
+    """The transposed step with one column per team, at the ends of its range and
+    of its blocks of three: the bits of one launch per step."""
+    w = _work(Nr, Nth, substeps=k)
+    assert np.array_equal(_adjoint(w, 0)[3], _adjoint(w, 1)[3])
