@@ -120,7 +120,7 @@ __device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long
 // blocks finished.  The last block to finish empties the queue for the next
 // launch and, after the last tick of an outer step, moves every member's
 // sample counter on (every block has read them by then).
-template <typename T>
+template <typename T, int KALL>
 __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 4 : 1)
 batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem *__restrict__ items,
                   int nitems, int tick, int kmax, int outer, unsigned int *ctr)
@@ -158,7 +158,9 @@ batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem
         if constexpr (F64) {
             SplitRing *ring = reinterpret_cast<SplitRing *>(sh_raw);
             unsigned long long *bar = bars[threadIdx.x >> 5];
-            switch (m.K) {
+            if constexpr (KALL > 0) {
+                sweep_teams<KALL>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now);
+            } else switch (m.K) {
             case 1: sweep_teams<1>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
             case 2: sweep_teams<2>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
             default: sweep_teams<4>(m, ring, bar, rows, st, u_in, u_out, w.i0, w.i1, obs_now); break;
@@ -191,30 +193,41 @@ batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem
 // Shared memory of the FP64 kernel's table rings.
 constexpr size_t kBatchSmem = kBatchThreads / 32 * sizeof(SplitRing);
 
-static int batch_resident_blocks(int precision)
+// The FP64 kernel for members that all have 32 kall rows (0: mixed).  With the
+// three sweeps in one kernel it spills 250 bytes, 20 loads and 12 stores per
+// column; alone none does: 6 x 1601 x 32 28.1 -> 25.8 us per tick.
+using BatchKernel = void (*)(const BatchMember *, int, const BatchItem *, int, int, int, int, unsigned int *);
+static BatchKernel batch_kernel_f64(int kall)
+{
+    return kall == 1 ? batch_step_kernel<double, 1>
+         : kall == 2 ? batch_step_kernel<double, 2>
+         : kall == 4 ? batch_step_kernel<double, 4>
+                     : batch_step_kernel<double, 0>;
+}
+
+static int batch_resident_blocks(int precision, int kall)
 {
     int n = 0;
     cudaError_t e = cudaSuccess;
     if (precision == 0) {
-        e = cudaFuncSetAttribute(batch_step_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBatchSmem);
+        const BatchKernel kern = batch_kernel_f64(kall);
+        e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<double>, kBatchThreads,
-                                                              kBatchSmem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kBatchThreads, kBatchSmem);
     } else {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<float>, kBatchThreads, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<float, 0>, kBatchThreads, 0);
     }
     return (e != cudaSuccess || n < 1) ? 1 : n;
 }
 
-static cudaError_t launch_batch_tick(int precision, int blocks, const BatchMember *mem, int nmem,
+static cudaError_t launch_batch_tick(int precision, int kall, int blocks, const BatchMember *mem, int nmem,
                                      const BatchItem *items, int nitems, int tick, int kmax,
                                      int outer, unsigned int *ctr, cudaStream_t st)
 {
     if (precision == 0)
-        return launch_chained(batch_step_kernel<double>, (unsigned)blocks, kBatchThreads, kBatchSmem, st, mem,
+        return launch_chained(batch_kernel_f64(kall), (unsigned)blocks, kBatchThreads, kBatchSmem, st, mem,
                               nmem, items, nitems, tick, kmax, outer, ctr);
-    return launch_chained(batch_step_kernel<float>, (unsigned)blocks, kBatchThreads, 0, st, mem, nmem,
+    return launch_chained(batch_step_kernel<float, 0>, (unsigned)blocks, kBatchThreads, 0, st, mem, nmem,
                           items, nitems, tick, kmax, outer, ctr);
 }
 
@@ -227,6 +240,7 @@ struct tk_batch {
     int n = 0;
     std::vector<tk_solver *> mem;
     int kmax = 1;
+    int kall = 0;      // the members' common K, 0 if they differ
     int blocks = 1;
     int seg = 32;
     // step the members one after another, each as tk_step would (segment
@@ -349,7 +363,7 @@ tk_status enqueue(tk_batch *B, int outer_steps, cudaStream_t st)
     for (int o = 0; o < outer_steps; ++o)
         for (int t = 0; t < B->kmax; ++t) {
             if (B->tick_n[t] == 0) continue;
-            TKB_CUDA(B, tk::launch_batch_tick(B->precision, B->blocks, B->d_mem, B->n,
+            TKB_CUDA(B, tk::launch_batch_tick(B->precision, B->kall, B->blocks, B->d_mem, B->n,
                                               B->d_items + B->tick_off[t], B->tick_n[t], t, B->kmax,
                                               o, B->d_ctr, st));
         }
@@ -428,13 +442,16 @@ tk_status tk_batch_create(tk_batch **out, tk_solver *const *members, int n)
         }
     }
     B->kmax = (int)lcm;
+    B->kall = S0->K;
+    for (tk_solver *S : B->mem)
+        if (S->K != S0->K) B->kall = 0;
     tk_status st = TK_OK;
     if (cudaSetDevice(B->device) != cudaSuccess) st = TK_ERR_CUDA;
     if (st == TK_OK && cudaMalloc(&B->d_mem, n * sizeof(tk::BatchMember)) != cudaSuccess) st = TK_ERR_OOM;
     if (st == TK_OK && cudaMalloc(&B->d_ctr, 2 * sizeof(unsigned int)) != cudaSuccess) st = TK_ERR_OOM;
     if (st == TK_OK && cudaMemset(B->d_ctr, 0, 2 * sizeof(unsigned int)) != cudaSuccess) st = TK_ERR_CUDA;
     if (st == TK_OK) {
-        B->blocks = S0->num_sms * tk::batch_resident_blocks(B->precision);
+        B->blocks = S0->num_sms * tk::batch_resident_blocks(B->precision, B->kall);
         long long cols = 0;
         for (tk_solver *S : B->mem) cols += S->Nr;
         // default: about four items per taker (FP64: a block, FP32: a warp) of
@@ -560,7 +577,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
     // (blocks per SM, up to the resident maximum; fewer blocks leave each
     // warp more items of the queue)
     const int candidates[] = {4, 8, 12, 16, 24, 32, 48, 64, 96, 128};
-    const int sms = B->mem[0]->num_sms, max_per_sm = tk::batch_resident_blocks(B->precision);
+    const int sms = B->mem[0]->num_sms, max_per_sm = tk::batch_resident_blocks(B->precision, B->kall);
     int best = B->seg, best_blocks = B->blocks;
     double best_t = 1e300;
     cudaEvent_t e0, e1;
