@@ -803,28 +803,39 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
 // lam0 = dL/du^0 (device layout) to dL/d(input planes) in [Ntheta][Nr].
 // independent_pi: the momentum planes were given (4 output planes); else
 // Pi_m = b_m (Phi_{m+1} - Phi_{m-1}) / (2 dr*) at interior m (2 output planes).
-template <typename T>
-__global__ void initial_transpose_kernel(int Nr, int Nth, int NP, double drs,
-                                         const T *__restrict__ lam0, const double *__restrict__ b_node,
-                                         int independent_pi, double *__restrict__ out)
+// Tiles of 32 rows by TI columns (tile_columns) go through shared memory so that
+// the planes are written in runs, and the spacing's inverse saves the divisions:
+// 16001 x 128 328 -> 36 us, 4001 x 64 48 -> 8.2.
+template <typename T, int TI>
+__global__ void __launch_bounds__(kTileThreads)
+initial_transpose_kernel(int Nr, int Nth, int NP, SpacingInverse d, const T *__restrict__ lam0,
+                         const double *__restrict__ b_node, int independent_pi, double *__restrict__ out)
 {
-    const int jp = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (jp >= Nth || i >= Nr) return;
-    const size_t plane = (size_t)Nth * Nr, k = (size_t)jp * Nr + i;
+    __shared__ double f[4][32][TI + 1];
+    const int j0 = blockIdx.x * 32, i0 = blockIdx.y * TI, lane = threadIdx.x & 31, jp = j0 + lane;
+    const size_t plane = (size_t)Nth * Nr;
+    const int nout = independent_pi ? 4 : 2;
     auto L = [&](int ii, int c) { return (double)lam0[((size_t)ii * 4 + c) * NP + jp]; };
-    double g[4] = {0.0, 0.0, 0.0, 0.0};
-    if (i > 0 && i < Nr - 1) {
-        for (int c = 0; c < 4; ++c) g[c] = L(i, c);
-        if (!independent_pi) {
-            for (int c = 0; c < 2; ++c) {
-                if (i - 1 >= 1) g[c] += b_node[(size_t)(i - 1) * NP + jp] * L(i - 1, 2 + c) / (2.0 * drs);
-                if (i + 1 <= Nr - 2) g[c] -= b_node[(size_t)(i + 1) * NP + jp] * L(i + 1, 2 + c) / (2.0 * drs);
+    for (int x = threadIdx.x >> 5; x < TI; x += kTileThreads / 32) {
+        const int i = i0 + x;
+        double g[4] = {0.0, 0.0, 0.0, 0.0};
+        if (i > 0 && i < Nr - 1) {
+            for (int c = 0; c < 4; ++c) g[c] = L(i, c);
+            if (!independent_pi) {
+                for (int c = 0; c < 2; ++c) {
+                    if (i - 1 >= 1) g[c] += d.over(b_node[(size_t)(i - 1) * NP + jp] * L(i - 1, 2 + c));
+                    if (i + 1 <= Nr - 2) g[c] -= d.over(b_node[(size_t)(i + 1) * NP + jp] * L(i + 1, 2 + c));
+                }
             }
         }
+        for (int c = 0; c < nout; ++c) f[c][lane][x] = g[c];
     }
-    const int nout = independent_pi ? 4 : 2;
-    for (int c = 0; c < nout; ++c) out[c * plane + k] = g[c];
+    __syncthreads();
+    for (int q = threadIdx.x; q < 32 * TI; q += kTileThreads) {
+        const int r = q / TI, x = q % TI, i = i0 + x;
+        if (j0 + r >= Nth || i >= Nr) continue;
+        for (int c = 0; c < nout; ++c) out[c * plane + (size_t)(j0 + r) * Nr + i] = f[c][r][x];
+    }
 }
 
 // ---- gradients with respect to the black-hole parameters (a or M) ----
@@ -1405,13 +1416,18 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
             return st;
         }
     }
-    dim3 block(32, 8), gridd((S->NP + 31) / 32, (S->Nr + 7) / 8);
+    const int ti = tk::tile_columns(S->Nr, S->NP);
+    const dim3 gridd(S->NP / 32, (S->Nr + ti - 1) / ti);
+    const tk::SpacingInverse d = tk::spacing_inverse(S->drs);
+    auto transpose = [&](auto kern, auto *lam) {
+        kern<<<gridd, tk::kTileThreads, 0, S->stream>>>(S->Nr, S->Nth, S->NP, d, lam, S->b_node, independent_pi, gdev);
+    };
     if (S->precision == 0)
-        tk::initial_transpose_kernel<double><<<gridd, block, 0, S->stream>>>(
-            S->Nr, S->Nth, S->NP, S->drs, (const double *)S->adj[cur], S->b_node, independent_pi, gdev);
+        transpose(ti == 8 ? tk::initial_transpose_kernel<double, 8> : tk::initial_transpose_kernel<double, 32>,
+                  (const double *)S->adj[cur]);
     else
-        tk::initial_transpose_kernel<float><<<gridd, block, 0, S->stream>>>(
-            S->Nr, S->Nth, S->NP, S->drs, (const float *)S->adj[cur], S->b_node, independent_pi, gdev);
+        transpose(ti == 8 ? tk::initial_transpose_kernel<float, 8> : tk::initial_transpose_kernel<float, 32>,
+                  (const float *)S->adj[cur]);
     e = cudaGetLastError();
     if (e == cudaSuccess && !grad_on_device)
         e = cudaMemcpyAsync(grad, gdev, nout * plane * sizeof(double), cudaMemcpyDeviceToHost, S->stream);

@@ -9,6 +9,7 @@
 // so a column of any plane or table is one contiguous, coalesced vector load.
 #pragma once
 
+#include <math.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -105,6 +106,26 @@ struct KerrSet {
     Kerr k[kShifts];
     double w[kShifts];
 };
+
+// Tiles of the transposes between the planes and the state: 32 rows by 32
+// columns, on small grids by 8 (64 bytes at a time, but four times the blocks).
+constexpr int kTileThreads = 256;
+inline int tile_columns(int Nr, int NP) { return (long long)(Nr / 32) * (NP / 32) < 304 ? 8 : 32; }
+
+// x / (2 dr*): a division costs the FP64 pipe some ten instructions of 64 cycles;
+// where 2 dr* is a power of two, one multiplication by its inverse gives the same bits.
+struct SpacingInverse {
+    double d2, inv;   // 2 dr*; its inverse, 0 where it is not a power of two
+#ifdef __CUDACC__
+    __device__ __forceinline__ double over(double x) const { return inv != 0.0 ? x * inv : x / d2; }
+#endif
+};
+inline SpacingInverse spacing_inverse(double drs)
+{
+    int e;
+    const double d2 = 2.0 * drs;
+    return SpacingInverse{d2, frexp(d2, &e) == 0.5 && e > -1000 && e < 1000 ? 1.0 / d2 : 0.0};
+}
 
 struct ObsDev {
     int n;                          // number of observers
