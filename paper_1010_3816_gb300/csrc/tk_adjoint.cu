@@ -808,7 +808,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
 // 16001 x 128 328 -> 36 us, 4001 x 64 48 -> 8.2.
 template <typename T, int TI>
 __global__ void __launch_bounds__(kTileThreads)
-initial_transpose_kernel(int Nr, int Nth, int NP, SpacingInverse d, const T *__restrict__ lam0,
+initial_transpose_kernel(int Nr, int Nth, int NP, Divisor d, const T *__restrict__ lam0,
                          const double *__restrict__ b_node, int independent_pi, double *__restrict__ out)
 {
     __shared__ double f[4][32][TI + 1];
@@ -823,8 +823,8 @@ initial_transpose_kernel(int Nr, int Nth, int NP, SpacingInverse d, const T *__r
             for (int c = 0; c < 4; ++c) g[c] = L(i, c);
             if (!independent_pi) {
                 for (int c = 0; c < 2; ++c) {
-                    if (i - 1 >= 1) g[c] += d.over(b_node[(size_t)(i - 1) * NP + jp] * L(i - 1, 2 + c));
-                    if (i + 1 <= Nr - 2) g[c] -= d.over(b_node[(size_t)(i + 1) * NP + jp] * L(i + 1, 2 + c));
+                    if (i - 1 >= 1) g[c] += d.under(b_node[(size_t)(i - 1) * NP + jp] * L(i - 1, 2 + c));
+                    if (i + 1 <= Nr - 2) g[c] -= d.under(b_node[(size_t)(i + 1) * NP + jp] * L(i + 1, 2 + c));
                 }
             }
         }
@@ -1418,7 +1418,7 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
     }
     const int ti = tk::tile_columns(S->Nr, S->NP);
     const dim3 gridd(S->NP / 32, (S->Nr + ti - 1) / ti);
-    const tk::SpacingInverse d = tk::spacing_inverse(S->drs);
+    const tk::Divisor d = tk::divisor(2.0 * S->drs);
     auto transpose = [&](auto kern, auto *lam) {
         kern<<<gridd, tk::kTileThreads, 0, S->stream>>>(S->Nr, S->Nth, S->NP, d, lam, S->b_node, independent_pi, gdev);
     };

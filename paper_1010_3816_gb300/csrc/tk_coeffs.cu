@@ -278,7 +278,7 @@ struct Entries {
 };
 
 // Of row jp < NP (polar angle th) and column i; all zero outside the grid.
-__device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr, int Nth, int NP, double drs, double dt,
+__device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr, int Nth, int NP, Divisor ds, Divisor de, double dt,
                                               double dth, double th, int i, int jp, const double *__restrict__ rad,
                                               const double *__restrict__ ang, const Angular &A,
                                               const double *__restrict__ raw_node,
@@ -312,8 +312,8 @@ __device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr
             if (i > 0 && i < Nr - 1) {
                 E.c4n = c.c4;
                 const double h2 = 0.5 * dt;
-                const double B = dt * c.b / drs;
-                const double g1r = dt * c.c1r / drs, g1i = dt * c.c1i / drs;
+                const double B = ds.under(dt * c.b);
+                const double g1r = ds.under(dt * c.c1r), g1i = ds.under(dt * c.c1i);
                 double kp, km;
                 if (variable == 0) {
                     kp = h2 * (c.c4 * ith2 + c.c5 * i2th);
@@ -346,8 +346,8 @@ __device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr
                                    : raw_coefficients(P, rad + (size_t)(Nr + i) * kRadial, A);
             E.c4h = c.c4;
             const double dtau = 0.5 * dt, e2 = 0.5 * dtau;
-            const double B = dtau * c.b / drs;
-            const double g1r = dtau * c.c1r / drs, g1i = dtau * c.c1i / drs;
+            const double B = ds.under(dtau * c.b);
+            const double g1r = ds.under(dtau * c.c1r), g1i = ds.under(dtau * c.c1i);
             double kp, km;
             if (variable == 0) {
                 kp = e2 * (c.c4 * ith2 + c.c5 * i2th);
@@ -362,8 +362,8 @@ __device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr
             if (variable == 0 && jp == Nth - 1) { far += p * kp; fcr += p * kp; kp = 0.0; }
             // the Phi half-node value is returned divided by e2 (= eh): its
             // Pi term e2 (Pi_a + Pi_c) then needs no multiplication
-            hv[H_HP] = (0.5 + B) / e2;
-            hv[H_HQ] = (0.5 - B) / e2;
+            hv[H_HP] = de.under(0.5 + B);
+            hv[H_HQ] = de.under(0.5 - B);
             hv[H_PAR] = 0.5 - B + e2 * c.c2r;
             hv[H_PCR] = 0.5 + B + e2 * c.c2r;
             hv[H_PI] = e2 * c.c2i;
@@ -382,12 +382,13 @@ __device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr
 // FP64 pipe: what depends on the radius alone comes from the inversion kernel,
 // what depends on the angle alone is formed once per thread, which takes
 // columns in turns (with both formed at every point 372 us at 4001 x 64, now
-// 217).
+// 217; with the divisions by dr* and e as multiplications where these are powers
+// of two 193).
 constexpr int kTableThreads = 256;
 
 template <typename T>
 __global__ void __launch_bounds__(kTableThreads)
-coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, double dt,
+coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, Divisor ds, Divisor de, double dt,
                     const double *__restrict__ rad, const double *__restrict__ ang, T *__restrict__ half,
                     T *__restrict__ node, double *__restrict__ b_node, double *__restrict__ w_row,
                     float *__restrict__ cmp, float *__restrict__ gpm, F32Derive fd,
@@ -412,7 +413,7 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
         T *hcol = half + (size_t)i * kNCH * NP + jp;
         T *ncol = node + (size_t)i * kNCN * NP + jp;
         Entries E;
-        table_entries(P, variable, Nr, Nth, NP, drs, dt, dth, th, i, jp, rad, ang, A, raw_node, raw_half, E);
+        table_entries(P, variable, Nr, Nth, NP, ds, de, dt, dth, th, i, jp, rad, ang, A, raw_node, raw_half, E);
         const double (&hv)[kNCH] = E.hv, (&nv)[kNCN] = E.nv;
         if (i == 0 && w_row)
             w_row[jp] = jp >= Nth ? 0.0 : (variable != 0) ? weight_w(P.s, P.m, th) : 1.0;
@@ -517,10 +518,11 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, double drs, 
 // The tables' derivative in a parameter of the black hole: the sum over q of
 // w[q] times the tables of kp.k[q], whose radial parts are rad[q].  One pass:
 // the tables of the shifted parameters stay in registers.  Bound by the FP64
-// pipe: 214 us at 1601 x 32; with each shifted table written out and added by
+// pipe: 187 us at 1601 x 32; with each shifted table written out and added by
 // kernels of their own the four took 350 us and twice the table memory.
 __global__ void __launch_bounds__(kTableThreads)
-table_derivative_kernel(const __grid_constant__ KerrSet kp, int variable, int Nr, int Nth, int NP, double drs, double dt,
+table_derivative_kernel(const __grid_constant__ KerrSet kp, int variable, int Nr, int Nth, int NP, Divisor ds,
+                        Divisor de, double dt,
                         const double *__restrict__ rad, const double *__restrict__ ang, double *__restrict__ half,
                         double *__restrict__ node, double *__restrict__ b_node)
 {
@@ -535,7 +537,7 @@ table_derivative_kernel(const __grid_constant__ KerrSet kp, int variable, int Nr
 #pragma unroll 1
         for (int q = 0; q < kShifts; ++q) {
             Entries E;
-            table_entries(geometry(kp.k[q]), variable, Nr, Nth, NP, drs, dt, dth, th, i, jp,
+            table_entries(geometry(kp.k[q]), variable, Nr, Nth, NP, ds, de, dt, dth, th, i, jp,
                           rad + (size_t)q * 2 * Nr * kRadial, ang, A, nullptr, nullptr, E);
             const double w = kp.w[q];
 #pragma unroll
@@ -665,7 +667,8 @@ cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_m
     if (e == cudaSuccess && variable != 0) e = launch_stencil(kp.k[0].s, kp.k[0].m, Ntheta, NP, ang, st);
     if (e != cudaSuccess) return e;
     const dim3 block(NP, kTableThreads / NP);
-    table_derivative_kernel<<<table_grid(Nr, block), block, 0, st>>>(kp, variable, Nr, Ntheta, NP, drs, dt_inner, rad,
+    table_derivative_kernel<<<table_grid(Nr, block), block, 0, st>>>(kp, variable, Nr, Ntheta, NP, divisor(drs),
+                                                                     divisor(0.25 * dt_inner), dt_inner, rad,
                                                                      ang, half, node, b_node);
     return cudaGetLastError();
 }
@@ -683,13 +686,14 @@ cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta,
     }
     dim3 block(NP, kTableThreads / NP);
     const dim3 grid = table_grid(Nr, block);
+    const Divisor ds = divisor(drs), de = divisor(0.25 * dt_inner);   // dr*, the half node's e
     if (precision == 0)
-        coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
+        coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, ds, de, dt_inner,
                                                              rad, ang, (double *)half,
                                                              (double *)node, b_node, w_row, nullptr,
                                                              nullptr, fd, raw_node, raw_half, step);
     else
-        coeff_tables_kernel<float><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, drs, dt_inner,
+        coeff_tables_kernel<float><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, ds, de, dt_inner,
                                                             rad, ang, (float *)half,
                                                             (float *)node, b_node, w_row, cmp, gpm, fd,
                                                             raw_node, raw_half, nullptr);

@@ -112,19 +112,19 @@ struct KerrSet {
 constexpr int kTileThreads = 256;
 inline int tile_columns(int Nr, int NP) { return (long long)(Nr / 32) * (NP / 32) < 304 ? 8 : 32; }
 
-// x / (2 dr*): a division costs the FP64 pipe some ten instructions of 64 cycles;
-// where 2 dr* is a power of two, one multiplication by its inverse gives the same bits.
-struct SpacingInverse {
-    double d2, inv;   // 2 dr*; its inverse, 0 where it is not a power of two
+// Division by a constant: a division costs the FP64 pipe some ten instructions of
+// 64 cycles; where the constant is a power of two, one multiplication by its
+// inverse gives the same bits (never contracted with what follows).
+struct Divisor {
+    double d, inv;   // the constant; its inverse, 0 where it is not a power of two
 #ifdef __CUDACC__
-    __device__ __forceinline__ double over(double x) const { return inv != 0.0 ? x * inv : x / d2; }
+    __device__ __forceinline__ double under(double x) const { return inv != 0.0 ? __dmul_rn(x, inv) : x / d; }
 #endif
 };
-inline SpacingInverse spacing_inverse(double drs)
+inline Divisor divisor(double d)
 {
     int e;
-    const double d2 = 2.0 * drs;
-    return SpacingInverse{d2, frexp(d2, &e) == 0.5 && e > -1000 && e < 1000 ? 1.0 / d2 : 0.0};
+    return Divisor{d, frexp(d, &e) == 0.5 && e > -1000 && e < 1000 ? 1.0 / d : 0.0};
 }
 
 struct ObsDev {

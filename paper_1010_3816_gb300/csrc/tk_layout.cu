@@ -19,7 +19,7 @@ namespace {
 // Both fields vanish on the radial edges; padding rows are zero.
 template <typename T, int TI>
 __global__ void __launch_bounds__(kTileThreads)
-import_kernel(int Nr, int Nth, int NP, SpacingInverse d, const double *__restrict__ phr,
+import_kernel(int Nr, int Nth, int NP, Divisor d, const double *__restrict__ phr,
               const double *__restrict__ phi, const double *__restrict__ pir, const double *__restrict__ pii,
               const double *__restrict__ b_node, T *__restrict__ u)
 {
@@ -55,8 +55,8 @@ import_kernel(int Nr, int Nth, int NP, SpacingInverse d, const double *__restric
                 v[3] = g[1][r][x];
             } else {
                 const double b = b_node[(size_t)i * NP + jp];
-                v[2] = d.over(b * (f[0][r][x + 2] - f[0][r][x]));
-                v[3] = d.over(b * (f[1][r][x + 2] - f[1][r][x]));
+                v[2] = d.under(b * (f[0][r][x + 2] - f[0][r][x]));
+                v[3] = d.under(b * (f[1][r][x + 2] - f[1][r][x]));
             }
         }
         T *col = u + (size_t)i * 4 * NP + jp;
@@ -197,7 +197,7 @@ cudaError_t launch_import_state(int precision, int Nr, int Ntheta, int NP, doubl
 {
     const int ti = tile_columns(Nr, NP);
     const dim3 grid(NP / 32, (Nr + ti - 1) / ti);
-    const SpacingInverse d = spacing_inverse(drs);
+    const Divisor d = divisor(2.0 * drs);
     auto go = [&](auto kern, auto *w) {
         kern<<<grid, kTileThreads, 0, st>>>(Nr, Ntheta, NP, d, phi_re, phi_im, pi_re, pi_im, b_node, w);
     };
