@@ -229,8 +229,8 @@ lw_adjoint_kernel(const T *__restrict__ lam, T *__restrict__ mu_out, const T *__
     constexpr int NP = 32 * K;
     constexpr size_t SP = 4 * NP, HP = (size_t)kNCH * NP, NQ = (size_t)kNCN * NP;
     extern __shared__ __align__(16) unsigned char sh_raw[];
-    T(*sh)[kAdjShared][NP] = reinterpret_cast<T(*)[kAdjShared][NP]>(sh_raw);
     chain_start();   // lam is the previous launch's output
+    T(*sh)[kAdjShared][NP] = reinterpret_cast<T(*)[kAdjShared][NP]>(sh_raw);
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     int i0, i1, left;
@@ -565,8 +565,8 @@ lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_o
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned long long bars[W][2];
     __shared__ SplitRows rows[W];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
     chain_start();   // lam is the previous launch's output
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
     split_ring_init(bars[wib], lane);
     SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
@@ -1546,7 +1546,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
             else kp.k[q].M += off[q];
         }
         e = tk::launch_table_derivative(kp, S->variable, S->rs_min, S->Nr, S->Nth, S->NP, S->drs, dt_in, tx, tang,
-                                        S->dhalf, S->dnode, S->db_node, S->stream);
+                                        S->dhalf, S->dnode, S->db_node, S->num_sms, S->stream);
     }
     if (e != cudaSuccess) return bail(tkh::fail(S, TK_ERR_CUDA, "tk_param_gradient: %s", cudaGetErrorString(e)));
     // 2. checkpoints of the trajectory every C outer steps, from u^0

@@ -292,12 +292,12 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
     S->kerr.s = s;
     S->kerr.m = m;
     if (S->auto_k) S->substeps = 1;
-    TK_CUDA(S, tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->rad,
-                                          S->stream));
+    TK_CUDA(S, tk::launch_radial_parts(S->kerr, S->rs_min, S->drs, S->Nr, S->rad, S->Nth, S->NP,
+                                       S->variable != 0 ? S->ang : nullptr, S->num_sms, S->stream));
     TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                        S->dt / S->substeps, S->rad, S->ang,
                                        S->precision, S->half, S->node, S->b_node, S->w_row,
-                                       S->cmp, S->gpm, S->stream, nullptr, nullptr, false, S->step));
+                                       S->cmp, S->gpm, S->stream, nullptr, nullptr, S->step));
     S->have_coeffs = true;
     S->have_state = false;
     S->coeffs_id++;
@@ -318,7 +318,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
                                                S->dt / S->substeps, S->rad, S->ang,
                                                S->precision, S->half, S->node, S->b_node,
                                                S->w_row, S->cmp, S->gpm, S->stream, nullptr, nullptr,
-                                               false, S->step));
+                                               S->step));
         }
     }
     return TK_OK;
@@ -367,11 +367,12 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, S->stream);
     }
     if (e == cudaSuccess)
-        e = tk::launch_invert_tortoise(S->kerr, S->rs_min, S->drs, S->Nr, S->rad, S->stream);
+        e = tk::launch_radial_parts(S->kerr, S->rs_min, S->drs, S->Nr, S->rad, S->Nth, S->NP,
+                                    S->variable != 0 && !ang_given ? S->ang : nullptr, S->num_sms, S->stream);
     if (e == cudaSuccess)
         e = tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs, S->dt / S->substeps,
                                     S->rad, S->ang, S->precision, S->half, S->node, S->b_node,
-                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, ang_given, S->step);
+                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, S->step);
     if (e == cudaSuccess && dev) e = cudaStreamSynchronize(S->stream);
     if (dev) cudaFree(dev);
     if (e != cudaSuccess) return fail(S, TK_ERR_CUDA, "tk_set_coefficients: %s", cudaGetErrorString(e));

@@ -14,7 +14,6 @@
 
 #include "tk_internal.h"
 #include "tk_split_tables.cuh"
-#include "tk_stencil.cuh"
 
 namespace tk {
 namespace {
@@ -115,20 +114,6 @@ __device__ Radial radial_part(const Geo &P, double x)
     return R;
 }
 
-// The tortoise inversion and the radial parts: nodes i in rad[i], half nodes
-// i + 1/2 in rad[Nr + i].
-// Black hole blockIdx.y of the set goes to rad + blockIdx.y 2 Nr kRadial.
-__global__ void invert_tortoise_kernel(const __grid_constant__ KerrSet kp, double rs_min, double drs, int Nr, double *rad)
-{
-    asm volatile("griddepcontrol.launch_dependents;");   // the angular stencil may run beside it
-    const Geo P = geometry(kp.k[blockIdx.y]);
-    rad += (size_t)blockIdx.y * 2 * Nr * kRadial;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= 2 * Nr - 1) return;
-    const double rs = k < Nr ? rs_min + k * drs : rs_min + (k - Nr + 0.5) * drs;
-    *reinterpret_cast<Radial *>(rad + (size_t)k * kRadial) = radial_part(P, x_of_rstar(P, rs));
-}
-
 // Coefficients of   d_t Phi + b d_* Phi = Pi,
 //                   d_t Pi - b d_* Pi - c1 d_* Phi = c2 Pi + c3 Phi + c4 Phi_thth + c5 Phi_th
 // obtained from Eq. 1 x (-Delta/(Sigma^2 r^3)) with Psi = e^{i m phi} r^3 Phi and
@@ -211,18 +196,15 @@ __device__ double sl_weight(int s, int m, double th)
 // chain of two powers, a sine and a cosine: ~10 us, so all of them at once);
 // then the first warp adds them, lane l those of sub-panels l and l + 32, and
 // the 32 partial sums in a fixed tree order: 32 us, with a warp per row that
-// took two panels a lane in turn 88.  Each block ends only after the kernel it
-// is chained to (the next kernel reads what both wrote).
+// took two panels a lane in turn 88.
 constexpr int kStencilPanels = 64;
 
-__global__ void __launch_bounds__(4 * kStencilPanels)
-regular_stencil_kernel(int s, int m, int Nth, int NP, double *__restrict__ ang)
+__device__ void stencil_row(int j, int s, int m, int Nth, int NP, double *__restrict__ ang)
 {
     __shared__ double val[kStencilPanels][4], face[2];
-    const int j = blockIdx.x, tid = threadIdx.x;
+    const int tid = threadIdx.x;
     if (j >= Nth) {
         if (tid == 0) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
             ang[j] = 0.0;
             ang[NP + j] = 0.0;
         }
@@ -246,9 +228,37 @@ regular_stencil_kernel(int s, int m, int Nth, int NP, double *__restrict__ ang)
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (tid != 0) return;
     const double Q = 0.5 * h * acc / dth;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     ang[j] = face[1] / (Q * dth * dth);
     ang[NP + j] = face[0] / (Q * dth * dth);
+}
+
+// The tortoise inversion with the radial parts, and beside it the angular
+// stencil: both are serial chains that leave most of the chip idle and share
+// nothing, so one launch holds the blocks of both (blockIdx.x < ninv: the
+// inversion's).  61 us for both at 1601 x 32 and 79 at 4001 x 64; one after the
+// other 57 + 32 and 75 + 32.  The stencil is the same for every black hole of
+// the set.
+//
+// Radii: nodes i in rad[i], half nodes i + 1/2 in rad[Nr + i]; black hole
+// blockIdx.y of the set goes to rad + blockIdx.y 2 Nr kRadial.  The first `use`
+// threads of a block take a radius each: one warp a block while the warps do
+// not exceed the SMs, then more.
+constexpr int kPartsThreads = 4 * kStencilPanels;
+
+__global__ void __launch_bounds__(kPartsThreads)
+radial_stencil_kernel(const __grid_constant__ KerrSet kp, double rs_min, double drs, int Nr, double *rad, int ninv,
+                      int use, int Nth, int NP, double *__restrict__ ang)
+{
+    if ((int)blockIdx.x >= ninv) {
+        if (blockIdx.y == 0) stencil_row((int)blockIdx.x - ninv, kp.k[0].s, kp.k[0].m, Nth, NP, ang);
+        return;
+    }
+    const int k = blockIdx.x * use + threadIdx.x;
+    if ((int)threadIdx.x >= use || k >= 2 * Nr - 1) return;
+    const Geo P = geometry(kp.k[blockIdx.y]);
+    rad += (size_t)blockIdx.y * 2 * Nr * kRadial;
+    const double rs = k < Nr ? rs_min + k * drs : rs_min + (k - Nr + 0.5) * drs;
+    *reinterpret_cast<Radial *>(rad + (size_t)k * kRadial) = radial_part(P, x_of_rstar(P, rs));
 }
 
 // Raw coefficients supplied by the caller: [9][Nth][Nr] in the order of Raw
@@ -632,26 +642,24 @@ cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, c
     return cudaGetLastError();
 }
 
-// The angular stencil, chained to the tortoise inversion: it needs nothing of
-// it, and that started after every earlier use of ang, so the two run side by side.
-static cudaError_t launch_stencil(int s, int m, int Ntheta, int NP, double *ang, cudaStream_t st)
+// n black holes of the set; ang NULL: the stencil is not wanted.
+static cudaError_t launch_parts(const KerrSet &kp, int n, double rs_min, double drs, int Nr, double *rad, int Ntheta,
+                                int NP, double *ang, int num_sms, cudaStream_t st)
 {
-    return launch_chained(regular_stencil_kernel, (unsigned)NP, 4 * kStencilPanels, 0, st, s, m, Ntheta, NP, ang);
-}
-
-// one warp per block: few warps, each a serial chain, over all the SMs
-static cudaError_t launch_inversion(const KerrSet &kp, int n, double rs_min, double drs, int Nr, double *rad,
-                                    cudaStream_t st)
-{
-    invert_tortoise_kernel<<<dim3((2 * Nr + 30) / 32, n), 32, 0, st>>>(kp, rs_min, drs, Nr, rad);
+    const int warps = (2 * Nr + 30) / 32;
+    const int use = 32 * std::min(kPartsThreads / 32, std::max(1, warps / num_sms));
+    const int ninv = (2 * Nr - 1 + use - 1) / use;
+    radial_stencil_kernel<<<dim3(ninv + (ang ? NP : 0), n), kPartsThreads, 0, st>>>(kp, rs_min, drs, Nr, rad, ninv,
+                                                                                    use, Ntheta, NP, ang);
     return cudaGetLastError();
 }
 
-cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr, double *rad, cudaStream_t st)
+cudaError_t launch_radial_parts(const Kerr &P, double rs_min, double drs, int Nr, double *rad, int Ntheta, int NP,
+                                double *ang, int num_sms, cudaStream_t st)
 {
     KerrSet kp = {};
     kp.k[0] = P;
-    return launch_inversion(kp, 1, rs_min, drs, Nr, rad, st);
+    return launch_parts(kp, 1, rs_min, drs, Nr, rad, Ntheta, NP, ang, num_sms, st);
 }
 
 static dim3 table_grid(int Nr, const dim3 &block)
@@ -661,10 +669,10 @@ static dim3 table_grid(int Nr, const dim3 &block)
 
 cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_min, int Nr, int Ntheta, int NP,
                                     double drs, double dt_inner, double *rad, double *ang, double *half,
-                                    double *node, double *b_node, cudaStream_t st)
+                                    double *node, double *b_node, int num_sms, cudaStream_t st)
 {
-    cudaError_t e = launch_inversion(kp, kShifts, rs_min, drs, Nr, rad, st);
-    if (e == cudaSuccess && variable != 0) e = launch_stencil(kp.k[0].s, kp.k[0].m, Ntheta, NP, ang, st);
+    cudaError_t e = launch_parts(kp, kShifts, rs_min, drs, Nr, rad, Ntheta, NP, variable != 0 ? ang : nullptr, num_sms,
+                                 st);
     if (e != cudaSuccess) return e;
     const dim3 block(NP, kTableThreads / NP);
     table_derivative_kernel<<<table_grid(Nr, block), block, 0, st>>>(kp, variable, Nr, Ntheta, NP, divisor(drs),
@@ -674,16 +682,12 @@ cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_m
 }
 
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                                double drs, double dt_inner, const double *rad, double *ang, int precision, void *half,
+                                double drs, double dt_inner, const double *rad, const double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node, const double *raw_half,
-                                bool ang_given, unsigned char *step)
+                                unsigned char *step)
 {
     const F32Derive fd = f32_derive(dt_inner);
-    if (variable != 0 && !ang_given) {
-        cudaError_t e = launch_stencil(P.s, P.m, Ntheta, NP, ang, st);
-        if (e != cudaSuccess) return e;
-    }
     dim3 block(NP, kTableThreads / NP);
     const dim3 grid = table_grid(Nr, block);
     const Divisor ds = divisor(drs), de = divisor(0.25 * dt_inner);   // dr*, the half node's e

@@ -156,26 +156,26 @@ struct WaveRead {
 // rad: the radial parts of the coefficients, kRadial doubles per radius, nodes
 // r*_i in rad[i], half nodes r*_{i+1/2} (i < Nr - 1) in rad[Nr + i].
 constexpr int kRadial = 12;
-cudaError_t launch_invert_tortoise(const Kerr &P, double rs_min, double drs, int Nr, double *rad, cudaStream_t st);
+// ang: the regularised angular stencil [2][NP], NULL where it is not wanted.
+cudaError_t launch_radial_parts(const Kerr &P, double rs_min, double drs, int Nr, double *rad, int Ntheta, int NP,
+                                double *ang, int num_sms, cudaStream_t st);
 // FP32 (precision 1) also writes the compact tables cmp and the theta
 // factors gpm[2][NP] (gp, then gm); both may be NULL for FP64.  raw_node,
 // raw_half (device, [9][Ntheta][Nr], half node i at r*_{i+1/2}): coefficients
-// supplied by the caller instead of computed (rad then unused);
-// ang_given: ang already holds the regularised stencil.  step: the FP64
-// step's tables (NULL: not wanted).
+// supplied by the caller instead of computed (rad then unused); ang: the
+// regularised stencil.  step: the FP64 step's tables (NULL: not wanted).
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
-                                double drs, double dt_inner, const double *rad, double *ang, int precision, void *half,
+                                double drs, double dt_inner, const double *rad, const double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
                                 cudaStream_t st, const double *raw_node = nullptr,
-                                const double *raw_half = nullptr, bool ang_given = false,
-                                unsigned char *step = nullptr);
+                                const double *raw_half = nullptr, unsigned char *step = nullptr);
 
 // The derivative of the FP64 tables in a parameter of the black hole, sum_q w[q]
 // tables(k[q]); rad: kShifts times the radial parts, ang: the angular stencil,
 // both scratch.
 cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_min, int Nr, int Ntheta, int NP,
                                     double drs, double dt_inner, double *rad, double *ang, double *half,
-                                    double *node, double *b_node, cudaStream_t st);
+                                    double *node, double *b_node, int num_sms, cudaStream_t st);
 
 // The raw coefficients of the precompute, [9][Ntheta][Nr] at nodes and half
 // nodes (device output buffers).
