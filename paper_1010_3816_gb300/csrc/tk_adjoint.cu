@@ -1037,13 +1037,13 @@ cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const 
     cudaError_t e = adj_smem_setup<T, K, W>();
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(T) == 8)
-        return launch_chained(lw_adjoint_team_kernel<K, W>, (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st,
-                              (const double *)lam, (double *)mu, (const double *)half, (const double *)node, tab, Nr,
-                              0.5 * dt_in, inj);
+        return launch_chained<lw_adjoint_team_kernel<K, W>>(
+            (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const double *)lam, (double *)mu,
+            (const double *)half, (const double *)node, tab, Nr, 0.5 * dt_in, inj);
     else
-        return launch_chained(lw_adjoint_kernel<T, K, W>, (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(),
-                              st, (const T *)lam, (T *)mu, (const T *)half, (const T *)node, Nr,
-                              (T)(0.25 * dt_in), (T)(0.5 * dt_in), inj);
+        return launch_chained<lw_adjoint_kernel<T, K, W>>(
+            (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const T *)lam, (T *)mu, (const T *)half,
+            (const T *)node, Nr, (T)(0.25 * dt_in), (T)(0.5 * dt_in), inj);
 }
 
 template <typename T, int K>

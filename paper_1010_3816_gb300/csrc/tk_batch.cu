@@ -224,11 +224,17 @@ static cudaError_t launch_batch_tick(int precision, int kall, int blocks, const 
                                      const BatchItem *items, int nitems, int tick, int kmax,
                                      int outer, unsigned int *ctr, cudaStream_t st)
 {
-    if (precision == 0)
-        return launch_chained(batch_kernel_f64(kall), (unsigned)blocks, kBatchThreads, kBatchSmem, st, mem,
-                              nmem, items, nitems, tick, kmax, outer, ctr);
-    return launch_chained(batch_step_kernel<float, 0>, (unsigned)blocks, kBatchThreads, 0, st, mem, nmem,
-                          items, nitems, tick, kmax, outer, ctr);
+    auto go = [&](auto launch, size_t smem) {
+        return launch((unsigned)blocks, (unsigned)kBatchThreads, smem, st, mem, nmem, items, nitems, tick, kmax, outer,
+                      ctr);
+    };
+#define TK_CHAINED(kern) [](auto... a) { return launch_chained<kern>(a...); }
+    if (precision != 0) return go(TK_CHAINED((batch_step_kernel<float, 0>)), 0);
+    return kall == 1 ? go(TK_CHAINED((batch_step_kernel<double, 1>)), kBatchSmem)
+         : kall == 2 ? go(TK_CHAINED((batch_step_kernel<double, 2>)), kBatchSmem)
+         : kall == 4 ? go(TK_CHAINED((batch_step_kernel<double, 4>)), kBatchSmem)
+                     : go(TK_CHAINED((batch_step_kernel<double, 0>)), kBatchSmem);
+#undef TK_CHAINED
 }
 
 }  // namespace tk

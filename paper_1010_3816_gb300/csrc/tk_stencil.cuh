@@ -46,10 +46,20 @@ __device__ __forceinline__ void chain_start()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                           cudaStream_t st, Args... args)
+// Whether the kernel keeps nothing in local memory.  Only such kernels are
+// launched with the programmatic edge: the compiler may touch a stack frame
+// ahead of the wait, and a kernel with one that worked there has faulted
+// (misaligned address) without an explanation.
+inline bool frameless(const void *kern)
 {
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, kern) == cudaSuccess && a.localSizeBytes == 0;
+}
+
+template <auto kern, typename... Args>
+cudaError_t launch_chained(unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args)
+{
+    static const bool chained = frameless((const void *)kern);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -59,7 +69,7 @@ cudaError_t launch_chained(void (*kern)(KArgs...), unsigned grid, unsigned block
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

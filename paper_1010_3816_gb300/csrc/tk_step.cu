@@ -1086,9 +1086,9 @@ cudaError_t launch_shape(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
             (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
         return cudaGetLastError();
     }
-    return launch_chained(lw_step_kernel<T, K, W>, (unsigned)L.blocks, W * 32, step_smem_bytes<T, K, W>(),
-                          st, (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node,
-                          L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
+    return launch_chained<lw_step_kernel<T, K, W>>(
+        (unsigned)L.blocks, W * 32, step_smem_bytes<T, K, W>(), st, (const T *)L.u_in, (T *)L.u_out, (const T *)L.half,
+        (const T *)L.node, L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
 }
 
 template <typename T, int K, int W>

@@ -28,7 +28,7 @@ def test_chained_kernels_wait_first():
     for _, text in _sources():
         for m in re.finditer(r"__global__[^{;]*?\b(\w+_kernel)\s*\([^{;]*\)\s*\{", text):
             kernels[m.group(1)] = text[m.end():]
-        for m in re.finditer(r"launch_chained\(\s*(\w+)", text):
+        for m in re.finditer(r"\b(?:launch_chained<|TK_CHAINED\(\()(\w+)", text):
             calls.add(m.group(1))
     chained = {c for c in calls if c.endswith("_kernel")}
     assert len(chained) >= 4
@@ -38,3 +38,17 @@ def test_chained_kernels_wait_first():
             if re.match(r"(if \(kUsePDL\) )?chain_start\(\)$", line):
                 break
             assert re.match(r"(constexpr|(extern )?__shared__)\b", line), (name, line)
+
+
+def test_programmatic_edge_only_for_kernels_without_a_stack_frame():
+    """The launch attribute stands in launch_chained alone, and goes with the launch
+    only where the kernel has no local memory."""
+    where = [(name, text) for name, text in _sources() if "ProgrammaticStreamSerialization" in text]
+    assert [name for name, _ in where] == ["tk_stencil.cuh"]
+    text = where[0][1]
+    assert text.count("cudaLaunchAttributeProgrammaticStreamSerialization") == 1
+    body = text[text.index("cudaError_t launch_chained("):]
+    body = body[:body.index("cudaLaunchKernelEx")]
+    assert re.search(r"bool chained = frameless\(\(const void \*\)kern\);", body)
+    assert re.search(r"numAttrs = chained \? 1 : 0;", body)
+    assert re.search(r"frameless\(const void \*kern\)\s*\{[^}]*localSizeBytes == 0", text)
