@@ -740,21 +740,21 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
             inject_row(col, Nr, row, inj, on, sample, a);
         }
         if (before && (owner || halves)) {
-            const int2 head = *reinterpret_cast<const int2 *>(left + kAdjExps + 256);
-            hot_a = adj_pair<K, false>(a, AdjTab<false>{left, lane}, head.y != 0, team, sa, sl);
+            const AdjTab<false> t{left, lane};
+            hot_a = adj_pair<K, false>(a, t, t.head(), team, sa, sl);
         }
         put(sh.lam[j], a);
         put_sums(0, sl, hot_a);
         double c[4];
         AdjSums sr;
         bool hot_c = false;
-        const int2 head = halves ? *reinterpret_cast<const int2 *>(own + kAdjExps + 256) : make_int2(0, 0);
+        const int2 head = halves ? AdjTab<false>{own, lane}.head() : make_int2(0, 0);
         const bool imag = head.y != 0;
         if (j == T && halves) {
             if (s > 0) warp_wait_flag(flags + (b + 1) * K + h, e, err);
             load_lam_row<K>(in, col + 1, Nr, row, inj, on, sample, c);
             AdjSums unused;
-            hot_c = adj_pair<K, false>(c, AdjTab<false>{own, lane}, imag, team, unused, sr);
+            hot_c = adj_pair<K, false>(c, AdjTab<false>{own, lane}, head, team, unused, sr);
         }
         __syncthreads();
         // eta
@@ -766,11 +766,11 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
                 get(sh.lam[j + 1], c);
                 hot_c = get_sums(0, j + 1, sr);
             }
-            if (hot_a || hot_c || head.x)
+            if (hot_a || hot_c)
                 eta_row_cold<K>(a, c, node + (size_t)col * (kNCN * NP) + row, en, team, ep);
             else
                 eta_row(a, c, sa, sr, imag, own, lane, en, k1, ep);
-            hot_p = adj_pair<K, true>(ep, AdjTab<true>{own, lane}, imag, team, s1, s2);
+            hot_p = adj_pair<K, true>(ep, AdjTab<true>{own, lane}, head, team, s1, s2);
             put(sh.eta[j], ep);
             put_sums(1, s2, hot_p);
         }
@@ -782,7 +782,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
                 AdjSums sm;
                 get(sh.eta[j - 1], em);
                 const bool hot_m = get_sums(1, j - 1, sm);
-                if (hot_p || hot_m || head.x)
+                if (hot_p || hot_m)
                     mu_row_cold<K>(a, ep, em, half + (size_t)col * (kNCH * NP) + row, team, o);
                 else
                     mu_row(a, ep, em, s1, sm, imag, own, lane, k1, o);

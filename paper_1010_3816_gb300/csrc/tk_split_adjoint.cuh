@@ -31,7 +31,9 @@ namespace {
 // row before, KM of the row after, the same of half node i + 1/2 (FAR, FCR,
 // FAI, FCI, KP, KM); [2][32] ints with the exponents of (F1, F2, KP, KM) and
 // (G1, G2); two ints, cold and has imaginary coefficients, over the column and
-// every table involved; padding.
+// every table involved; padding.  A cold block's integers are zero, also where
+// the sums formed with them go to a column that is not cold: such sums are marked
+// as those of values that call for the FP64 instructions (adj_pair).
 enum { A_BA = 0, A_PP, A_CA, A_BC, A_PM, A_CC, A_HP, A_PA, A_PI, A_HQ, A_PC, A_PJ };
 enum { A_F1 = 0, A_F2, A_G1, A_G2, A_KP, A_KM };
 constexpr int kAdjF64 = 12;
@@ -50,6 +52,7 @@ struct AdjTab {
     {
         return *reinterpret_cast<const int *>(p + kAdjExps + (HALF ? 128 : 0) + lane * 4);
     }
+    __device__ __forceinline__ int2 head() const { return *reinterpret_cast<const int2 *>(p + kAdjExps + 256); }
 };
 
 __device__ __forceinline__ double adj_f64(const unsigned char *p, int q, int lane)
@@ -155,19 +158,22 @@ __device__ __forceinline__ void adj_zero(AdjSums &a)
     a.O[0] = a.O[1] = kSplitAbsent;
 }
 
-// Both sums of the Pi values v[2], v[3]; whether the FP64 instructions are
-// called for anywhere in the team (a barrier of the team).
+// Both sums of the Pi values v[2], v[3] with the block of tab, whose head is
+// given; whether the FP64 instructions are called for anywhere in the team, by
+// the values or by the tables (a barrier of the team): the sums are then not
+// valid, for any column that they go to.
 template <int K, bool HALF>
-__device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF> &tab, bool imag,
+__device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF> &tab, int2 head,
                                          SplitTeam<K> &team, AdjSums &s1, AdjSums &s2)
 {
+    const bool imag = head.y != 0;
     SplitInts p;
     split_ints<2>(v, p);
     int4 su, sd;
     int2 eu2, ed2;
     const bool hot = team.exchange(
         make_int4((int)(p.x[0] >> 32), (int)p.x[0], (int)(p.x[1] >> 32), (int)p.x[1]), make_int2(p.e[0], p.e[1]),
-        max(p.e[0], p.e[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
+        head.x != 0 || max(p.e[0], p.e[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
     const int rx = tab.row_exp();
     AdjSums g1, g2;
 #pragma unroll
@@ -405,8 +411,9 @@ struct AdjSweep {
         adj_zero(sm);
         if (ib > 0) {
             const unsigned char *block = tab + (size_t)(ib - 1) * (K * kAdjBytes);
+            const AdjTab<false> t{block, lane};
             AdjSums s2;
-            hot_a = adj_pair<K, false>(a, AdjTab<false>{block, lane}, true, team, sa, s2);
+            hot_a = adj_pair<K, false>(a, t, t.head(), team, sa, s2);
         }
 #pragma unroll 1
         for (int i = ib; i < i1; ++i) {
@@ -425,11 +432,11 @@ struct AdjSweep {
                 await(st, st.cur);
                 const unsigned char *p = ring->tab[st.cur];
                 st.cur ^= 1;
-                const int2 head = *reinterpret_cast<const int2 *>(p + kAdjExps + 256);
+                const int2 head = AdjTab<false>{p, lane}.head();
                 const bool imag = head.y != 0;
                 // eta at half node i + 1/2
-                const bool hot_c = adj_pair<K, false>(c, AdjTab<false>{p, lane}, imag, team, sc, sr);
-                if (hot_a || hot_c || head.x) {
+                const bool hot_c = adj_pair<K, false>(c, AdjTab<false>{p, lane}, head, team, sc, sr);
+                if (hot_a || hot_c) {
                     double za[2], zc[2];
                     const double *ta = node64 + (size_t)i * (kNCN * NP) + row, *tc = ta + kNCN * NP;
                     cold_sources<K>(a, ta + N_KP * NP, ta + N_KM * NP, team, za);
@@ -454,12 +461,12 @@ struct AdjSweep {
                     ep[3] = fma(PM, c[3], y);
                 }
                 // mu at node i
-                const bool hot_p = adj_pair<K, true>(ep, AdjTab<true>{p, lane}, imag, team, s1, s2);
+                const bool hot_p = adj_pair<K, true>(ep, AdjTab<true>{p, lane}, head, team, s1, s2);
                 if (i >= i0) {
                     if (i == 0) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) o[k] = 0.0;
-                    } else if (hot_p || hot_m || head.x) {
+                    } else if (hot_p || hot_m) {
                         double yp[2], ym[2];
                         const double *tp = half64 + (size_t)i * (kNCH * NP) + row, *tm = tp - kNCH * NP;
                         cold_sources<K>(ep, tp + H_KP * NP, tp + H_KM * NP, team, yp);
