@@ -231,7 +231,7 @@ tk_status tk_extract_noalloc(tk_solver *S, int obs_id, int first, int count, dou
  *              independent_pi = 1, planes4 including dL/d(pi planes)
  *   grad_on_device location of grad
  * The solver's state is not touched.  Allocates two adjoint state levels on
- * first use and, in FP64, the transposed tables (6416 bytes per column and 32
+ * first use and, in FP64, the transposed tables (6544 bytes per column and 32
  * rows), all kept until tk_destroy, and temporary buffers for host inputs.
  * Synchronizes the stream when an input or the output is in host memory. */
 tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfinal, int on_device,

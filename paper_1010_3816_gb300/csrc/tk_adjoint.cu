@@ -564,11 +564,11 @@ lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_o
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned long long bars[W][2];
-    __shared__ SplitRows rows[W];
+    __shared__ AdjRows rows[W];
     chain_start();   // lam is the previous launch's output
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
     split_ring_init(bars[wib], lane);
-    SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
+    AdjTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
                          en, nullptr};
     int i0, i1;
@@ -596,14 +596,14 @@ lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restri
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned int step_done[W];
     __shared__ unsigned long long bars[W][2];
-    __shared__ SplitRows rows[W];
+    __shared__ AdjRows rows[W];
     constexpr int TEAMS = W / K;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K, h = wib % K, row = 32 * h + lane;
     if (threadIdx.x < W) step_done[threadIdx.x] = 0;
     split_ring_init(bars[wib], lane);
     __syncthreads();
     const int nb = (int)gridDim.x, b = (int)blockIdx.x;
-    SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
+    AdjTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
                          en, err};
     int i0, i1;
@@ -658,7 +658,7 @@ struct AdjColumnShared {
     long long sum[2][T + 1][2][NP];                       // of lam~ to the left, of eta to the right
     int exp[2][T + 1][2][NP];
     int hot[2][T + 1];
-    SplitRows rows[(T + 1) * K];
+    AdjRows rows[(T + 1) * K];
     unsigned long long bars[(T + 1) * K];
 };
 
@@ -678,7 +678,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
     const bool halves = col >= 0 && col + 1 < Nr;      // there is a half node right of it
     const bool before = col > 0 && col < Nr;           // and one left of it
     const FmaK<double> k1 = fma_k<double>();
-    SplitTeam<K> team{sh.rows + j * K, h, lane, 1 + j};
+    AdjTeam<K> team{sh.rows + j * K, h, lane, 1 + j};
     const unsigned char *left = sh.tab[j][h], *own = sh.tab[j + 1][h];   // of columns col - 1 and col
     auto put = [&](double (*p)[NP], const double (&x)[4]) {
 #pragma unroll

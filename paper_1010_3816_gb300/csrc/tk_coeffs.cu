@@ -432,35 +432,38 @@ coeff_tables_kernel(Kerr KP, int variable, int Nr, int Nth, int NP, Divisor ds, 
             const double hs[kSplitEntries] = {hv[H_FAR], hv[H_FCR], hv[H_KP], hv[H_KM], hv[H_FAI], hv[H_FCI]};
             const double nd[kStepNodeF64] = {nv[N_B], nv[N_PPR], nv[N_PMR], nv[N_C2I]};
             const double ns[kSplitEntries] = {nv[N_FMR], nv[N_FPR], nv[N_KP], nv[N_KM], nv[N_FMI], nv[N_FPI]};
-            int ex[2][2];
             int cold = 0;
-            for (int w = 0; w < 2; ++w) {
-                const double *v = w ? ns : hs;
-                ex[w][0] = class_exponent((fabs(v[S_FA]) + fabs(v[S_FC])) + 2.0 * (fabs(v[S_KP]) + fabs(v[S_KM])),
-                                          &cold);
-                ex[w][1] = class_exponent(fabs(v[S_GA]) + fabs(v[S_GC]), &cold);
-            }
+            auto terms = [](const double *v) {
+                return RowTerms{fabs(v[S_FA]) + fabs(v[S_FC]), 2.0 * fabs(v[S_KP]), 2.0 * fabs(v[S_KM])};
+            };
+            auto other = [](const double *v) { return fabs(v[S_GA]) + fabs(v[S_GC]); };
+            const RowTerms ht = terms(hs), nt = terms(ns);
+            const double hg = other(hs), ng = other(ns);
+            const RowLifts lift(ht, nt, &cold);
+            const RowExps hx(ht, lift, hg, &cold), nx(nt, lift, ng, &cold);
             // plain stores of the same value
             if (cold) flags[threadIdx.y][0] = 1;
-            if (ex[0][1] != kSplitAbsent || ex[1][1] != kSplitAbsent || hv[H_PI] != 0.0 || nv[N_C2I] != 0.0)
-                flags[threadIdx.y][1] = 1;
+            if (hg != 0.0 || ng != 0.0 || hv[H_PI] != 0.0 || nv[N_C2I] != 0.0) flags[threadIdx.y][1] = 1;
             __syncthreads();
             if (i < Nr) {
                 const int lane = jp & 31;
                 unsigned char *block = step + ((size_t)i * (NP / 32) + jp / 32) * kStepBytes;
                 double *d = reinterpret_cast<double *>(block) + lane;
-                auto entries = [&](const double *v, const int (&e)[2]) {
-                    for (int q = 0; q < kSplitEntries; ++q, d += 32)
-                        *reinterpret_cast<int2 *>(d) = flags[threadIdx.y][0] ? make_int2(0, 0)
-                                                                             : split_entry(v[q], e[q >= S_GA]);
+                auto entries = [&](const double *v, const RowExps &e) {
+                    for (int q = 0; q < kSplitEntries; ++q, d += 32) {
+                        const int C = q >= S_GA ? e.g : q == S_KP ? e.f - lift.u : q == S_KM ? e.f - lift.d : e.f;
+                        *reinterpret_cast<int2 *>(d) = flags[threadIdx.y][0] ? make_int2(0, 0) : split_entry(v[q], C);
+                    }
                 };
                 for (int q = 0; q < kStepHalfF64; ++q, d += 32) *d = hd[q];
-                entries(hs, ex[0]);
+                entries(hs, hx);
                 for (int q = 0; q < kStepNodeF64; ++q, d += 32) *d = nd[q];
-                entries(ns, ex[1]);
+                entries(ns, nx);
                 int *x = reinterpret_cast<int *>(block + kStepExps);
-                for (int w = 0; w < 2; ++w) x[32 * w + lane] = (ex[w][0] & 0xffff) | (ex[w][1] << 16);
-                if (lane < 4) x[64 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
+                x[lane] = hx.packed();
+                x[32 + lane] = nx.packed();
+                x[64 + lane] = lift.packed();
+                if (lane < 4) x[96 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
             }
         }
         if (i >= Nr) continue;

@@ -81,17 +81,21 @@ inline F32Derive f32_derive(double dt_inner)
 // One contiguous block of kStepBytes per column and 32 rows, step[i][row /
 // 32]: the half node's FP64 entries and limb pairs, then the node's, each
 // [entry][32] (8 bytes); [2][32] ints with the row's exponents of the two
-// integer classes of the half node and of the node (the low half bounds |FA| +
-// |FC| + 2 |KP| + 2 |KM|, the high half |GA| + |GC|); then two ints, cold and
-// has imaginary coefficients (over the whole column), and eight bytes of padding.
+// integer classes of the half node and of the node (the low half F's, the high
+// half G's); [32] ints with the row's lifts of KP (low half) and KM (high half),
+// the same for both (RowLifts, tk_split_tables.cuh); then two ints, cold and has
+// imaginary coefficients (over the whole column), and eight bytes of padding.
 enum { D_HP = 0, D_HQ, D_PAR, D_PCR, D_PI };
 enum { D_B = 0, D_PPR, D_PMR, D_C2I };
 constexpr int kStepHalfF64 = 5, kStepNodeF64 = 4;
 constexpr int kSplitEntries = 6;
 enum { S_FA = 0, S_FC, S_KP, S_KM, S_GA, S_GC };
 constexpr int kStepExps = (kStepHalfF64 + kStepNodeF64 + 2 * kSplitEntries) * 256;   // offset of the exponents
-constexpr int kStepBytes = kStepExps + 256 + 16;
-constexpr int kSplitAbsent = -20000;    // exponent of a class whose entries are all zero
+constexpr int kStepHead = kStepExps + 256 + 128;   // offset of the column's two flags
+constexpr int kStepBytes = kStepHead + 16;
+constexpr int kSplitAbsent = -14000;    // exponent of a class whose entries are all zero
+constexpr int kLiftAbsent = 14000;      // lift of a neighbour's coefficient that is zero
+constexpr int kLiftSpread = 6;          // largest difference of the lifts that two tables share
 constexpr int kSplitMaxClass = 20;      // largest class exponent; larger tables are cold
 constexpr int kSplitMaxExp = 1900;      // columns with this exponent field or more are cold
 

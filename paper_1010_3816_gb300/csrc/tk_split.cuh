@@ -24,21 +24,22 @@
 //
 // Numbers.  A value is an integer X, 2^59 <= |X| < 2^60, with its own exponent
 // e: X 2^(e - 1082), exact.  A table entry is an integer Q with an exponent C
-// shared by a class of entries of its row, Q 2^(C - 62), where the class's
-// absolute sum is at most 2^62.  Multiplicands are taken as two 32-bit limbs,
+// shared by a class of entries of its row, Q 2^(C - 62), but for the theta
+// neighbours' coefficients, which have their own (lower by their lift,
+// tk_split_tables.cuh).  Multiplicands are taken as two 32-bit limbs,
 // h 2^32 + l with l in [-2^31, 2^31); a sum keeps two 64-bit accumulators, of
-// weight 2^64 (h h) and 2^32 (h l + l h), which cannot overflow whatever the
-// data; the l l products, zero in the mean and below 2^-60 of the class's
-// bound, are left out.
+// weight 2^64 (h h) and 2^32 (h l + l h).  These cannot overflow whatever the
+// data: the integers of class F (F and the lifted K) add up to 2^62, those of G to
+// 2^61, so that the first stays below 2^59 and the second below 3.5 2^61.
 //
-// Alignment.  The values of one component that meet in a sum are shifted right
-// to the largest of their exponents, per row: what is lost lies 2^-60 below
-// the largest value of the sum, where an FP64 sum with it ends at 2^-53.  Each
-// class's sum T = sum / 2^64 stands for T 2^(C + e - 1080); the two classes'
-// sums are aligned to the larger exponent, the total is converted to FP64 once
-// (split_value).
-// The errors are below those of the FMA chain it replaces, which rounds at
-// every product.  Every operation treats both signs alike, so that conjugate
+// Alignment.  Each product has the exponent of its value plus that of its entry;
+// the values are shifted right to the largest of these, per row and component:
+// what is lost lies 2^-60 below a product of the sum's largest exponent.  The
+// sum, T = sum / 2^64, stands for T 2^(E - 1080) and is converted to FP64 once
+// (split_value).  The l l products, zero in the mean, are left out.  T's last
+// place is at most 2^-53 of the sum's largest product, typically 2^-55: an FMA
+// chain rounds to 2^-53 of its partial sum at every product.
+// Every operation treats both signs alike, so that conjugate
 // data and a -> -a still give conjugate results to the bit.
 //
 // A team of K warps (NP = 32 K rows, one per lane) walks the columns together;
@@ -166,13 +167,15 @@ __device__ __forceinline__ double split_value(long long T, int o)
 // twelve shuffles took longer.
 struct SplitRows {
     int4 s[2][32];
-    int2 e[2][32];
+    int2 x[2][32];
+    __device__ __forceinline__ void put_exps(int b, int l, int2 e) { x[b][l] = e; }
+    __device__ __forceinline__ int2 exps(int b, int l) const { return x[b][l]; }
 };
 
 // A warp's place in its team.
-template <int K>
+template <int K, class Rows = SplitRows>
 struct SplitTeam {
-    SplitRows *rows;   // the team's K
+    Rows *rows;        // the team's K
     int h;             // this warp's rows are 32 h ..
     int lane;
     int bar;           // the team's named barrier
@@ -201,14 +204,14 @@ struct SplitTeam {
     __device__ __forceinline__ bool exchange(int4 s, int2 e, bool p, int4 &su, int2 &eu, int4 &sd, int2 &ed)
     {
         rows[h].s[buf][lane] = s;
-        rows[h].e[buf][lane] = e;
+        rows[h].put_exps(buf, lane, e);
         const bool r = any(p);
         const int row = 32 * h + lane;
         const int u = min(row + 1, 32 * K - 1), d = max(row - 1, 0);
         su = rows[u >> 5].s[buf][u & 31];
-        eu = rows[u >> 5].e[buf][u & 31];
+        eu = rows[u >> 5].exps(buf, u & 31);
         sd = rows[d >> 5].s[buf][d & 31];
-        ed = rows[d >> 5].e[buf][d & 31];
+        ed = rows[d >> 5].exps(buf, d & 31);
         buf ^= 1;
         return r;
     }
@@ -246,7 +249,11 @@ struct StepTab {
     {
         return *reinterpret_cast<const int *>(p + kStepExps + (NODE ? 128 : 0) + lane * 4);
     }
-    __device__ __forceinline__ int2 head() const { return *reinterpret_cast<const int2 *>(p + kStepExps + 256); }
+    __device__ __forceinline__ int lifts() const
+    {
+        return *reinterpret_cast<const int *>(p + kStepExps + 256 + lane * 4);
+    }
+    __device__ __forceinline__ int2 head() const { return *reinterpret_cast<const int2 *>(p + kStepHead); }
 };
 
 // The coupling of Phi (values a left and c right of the point) to Pi_R and
@@ -271,38 +278,37 @@ __device__ __forceinline__ bool split_coupling(const SplitInts &a, const SplitIn
         team.exchange(make_int4(sh[0], sl[0], sh[1], sl[1]), make_int2(e1[0], e1[1]),
                       cold || max(e1[0], e1[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
     if (over) return false;
-    const int rx = tab.row_exp();
-    long long G[2];   // the other part's share
-    int OG[2];
+    // exponents of the products over the F class's: the largest of each sum
+    const int rx = tab.row_exp(), cf = (short)(rx & 0xffff), cg = (rx >> 16) - cf;
+    const int lx = tab.lifts(), lu = (short)(lx & 0xffff), ld = lx >> 16;
+    int f[2];
+    f[0] = max(max(eu2.x - lu, ed2.x - ld), e1[0]);
+    f[1] = max(max(eu2.y - lu, ed2.y - ld), e1[1]);
+    if (imag) {
+        f[0] = max(f[0], e1[1] + cg);
+        f[1] = max(f[1], e1[0] + cg);
+    }
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
         const int uh = g ? su.z : su.x, ul = g ? su.w : su.y, eu = g ? eu2.y : eu2.x;
         const int dh = g ? sd.z : sd.x, dl = g ? sd.w : sd.y, ed = g ? ed2.y : ed2.x;
-        const int ef = max(max(eu, ed), e1[g]);
-        const int2 la = limbs(cut(a.x[g], ef - a.e[g], a.j[g]));
-        const int2 lc = limbs(cut(c.x[g], ef - c.e[g], c.j[g]));
         SplitSum s;
-        s.add(la, tab.entry(S_FA));
-        s.add(lc, tab.entry(S_FC));
-        s.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, ef - eu, nonzero(uh, ul))), tab.entry(S_KP));
-        s.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, ef - ed, nonzero(dh, dl))), tab.entry(S_KM));
+        s.add(limbs(cut(a.x[g], f[g] - a.e[g], a.j[g])), tab.entry(S_FA));
+        s.add(limbs(cut(c.x[g], f[g] - c.e[g], c.j[g])), tab.entry(S_FC));
+        s.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, f[g] + lu - eu, nonzero(uh, ul))), tab.entry(S_KP));
+        s.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, f[g] + ld - ed, nonzero(dh, dl))), tab.entry(S_KM));
+        if (imag) {   // the other part's, subtracted from the real part
+            const int o = 1 - g, n = f[g] - cg;
+            int2 la = limbs(cut(a.x[o], n - a.e[o], a.j[o])), lc = limbs(cut(c.x[o], n - c.e[o], c.j[o]));
+            if (g == 0) {
+                la = make_int2(-la.x, -la.y);
+                lc = make_int2(-lc.x, -lc.y);
+            }
+            s.add(la, tab.entry(S_GA));
+            s.add(lc, tab.entry(S_GC));
+        }
         T[g] = s.take();
-        O[g] = (short)(rx & 0xffff) + ef;
-        if (imag) {
-            SplitSum q;
-            q.add(la, tab.entry(S_GA));
-            q.add(lc, tab.entry(S_GC));
-            G[1 - g] = g == 0 ? q.take() : -q.take();
-            OG[1 - g] = (rx >> 16) + ef;
-        }
-    }
-    if (imag) {
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            const int o = max(O[g], OG[g]);
-            T[g] = shr_zero(T[g], o - O[g]) + shr_zero(G[g], o - OG[g]);
-            O[g] = o;
-        }
+        O[g] = cf + f[g];
     }
     return true;
 }

@@ -30,15 +30,32 @@ namespace {
 // HQ, PCR, PI; limb pairs [12][32]: of node i + 1 FPR, FMR, FPI, FMI, KP of the
 // row before, KM of the row after, the same of half node i + 1/2 (FAR, FCR,
 // FAI, FCI, KP, KM); [2][32] ints with the exponents of (F1, F2, KP, KM) and
-// (G1, G2); two ints, cold and has imaginary coefficients, over the column and
-// every table involved; padding.  A cold block's integers are zero, also where
+// (G1, G2); [32] ints with the lifts of KM (low half, it multiplies the row
+// above) and KP (high half), the same for both; two ints, cold and has imaginary
+// coefficients, over the column and every table involved; padding.  A cold block's integers are zero, also where
 // the sums formed with them go to a column that is not cold: such sums are marked
 // as those of values that call for the FP64 instructions (adj_pair).
 enum { A_BA = 0, A_PP, A_CA, A_BC, A_PM, A_CC, A_HP, A_PA, A_PI, A_HQ, A_PC, A_PJ };
 enum { A_F1 = 0, A_F2, A_G1, A_G2, A_KP, A_KM };
 constexpr int kAdjF64 = 12;
 constexpr int kAdjExps = (kAdjF64 + 12) * 256;
-constexpr int kAdjBytes = kAdjExps + 256 + 16;
+constexpr int kAdjHead = kAdjExps + 256 + 128;   // offset of the column's two flags
+constexpr int kAdjBytes = kAdjHead + 16;
+
+// The rows' records with the two exponents in one word: sixteen warps' rings
+// leave no room for more.
+struct AdjRows {
+    int4 s[2][32];
+    unsigned x[2][32];
+    __device__ __forceinline__ void put_exps(int b, int l, int2 e) { x[b][l] = (unsigned)e.x | ((unsigned)e.y << 16); }
+    __device__ __forceinline__ int2 exps(int b, int l) const
+    {
+        return make_int2((int)(x[b][l] & 0xffff), (int)(x[b][l] >> 16));
+    }
+};
+
+template <int K>
+using AdjTeam = SplitTeam<K, AdjRows>;
 
 template <bool HALF>
 struct AdjTab {
@@ -52,7 +69,11 @@ struct AdjTab {
     {
         return *reinterpret_cast<const int *>(p + kAdjExps + (HALF ? 128 : 0) + lane * 4);
     }
-    __device__ __forceinline__ int2 head() const { return *reinterpret_cast<const int2 *>(p + kAdjExps + 256); }
+    __device__ __forceinline__ int lifts() const
+    {
+        return *reinterpret_cast<const int *>(p + kAdjExps + 256 + lane * 4);
+    }
+    __device__ __forceinline__ int2 head() const { return *reinterpret_cast<const int2 *>(p + kAdjHead); }
 };
 
 __device__ __forceinline__ double adj_f64(const unsigned char *p, int q, int lane)
@@ -67,8 +88,8 @@ adj_tables_kernel(int Nr, int NP, const double *__restrict__ half, const double 
                   unsigned char *__restrict__ out)
 {
     __shared__ int flags[kAdjTableThreads / 32][2];
-    const int jp = threadIdx.x, i = blockIdx.x * blockDim.y + threadIdx.y;
-    const int k = threadIdx.y * blockDim.x + threadIdx.x;
+    const int jp = threadIdx.x, k = threadIdx.y * blockDim.x + threadIdx.x;
+    int i = blockIdx.x * blockDim.y + threadIdx.y;
     if (k < kAdjTableThreads / 32 * 2) (&flags[0][0])[k] = 0;
     __syncthreads();
     auto H = [&](int c, int q, int j) {
@@ -78,7 +99,7 @@ adj_tables_kernel(int Nr, int NP, const double *__restrict__ half, const double 
         return (c < 1 || c >= Nr - 1 || j < 0 || j >= NP) ? 0.0 : node[((size_t)c * kNCN + q) * NP + j];
     };
     // integers of node c (w = 0) or half node c (w = 1)
-    auto entries = [&](int c, int w, double (&v)[6], int (&e)[2], int *cold) {
+    auto entries = [&](int c, int w, double (&v)[6]) {
         if (w == 0) {
             v[A_F1] = N(c, N_FPR, jp), v[A_F2] = N(c, N_FMR, jp), v[A_G1] = N(c, N_FPI, jp), v[A_G2] = N(c, N_FMI, jp);
             v[A_KP] = N(c, N_KP, jp - 1), v[A_KM] = N(c, N_KM, jp + 1);
@@ -86,26 +107,37 @@ adj_tables_kernel(int Nr, int NP, const double *__restrict__ half, const double 
             v[A_F1] = H(c, H_FAR, jp), v[A_F2] = H(c, H_FCR, jp), v[A_G1] = H(c, H_FAI, jp), v[A_G2] = H(c, H_FCI, jp);
             v[A_KP] = H(c, H_KP, jp - 1), v[A_KM] = H(c, H_KM, jp + 1);
         }
-        e[0] = class_exponent((fabs(v[A_F1]) + fabs(v[A_F2])) + (fabs(v[A_KP]) + fabs(v[A_KM])), cold);
-        e[1] = class_exponent(fabs(v[A_G1]) + fabs(v[A_G2]), cold);
     };
-    double vn[6], vh[6], vx[6];
-    int en[2], eh[2], ex[2], cold = 0;
+    auto terms = [](const double (&v)[6]) {
+        return RowTerms{fabs(v[A_F1]) + fabs(v[A_F2]), fabs(v[A_KM]), fabs(v[A_KP])};
+    };
+    auto other = [](const double (&v)[6]) { return fabs(v[A_G1]) + fabs(v[A_G2]); };
+    double vn[6], vh[6];
+    int cold = 0;
     const bool in = i < Nr - 1;
-    if (in) {
-        bool imag = false;
-        entries(i, 0, vx, ex, &cold);          // node i and half node i - 1/2: flags only
-        imag |= ex[1] != kSplitAbsent;
-        entries(i - 1, 1, vx, ex, &cold);
-        imag |= ex[1] != kSplitAbsent;
-        entries(i + 1, 0, vn, en, &cold);
-        entries(i, 1, vh, eh, &cold);
-        imag |= en[1] != kSplitAbsent || eh[1] != kSplitAbsent || N(i, N_C2I, jp) != 0.0 ||
-                N(i + 1, N_C2I, jp) != 0.0 || H(i, H_PI, jp) != 0.0 || H(i - 1, H_PI, jp) != 0.0;
-        // plain stores of the same value
-        if (cold) flags[threadIdx.y][0] = 1;
-        if (imag) flags[threadIdx.y][1] = 1;
+    if (!in) i = Nr - 2;   // (the block's threads meet below)
+    {   // node i and half node i - 1/2: flags only
+        double wn[6], wh[6];
+        entries(i, 0, wn);
+        entries(i - 1, 1, wh);
+        const RowTerms tn = terms(wn), th = terms(wh);
+        const RowLifts lift(tn, th, &cold);
+        const double gn = other(wn), gh = other(wh);
+        RowExps(tn, lift, gn, &cold);
+        RowExps(th, lift, gh, &cold);
+        if (in && (gn != 0.0 || gh != 0.0)) flags[threadIdx.y][1] = 1;
     }
+    entries(i + 1, 0, vn);
+    entries(i, 1, vh);
+    const RowTerms tn = terms(vn), th = terms(vh);
+    const RowLifts lift(tn, th, &cold);
+    const double gn = other(vn), gh = other(vh);
+    const RowExps xn(tn, lift, gn, &cold), xh(th, lift, gh, &cold);
+    // plain stores of the same value
+    if (in && cold) flags[threadIdx.y][0] = 1;
+    if (in && (gn != 0.0 || gh != 0.0 || N(i, N_C2I, jp) != 0.0 || N(i + 1, N_C2I, jp) != 0.0 ||
+               H(i, H_PI, jp) != 0.0 || H(i - 1, H_PI, jp) != 0.0))
+        flags[threadIdx.y][1] = 1;
     __syncthreads();
     if (!in) return;
     const int lane = jp & 31;
@@ -117,17 +149,19 @@ adj_tables_kernel(int Nr, int NP, const double *__restrict__ half, const double 
                                H(i - 1, H_HQ, jp), H(i - 1, H_PCR, jp), H(i - 1, H_PI, jp)};
     for (int q = 0; q < kAdjF64; ++q, d += 32) *d = f[q];
     const bool none = flags[threadIdx.y][0] != 0;
-    auto put = [&](const double (&v)[6], const int (&e)[2]) {
-        for (int q = 0; q < 6; ++q, d += 32)
-            *reinterpret_cast<int2 *>(d) = none ? make_int2(0, 0)
-                                                : split_entry(v[q], e[q == A_G1 || q == A_G2]);
+    auto put = [&](const double (&v)[6], const RowExps &e) {
+        for (int q = 0; q < 6; ++q, d += 32) {
+            const int C = q == A_G1 || q == A_G2 ? e.g : q == A_KM ? e.f - lift.u : q == A_KP ? e.f - lift.d : e.f;
+            *reinterpret_cast<int2 *>(d) = none ? make_int2(0, 0) : split_entry(v[q], C);
+        }
     };
-    put(vn, en);
-    put(vh, eh);
+    put(vn, xn);
+    put(vh, xh);
     int *x = reinterpret_cast<int *>(block + kAdjExps);
-    x[lane] = (en[0] & 0xffff) | (en[1] << 16);
-    x[32 + lane] = (eh[0] & 0xffff) | (eh[1] << 16);
-    if (lane < 4) x[64 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
+    x[lane] = xn.packed();
+    x[32 + lane] = xh.packed();
+    x[64 + lane] = lift.packed();
+    if (lane < 4) x[96 + lane] = lane < 2 ? flags[threadIdx.y][lane] : 0;
 }
 
 // ---- sums ----
@@ -164,7 +198,7 @@ __device__ __forceinline__ void adj_zero(AdjSums &a)
 // valid, for any column that they go to.
 template <int K, bool HALF>
 __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF> &tab, int2 head,
-                                         SplitTeam<K> &team, AdjSums &s1, AdjSums &s2)
+                                         AdjTeam<K> &team, AdjSums &s1, AdjSums &s2)
 {
     const bool imag = head.y != 0;
     SplitInts p;
@@ -174,36 +208,36 @@ __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF
     const bool hot = team.exchange(
         make_int4((int)(p.x[0] >> 32), (int)p.x[0], (int)(p.x[1] >> 32), (int)p.x[1]), make_int2(p.e[0], p.e[1]),
         head.x != 0 || max(p.e[0], p.e[1]) >= kSplitMaxExp, su, eu2, sd, ed2);
-    const int rx = tab.row_exp();
-    AdjSums g1, g2;
+    // exponents of the products over the F class's: the largest of each sum
+    const int rx = tab.row_exp(), cf = (short)(rx & 0xffff), cg = (rx >> 16) - cf;
+    const int lx = tab.lifts(), lu = (short)(lx & 0xffff), ld = lx >> 16;
+    int f[2];
+    f[0] = max(max(eu2.x - lu, ed2.x - ld), p.e[0]);
+    f[1] = max(max(eu2.y - lu, ed2.y - ld), p.e[1]);
+    if (imag) {
+        f[0] = max(f[0], p.e[1] + cg);
+        f[1] = max(f[1], p.e[0] + cg);
+    }
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
         const int uh = g ? su.z : su.x, ul = g ? su.w : su.y, eu = g ? eu2.y : eu2.x;
         const int dh = g ? sd.z : sd.x, dl = g ? sd.w : sd.y, ed = g ? ed2.y : ed2.x;
-        const int ef = max(max(eu, ed), p.e[g]);
-        const int2 l = limbs(cut(p.x[g], ef - p.e[g], p.j[g]));
+        const int2 l = limbs(cut(p.x[g], f[g] - p.e[g], p.j[g]));
         SplitSum a, b;
-        a.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, ef - eu, min(eu, 1))), tab.entry(A_KM));
-        a.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, ef - ed, min(ed, 1))), tab.entry(A_KP));
+        a.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, f[g] + lu - eu, min(eu, 1))), tab.entry(A_KM));
+        a.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, f[g] + ld - ed, min(ed, 1))), tab.entry(A_KP));
         b = a;
         a.add(l, tab.entry(A_F1));
         b.add(l, tab.entry(A_F2));
+        if (imag) {   // the other part's, subtracted from the imaginary part
+            int2 m = limbs(cut(p.x[1 - g], f[g] - cg - p.e[1 - g], p.j[1 - g]));
+            if (g == 1) m = make_int2(-m.x, -m.y);
+            a.add(m, tab.entry(A_G1));
+            b.add(m, tab.entry(A_G2));
+        }
         s1.T[g] = a.take();
         s2.T[g] = b.take();
-        s1.O[g] = s2.O[g] = (short)(rx & 0xffff) + ef;
-        if (imag) {
-            SplitSum c, d;
-            c.add(l, tab.entry(A_G1));
-            d.add(l, tab.entry(A_G2));
-            const long long tc = c.take(), td = d.take();
-            g1.T[1 - g] = g == 0 ? -tc : tc;
-            g2.T[1 - g] = g == 0 ? -td : td;
-            g1.O[1 - g] = g2.O[1 - g] = (rx >> 16) + ef;
-        }
-    }
-    if (imag) {
-        s1 = adj_add(s1, g1);
-        s2 = adj_add(s2, g2);
+        s1.O[g] = s2.O[g] = cf + f[g];
     }
     return hot;
 }
@@ -213,7 +247,7 @@ __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF
 // (KP x)(j-1) + (KM x)(j+1) of x = v[2], v[3], from the unsplit table's row.
 template <int K>
 __device__ __forceinline__ void cold_sources(const double (&v)[4], const double *kp, const double *km,
-                                             SplitTeam<K> &team, double (&z)[2])
+                                             AdjTeam<K> &team, double (&z)[2])
 {
     double up[2], dn[2];
     team.neighbours(v[2], v[3], up, dn);
@@ -300,7 +334,7 @@ __device__ __forceinline__ void eta_row(const double (&a)[4], const double (&c)[
 // unsplit node table.
 template <int K>
 __device__ __forceinline__ void eta_row_cold(const double (&a)[4], const double (&c)[4], const double *ta, double E,
-                                             SplitTeam<K> &team, double (&ep)[4])
+                                             AdjTeam<K> &team, double (&ep)[4])
 {
     constexpr int NP = 32 * K;
     double za[2], zc[2];
@@ -337,7 +371,7 @@ __device__ __forceinline__ void mu_row(const double (&a)[4], const double (&ep)[
 // tp: the node's row of the unsplit half-node table.
 template <int K>
 __device__ __forceinline__ void mu_row_cold(const double (&a)[4], const double (&ep)[4], const double (&em)[4],
-                                            const double *tp, SplitTeam<K> &team, double (&o)[4])
+                                            const double *tp, AdjTeam<K> &team, double (&o)[4])
 {
     constexpr int NP = 32 * K;
     double yp[2], ym[2];
@@ -390,7 +424,7 @@ struct AdjSweep {
     // (with the waveform gradient added, zero on the radial edges).  The edges'
     // own mu, which nothing uses, is stored as zero.
     template <typename Load, typename Right, typename Store>
-    __device__ __forceinline__ void run(SplitRingState &st, SplitTeam<K> &team, Load load, int i0, int i1,
+    __device__ __forceinline__ void run(SplitRingState &st, AdjTeam<K> &team, Load load, int i0, int i1,
                                         bool again, Right before_right, Store store) const
     {
         constexpr int NP = 32 * K;
