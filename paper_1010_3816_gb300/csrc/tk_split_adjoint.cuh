@@ -174,14 +174,14 @@ struct AdjSums {
 };
 
 // a + b, the smaller one's last places cut off (a place is below 2^-57 of the
-// sum's bound).
+// sum's bound), of either sign alike.
 __device__ __forceinline__ AdjSums adj_add(const AdjSums &a, const AdjSums &b)
 {
     AdjSums r;
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
         r.O[g] = max(a.O[g], b.O[g]);
-        r.T[g] = shr_s64(a.T[g], r.O[g] - a.O[g]) + shr_s64(b.T[g], r.O[g] - b.O[g]);
+        r.T[g] = shr_zero(a.T[g], r.O[g] - a.O[g]) + shr_zero(b.T[g], r.O[g] - b.O[g]);
     }
     return r;
 }

@@ -177,3 +177,29 @@ def test_neighbours_of_very_different_size(kw, Nth, mode, spread):
     g.close()
     _check(got, E.step(u.astype(LD)), E.step(np.abs(u).astype(LD), np.abs))
     _check(grad, E.transpose(dL.astype(LD)), E.transpose(np.abs(dL).astype(LD), np.abs))
+
+
+# every number of 32-row pieces, with one column per team and with several
+SIZES = [(60, 20), (60, 50), (60, 97), (2300, 30), (2200, 64), (1300, 128)]
+
+
+@pytest.mark.parametrize("Nr,Nth", SIZES)
+@pytest.mark.parametrize("mode", [0, 1])
+def test_both_signs_alike(Nr, Nth, mode):
+    """The step of -u and the gradient of -dL are the negatives of those of u and
+    dL to the bit, with neighbours of very different size."""
+    w = _work(Nr, Nth)
+    rng = np.random.default_rng(2)
+    shape = (4, Nth, Nr)
+    u0, dL = (rng.standard_normal(shape) * 2.0 ** rng.integers(-30, 30, shape) for _ in range(2))
+    g = _solver(w, mode)
+    out = []
+    for sign in (1.0, -1.0):
+        g.set_initial(*(sign * u0))
+        g.step(3)
+        grad = np.empty(shape)
+        g.adjoint(grad, dL_dfinal=sign * dL, independent_pi=True)
+        out.append((g.state(), grad))
+    g.close()
+    assert np.array_equal(out[0][0], -out[1][0])
+    assert np.array_equal(out[0][1], -out[1][1])
