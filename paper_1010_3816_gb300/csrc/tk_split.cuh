@@ -140,9 +140,9 @@ struct SplitSum {
     }
 };
 
-// T 2^(o - 1080) in FP64, 0 below the normal numbers.  The bits beyond the 53
-// are replaced by a 1 in the last place (unbiased, as in cut).  In integers:
-// the conversion instruction holds the FP64 pipe as long as a DFMA does.
+// T 2^(o - 1080) in FP64, rounded to the nearest (ties to even), 0 below the
+// normal numbers.  In integers: the conversion instruction holds the FP64 pipe as
+// long as a DFMA does.
 __device__ __forceinline__ double split_value(long long T, int o)
 {
     const long long s = T >> 63;
@@ -150,11 +150,12 @@ __device__ __forceinline__ double split_value(long long T, int o)
     const unsigned mh = (unsigned)(m >> 32), ml = (unsigned)m;
     int n = __clz((int)mh);
     if (mh == 0) n = 32 + __clz((int)ml);
-    const unsigned long long q = m << n;
+    unsigned long long q = m << (n - 1);             // the leading bit at place 62 (|T| < 2^62)
+    q += 0x1ffu + (((unsigned)q >> 10) & 1u);        // 53 bits stay, a carry goes into the exponent
     const unsigned qh = (unsigned)(q >> 32), ql = (unsigned)q;
     const int e = o - n + 6;   // exponent field
-    const unsigned lo = __funnelshift_r(ql, qh, 11) | 1u;
-    const unsigned hi = ((qh >> 11) + ((unsigned)(e - 1) << 20)) | ((unsigned)s & 0x80000000u);
+    const unsigned lo = __funnelshift_r(ql, qh, 10);
+    const unsigned hi = ((qh >> 10) + ((unsigned)(e - 1) << 20)) | ((unsigned)s & 0x80000000u);
     const bool normal = e > 0 && m != 0;
     return __hiloint2double(normal ? (int)hi : 0, normal ? (int)lo : 0);
 }

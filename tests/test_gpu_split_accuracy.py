@@ -203,3 +203,34 @@ def test_both_signs_alike(Nr, Nth, mode):
     g.close()
     assert np.array_equal(out[0][0], -out[1][0])
     assert np.array_equal(out[0][1], -out[1][1])
+
+
+@pytest.mark.parametrize("Nr,Nth", SIZES)
+@pytest.mark.parametrize("mode", [0, 1])
+def test_representable_couplings_are_exact(Nr, Nth, mode):
+    """With c3 alone and Phi = 1 the new Pi is dt c3, a number of 53 bits, and
+    the transpose of a single Pi = 1 gives Phi such numbers (its Pi, 1 + dt^2 c3 / 4,
+    is none): nothing but the rounding of the integer sum to FP64 can change a bit."""
+    import paper_1010_3816_gb300 as tk
+    w = _work(Nr, Nth)
+    rng = np.random.default_rng(9)
+    node, half = np.zeros((2, 9, Nth, Nr))
+    node[5:7] = rng.standard_normal((2, Nth, Nr))
+    g = tk.Solver(rstar_min=w.rs_min, rstar_max=w.rs_max, Nr=w.Nr, Ntheta=w.Ntheta, dt=w.dt)
+    tk.tk_set_coefficients(g.h, w.a, w.M, w.s, w.m, node, half, np.zeros((2, Nth)))
+    g.set_steps_per_launch(mode)
+    E = Exact(w, node, half, np.zeros((2, Nth)))
+    u = np.zeros((4, Nth, Nr))
+    u[0, :, 1:-1] = 1.0
+    dL = np.zeros_like(u)
+    dL[2, :, 2:-2:4] = 1.0
+    grad = _transpose(g, w, dL)
+    g.set_initial(*u)
+    g.step(1)
+    got = g.state()
+    g.close()
+    inner = np.s_[:, :, 2:-2]      # (next to the edges Phi's half nodes are 1/2)
+    want = E.step(u.astype(LD))
+    assert np.array_equal(got[inner], want[inner].astype(float))
+    assert np.array_equal(np.abs(got[2][:, 2:-2]), np.abs(w.dt * node[5][:, 2:-2]))
+    assert np.array_equal(grad[:2], E.transpose(dL.astype(LD))[:2].astype(float))
