@@ -95,6 +95,14 @@ __device__ void sweep(const BatchMember &m, const T *__restrict__ u_in, T *__res
     }
 }
 
+// A member's unsplit tables, looked up where they are used: four registers less in
+// the sweep.
+struct MemberTables {
+    const BatchMember *m;
+    __device__ __forceinline__ const double *half() const { return (const double *)m->half; }
+    __device__ __forceinline__ const double *node() const { return (const double *)m->node; }
+};
+
 // The block's share of an FP64 item: its teams take equal parts of the columns.
 template <int K>
 __device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long long *bar, SplitRows *rows,
@@ -104,8 +112,7 @@ __device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long
     constexpr int TEAMS = kBatchThreads / 32 / K, NP = 32 * K;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
     SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
-    const SplitSweep<K> sw{ring + wib, bar, m.step + team.h * kStepBytes, (const double *)m.half,
-                           (const double *)m.node, m.Nr, m.en, nullptr};
+    const SplitSweep<K, MemberTables> sw{ring + wib, bar, m.step + team.h * kStepBytes, {&m}, m.Nr, m.en, nullptr};
     const int a = i0 + t * (i1 - i0) / TEAMS, b = i0 + (t + 1) * (i1 - i0) / TEAMS;
     if (b <= a) return;
     sw.run(st, team, u_in, a, b, false, [] {}, [&](int i, const double (&o)[4]) {

@@ -49,8 +49,8 @@
 // rows per lane (three warps, 168 registers) the same arithmetic took 124 us.
 // 20 warps (96 registers, spills): 120 us.
 //
-// Subnormal values count as zero in the coupling, and a coupling below 2^-1022
-// is dropped.  Columns with a Phi above 1e263, infinite or NaN, and columns whose
+// Subnormal values and couplings are taken and rounded like any other.  Columns
+// with a Phi above 1e263, infinite or NaN, and columns whose
 // tables are not finite or too large, take the FP64 instructions alone, so that
 // such values propagate as IEEE arithmetic has them; Pi only ever meets FP64
 // instructions (testing it too took 89.6 instead of 88.8 us on 25601 x 64).
@@ -66,7 +66,8 @@ namespace {
 
 // Two components of a lane's row as integers: the magnitude, all its bits
 // inverted where the value is negative (so that a right shift cuts both signs
-// alike), the exponent field, and 1 unless the value is zero (or subnormal).
+// alike), the exponent field (1 for zeros and subnormals, whose magnitudes have no
+// leading one), and 1 unless the value is zero.
 struct SplitInts {
     long long x[2];
     int e[2];
@@ -112,8 +113,8 @@ __device__ __forceinline__ void split_ints(const double (&u)[4], SplitInts &o)
     for (int k = C0; k < C0 + 2; ++k) {
         const unsigned hi = (unsigned)__double2hiint(u[k]);
         const unsigned lo = (unsigned)__double2loint(u[k]);
-        const int e = (int)((hi >> 20) & 0x7ffu), j = min(e, 1);
-        const unsigned m = (hi & 0xfffffu) | 0x100000u;
+        const int f = (int)((hi >> 20) & 0x7ffu), e = max(f, 1), j = nonzero((int)(hi & 0x7fffffffu), (int)lo);
+        const unsigned m = (hi & 0xfffffu) + ((unsigned)min(f, 1) << 20);
         const unsigned s = (unsigned)((int)hi >> 31), mask = (unsigned)-j;
         const unsigned xh = (__funnelshift_l(lo, m, 7) ^ s) & mask, xl = ((lo << 7) ^ s) & mask;
         o.x[k - C0] = ((long long)(int)xh << 32) | xl;
@@ -140,9 +141,9 @@ struct SplitSum {
     }
 };
 
-// T 2^(o - 1080) in FP64, rounded to the nearest (ties to even), 0 below the
-// normal numbers.  In integers: the conversion instruction holds the FP64 pipe as
-// long as a DFMA does.
+// T 2^(o - 1080) in FP64, rounded to the nearest (ties to even); subnormal ones
+// are rounded once more by a product with 2^-64.  In integers: the conversion
+// instruction holds the FP64 pipe as long as a DFMA does.
 __device__ __forceinline__ double split_value(long long T, int o)
 {
     const long long s = T >> 63;
@@ -156,8 +157,10 @@ __device__ __forceinline__ double split_value(long long T, int o)
     const int e = o - n + 6;   // exponent field
     const unsigned lo = __funnelshift_r(ql, qh, 10);
     const unsigned hi = ((qh >> 10) + ((unsigned)(e - 1) << 20)) | ((unsigned)s & 0x80000000u);
-    const bool normal = e > 0 && m != 0;
-    return __hiloint2double(normal ? (int)hi : 0, normal ? (int)lo : 0);
+    if (e > 0 || m == 0) return __hiloint2double(m != 0 ? (int)hi : 0, (int)lo);
+    return e < -60 ? 0.0
+                   : __hiloint2double((int)(((qh >> 10) + ((unsigned)(e + 63) << 20)) | ((unsigned)s & 0x80000000u)),
+                                      (int)lo) * 0x1p-64;
 }
 
 // ---- teams ----
@@ -505,12 +508,19 @@ __device__ __forceinline__ void split_ring_init(unsigned long long *bar, int lan
     __syncwarp();
 }
 
-template <int K>
+// The unsplit tables, for the FP64 instructions alone.
+struct Unsplit {
+    const double *h, *n;
+    __device__ __forceinline__ const double *half() const { return h; }
+    __device__ __forceinline__ const double *node() const { return n; }
+};
+
+template <int K, class Tables = Unsplit>
 struct SplitSweep {
     SplitRing *ring;
     unsigned long long *bar;   // the warp's two mbarriers, in shared memory (split_ring_init)
     const unsigned char *tab;  // the warp's block of column 0
-    const double *half64, *node64;
+    Tables unsplit;
     int Nr;
     double en;
     int *err;                  // raised when a wait for a copy gives up
@@ -590,12 +600,13 @@ struct SplitSweep {
                 await(st, st.cur);
                 const unsigned char *block = ring->tab[st.cur];
                 st.cur ^= 1;
-                split_half_node<K>(a, pa, c, pc, block, team, half64 + (size_t)i * (kNCH * NP) + row, k1, hp);
+                split_half_node<K>(a, pa, c, pc, block, team, unsplit.half() + (size_t)i * (kNCH * NP) + row, k1,
+                                   hp);
                 split_ints<0>(hp, pp);
                 if (i >= i0) {
                     if (i > 0) {
-                        split_full_node<K>(hm, pm, hp, pp, a, block, team, node64 + (size_t)i * (kNCN * NP) + row,
-                                           en, k1, o);
+                        split_full_node<K>(hm, pm, hp, pp, a, block, team,
+                                           unsplit.node() + (size_t)i * (kNCN * NP) + row, en, k1, o);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) o[k] = 0.0;

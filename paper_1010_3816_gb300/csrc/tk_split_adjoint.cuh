@@ -224,8 +224,8 @@ __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF
         const int dh = g ? sd.z : sd.x, dl = g ? sd.w : sd.y, ed = g ? ed2.y : ed2.x;
         const int2 l = limbs(cut(p.x[g], f[g] - p.e[g], p.j[g]));
         SplitSum a, b;
-        a.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, f[g] + lu - eu, min(eu, 1))), tab.entry(A_KM));
-        a.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, f[g] + ld - ed, min(ed, 1))), tab.entry(A_KP));
+        a.add(limbs(cut(((long long)uh << 32) | (unsigned)ul, f[g] + lu - eu, nonzero(uh, ul))), tab.entry(A_KM));
+        a.add(limbs(cut(((long long)dh << 32) | (unsigned)dl, f[g] + ld - ed, nonzero(dh, dl))), tab.entry(A_KP));
         b = a;
         a.add(l, tab.entry(A_F1));
         b.add(l, tab.entry(A_F2));

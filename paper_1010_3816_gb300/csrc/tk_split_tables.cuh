@@ -23,7 +23,8 @@ namespace {
 __device__ int split_exponent(double v)
 {
     if (v == 0.0) return kSplitAbsent;
-    return ((__double2hiint(v) >> 20) & 0x7ff) - 1022;
+    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    return e != 0 ? e - 1022 : -1010 - __clzll(__double_as_longlong(v));
 }
 
 // The magnitudes of a table's class F: the own coefficients' sum, and each
@@ -85,10 +86,12 @@ struct RowExps {
 __device__ int2 split_entry(double c, int C)
 {
     const long long b = __double_as_longlong(c);
-    const int e = (int)((b >> 52) & 0x7ff);
-    if (e == 0) return make_int2(0, 0);
-    long long v = (b & 0xfffffffffffffll) | (1ll << 52);
-    const int up = e - 1075 + 62 - C;    // <= 9
+    int e = (int)((b >> 52) & 0x7ff);
+    long long v = b & 0xfffffffffffffll;
+    if (e != 0) v |= 1ll << 52;
+    else e = 1;
+    if (v == 0) return make_int2(0, 0);
+    const int up = e - 1075 + 62 - C;    // |c| < 2^C: v stays below 2^62
     if (up >= 0) v <<= up;
     else v = up < -54 ? 0 : (v + (1ll << (-up - 1))) >> -up;
     v |= 1;   // odd, so that the limbs of -c are those of c with the other sign

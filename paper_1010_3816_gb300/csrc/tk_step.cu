@@ -175,7 +175,7 @@ lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__res
         split_ring_init(bars[wib], lane);
         SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
         const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib],
-                               step + (wib % K) * kStepBytes, half, node, Nr, en, nullptr};
+                               step + (wib % K) * kStepBytes, {half, node}, Nr, en, nullptr};
         int i0, i1;
         team_range<W, K>(Nr, t, &i0, &i1);
         SplitRingState st;
@@ -258,8 +258,8 @@ lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, co
     __syncthreads();
     const int nb = (int)gridDim.x, b = (int)blockIdx.x;
     SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
-    const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib], step + h * kStepBytes, half,
-                           node, Nr, en, err};
+    const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib], step + h * kStepBytes,
+                           {half, node}, Nr, en, err};
     // The launch has at most Nr / TEAMS blocks, so every team has a column; one
     // without would never publish, and its neighbours' waits would run out.
     int i0, i1;

@@ -234,3 +234,27 @@ def test_representable_couplings_are_exact(Nr, Nth, mode):
     assert np.array_equal(got[inner], want[inner].astype(float))
     assert np.array_equal(np.abs(got[2][:, 2:-2]), np.abs(w.dt * node[5][:, 2:-2]))
     assert np.array_equal(grad[:2], E.transpose(dL.astype(LD))[:2].astype(float))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("Nth", [30, 64, 97])
+@pytest.mark.parametrize("p", [-960, -1010, -1040, -1060])
+@pytest.mark.parametrize("kw", [dict(), dict(s=0, m=0, rs_min=-1440.0)])
+def test_gradual_underflow(kw, p, Nth, mode):
+    """Tiny data: each of at most 64 roundings costs 2^-1075 at least, and 4 / dt as
+    much in the Phi that the transposed half nodes keep times dt / 4 (near the horizon
+    the neighbours' coefficients are subnormal too)."""
+    w = _work(9, Nth, **kw)
+    rng = np.random.default_rng(-p)
+    shape = (4, Nth, w.Nr)
+    u, dL = (rng.standard_normal(shape) * 2.0 ** p for _ in range(2))
+    u[:, :, [0, -1]] = dL[:, :, [0, -1]] = 0.0
+    g, E = _case(w, mode)
+    grad = _transpose(g, w, dL)
+    g.set_initial(*u)
+    g.step(1)
+    got = g.state()
+    g.close()
+    floor = 64 * 4 / w.dt * LD(2.0) ** -1075 / TOL
+    _check(got, E.step(u.astype(LD)), E.step(np.abs(u).astype(LD), np.abs) + floor)
+    _check(grad, E.transpose(dL.astype(LD)), E.transpose(np.abs(dL).astype(LD), np.abs) + floor)
