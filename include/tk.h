@@ -163,7 +163,12 @@ tk_status tk_add_observer(tk_solver *S, double rstar_obs, double theta_obs, int 
  * outer step.  In the persistent mode of tk_set_steps_per_launch (-1, the
  * default) every step of the call runs in one cooperative launch and the call
  * synchronizes the stream to check that launch's bounded waits; in the other
- * modes it is asynchronous.  The persistent launch needs all its blocks
+ * modes it is asynchronous, and the bounded waits of its FP64 launches (for
+ * their own copies of tables) are checked by the next call on this solver that
+ * waits for the stream (tk_extract and tk_get_state to the host,
+ * tk_check_finite, tk_synchronize, a persistent tk_step, tk_adjoint with host
+ * arrays), which then returns TK_ERR_INTERNAL; the samples are then invalid like
+ * the state.  The persistent launch needs all its blocks
  * resident at once, as the grid was sized for at tk_make_grid; where fewer
  * fit (a limit on active threads set for the process) the launch fails with
  * TK_ERR_CUDA and nothing is stepped, and tk_set_steps_per_launch(S, 1) runs
@@ -233,7 +238,9 @@ tk_status tk_extract_noalloc(tk_solver *S, int obs_id, int first, int count, dou
  * The solver's state is not touched.  Allocates two adjoint state levels on
  * first use and, in FP64, the transposed tables (6544 bytes per column and 32
  * rows), all kept until tk_destroy, and temporary buffers for host inputs.
- * Synchronizes the stream when an input or the output is in host memory. */
+ * Synchronizes the stream when an input or the output is in host memory, and
+ * where it runs as one persistent launch (the mode of tk_set_steps_per_launch);
+ * otherwise bounded waits that ran out are reported by the next call that does. */
 tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfinal, int on_device,
                      double *grad, int grad_on_device, int independent_pi);
 
@@ -320,7 +327,8 @@ tk_status tk_steps_done(const tk_solver *S, int64_t *steps);
  * not.  Synchronizes the stream. */
 tk_status tk_check_finite(tk_solver *S);
 
-/* Wait for all work queued by this solver. */
+/* Wait for all work queued by this solver.  TK_ERR_INTERNAL if a bounded wait of
+ * an asynchronous launch ran out (tk_step, tk_batch_step, tk_adjoint). */
 tk_status tk_synchronize(tk_solver *S);
 
 /* ---- Batches: many solvers advanced together ----------------------------
@@ -341,7 +349,9 @@ typedef struct tk_batch tk_batch;
  * device, precision and dt, or lcm(k_i) > 64. */
 tk_status tk_batch_create(tk_batch **out, tk_solver *const *members, int n);
 
-/* Advance every member by n outer steps (samples appended as by tk_step). */
+/* Advance every member by n outer steps (samples appended as by tk_step).
+ * Asynchronous; bounded waits that ran out are reported on the members as for
+ * the asynchronous modes of tk_step. */
 tk_status tk_batch_step(tk_batch *B, int n);
 
 /* Autotuner (the counterpart of the paper's tuning of the work-group size,
@@ -380,9 +390,11 @@ void tk_batch_destroy(tk_batch *B);
  * kernels' blocks do between steps and then as the one-step sweep's edge
  * warps do -- except block `silent` (-1: none), which never publishes and
  * instead waits on a shared-memory counter that nothing sets, as the one-step
- * sweep's warps wait for their siblings.  All three kinds of wait run out,
- * each sets its own error flag, and every block returns; the context stays
- * usable.  *timed_out = 1 if all three error flags were set (where tk_step
+ * sweep's warps wait for their siblings, and for a copy into shared memory that
+ * nothing starts, as they wait for their tables (a quarter of max_polls).  All
+ * four kinds of wait run out, each sets its own error flag, and every block
+ * returns; the context stays
+ * usable.  *timed_out = 1 if all four error flags were set (where tk_step
  * reports TK_ERR_INTERNAL), 0 if none was; TK_ERR_INTERNAL if only some were.  The persistent kernels use 2^24 polls.
  * Runs on the legacy default stream and synchronizes.  TK_ERR_ARG for
  * arguments out of range (message in tk_last_error(NULL)). */
@@ -403,7 +415,8 @@ tk_status tk_probe_fp64_fma(int blocks_per_sm, int threads, int iters, double *s
 /* Test hook, host-side fault injection (not in the paper): the next tk_step
  * on this solver that runs a persistent launch completes its device work
  * normally and then reports its bounded waits as having run out, with the
- * consequences described at tk_step.  For testing a caller's recovery path
+ * consequences described at tk_step; the next asynchronous tk_step,
+ * tk_batch_step or tk_adjoint has its error word set behind its launches.  For testing a caller's recovery path
  * without a device fault.  Cleared when it fires. */
 tk_status tk_inject_wait_timeout(tk_solver *S);
 

@@ -560,7 +560,7 @@ template <int K, int W>
 __global__ void __launch_bounds__(W * 32, adj_wide_warps<double, K>() / W)
 lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_out, const double *__restrict__ half,
                        const double *__restrict__ node, const unsigned char *__restrict__ tab, int Nr, double en,
-                       const InjectArgs inj)
+                       const InjectArgs inj, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned long long bars[W][2];
@@ -570,7 +570,7 @@ lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_o
     split_ring_init(bars[wib], lane);
     AdjTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
-                         en, nullptr};
+                         en, err};
     int i0, i1;
     team_range<W, K>(Nr, t, &i0, &i1);
     SplitRingState st;
@@ -705,6 +705,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
         return sh.hot[w][t] != 0;
     };
     const bool extra = j == 0 && before;               // the block left of the first
+    bool lost = false;                                 // the tables did not come
     if (halves || extra) {
         if (lane == 0) {
             unsigned long long *bar = &sh.bars[wib];
@@ -715,7 +716,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
             if (extra) bulk_fetch(sh.tab[0][h], tab + ((size_t)(col - 1) * K + h) * kAdjBytes, kAdjBytes, bar);
         }
         __syncwarp();
-        if (!mbar_wait(&sh.bars[wib], 0)) atomicExch(err, 1);
+        lost = !warp_mbar_wait(&sh.bars[wib], 0, ErrWord{err});
     }
     double a[4];   // the column's adjoint state
 #pragma unroll
@@ -797,6 +798,7 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
             if (j == T) warp_publish_gpu(flags + (nb + b) * K + h, e + 1);
         }
     }
+    if (lost) mbar_wait(&sh.bars[wib], 0);
 }
 
 // Transpose of the initial-data map of tk_set_initial_data: the adjoint state
@@ -1031,7 +1033,7 @@ cudaError_t adj_smem_setup()
 
 template <typename T, int K, int W>
 cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab,
-                             int Nr, int blocks, double dt_in, const InjectArgs &inj,
+                             int Nr, int blocks, double dt_in, const InjectArgs &inj, int *err,
                              cudaStream_t st)
 {
     cudaError_t e = adj_smem_setup<T, K, W>();
@@ -1039,7 +1041,7 @@ cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const 
     if constexpr (sizeof(T) == 8)
         return launch_chained<lw_adjoint_team_kernel<K, W>>(
             (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const double *)lam, (double *)mu,
-            (const double *)half, (const double *)node, tab, Nr, 0.5 * dt_in, inj);
+            (const double *)half, (const double *)node, tab, Nr, 0.5 * dt_in, inj, err);
     else
         return launch_chained<lw_adjoint_kernel<T, K, W>>(
             (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const T *)lam, (T *)mu, (const T *)half,
@@ -1048,28 +1050,28 @@ cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const 
 
 template <typename T, int K>
 cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab, int Nr,
-                       int blocks, int warps, double dt_in, const InjectArgs &inj, cudaStream_t st)
+                       int blocks, int warps, double dt_in, const InjectArgs &inj, int *err, cudaStream_t st)
 {
     constexpr int WW = adj_wide_warps<T, K>();
     if (warps == WW)
-        return launch_adj_shape<T, K, WW>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, st);
+        return launch_adj_shape<T, K, WW>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, err, st);
     if (warps == kNarrowWarps)
-        return launch_adj_shape<T, K, kNarrowWarps>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, st);
+        return launch_adj_shape<T, K, kNarrowWarps>(lam, mu, half, node, tab, Nr, blocks, dt_in, inj, err, st);
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_adjoint_step(int precision, int K, const void *lam, void *mu, const void *half,
                                 const void *node, const unsigned char *tab, int Nr, int blocks, int warps, double dt_in,
-                                const InjectArgs &inj, cudaStream_t st)
+                                const InjectArgs &inj, int *err, cudaStream_t st)
 {
     if (precision == 0) {
-        if (K == 1) return launch_adj<double, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
-        if (K == 2) return launch_adj<double, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
-        return launch_adj<double, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+        if (K == 1) return launch_adj<double, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
+        if (K == 2) return launch_adj<double, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
+        return launch_adj<double, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
     }
-    if (K == 1) return launch_adj<float, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
-    if (K == 2) return launch_adj<float, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
-    return launch_adj<float, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, st);
+    if (K == 1) return launch_adj<float, 1>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
+    if (K == 2) return launch_adj<float, 2>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
+    return launch_adj<float, 4>(lam, mu, half, node, tab, Nr, blocks, warps, dt_in, inj, err, st);
 }
 
 template <typename T, int K, int W>
@@ -1397,9 +1399,10 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
                 inj.sample = t;
                 e = tk::launch_adjoint_step(S->precision, S->K, S->adj[cur], S->adj[cur ^ 1], S->half,
                                             S->node, S->adj_tab, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj,
-                                            S->stream);
+                                            S->lost + 1, S->stream);
                 cur ^= 1;
             }
+        if (e == cudaSuccess) e = tkh::mark_unchecked(S, S->stream, 1);
     }
     if (e != cudaSuccess) {
         cleanup();
@@ -1434,7 +1437,7 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
     if (e == cudaSuccess && (!grad_on_device || !on_device)) e = cudaStreamSynchronize(S->stream);
     cleanup();
     if (e != cudaSuccess) return tkh::fail(S, TK_ERR_CUDA, "tk_adjoint: %s", cudaGetErrorString(e));
-    return TK_OK;
+    return grad_on_device && on_device ? TK_OK : tkh::check_lost(S, "tk_adjoint");
 }
 
 // Gradient of a waveform loss with respect to the spin a (param 0) or the mass
@@ -1555,6 +1558,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     L.write_wave = 0;
     unsigned int *flags = (unsigned int *)pflags;
     int *perr = (int *)(flags + nflags);
+    L.err = perr;
     if (e == cudaSuccess) e = cudaMemsetAsync(perr, 0, sizeof(int), S->stream);
     // n >= 1 levels after src, to dst, dst + se, ..
     auto levels = [&](const double *src, double *dst, long long n) {
@@ -1628,7 +1632,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
                 inj.on = (g + q) % k == 0;
                 inj.sample = t0 + len - 1 - (g + q) / k;
                 e = tk::launch_adjoint_step(0, S->K, lam[cur], lam[nxt], S->half, S->node, S->adj_tab, S->Nr,
-                                            S->adj_blocks, S->adj_warps, dt_in, inj, S->stream);
+                                            S->adj_blocks, S->adj_warps, dt_in, inj, perr, S->stream);
                 cur = nxt;
             }
             if (e == cudaSuccess)

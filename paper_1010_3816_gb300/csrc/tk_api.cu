@@ -47,7 +47,7 @@ void release(tk_solver *S)
     void *ptrs[] = {S->u[0], S->u[1], S->half, S->node, S->b_node, S->w_row,
                     S->rad, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
                     S->adj[0], S->adj[1], S->u_init, S->dhalf, S->dnode, S->db_node, S->pflags,
-                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step, S->adj_tab};
+                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step, S->adj_tab, S->lost};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (int k = 0; k < 2; ++k)
@@ -104,6 +104,32 @@ tk_status need_state(tk_solver *S, const char *what)
     return TK_OK;
 }
 
+tk_status check_lost(tk_solver *S, const char *what)
+{
+    if (!S->unchecked) return TK_OK;
+    int h[2] = {0, 0};
+    TK_CUDA(S, cudaMemcpyAsync(h, S->lost, sizeof h, cudaMemcpyDeviceToHost, S->stream));
+    TK_CUDA(S, cudaStreamSynchronize(S->stream));
+    S->unchecked = false;
+    if (!h[0] && !h[1]) return TK_OK;
+    TK_CUDA(S, cudaMemsetAsync(S->lost, 0, sizeof h, S->stream));
+    if (h[0]) {
+        S->state_valid = false;
+        S->init_valid = false;
+    }
+    return fail(S, TK_ERR_INTERNAL, "%s: a copy of tables did not come in an earlier %s; %s", what,
+                h[0] ? "tk_step or tk_batch_step" : "tk_adjoint",
+                h[0] ? "the state and its samples are invalid" : "its gradient is not valid");
+}
+
+cudaError_t mark_unchecked(tk_solver *S, cudaStream_t st, int which)
+{
+    S->unchecked = true;
+    if (!S->inject_wait_timeout) return cudaSuccess;
+    S->inject_wait_timeout = false;
+    return cudaMemsetAsync(S->lost + which, 1, sizeof(int), st);
+}
+
 tk::WaveRead wave_read(const tk_solver *S, int k)
 {
     tk::WaveRead r;
@@ -134,6 +160,7 @@ void fill_launch(const tk_solver *S, tk::StepLaunch &L)
     L.cmp = S->cmp;
     L.gpm = S->gpm;
     L.step = S->step;
+    L.err = S->lost;
     L.wave_cap = S->wave_cap;
     L.wave = S->wave;
     L.w_row = S->w_row;
@@ -152,6 +179,7 @@ void fill_launch(const tk_solver *S, tk::StepLaunch &L)
 }  // namespace tkh
 
 using tkh::alloc;
+using tkh::check_lost;
 using tkh::ensure_staging;
 using tkh::release;
 using tkh::state_elems;
@@ -260,6 +288,7 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     if (st == TK_OK) st = alloc(S, (void **)&S->flag, sizeof(int));
     if (st == TK_OK) st = alloc(S, (void **)&S->stiff, 2 * sizeof(unsigned long long));
     if (st == TK_OK) st = alloc(S, (void **)&S->ctr, 2 * sizeof(long long));
+    if (st == TK_OK) st = alloc(S, (void **)&S->lost, 2 * sizeof(int));
     if (st != TK_OK) {
         snprintf(g_err, sizeof g_err, "%s", S->err);
         release(S);
@@ -269,6 +298,7 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     e = cudaMemsetAsync(S->u[0], 0, se * S->esz, S->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(S->u[1], 0, se * S->esz, S->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(S->ctr, 0, 2 * sizeof(long long), S->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(S->lost, 0, 2 * sizeof(int), S->stream);
     if (e != cudaSuccess) {
         fail(nullptr, TK_ERR_CUDA, "tk_make_grid: %s", cudaGetErrorString(e));
         release(S);
@@ -441,6 +471,7 @@ static tk_status import_planes(tk_solver *S, const double *pr, const double *pi,
         qr = qr ? S->staging + 2 * plane : nullptr;
         qi = qi ? S->staging + 3 * plane : nullptr;
     }
+    if (S->unchecked) TK_CUDA(S, cudaMemsetAsync(S->lost, 0, sizeof(int), S->stream));   // of the state replaced
     void *dst = S->u[S->cur];
     TK_CUDA(S, tk::launch_import_state(S->precision, S->Nr, S->Nth, S->NP, S->drs, pr, pi, qr, qi,
                                        S->b_node, dst, S->stream));
@@ -626,6 +657,8 @@ tk_status tk_step(tk_solver *S, int n)
     st = ensure_wave(S, S->count + n);
     if (st != TK_OK) return st;
     if (S->persist && (long long)n * S->substeps >= 2) {
+        st = check_lost(S, "tk_step");   // this call waits for the stream anyway
+        if (st != TK_OK) return st;
         // every inner step of the call in one cooperative launch; its waits
         // are bounded, and a wait that timed out is reported here
         // the one-step sweep keeps two flags per block and 32 rows (its first and last team)
@@ -730,6 +763,7 @@ tk_status tk_step(tk_solver *S, int n)
         st = get_graph(S, chunk, &ge);
         if (st != TK_OK) return st;
         TK_CUDA(S, cudaGraphLaunch(ge, S->stream));
+        TK_CUDA(S, tkh::mark_unchecked(S, S->stream));
         S->count += chunk;
         S->steps_done += chunk;
         n -= chunk;
@@ -737,6 +771,7 @@ tk_status tk_step(tk_solver *S, int n)
     if (n > 0) {
         int cur = S->cur;
         TK_CUDA(S, enqueue_steps(S, S->cur, n, S->stream, &cur));
+        TK_CUDA(S, tkh::mark_unchecked(S, S->stream));
         S->cur = cur;
         S->count += n;
         S->steps_done += n;
@@ -785,6 +820,8 @@ tk_status tk_extract(tk_solver *S, int obs_id, double *re, double *im, int capac
         TK_CUDA(S, tk::launch_wave_sum(src, 0, n, rd, re, im, S->stream));
         return TK_OK;
     }
+    st = check_lost(S, "tk_extract");
+    if (st != TK_OK) return st;
     // host read-out through a device buffer the solver keeps (sized to the
     // waveform buffer's capacity, reallocated only when that grows)
     if (S->xbuf_cap < S->wave_cap) {
@@ -826,6 +863,8 @@ tk_status tk_get_state(tk_solver *S, double *planes4, int on_device)
                                            S->stream));
         return TK_OK;
     }
+    st = check_lost(S, "tk_get_state");
+    if (st != TK_OK) return st;
     st = ensure_staging(S);
     if (st != TK_OK) return st;
     TK_CUDA(S, tk::launch_export_state(S->precision, S->Nr, S->Nth, S->NP, S->u[S->cur], S->staging,
@@ -890,6 +929,8 @@ tk_status tk_check_finite(tk_solver *S)
     if (st != TK_OK) return st;
     st = need_state(S, "tk_check_finite");
     if (st != TK_OK) return st;
+    st = check_lost(S, "tk_check_finite");
+    if (st != TK_OK) return st;
     int h = 0;
     TK_CUDA(S, cudaMemsetAsync(S->flag, 0, sizeof(int), S->stream));
     TK_CUDA(S, tk::launch_finite_check(S->precision, state_elems(S), S->u[S->cur], S->flag, S->stream));
@@ -905,7 +946,7 @@ tk_status tk_synchronize(tk_solver *S)
     tk_status st = enter(S);
     if (st != TK_OK) return st;
     TK_CUDA(S, cudaStreamSynchronize(S->stream));
-    return TK_OK;
+    return check_lost(S, "tk_synchronize");
 }
 
 tk_status tk_check_bounded_wait(int n_blocks, int silent, int64_t max_polls, int *timed_out)
@@ -915,27 +956,27 @@ tk_status tk_check_bounded_wait(int n_blocks, int silent, int64_t max_polls, int
         return TK_ERR_ARG;
     }
     unsigned int *flags = nullptr;
-    const size_t bytes = (size_t)n_blocks * sizeof(unsigned int) + 3 * sizeof(int);
+    const size_t bytes = (size_t)n_blocks * sizeof(unsigned int) + 4 * sizeof(int);
     cudaError_t e = cudaMalloc((void **)&flags, bytes);
     if (e == cudaSuccess) e = cudaMemset(flags, 0, bytes);
     // [0] the blocks' neighbour barrier, [1] a warp on a global flag, [2] a
-    // warp on a shared-memory counter
+    // warp on a shared-memory counter, [3] a warp on a copy
     int *err = (int *)(flags + n_blocks);
     if (e == cudaSuccess) e = tk::launch_wait_check(n_blocks, silent, (long long)max_polls, flags, err, 0);
-    int h[3] = {0, 0, 0};
+    int h[4] = {0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpy(h, err, sizeof h, cudaMemcpyDeviceToHost);
     if (flags) cudaFree(flags);
     if (e != cudaSuccess) {
         snprintf(g_err, sizeof g_err, "tk_check_bounded_wait: %s", cudaGetErrorString(e));
         return TK_ERR_CUDA;
     }
-    const int n_out = (h[0] != 0) + (h[1] != 0) + (h[2] != 0);
-    if (n_out != 0 && n_out != 3) {
-        snprintf(g_err, sizeof g_err, "tk_check_bounded_wait: only some waits ran out (%d %d %d)", h[0] != 0,
-                 h[1] != 0, h[2] != 0);
+    const int n_out = (h[0] != 0) + (h[1] != 0) + (h[2] != 0) + (h[3] != 0);
+    if (n_out != 0 && n_out != 4) {
+        snprintf(g_err, sizeof g_err, "tk_check_bounded_wait: only some waits ran out (%d %d %d %d)", h[0] != 0,
+                 h[1] != 0, h[2] != 0, h[3] != 0);
         return TK_ERR_INTERNAL;
     }
-    *timed_out = n_out == 3;
+    *timed_out = n_out == 4;
     return TK_OK;
 }
 

@@ -35,6 +35,7 @@ struct BatchMember {
     void *u0, *u1;            // the member's two time levels
     const void *half, *node;  // folded coefficient tables
     const unsigned char *step;   // FP64: the step's tables
+    int *err;                 // raised where a copy of them did not come
     int Nr, K;
     int substeps, ratio;      // k_i and kmax / k_i
     int level0;               // level holding the state when the call started
@@ -95,12 +96,13 @@ __device__ void sweep(const BatchMember &m, const T *__restrict__ u_in, T *__res
     }
 }
 
-// A member's unsplit tables, looked up where they are used: four registers less in
-// the sweep.
-struct MemberTables {
+// A member's unsplit tables and error word, looked up where they are used: six
+// registers less in the sweep, which spills otherwise.
+struct MemberRare {
     const BatchMember *m;
     __device__ __forceinline__ const double *half() const { return (const double *)m->half; }
     __device__ __forceinline__ const double *node() const { return (const double *)m->node; }
+    __device__ __forceinline__ int *err() const { return m->err; }
 };
 
 // The block's share of an FP64 item: its teams take equal parts of the columns.
@@ -112,7 +114,7 @@ __device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long
     constexpr int TEAMS = kBatchThreads / 32 / K, NP = 32 * K;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
     SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
-    const SplitSweep<K, MemberTables> sw{ring + wib, bar, m.step + team.h * kStepBytes, {&m}, m.Nr, m.en, nullptr};
+    const SplitSweep<K, MemberRare> sw{ring + wib, bar, m.step + team.h * kStepBytes, {&m}, m.Nr, m.en};
     const int a = i0 + t * (i1 - i0) / TEAMS, b = i0 + (t + 1) * (i1 - i0) / TEAMS;
     if (b <= a) return;
     sw.run(st, team, u_in, a, b, false, [] {}, [&](int i, const double (&o)[4]) {
@@ -364,6 +366,7 @@ tk_status upload_members(tk_batch *B)
         tkh::fill_launch(S, L);
         m.obs = L.obs;
         m.step = L.step;
+        m.err = L.err;
     }
     TKB_CUDA(B, cudaMemcpyAsync(B->d_mem, h.data(), B->n * sizeof(tk::BatchMember),
                                 cudaMemcpyHostToDevice, B->stream));
@@ -410,6 +413,7 @@ tk_status advance_members(tk_batch *B, int n)
         if ((long long)n * S->substeps % 2) S->cur ^= 1;
         S->count += n;
         S->steps_done += n;
+        TKB_CUDA(B, tkh::mark_unchecked(S, B->stream));
     }
     return TK_OK;
 }
@@ -716,6 +720,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
         best_t = per_member ? ms : (queue_ms > 0.0 && queue_ms < 1e300 ? queue_ms : best_t);
     }
     for (void *p : keep) cudaFree(p);
+    for (tk_solver *S : B->mem) S->unchecked = true;
     B->graph_chunk = old_chunk;
     B->blocks = best_blocks;
     if (st != TK_OK) return st;

@@ -225,6 +225,7 @@ struct StepLaunch {
     const float *cmp;     // FP32: compact tables [i][kNCC][jp] (the four-step sweep)
     const float *gpm;     // FP32: theta factors gp[NP], gm[NP]
     const unsigned char *step;   // FP64: the step's tables
+    int *err;             // one-step launch: raised where a copy of tables did not come
     // waveform (only on the last inner step of an outer step)
     int write_wave;
     const long long *sample_ctr;  // device: index of the sample the outer step writes

@@ -43,6 +43,11 @@ struct tk_solver {
     // then invalid until tk_set_initial_data or tk_set_state replaces it
     bool state_valid = true;
     bool inject_wait_timeout = false;   // tk_inject_wait_timeout (host-side test hook)
+    // Launches that the host does not wait for raise these words where a copy of
+    // tables did not come: [0] of steps, [1] of transposed steps.  unchecked: such
+    // launches have been made since the words were last looked at.
+    int *lost = nullptr;
+    bool unchecked = false;
     // observers and waveform samples
     struct Obs {
         double rs, th;
@@ -96,6 +101,11 @@ tk::WaveRead wave_read(const tk_solver *S, int k);
 // TK_ERR_STATE unless the solver holds a valid state (initial data set, and
 // no persistent launch failed since); `what` names the call.
 tk_status need_state(tk_solver *S, const char *what);
+// Waits for the stream and looks at the solver's error words, where launches have
+// been made that may have raised them; raised ones are reported and cleared.
+tk_status check_lost(tk_solver *S, const char *what);
+// Steps (transposed ones: which = 1) have been enqueued that may raise them.
+cudaError_t mark_unchecked(tk_solver *S, cudaStream_t st, int which = 0);
 
 }  // namespace tkh
 

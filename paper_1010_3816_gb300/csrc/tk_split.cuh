@@ -496,6 +496,7 @@ struct SplitRing {
 // per slot the parity of the next wait and of the copies issued.
 struct SplitRingState {
     unsigned cur = 0, wait = 0, issue = 0;
+    bool lost = false;   // a wait gave up
 };
 
 __device__ __forceinline__ void split_ring_init(unsigned long long *bar, int lane)
@@ -508,26 +509,29 @@ __device__ __forceinline__ void split_ring_init(unsigned long long *bar, int lan
     __syncwarp();
 }
 
-// The unsplit tables, for the FP64 instructions alone.
-struct Unsplit {
+// What a sweep rarely needs: the unsplit tables, for the FP64 instructions alone,
+// and the word that is raised when a wait for a copy gives up.
+struct SweepRare {
     const double *h, *n;
+    int *e;
     __device__ __forceinline__ const double *half() const { return h; }
     __device__ __forceinline__ const double *node() const { return n; }
+    __device__ __forceinline__ int *err() const { return e; }
 };
 
-template <int K, class Tables = Unsplit>
+template <int K, class Rare = SweepRare>
 struct SplitSweep {
     SplitRing *ring;
     unsigned long long *bar;   // the warp's two mbarriers, in shared memory (split_ring_init)
     const unsigned char *tab;  // the warp's block of column 0
-    Tables unsplit;
+    Rare rare;
     int Nr;
     double en;
-    int *err;                  // raised when a wait for a copy gives up
 
     // Copy column i's block into a slot; the warp has used its last contents.
     __device__ __forceinline__ void fetch(SplitRingState &st, int slot, int i, int lane) const
     {
+        if (st.lost) return;
         __syncwarp();
         if (lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -536,16 +540,22 @@ struct SplitSweep {
         }
         st.issue ^= 1u << slot;
     }
+    // After a wait that gave up, a warp fetches and waits no more (its results are
+    // then not valid; everything else goes on, so that its team's barriers hold).
     __device__ __forceinline__ void await(SplitRingState &st, int slot) const
     {
-        if (!mbar_wait(&bar[slot], (st.wait >> slot) & 1u) && err) atomicExch(err, 1);
+        const unsigned parity = (st.wait >> slot) & 1u;
+        if (!__all_sync(kFull, mbar_test(&bar[slot], parity))) {
+            if (!st.lost) st.lost = !warp_mbar_wait(&bar[slot], parity, rare);
+            if (st.lost) return;
+        }
         st.wait ^= 1u << slot;
     }
-    // Wait for a copy still in flight (before the block exits).
+    // Wait (with a limit) for the copies still in flight before the block exits.
     __device__ __forceinline__ void drain(SplitRingState &st) const
     {
         for (int s = 0; s < 2; ++s)
-            if (((st.wait ^ st.issue) >> s) & 1u) await(st, s);
+            if (((st.wait ^ st.issue) >> s) & 1u) mbar_wait(&bar[s], (st.wait >> s) & 1u);
     }
 
     // Columns [i0, i1) of one step.  The half node left of i0 is formed here
@@ -600,13 +610,13 @@ struct SplitSweep {
                 await(st, st.cur);
                 const unsigned char *block = ring->tab[st.cur];
                 st.cur ^= 1;
-                split_half_node<K>(a, pa, c, pc, block, team, unsplit.half() + (size_t)i * (kNCH * NP) + row, k1,
+                split_half_node<K>(a, pa, c, pc, block, team, rare.half() + (size_t)i * (kNCH * NP) + row, k1,
                                    hp);
                 split_ints<0>(hp, pp);
                 if (i >= i0) {
                     if (i > 0) {
                         split_full_node<K>(hm, pm, hp, pp, a, block, team,
-                                           unsplit.node() + (size_t)i * (kNCN * NP) + row, en, k1, o);
+                                           rare.node() + (size_t)i * (kNCN * NP) + row, en, k1, o);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) o[k] = 0.0;

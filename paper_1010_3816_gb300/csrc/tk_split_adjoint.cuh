@@ -401,6 +401,7 @@ struct AdjSweep {
 
     __device__ __forceinline__ void fetch(SplitRingState &st, int slot, int i, int lane) const
     {
+        if (st.lost) return;
         __syncwarp();
         if (lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -411,13 +412,17 @@ struct AdjSweep {
     }
     __device__ __forceinline__ void await(SplitRingState &st, int slot) const
     {
-        if (!mbar_wait(&bar[slot], (st.wait >> slot) & 1u) && err) atomicExch(err, 1);
+        const unsigned parity = (st.wait >> slot) & 1u;
+        if (!__all_sync(kFull, mbar_test(&bar[slot], parity))) {
+            if (!st.lost) st.lost = !warp_mbar_wait(&bar[slot], parity, ErrWord{err});
+            if (st.lost) return;
+        }
         st.wait ^= 1u << slot;
     }
     __device__ __forceinline__ void drain(SplitRingState &st) const
     {
         for (int s = 0; s < 2; ++s)
-            if (((st.wait ^ st.issue) >> s) & 1u) await(st, s);
+            if (((st.wait ^ st.issue) >> s) & 1u) mbar_wait(&bar[s], (st.wait >> s) & 1u);
     }
 
     // Columns [i0, i1): as SplitSweep::run, load(i, l) giving lam~ of column i

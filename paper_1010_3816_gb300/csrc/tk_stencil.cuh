@@ -639,14 +639,33 @@ __device__ __forceinline__ bool mbar_test(unsigned long long *bar, unsigned pari
 }
 
 // Polls of a ring slot's mbarrier before the wait gives up (each try_wait
-// itself suspends the warp for a while); a copy of valid memory completes
-// long before.
+// itself suspends the warp for 1.5 us: 6 s); a copy of valid memory completes
+// long before.  Once *err is set (looked at after every 64th poll) it gives up too.
 constexpr long long kMaxMbarPolls = 1ll << 22;
 
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity)
+__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, const int *err = nullptr,
+                                          long long polls = kMaxMbarPolls)
 {
-    for (long long i = 0; i < kMaxMbarPolls; ++i)
+    for (long long i = 0; i < polls; ++i) {
         if (mbar_test(bar, parity)) return true;
+        if ((i & 63) == 63 && err && *(const volatile int *)err != 0) return false;
+    }
+    return false;
+}
+
+// For the whole warp alike; raises *where.err() (looked up where it is needed)
+// where the copy did not come.
+struct ErrWord {
+    int *p;
+    __device__ __forceinline__ int *err() const { return p; }
+};
+
+template <class Where>
+__device__ __forceinline__ bool warp_mbar_wait(unsigned long long *bar, unsigned parity, const Where &where,
+                                               long long polls = kMaxMbarPolls)
+{
+    if (__all_sync(0xffffffffu, mbar_wait(bar, parity, where.err(), polls))) return true;
+    if ((threadIdx.x & 31) == 0) atomicExch(where.err(), 1);
     return false;
 }
 

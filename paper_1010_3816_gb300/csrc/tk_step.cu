@@ -164,7 +164,7 @@ template <typename T, int K, int W>
 __global__ void __launch_bounds__(W * 32, wide_warps<T, K>() / W)
 lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__restrict__ half,
                const T *__restrict__ node, const unsigned char *__restrict__ step, int Nr, T eh, T en,
-               const WaveArgs wa)
+               const WaveArgs wa, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     if (kUsePDL) chain_start();
@@ -175,7 +175,7 @@ lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__res
         split_ring_init(bars[wib], lane);
         SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
         const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib],
-                               step + (wib % K) * kStepBytes, {half, node}, Nr, en, nullptr};
+                               step + (wib % K) * kStepBytes, {half, node, err}, Nr, en};
         int i0, i1;
         team_range<W, K>(Nr, t, &i0, &i1);
         SplitRingState st;
@@ -235,7 +235,8 @@ __device__ __forceinline__ bool neighbour_barrier(unsigned int *flags, unsigned 
 // reads that column.  The progress counters are in shared memory, for a block's
 // first and last team also in global memory (flags[b K + h] and flags[(blocks +
 // b) K + h] for the rows from 32 h).  Every wait is bounded: after kMaxSpins
-// polls the warp sets *err, and from then on every wait returns at once, so this
+// (kMaxMbarPolls) polls the warp sets *err, and from then on every wait for a flag
+// returns at once and one for a table after 64 polls, a warp's last one, so this
 // kernel runs its remaining steps without waiting and the persistent kernels
 // below leave their loops (the state is then invalid and the host reports the
 // error); the barriers of a team are outside this, all its warps run the same
@@ -259,7 +260,7 @@ lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, co
     const int nb = (int)gridDim.x, b = (int)blockIdx.x;
     SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
     const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib], step + h * kStepBytes,
-                           {half, node}, Nr, en, err};
+                           {half, node, err}, Nr, en};
     // The launch has at most Nr / TEAMS blocks, so every team has a column; one
     // without would never publish, and its neighbours' waits would run out.
     int i0, i1;
@@ -362,6 +363,7 @@ lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const 
 #pragma unroll
         for (int k = 0; k < 4; ++k) x[k] = p[(t * 4 + k) * NP + row];
     };
+    bool lost = false;   // the tables did not come
     if (halves) {
         if (lane == 0) {
             mbar_init(&bars[wib]);
@@ -370,7 +372,7 @@ lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const 
             bulk_fetch(sh_raw + wib * kStepBytes, step + ((size_t)col * K + h) * kStepBytes, kStepBytes, &bars[wib]);
         }
         __syncwarp();
-        if (!mbar_wait(&bars[wib], 0)) atomicExch(err, 1);
+        lost = !warp_mbar_wait(&bars[wib], 0, ErrWord{err});
     }
     double a[4];   // column col
     if (owner) {
@@ -425,6 +427,7 @@ lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const 
         }
         __syncthreads();
     }
+    if (lost) mbar_wait(&bars[wib], 0);
     if (wa.write) advance_sample(wa, n_inner / substeps);
 }
 
@@ -434,8 +437,9 @@ lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const 
 // as the edge warps of the one-step sweep do (the warp-level wait on a global
 // flag, err[1]).  `silent` instead waits on a shared-memory counter that
 // nothing sets, as the one-step sweep's warps wait for their siblings (err[2]),
-// and returns without publishing; so all three kinds of wait run out after
-// max_spins polls and set their error words.
+// and for a copy that nothing starts, as they do for their tables (a quarter of the
+// polls, err[3]), and returns without publishing; so all kinds of wait run out
+// after max_spins polls and set their error words.
 __global__ void wait_check_kernel(unsigned int *flags, int *err, int silent, long long max_spins)
 {
     __shared__ unsigned int never;
@@ -443,6 +447,13 @@ __global__ void wait_check_kernel(unsigned int *flags, int *err, int silent, lon
         if (threadIdx.x == 0) never = 0;
         __syncwarp();
         warp_wait_cta(&never, 1u, err + 2, max_spins);
+        __shared__ unsigned long long bar;
+        if (threadIdx.x == 0) {
+            mbar_init(&bar);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        warp_mbar_wait(&bar, 0, ErrWord{err + 3}, max_spins > 4 ? max_spins / 4 : 1);
         return;
     }
     neighbour_barrier(flags, 1u, err, max_spins);
@@ -1083,12 +1094,12 @@ cudaError_t launch_shape(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
     if (!kUsePDL) {
         lw_step_kernel<T, K, W><<<L.blocks, W * 32, step_smem_bytes<T, K, W>(), st>>>(
             (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr,
-            (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
+            (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa, L.err);
         return cudaGetLastError();
     }
     return launch_chained<lw_step_kernel<T, K, W>>(
         (unsigned)L.blocks, W * 32, step_smem_bytes<T, K, W>(), st, (const T *)L.u_in, (T *)L.u_out, (const T *)L.half,
-        (const T *)L.node, L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa);
+        (const T *)L.node, L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa, L.err);
 }
 
 template <typename T, int K, int W>
