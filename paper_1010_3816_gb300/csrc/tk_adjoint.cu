@@ -1026,8 +1026,8 @@ const void *adj_persistent_kernel()
 template <typename T, int K, int W>
 cudaError_t adj_smem_setup()
 {
-    static cudaError_t e = cudaFuncSetAttribute(adj_kernel<T, K, W>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)adj_smem_bytes<T, K, W>());
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, adj_kernel<T, K, W>(), adj_smem_bytes<T, K, W>());
     return e;
 }
 
@@ -1078,8 +1078,8 @@ template <typename T, int K, int W>
 int adj_persistent_blocks_w(int Nr, int num_sms)
 {
     const void *kern = adj_persistent_kernel<T, K, W>();
-    static cudaError_t e0 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)adj_smem_bytes<T, K, W>());
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, kern, adj_smem_bytes<T, K, W>());
     int n = 0;
     if (e0 != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, W * 32, adj_smem_bytes<T, K, W>()) != cudaSuccess ||
@@ -1139,9 +1139,8 @@ template <int K>
 int adj_column_blocks(int Nr, int num_sms)
 {
     int n = 0;
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_adjoint_column_kernel<K>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)sizeof(AdjColumnShared<K>));
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, (const void *)lw_adjoint_column_kernel<K>, sizeof(AdjColumnShared<K>));
     if (e0 != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_adjoint_column_kernel<K>, (kAdjColumns + 1) * K * 32,
                                                       sizeof(AdjColumnShared<K>)) != cudaSuccess)

@@ -4,6 +4,7 @@
 // K*l .. K*l+K-1; u[c][t] is component c (Phi_R, Phi_I, Pi_R, Pi_I) of row K*l+t.
 #pragma once
 
+#include "tk_device_once.h"
 #include "tk_internal.h"
 
 namespace tk {

@@ -1080,9 +1080,8 @@ constexpr size_t step_smem_bytes()
 template <typename T, int K, int W>
 cudaError_t step_smem_setup()
 {
-    static cudaError_t e = cudaFuncSetAttribute(lw_step_kernel<T, K, W>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)step_smem_bytes<T, K, W>());
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, (const void *)lw_step_kernel<T, K, W>, step_smem_bytes<T, K, W>());
     return e;
 }
 
@@ -1105,9 +1104,9 @@ cudaError_t launch_shape(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
 template <typename T, int K, int W>
 cudaError_t ring_smem_setup()
 {
-    static cudaError_t e = cudaFuncSetAttribute(
-        lw_step2_ring_kernel<T, K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)(ring_smem_bytes<T, K>() / ring_warps<T, K>() * W));
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, (const void *)lw_step2_ring_kernel<T, K, W>,
+                                      ring_smem_bytes<T, K>() / ring_warps<T, K>() * W);
     return e;
 }
 
@@ -1230,9 +1229,8 @@ template <int K, int W>
 int persistent_blocks_w(int Nr, int num_sms)
 {
     int n = 0;
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_persistent_kernel<K, W>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)step_smem_bytes<double, K, W>());
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, (const void *)lw_persistent_kernel<K, W>, step_smem_bytes<double, K, W>());
     if (e0 != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_persistent_kernel<K, W>, W * 32,
                                                       step_smem_bytes<double, K, W>()) != cudaSuccess ||
@@ -1257,8 +1255,8 @@ template <int K, int T>
 int column_blocks_t(int Nr, int num_sms)
 {
     int n = 0;
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_column_kernel<K, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)column_smem_bytes<K, T>());
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, (const void *)lw_column_kernel<K, T>, column_smem_bytes<K, T>());
     if (e0 != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lw_column_kernel<K, T>, column_warps<K, T>() * 32,
                                                       column_smem_bytes<K, T>()) != cudaSuccess)
@@ -1328,9 +1326,9 @@ cudaError_t launch_ring_persistent_w(const StepLaunch &L, void *u_other, int n_p
 {
     cudaError_t e = ring_smem_setup<T, K, W>();
     if (e != cudaSuccess) return e;
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_ring_persistent_kernel<T, K, W>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(ring_smem_bytes<T, K>() / ring_warps<T, K>() * W));
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, (const void *)lw_ring_persistent_kernel<T, K, W>,
+                                      ring_smem_bytes<T, K>() / ring_warps<T, K>() * W);
     if (e0 != cudaSuccess) return e0;
     WaveArgs wa;
     wa.write = L.write_wave;
@@ -1379,8 +1377,8 @@ cudaError_t launch_multi_persistent_w(const StepLaunch &L, void *u_other, int n_
                                       unsigned int *flags, int *err, void *scratch, cudaStream_t st)
 {
     constexpr size_t smem = multi_smem_bytes<K, W, kSweepLevels>();
-    static cudaError_t e0 = cudaFuncSetAttribute(lw_multi_persistent_kernel<T, K, W, kSweepLevels>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, (const void *)lw_multi_persistent_kernel<T, K, W, kSweepLevels>, smem);
     if (e0 != cudaSuccess) return e0;
     if (!L.cmp || !L.gpm) return cudaErrorInvalidValue;
     WaveArgs wa;
