@@ -81,7 +81,11 @@ enum {
  *   angular_variable        TK_VAR_LITERAL or TK_VAR_REGULARISED
  *   precision               TK_PREC_F64 or TK_PREC_F32
  *   cuda_stream             cudaStream_t to run on (NULL: the legacy default stream)
- * Allocates the device state (two time levels) and nothing else yet.
+ * Allocates the device state (two time levels) and the coefficient tables, per
+ * point 240 bytes in FP64 and 180 more for the step's split tables.  Where
+ * the memory does not reach for these (here or in a later call), the solver runs
+ * on the plain tables alone: the same results but for roundings, at the speed of
+ * the FP64 instructions.
  * Returns TK_ERR_ARG on a bad size, TK_ERR_OOM if allocation fails. */
 tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int Nr, int Ntheta,
                        double dt, int substeps, int angular_variable, int precision,

@@ -30,6 +30,10 @@
 #include "tk_stencil.cuh"
 
 namespace tk {
+
+int adj_block_bytes() { return kAdjBytes; }
+int adj_block_head() { return kAdjHead; }
+
 namespace {
 
 struct InjectArgs {
@@ -559,8 +563,8 @@ __device__ __forceinline__ void store_row(double *__restrict__ u, int i, int row
 template <int K, int W>
 __global__ void __launch_bounds__(W * 32, adj_wide_warps<double, K>() / W)
 lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_out, const double *__restrict__ half,
-                       const double *__restrict__ node, const unsigned char *__restrict__ tab, int Nr, double en,
-                       const InjectArgs inj, int *err)
+                       const double *__restrict__ node, const unsigned char *__restrict__ tab, size_t pitch, int Nr,
+                       double en, const InjectArgs inj, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned long long bars[W][2];
@@ -570,7 +574,7 @@ lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_o
     split_ring_init(bars[wib], lane);
     AdjTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
-                         en, err};
+                         en, err, pitch};
     int i0, i1;
     team_range<W, K>(Nr, t, &i0, &i1);
     SplitRingState st;
@@ -589,8 +593,8 @@ lw_adjoint_team_kernel(const double *__restrict__ lam, double *__restrict__ mu_o
 template <int K, int W>
 __global__ void __launch_bounds__(W * 32, adj_wide_warps<double, K>() / W)
 lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restrict__ half,
-                                  const double *__restrict__ node, const unsigned char *__restrict__ tab, int Nr,
-                                  double en, const InjectArgs inj, int inject, long long n_inner, int substeps,
+                                  const double *__restrict__ node, const unsigned char *__restrict__ tab, size_t pitch,
+                                  int Nr, double en, const InjectArgs inj, int inject, long long n_inner, int substeps,
                                   unsigned int *flags, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
@@ -605,7 +609,7 @@ lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restri
     const int nb = (int)gridDim.x, b = (int)blockIdx.x;
     AdjTeam<K> team{rows + t * K, h, lane, 1 + t};
     const AdjSweep<K> sw{reinterpret_cast<AdjRing *>(sh_raw) + wib, bars[wib], tab + h * kAdjBytes, half, node, Nr,
-                         en, err};
+                         en, err, pitch};
     int i0, i1;
     team_range<W, K>(Nr, t, &i0, &i1);   // at most Nr / TEAMS blocks: every team has a column
     SplitRingState st;
@@ -665,7 +669,8 @@ struct AdjColumnShared {
 template <int K>
 __global__ void __launch_bounds__((kAdjColumns + 1) * K * 32, 4 / K)
 lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half, const double *__restrict__ node,
-                         const unsigned char *__restrict__ tab, int Nr, double en, const InjectArgs inj, int inject,
+                         const unsigned char *__restrict__ tab, size_t pitch, int Nr, double en,
+                         const InjectArgs inj, int inject,
                          long long n_inner, int substeps, unsigned int *flags, int *err, long long first,
                          size_t stride)
 {
@@ -712,8 +717,8 @@ lw_adjoint_column_kernel(double *a0, double *a1, const double *__restrict__ half
             mbar_init(bar);
             mbar_init_fence();
             mbar_expect(bar, ((halves ? 1 : 0) + (extra ? 1 : 0)) * kAdjBytes);
-            if (halves) bulk_fetch(sh.tab[j + 1][h], tab + ((size_t)col * K + h) * kAdjBytes, kAdjBytes, bar);
-            if (extra) bulk_fetch(sh.tab[0][h], tab + ((size_t)(col - 1) * K + h) * kAdjBytes, kAdjBytes, bar);
+            if (halves) bulk_fetch(sh.tab[j + 1][h], tab + col * pitch + h * kAdjBytes, kAdjBytes, bar);
+            if (extra) bulk_fetch(sh.tab[0][h], tab + (col - 1) * pitch + h * kAdjBytes, kAdjBytes, bar);
         }
         __syncwarp();
         lost = !warp_mbar_wait(&sh.bars[wib], 0, ErrWord{err});
@@ -1002,6 +1007,12 @@ cudaError_t launch_param_tangent(int K, int blocks, int steps, const double *u_l
     return cudaGetLastError();
 }
 
+// The FP64 tables and the bytes from a column's to the next's (0: one cold block).
+struct AdjTables {
+    const unsigned char *p;
+    size_t pitch;
+};
+
 template <typename T, int K, int W>
 constexpr size_t adj_smem_bytes()
 {
@@ -1032,7 +1043,7 @@ cudaError_t adj_smem_setup()
 }
 
 template <typename T, int K, int W>
-cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab,
+cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const void *node, AdjTables tab,
                              int Nr, int blocks, double dt_in, const InjectArgs &inj, int *err,
                              cudaStream_t st)
 {
@@ -1041,7 +1052,7 @@ cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const 
     if constexpr (sizeof(T) == 8)
         return launch_chained<lw_adjoint_team_kernel<K, W>>(
             (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const double *)lam, (double *)mu,
-            (const double *)half, (const double *)node, tab, Nr, 0.5 * dt_in, inj, err);
+            (const double *)half, (const double *)node, tab.p, tab.pitch, Nr, 0.5 * dt_in, inj, err);
     else
         return launch_chained<lw_adjoint_kernel<T, K, W>>(
             (unsigned)blocks, W * 32, adj_smem_bytes<T, K, W>(), st, (const T *)lam, (T *)mu, (const T *)half,
@@ -1049,7 +1060,7 @@ cudaError_t launch_adj_shape(const void *lam, void *mu, const void *half, const 
 }
 
 template <typename T, int K>
-cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *node, const unsigned char *tab, int Nr,
+cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *node, AdjTables tab, int Nr,
                        int blocks, int warps, double dt_in, const InjectArgs &inj, int *err, cudaStream_t st)
 {
     constexpr int WW = adj_wide_warps<T, K>();
@@ -1061,7 +1072,7 @@ cudaError_t launch_adj(const void *lam, void *mu, const void *half, const void *
 }
 
 cudaError_t launch_adjoint_step(int precision, int K, const void *lam, void *mu, const void *half,
-                                const void *node, const unsigned char *tab, int Nr, int blocks, int warps, double dt_in,
+                                const void *node, AdjTables tab, int Nr, int blocks, int warps, double dt_in,
                                 const InjectArgs &inj, int *err, cudaStream_t st)
 {
     if (precision == 0) {
@@ -1102,7 +1113,7 @@ int adj_persistent_blocks_t(int Nr, int num_sms, int warps)
 
 template <typename T, int K, int W>
 cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const void *node,
-                                    const unsigned char *tab, int Nr, int blocks,
+                                    AdjTables tab, int Nr, int blocks,
                                     double dt_in, const InjectArgs &inj, int inject, long long n_inner,
                                     int substeps, unsigned int *flags, int *err, cudaStream_t st)
 {
@@ -1110,7 +1121,7 @@ cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const 
     const T *h = (const T *)half, *nd = (const T *)node;
     T en = (T)(0.5 * dt_in);
     InjectArgs in = inj;
-    void *args64[] = {&p0, &p1, &h, &nd, &tab, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
+    void *args64[] = {&p0, &p1, &h, &nd, &tab.p, &tab.pitch, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
     void *args32[] = {&p0, &p1, &h, &nd, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err};
     return cudaLaunchCooperativeKernel(adj_persistent_kernel<T, K, W>(), dim3(blocks), dim3(W * 32),
                                        sizeof(T) == 8 ? args64 : args32, adj_smem_bytes<T, K, W>(), st);
@@ -1118,7 +1129,7 @@ cudaError_t launch_adj_persistent_w(void *a0, void *a1, const void *half, const 
 
 template <typename T, int K>
 cudaError_t launch_adj_persistent_t(void *a0, void *a1, const void *half, const void *node,
-                                    const unsigned char *tab, int Nr, int blocks,
+                                    AdjTables tab, int Nr, int blocks,
                                     int warps, double dt_in, const InjectArgs &inj, int inject,
                                     long long n_inner, int substeps, unsigned int *flags, int *err,
                                     cudaStream_t st)
@@ -1158,7 +1169,7 @@ int adjoint_column_blocks(int precision, int K, int Nr, int num_sms)
 }
 
 template <int K>
-cudaError_t launch_adj_columns(double *a0, double *a1, const void *half, const void *node, const unsigned char *tab,
+cudaError_t launch_adj_columns(double *a0, double *a1, const void *half, const void *node, AdjTables tab,
                                int Nr, int blocks, double dt_in, const InjectArgs &inj, int inject, long long n_inner,
                                int substeps, unsigned int *flags, int *err, long long first, size_t stride,
                                cudaStream_t st)
@@ -1166,13 +1177,14 @@ cudaError_t launch_adj_columns(double *a0, double *a1, const void *half, const v
     const double *h = (const double *)half, *nd = (const double *)node;
     double en = 0.5 * dt_in;
     InjectArgs in = inj;
-    void *args[] = {&a0, &a1, &h, &nd, &tab, &Nr, &en, &in, &inject, &n_inner, &substeps, &flags, &err, &first, &stride};
+    void *args[] = {&a0,     &a1,      &h,        &nd,    &tab.p, &tab.pitch, &Nr,    &en, &in,
+                    &inject, &n_inner, &substeps, &flags, &err,   &first,     &stride};
     return cudaLaunchCooperativeKernel((const void *)lw_adjoint_column_kernel<K>, dim3(blocks),
                                        dim3((kAdjColumns + 1) * K * 32), args, sizeof(AdjColumnShared<K>), st);
 }
 
 cudaError_t launch_adjoint_columns(int K, double *a0, double *a1, const void *half, const void *node,
-                                   const unsigned char *tab, int Nr, int blocks, double dt_in, const InjectArgs &inj,
+                                   AdjTables tab, int Nr, int blocks, double dt_in, const InjectArgs &inj,
                                    int inject, long long n_inner, int substeps, unsigned int *flags, int *err,
                                    long long first, size_t stride, cudaStream_t st)
 {
@@ -1197,7 +1209,7 @@ int adjoint_persistent_blocks(int precision, int K, int Nr, int num_sms, int war
 }
 
 cudaError_t launch_adjoint_persistent(int precision, int K, void *a0, void *a1, const void *half,
-                                      const void *node, const unsigned char *tab, int Nr, int blocks, int warps, double dt_in,
+                                      const void *node, AdjTables tab, int Nr, int blocks, int warps, double dt_in,
                                       const InjectArgs &inj, int inject, long long n_inner, int substeps,
                                       unsigned int *flags, int *err, cudaStream_t st)
 {
@@ -1269,9 +1281,14 @@ static tk_status adjoint_tables(tk_solver *S)
 {
     if (S->precision != TK_PREC_F64 || S->adj_tab_of == S->coeffs_id) return TK_OK;
     if (!S->adj_tab) {
-        tk_status st = tkh::alloc(S, (void **)&S->adj_tab, (size_t)S->Nr * S->K * tk::kAdjBytes);
-        if (st != TK_OK) return st;
+        if (tkh::alloc(S, (void **)&S->adj_tab, (size_t)S->Nr * S->K * tk::kAdjBytes, true) == TK_OK)
+            S->adj_pitch = S->K * tk::kAdjBytes;
+        else if (tkh::cold_tables(S))
+            S->adj_tab = S->cold + (size_t)S->K * tk::kStepBytes;
+        else
+            return TK_ERR_OOM;
     }
+    if (S->adj_pitch == 0) return TK_OK;
     const dim3 block(S->NP, tk::kAdjTableThreads / S->NP), grid((S->Nr + block.y - 1) / block.y);
     tk::adj_tables_kernel<<<grid, block, 0, S->stream>>>(S->Nr, S->NP, (const double *)S->half,
                                                          (const double *)S->node, S->adj_tab);
@@ -1279,6 +1296,8 @@ static tk_status adjoint_tables(tk_solver *S)
     S->adj_tab_of = S->coeffs_id;
     return TK_OK;
 }
+
+static tk::AdjTables tables_of(const tk_solver *S) { return {S->adj_tab, S->adj_pitch}; }
 
 extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const double *dL_dfinal,
                                 int on_device, double *grad, int grad_on_device, int independent_pi)
@@ -1375,12 +1394,12 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
         int herr = 0;
         e = cudaMemsetAsync(flags, 0, fbytes, S->stream);
         if (e == cudaSuccess && cblocks > 0)
-            e = tk::launch_adjoint_columns(S->K, (double *)S->adj[0], (double *)S->adj[1], S->half, S->node, S->adj_tab,
+            e = tk::launch_adjoint_columns(S->K, (double *)S->adj[0], (double *)S->adj[1], S->half, S->node, tables_of(S),
                                            S->Nr, cblocks, dt_in, inj, dwave != nullptr, n_inner, S->substeps, flags,
                                            derr, 0, 0, S->stream);
         else if (e == cudaSuccess)
-            e = tk::launch_adjoint_persistent(S->precision, S->K, S->adj[0], S->adj[1], S->half, S->node, S->adj_tab, S->Nr,
-                                              pblocks, S->adj_warps, dt_in, inj, dwave != nullptr, n_inner,
+            e = tk::launch_adjoint_persistent(S->precision, S->K, S->adj[0], S->adj[1], S->half, S->node, tables_of(S),
+                                              S->Nr, pblocks, S->adj_warps, dt_in, inj, dwave != nullptr, n_inner,
                                               S->substeps, flags, derr, S->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, S->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(S->stream);
@@ -1397,7 +1416,7 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
                 inj.on = (k == 0) && dwave != nullptr;
                 inj.sample = t;
                 e = tk::launch_adjoint_step(S->precision, S->K, S->adj[cur], S->adj[cur ^ 1], S->half,
-                                            S->node, S->adj_tab, S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj,
+                                            S->node, tables_of(S), S->Nr, S->adj_blocks, S->adj_warps, dt_in, inj,
                                             S->lost + 1, S->stream);
                 cur ^= 1;
             }
@@ -1509,7 +1528,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
             {&acc, (size_t)(blocks + pblocks)}, {&parts, (size_t)Q * blocks}, {&pflags, 1 + (nflags + 1) / 2}};
         size_t total = 0;
         for (auto &x : piece) total += (x.n + 31) / 32 * 32;
-        st = tkh::alloc(S, (void **)&scratch, total * sizeof(double));
+        st = tkh::alloc(S, (void **)&scratch, total * sizeof(double), Q > 1 || cblocks);
         if (st == TK_OK) {
             double *at = scratch;
             for (auto &x : piece) {
@@ -1621,7 +1640,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
                 for (int q = 0; q < n; ++q) set.p[q] = lam[q];
                 e = cudaMemsetAsync(flags, 0, nflags * sizeof(unsigned int), S->stream);
                 if (e == cudaSuccess)
-                    e = tk::launch_adjoint_columns(S->K, lam[0], lam[1], S->half, S->node, S->adj_tab, S->Nr, cblocks,
+                    e = tk::launch_adjoint_columns(S->K, lam[0], lam[1], S->half, S->node, tables_of(S), S->Nr, cblocks,
                                                    dt_in, inj, 1, n, k, flags, perr,
                                                    (count - t0 - len) * k + g, se, S->stream);
             }
@@ -1630,7 +1649,7 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
                 set.p[q] = lam[cur];
                 inj.on = (g + q) % k == 0;
                 inj.sample = t0 + len - 1 - (g + q) / k;
-                e = tk::launch_adjoint_step(0, S->K, lam[cur], lam[nxt], S->half, S->node, S->adj_tab, S->Nr,
+                e = tk::launch_adjoint_step(0, S->K, lam[cur], lam[nxt], S->half, S->node, tables_of(S), S->Nr,
                                             S->adj_blocks, S->adj_warps, dt_in, inj, perr, S->stream);
                 cur = nxt;
             }

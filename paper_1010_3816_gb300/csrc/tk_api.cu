@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include <new>
+#include <vector>
 
 #include "tk_solver_impl.h"
 
@@ -31,9 +32,57 @@ tk_status fail(tk_solver *S, tk_status st, const char *fmt, ...)
 
 size_t state_elems(const tk_solver *S) { return (size_t)S->Nr * 4 * S->NP; }
 
-tk_status alloc(tk_solver *S, void **p, size_t bytes)
+// (allocated where it is needed: a few KB more among the small allocations of six
+// solvers cost their batch 4 % of a tick)
+bool cold_tables(tk_solver *S)
+{
+    if (S->cold) return true;
+    const size_t sb = tk::kStepBytes, ab = tk::adj_block_bytes();
+    std::vector<unsigned char> h(S->K * (sb + ab), 0);
+    for (int k = 0; k < S->K; ++k) {
+        h[k * sb + tk::kStepHead] = 1;
+        h[S->K * sb + k * ab + tk::adj_block_head()] = 1;
+    }
+    if (cudaMalloc((void **)&S->cold, h.size()) == cudaSuccess &&
+        cudaMemcpy(S->cold, h.data(), h.size(), cudaMemcpyHostToDevice) == cudaSuccess)
+        return true;
+    if (S->cold) cudaFree(S->cold);
+    S->cold = nullptr;
+    cudaGetLastError();
+    return false;
+}
+
+bool give_up_tables(tk_solver *S)
+{
+    if (!S || (S->step_pitch == 0 && S->adj_pitch == 0)) return false;
+    cudaDeviceSynchronize();   // no launch reads them any more
+    if (S->step_pitch) {
+        cudaFree(S->step);
+        S->step = nullptr;
+        S->step_pitch = 0;
+    }
+    if (S->adj_pitch) {
+        cudaFree(S->adj_tab);
+        S->adj_tab = nullptr;
+        S->adj_pitch = 0;
+    }
+    S->epoch++;   // graphs hold the pointer
+    if (!cold_tables(S)) {   // nothing to step with
+        S->have_coeffs = S->have_state = false;
+        return false;
+    }
+    S->step = S->cold;
+    S->adj_tab = S->cold + (size_t)S->K * tk::kStepBytes;
+    return true;
+}
+
+tk_status alloc(tk_solver *S, void **p, size_t bytes, bool keep_tables)
 {
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && !keep_tables) {
+        cudaGetLastError();
+        if (give_up_tables(S)) e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
@@ -47,7 +96,8 @@ void release(tk_solver *S)
     void *ptrs[] = {S->u[0], S->u[1], S->half, S->node, S->b_node, S->w_row,
                     S->rad, S->ang, S->staging, S->flag, S->stiff, S->ctr, S->wave,
                     S->adj[0], S->adj[1], S->u_init, S->dhalf, S->dnode, S->db_node, S->pflags,
-                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step, S->adj_tab, S->lost};
+                    S->obs_scr, S->xbuf, S->cmp, S->gpm, S->step_pitch ? S->step : nullptr,
+                    S->adj_pitch ? S->adj_tab : nullptr, S->cold, S->lost};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (int k = 0; k < 2; ++k)
@@ -160,6 +210,7 @@ void fill_launch(const tk_solver *S, tk::StepLaunch &L)
     L.cmp = S->cmp;
     L.gpm = S->gpm;
     L.step = S->step;
+    L.pitch = S->step_pitch;
     L.err = S->lost;
     L.wave_cap = S->wave_cap;
     L.wave = S->wave;
@@ -275,8 +326,6 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     if (st == TK_OK) st = alloc(S, &S->u[1], se * S->esz);
     if (st == TK_OK) st = alloc(S, &S->half, (size_t)Nr * tk::kNCH * S->NP * S->esz);
     if (st == TK_OK) st = alloc(S, &S->node, (size_t)Nr * tk::kNCN * S->NP * S->esz);
-    if (st == TK_OK && precision == TK_PREC_F64)
-        st = alloc(S, (void **)&S->step, (size_t)Nr * S->K * tk::kStepBytes);
     if (st == TK_OK && precision == TK_PREC_F32)
         st = alloc(S, (void **)&S->cmp, (size_t)Nr * tk::kNCC * S->NP * sizeof(float));
     if (st == TK_OK && precision == TK_PREC_F32)
@@ -289,6 +338,15 @@ tk_status tk_make_grid(tk_solver **out, double rstar_min, double rstar_max, int 
     if (st == TK_OK) st = alloc(S, (void **)&S->stiff, 2 * sizeof(unsigned long long));
     if (st == TK_OK) st = alloc(S, (void **)&S->ctr, 2 * sizeof(long long));
     if (st == TK_OK) st = alloc(S, (void **)&S->lost, 2 * sizeof(int));
+    if (st == TK_OK && precision == TK_PREC_F64) {   // last: the rest of the grid comes first
+        st = alloc(S, (void **)&S->step, (size_t)Nr * S->K * tk::kStepBytes, true);
+        if (st == TK_OK) {
+            S->step_pitch = S->K * tk::kStepBytes;
+        } else if (st == TK_ERR_OOM && tkh::cold_tables(S)) {
+            S->step = S->cold;
+            st = TK_OK;
+        }
+    }
     if (st != TK_OK) {
         snprintf(g_err, sizeof g_err, "%s", S->err);
         release(S);
@@ -327,7 +385,8 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
     TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                        S->dt / S->substeps, S->rad, S->ang,
                                        S->precision, S->half, S->node, S->b_node, S->w_row,
-                                       S->cmp, S->gpm, S->stream, nullptr, nullptr, S->step));
+                                       S->cmp, S->gpm, S->stream, nullptr, nullptr,
+                                       S->step_pitch ? S->step : nullptr));
     S->have_coeffs = true;
     S->have_state = false;
     S->coeffs_id++;
@@ -348,7 +407,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
                                                S->dt / S->substeps, S->rad, S->ang,
                                                S->precision, S->half, S->node, S->b_node,
                                                S->w_row, S->cmp, S->gpm, S->stream, nullptr, nullptr,
-                                               S->step));
+                                               S->step_pitch ? S->step : nullptr));
         }
     }
     return TK_OK;
@@ -402,7 +461,7 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
     if (e == cudaSuccess)
         e = tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs, S->dt / S->substeps,
                                     S->rad, S->ang, S->precision, S->half, S->node, S->b_node,
-                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, S->step);
+                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, S->step_pitch ? S->step : nullptr);
     if (e == cudaSuccess && dev) e = cudaStreamSynchronize(S->stream);
     if (dev) cudaFree(dev);
     if (e != cudaSuccess) return fail(S, TK_ERR_CUDA, "tk_set_coefficients: %s", cudaGetErrorString(e));

@@ -35,6 +35,7 @@ struct BatchMember {
     void *u0, *u1;            // the member's two time levels
     const void *half, *node;  // folded coefficient tables
     const unsigned char *step;   // FP64: the step's tables
+    size_t pitch;             // (StepLaunch)
     int *err;                 // raised where a copy of them did not come
     int Nr, K;
     int substeps, ratio;      // k_i and kmax / k_i
@@ -103,6 +104,7 @@ struct MemberRare {
     __device__ __forceinline__ const double *half() const { return (const double *)m->half; }
     __device__ __forceinline__ const double *node() const { return (const double *)m->node; }
     __device__ __forceinline__ int *err() const { return m->err; }
+    __device__ __forceinline__ size_t pitch() const { return m->pitch; }
 };
 
 // The block's share of an FP64 item: its teams take equal parts of the columns.
@@ -366,6 +368,7 @@ tk_status upload_members(tk_batch *B)
         tkh::fill_launch(S, L);
         m.obs = L.obs;
         m.step = L.step;
+        m.pitch = L.pitch;
         m.err = L.err;
     }
     TKB_CUDA(B, cudaMemcpyAsync(B->d_mem, h.data(), B->n * sizeof(tk::BatchMember),

@@ -99,6 +99,10 @@ constexpr int kLiftSpread = 6;          // largest difference of the lifts that 
 constexpr int kSplitMaxClass = 20;      // largest class exponent; larger tables are cold
 constexpr int kSplitMaxExp = 1900;      // columns with this exponent field or more are cold
 
+// Of the adjoint's blocks: their size, and where a block's flags are.
+int adj_block_bytes();
+int adj_block_head();
+
 struct Kerr {
     double M, a;  // black-hole mass and spin
     int s, m;     // spin weight, azimuthal mode
@@ -225,6 +229,7 @@ struct StepLaunch {
     const float *cmp;     // FP32: compact tables [i][kNCC][jp] (the four-step sweep)
     const float *gpm;     // FP32: theta factors gp[NP], gm[NP]
     const unsigned char *step;   // FP64: the step's tables
+    size_t pitch;         // bytes from a column's to the next's (0: one cold block for all)
     int *err;             // one-step launch: raised where a copy of tables did not come
     // waveform (only on the last inner step of an outer step)
     int write_wave;

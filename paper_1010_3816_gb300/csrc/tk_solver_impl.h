@@ -20,7 +20,13 @@ struct tk_solver {
     int cur = 0;
     void *half = nullptr, *node = nullptr;
     float *cmp = nullptr, *gpm = nullptr;   // FP32: compact tables, theta factors (tk_internal.h)
-    unsigned char *step = nullptr;   // FP64: the step's tables (tk_internal.h)
+    // FP64: the step's tables (tk_internal.h) and the bytes from a column's blocks to
+    // the next's.  Where the memory does not reach for them (or for anything else
+    // while they hold it), one column of cold blocks stands for all, pitch 0: every
+    // column then takes the FP64 instructions and the unsplit tables alone.
+    unsigned char *step = nullptr;
+    size_t step_pitch = 0;
+    unsigned char *cold = nullptr;   // [K] of the step's blocks, [K] of the adjoint's
     double *b_node = nullptr, *w_row = nullptr;
     double *rad = nullptr;      // radial parts of the coefficients (tk_internal.h)
     double *ang = nullptr;      // regularised angular stencil [2][NP]
@@ -29,6 +35,7 @@ struct tk_solver {
     unsigned long long *stiff = nullptr;  // [max omega^2, max b] as double bit patterns
     long long *ctr = nullptr;   // [0]: sample index of the next outer step, [1]: blocks done
     unsigned char *adj_tab = nullptr;   // FP64 adjoint: its tables, allocated and formed on use
+    size_t adj_pitch = 0;               // as step_pitch
     long long coeffs_id = 0, adj_tab_of = -1;   // which coefficients are set, which adj_tab was formed from
     void *adj[2] = {nullptr, nullptr};  // adjoint state levels (tk_adjoint), allocated on use
     // parameter gradients (tk_param_gradient): u^0 and the derivative tables
@@ -92,7 +99,12 @@ namespace tkh {
 
 // Record a one-line message on the solver (or thread-locally if S is NULL).
 tk_status fail(tk_solver *S, tk_status st, const char *fmt, ...);
-tk_status alloc(tk_solver *S, void **p, size_t bytes);
+// Where the memory does not reach, the solver's split tables are given up for it
+// (not with keep_tables).
+tk_status alloc(tk_solver *S, void **p, size_t bytes, bool keep_tables = false);
+// False if there was nothing to give up, or not even room for the cold blocks.
+bool give_up_tables(tk_solver *S);
+bool cold_tables(tk_solver *S);   // S->cold is there
 tk_status ensure_wave(tk_solver *S, int64_t need);
 tk_status enter(tk_solver *S);
 void fill_launch(const tk_solver *S, tk::StepLaunch &L);

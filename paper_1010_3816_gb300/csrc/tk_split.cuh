@@ -510,13 +510,17 @@ __device__ __forceinline__ void split_ring_init(unsigned long long *bar, int lan
 }
 
 // What a sweep rarely needs: the unsplit tables, for the FP64 instructions alone,
-// and the word that is raised when a wait for a copy gives up.
+// the word that is raised when a wait for a copy gives up, and (one lane, once a
+// column) the bytes from a column's blocks to the next's: 0 where one cold block
+// stands for all of them.
 struct SweepRare {
     const double *h, *n;
     int *e;
+    size_t p;
     __device__ __forceinline__ const double *half() const { return h; }
     __device__ __forceinline__ const double *node() const { return n; }
     __device__ __forceinline__ int *err() const { return e; }
+    __device__ __forceinline__ size_t pitch() const { return p; }
 };
 
 template <int K, class Rare = SweepRare>
@@ -536,7 +540,7 @@ struct SplitSweep {
         if (lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_expect(&bar[slot], kStepBytes);
-            bulk_fetch(ring->tab[slot], tab + (size_t)i * (K * kStepBytes), kStepBytes, &bar[slot]);
+            bulk_fetch(ring->tab[slot], tab + (size_t)i * rare.pitch(), kStepBytes, &bar[slot]);
         }
         st.issue ^= 1u << slot;
     }

@@ -398,6 +398,7 @@ struct AdjSweep {
     int Nr;
     double E;                   // dt/2
     int *err;
+    size_t pitch;               // bytes from a column's blocks to the next's, 0: one for all
 
     __device__ __forceinline__ void fetch(SplitRingState &st, int slot, int i, int lane) const
     {
@@ -406,7 +407,7 @@ struct AdjSweep {
         if (lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_expect(&bar[slot], kAdjBytes);
-            bulk_fetch(ring->tab[slot], tab + (size_t)i * (K * kAdjBytes), kAdjBytes, &bar[slot]);
+            bulk_fetch(ring->tab[slot], tab + (size_t)i * pitch, kAdjBytes, &bar[slot]);
         }
         st.issue ^= 1u << slot;
     }
@@ -449,7 +450,7 @@ struct AdjSweep {
         adj_zero(sa);
         adj_zero(sm);
         if (ib > 0) {
-            const unsigned char *block = tab + (size_t)(ib - 1) * (K * kAdjBytes);
+            const unsigned char *block = tab + (size_t)(ib - 1) * pitch;
             const AdjTab<false> t{block, lane};
             AdjSums s2;
             hot_a = adj_pair<K, false>(a, t, t.head(), team, sa, s2);

@@ -163,7 +163,7 @@ __device__ __forceinline__ void step_sweep(unsigned char *sh_raw, const T *__res
 template <typename T, int K, int W>
 __global__ void __launch_bounds__(W * 32, wide_warps<T, K>() / W)
 lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__restrict__ half,
-               const T *__restrict__ node, const unsigned char *__restrict__ step, int Nr, T eh, T en,
+               const T *__restrict__ node, const unsigned char *__restrict__ step, size_t pitch, int Nr, T eh, T en,
                const WaveArgs wa, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
@@ -175,7 +175,7 @@ lw_step_kernel(const T *__restrict__ u_in, T *__restrict__ u_out, const T *__res
         split_ring_init(bars[wib], lane);
         SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
         const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib],
-                               step + (wib % K) * kStepBytes, {half, node, err}, Nr, en};
+                               step + (wib % K) * kStepBytes, {half, node, err, pitch}, Nr, en};
         int i0, i1;
         team_range<W, K>(Nr, t, &i0, &i1);
         SplitRingState st;
@@ -245,8 +245,8 @@ __device__ __forceinline__ bool neighbour_barrier(unsigned int *flags, unsigned 
 template <int K, int W>
 __global__ void __launch_bounds__(W * 32, wide_warps<double, K>() / W)
 lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, const double *__restrict__ node,
-                     const unsigned char *__restrict__ step, int Nr, double en, const WaveArgs wa, int n_inner,
-                     int substeps, unsigned int *flags, int *err)
+                     const unsigned char *__restrict__ step, size_t pitch, int Nr, double en, const WaveArgs wa,
+                     int n_inner, int substeps, unsigned int *flags, int *err)
 {
     extern __shared__ __align__(16) unsigned char sh_raw[];
     __shared__ unsigned int step_done[W];
@@ -260,7 +260,7 @@ lw_persistent_kernel(double *u0, double *u1, const double *__restrict__ half, co
     const int nb = (int)gridDim.x, b = (int)blockIdx.x;
     SplitTeam<K> team{rows + t * K, h, lane, 1 + t};
     const SplitSweep<K> sw{reinterpret_cast<SplitRing *>(sh_raw) + wib, bars[wib], step + h * kStepBytes,
-                           {half, node, err}, Nr, en};
+                           {half, node, err, pitch}, Nr, en};
     // The launch has at most Nr / TEAMS blocks, so every team has a column; one
     // without would never publish, and its neighbours' waits would run out.
     int i0, i1;
@@ -335,8 +335,8 @@ constexpr size_t column_smem_bytes()
 template <int K, int T>
 __global__ void __launch_bounds__(column_warps<K, T>() * 32, 16 / column_warps<K, T>())
 lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const double *__restrict__ node,
-                 const unsigned char *__restrict__ step, int Nr, double en, const WaveArgs wa, int n_inner,
-                 int substeps, unsigned int *flags, int *err, size_t stride)
+                 const unsigned char *__restrict__ step, size_t pitch, int Nr, double en, const WaveArgs wa,
+                 int n_inner, int substeps, unsigned int *flags, int *err, size_t stride)
 {
     constexpr int W = (T + 1) * K, NP = 32 * K;
     extern __shared__ __align__(16) unsigned char sh_raw[];
@@ -369,7 +369,7 @@ lw_column_kernel(double *u0, double *u1, const double *__restrict__ half, const 
             mbar_init(&bars[wib]);
             mbar_init_fence();
             mbar_expect(&bars[wib], kStepBytes);
-            bulk_fetch(sh_raw + wib * kStepBytes, step + ((size_t)col * K + h) * kStepBytes, kStepBytes, &bars[wib]);
+            bulk_fetch(sh_raw + wib * kStepBytes, step + col * pitch + h * kStepBytes, kStepBytes, &bars[wib]);
         }
         __syncwarp();
         lost = !warp_mbar_wait(&bars[wib], 0, ErrWord{err});
@@ -483,8 +483,8 @@ constexpr int fused_warps()
 template <int K, int W>
 __global__ void __launch_bounds__(W * 32, fused_warps<double, K>() / W)
 lw_step2_kernel(const double *__restrict__ u_in, double *__restrict__ u_out, const double *__restrict__ half,
-                const double *__restrict__ node, const unsigned char *__restrict__ step, int Nr, double en,
-                const WaveArgs wa, int obs_mask)
+                const double *__restrict__ node, const unsigned char *__restrict__ step, size_t pitch, int Nr,
+                double en, const WaveArgs wa, int obs_mask)
 {
     constexpr int NP = 32 * K;
     __shared__ SplitRows rows[W];
@@ -500,7 +500,7 @@ lw_step2_kernel(const double *__restrict__ u_in, double *__restrict__ u_out, con
         for (int k = 0; k < 4; ++k) x[k] = 0.0;
     };
     // the half node between columns i and i + 1, the node i, their tables read from global memory
-    auto block = [&](int i) { return step + ((size_t)i * K + team.h) * kStepBytes; };
+    auto block = [&](int i) { return step + i * pitch + team.h * kStepBytes; };
     auto half_at = [&](int i, const double (&x)[4], const SplitInts &px, const double (&y)[4], const SplitInts &py,
                        double (&o)[4]) {
         split_half_node<K>(x, px, y, py, block(i), team, half + (size_t)i * (kNCH * NP) + row, k1, o);
@@ -1092,13 +1092,13 @@ cudaError_t launch_shape(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
     if (e != cudaSuccess) return e;
     if (!kUsePDL) {
         lw_step_kernel<T, K, W><<<L.blocks, W * 32, step_smem_bytes<T, K, W>(), st>>>(
-            (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr,
+            (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.pitch, L.Nr,
             (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa, L.err);
         return cudaGetLastError();
     }
     return launch_chained<lw_step_kernel<T, K, W>>(
         (unsigned)L.blocks, W * 32, step_smem_bytes<T, K, W>(), st, (const T *)L.u_in, (T *)L.u_out, (const T *)L.half,
-        (const T *)L.node, L.step, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa, L.err);
+        (const T *)L.node, L.step, L.pitch, L.Nr, (T)(0.25 * L.dt_inner), (T)(0.5 * L.dt_inner), wa, L.err);
 }
 
 template <typename T, int K, int W>
@@ -1137,12 +1137,12 @@ cudaError_t launch_fused(const StepLaunch &L, const WaveArgs &wa, cudaStream_t s
         constexpr int WF = fused_warps<T, K>();
         if (L.warps == WF)
             lw_step2_kernel<K, WF><<<L.blocks, WF * 32, 0, st>>>(
-                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr, en, wa,
-                mask);
+                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.pitch, L.Nr, en,
+                wa, mask);
         else if (L.warps == kNarrowWarps)
             lw_step2_kernel<K, kNarrowWarps><<<L.blocks, kNarrowWarps * 32, 0, st>>>(
-                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.Nr, en, wa,
-                mask);
+                (const T *)L.u_in, (T *)L.u_out, (const T *)L.half, (const T *)L.node, L.step, L.pitch, L.Nr, en,
+                wa, mask);
         else
             return cudaErrorInvalidValue;
         return cudaGetLastError();
@@ -1293,10 +1293,11 @@ cudaError_t launch_persistent_w(const StepLaunch &L, void *u_other, int n_inner,
     double *u0 = (double *)L.u_in, *u1 = (double *)u_other;
     const double *half = (const double *)L.half, *node = (const double *)L.node;
     const unsigned char *step = L.step;
+    size_t pitch = L.pitch;
     int Nr = L.Nr;
     double en = 0.5 * L.dt_inner;
     size_t stride = L.stride;
-    void *args[] = {&u0, &u1, &half, &node, &step, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err, &stride};
+    void *args[] = {&u0, &u1, &half, &node, &step, &pitch, &Nr, &en, &wa, &n_inner, &substeps, &flags, &err, &stride};
     if (L.columns == 3)
         return cudaLaunchCooperativeKernel((const void *)lw_column_kernel<K, 3>, dim3(L.blocks),
                                            dim3(column_warps<K, 3>() * 32), args, column_smem_bytes<K, 3>(), st);
