@@ -1358,7 +1358,8 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
         }
         if (e == cudaSuccess)
             e = tk::launch_import_state(S->precision, S->Nr, S->Nth, S->NP, S->drs, src, src + plane,
-                                        src + 2 * plane, src + 3 * plane, S->b_node, S->adj[0], S->stream);
+                                        src + 2 * plane, src + 3 * plane, S->b_node, S->adj[0], S->num_sms,
+                                        S->stream);
     } else {
         e = cudaMemsetAsync(S->adj[0], 0, se * S->esz, S->stream);
     }
@@ -1437,7 +1438,7 @@ extern "C" tk_status tk_adjoint(tk_solver *S, const double *dL_dwave, const doub
             return st;
         }
     }
-    const int ti = tk::tile_columns(S->Nr, S->NP);
+    const int ti = tk::tile_columns(S->Nr, S->NP, S->num_sms);
     const dim3 gridd(S->NP / 32, (S->Nr + ti - 1) / ti);
     const tk::Divisor d = tk::divisor(2.0 * S->drs);
     auto transpose = [&](auto kern, auto *lam) {

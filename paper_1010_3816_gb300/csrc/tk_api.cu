@@ -385,7 +385,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
     TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                        S->dt / S->substeps, S->rad, S->ang,
                                        S->precision, S->half, S->node, S->b_node, S->w_row,
-                                       S->cmp, S->gpm, S->stream, nullptr, nullptr,
+                                       S->cmp, S->gpm, S->num_sms, S->stream, nullptr, nullptr,
                                        S->step_pitch ? S->step : nullptr));
     S->have_coeffs = true;
     S->have_state = false;
@@ -406,7 +406,7 @@ tk_status tk_precompute_coeffs(tk_solver *S, double a, double M, int s, int m)
             TK_CUDA(S, tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs,
                                                S->dt / S->substeps, S->rad, S->ang,
                                                S->precision, S->half, S->node, S->b_node,
-                                               S->w_row, S->cmp, S->gpm, S->stream, nullptr, nullptr,
+                                               S->w_row, S->cmp, S->gpm, S->num_sms, S->stream, nullptr, nullptr,
                                                S->step_pitch ? S->step : nullptr));
         }
     }
@@ -461,7 +461,8 @@ tk_status tk_set_coefficients(tk_solver *S, double a, double M, int s, int m, co
     if (e == cudaSuccess)
         e = tk::launch_coeff_tables(S->kerr, S->variable, S->Nr, S->Nth, S->NP, S->drs, S->dt / S->substeps,
                                     S->rad, S->ang, S->precision, S->half, S->node, S->b_node,
-                                    S->w_row, S->cmp, S->gpm, S->stream, dn, dh, S->step_pitch ? S->step : nullptr);
+                                    S->w_row, S->cmp, S->gpm, S->num_sms, S->stream, dn, dh,
+                                    S->step_pitch ? S->step : nullptr);
     if (e == cudaSuccess && dev) e = cudaStreamSynchronize(S->stream);
     if (dev) cudaFree(dev);
     if (e != cudaSuccess) return fail(S, TK_ERR_CUDA, "tk_set_coefficients: %s", cudaGetErrorString(e));
@@ -481,14 +482,14 @@ tk_status tk_get_coefficients(tk_solver *S, double *node9, double *half9, int on
     const size_t n9 = (size_t)9 * S->Nth * S->Nr;
     if (on_device) {
         TK_CUDA(S, tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->rad, node9,
-                                         half9, S->stream));
+                                         half9, S->num_sms, S->stream));
         return TK_OK;
     }
     double *dev = nullptr;
     st = alloc(S, (void **)&dev, 2 * n9 * sizeof(double));
     if (st != TK_OK) return st;
     cudaError_t e = tk::launch_raw_export(S->kerr, S->variable, S->Nr, S->Nth, S->rad, dev,
-                                          dev + n9, S->stream);
+                                          dev + n9, S->num_sms, S->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(node9, dev, n9 * sizeof(double), cudaMemcpyDeviceToHost, S->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(half9, dev + n9, n9 * sizeof(double), cudaMemcpyDeviceToHost, S->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(S->stream);
@@ -533,7 +534,7 @@ static tk_status import_planes(tk_solver *S, const double *pr, const double *pi,
     if (S->unchecked) TK_CUDA(S, cudaMemsetAsync(S->lost, 0, sizeof(int), S->stream));   // of the state replaced
     void *dst = S->u[S->cur];
     TK_CUDA(S, tk::launch_import_state(S->precision, S->Nr, S->Nth, S->NP, S->drs, pr, pi, qr, qi,
-                                       S->b_node, dst, S->stream));
+                                       S->b_node, dst, S->num_sms, S->stream));
     return TK_OK;
 }
 
@@ -919,7 +920,7 @@ tk_status tk_get_state(tk_solver *S, double *planes4, int on_device)
     if (!planes4) return fail(S, TK_ERR_ARG, "tk_get_state: planes4 is NULL");
     if (on_device) {
         TK_CUDA(S, tk::launch_export_state(S->precision, S->Nr, S->Nth, S->NP, S->u[S->cur], planes4,
-                                           S->stream));
+                                           S->num_sms, S->stream));
         return TK_OK;
     }
     st = check_lost(S, "tk_get_state");
@@ -927,7 +928,7 @@ tk_status tk_get_state(tk_solver *S, double *planes4, int on_device)
     st = ensure_staging(S);
     if (st != TK_OK) return st;
     TK_CUDA(S, tk::launch_export_state(S->precision, S->Nr, S->Nth, S->NP, S->u[S->cur], S->staging,
-                                       S->stream));
+                                       S->num_sms, S->stream));
     TK_CUDA(S, cudaMemcpyAsync(planes4, S->staging, (size_t)4 * S->Nth * S->Nr * sizeof(double),
                                cudaMemcpyDeviceToHost, S->stream));
     TK_CUDA(S, cudaStreamSynchronize(S->stream));

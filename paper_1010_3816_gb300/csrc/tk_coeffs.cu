@@ -637,10 +637,10 @@ cudaError_t launch_stiffness(const Kerr &P, int variable, int Nr, int Ntheta, in
 }
 
 cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *rad, double *out_node,
-                              double *out_half, cudaStream_t st)
+                              double *out_half, int num_sms, cudaStream_t st)
 {
     const size_t n = (size_t)Ntheta * Nr;
-    const int blocks = (int)std::min<size_t>((n + 255) / 256, 152 * 8);
+    const int blocks = (int)std::min<size_t>((n + 255) / 256, num_sms * 8);
     raw_export_kernel<<<blocks, 256, 0, st>>>(P, variable, Nr, Ntheta, rad, out_node, out_half);
     return cudaGetLastError();
 }
@@ -665,9 +665,10 @@ cudaError_t launch_radial_parts(const Kerr &P, double rs_min, double drs, int Nr
     return launch_parts(kp, 1, rs_min, drs, Nr, rad, Ntheta, NP, ang, num_sms, st);
 }
 
-static dim3 table_grid(int Nr, const dim3 &block)
+// at most four blocks per SM, whose threads take the columns in turns
+static dim3 table_grid(int Nr, const dim3 &block, int num_sms)
 {
-    return dim3(std::min<unsigned>((Nr + block.y - 1) / block.y, 152 * 4));
+    return dim3(std::min<unsigned>((Nr + block.y - 1) / block.y, num_sms * 4));
 }
 
 cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_min, int Nr, int Ntheta, int NP,
@@ -678,21 +679,20 @@ cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_m
                                  st);
     if (e != cudaSuccess) return e;
     const dim3 block(NP, kTableThreads / NP);
-    table_derivative_kernel<<<table_grid(Nr, block), block, 0, st>>>(kp, variable, Nr, Ntheta, NP, divisor(drs),
-                                                                     divisor(0.25 * dt_inner), dt_inner, rad,
-                                                                     ang, half, node, b_node);
+    table_derivative_kernel<<<table_grid(Nr, block, num_sms), block, 0, st>>>(
+        kp, variable, Nr, Ntheta, NP, divisor(drs), divisor(0.25 * dt_inner), dt_inner, rad, ang, half, node, b_node);
     return cudaGetLastError();
 }
 
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
                                 double drs, double dt_inner, const double *rad, const double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
-                                cudaStream_t st, const double *raw_node, const double *raw_half,
+                                int num_sms, cudaStream_t st, const double *raw_node, const double *raw_half,
                                 unsigned char *step)
 {
     const F32Derive fd = f32_derive(dt_inner);
     dim3 block(NP, kTableThreads / NP);
-    const dim3 grid = table_grid(Nr, block);
+    const dim3 grid = table_grid(Nr, block, num_sms);
     const Divisor ds = divisor(drs), de = divisor(0.25 * dt_inner);   // dr*, the half node's e
     if (precision == 0)
         coeff_tables_kernel<double><<<grid, block, 0, st>>>(P, variable, Nr, Ntheta, NP, ds, de, dt_inner,

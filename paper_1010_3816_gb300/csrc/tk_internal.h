@@ -116,9 +116,13 @@ struct KerrSet {
 };
 
 // Tiles of the transposes between the planes and the state: 32 rows by 32
-// columns, on small grids by 8 (64 bytes at a time, but four times the blocks).
+// columns, by 8 on grids with fewer of these than two per SM (64 bytes at a time,
+// but four times the blocks: 1 % of the 6 x 1601 x 32 batch's pass).
 constexpr int kTileThreads = 256;
-inline int tile_columns(int Nr, int NP) { return (long long)(Nr / 32) * (NP / 32) < 304 ? 8 : 32; }
+inline int tile_columns(int Nr, int NP, int num_sms)
+{
+    return (long long)(Nr / 32) * (NP / 32) < 2 * num_sms ? 8 : 32;
+}
 
 // Division by a constant: a division costs the FP64 pipe some ten instructions of
 // 64 cycles; where the constant is a power of two, one multiplication by its
@@ -175,7 +179,7 @@ cudaError_t launch_radial_parts(const Kerr &P, double rs_min, double drs, int Nr
 cudaError_t launch_coeff_tables(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
                                 double drs, double dt_inner, const double *rad, const double *ang, int precision, void *half,
                                 void *node, double *b_node, double *w_row, float *cmp, float *gpm,
-                                cudaStream_t st, const double *raw_node = nullptr,
+                                int num_sms, cudaStream_t st, const double *raw_node = nullptr,
                                 const double *raw_half = nullptr, unsigned char *step = nullptr);
 
 // The derivative of the FP64 tables in a parameter of the black hole, sum_q w[q]
@@ -188,7 +192,7 @@ cudaError_t launch_table_derivative(const KerrSet &kp, int variable, double rs_m
 // The raw coefficients of the precompute, [9][Ntheta][Nr] at nodes and half
 // nodes (device output buffers).
 cudaError_t launch_raw_export(const Kerr &P, int variable, int Nr, int Ntheta, const double *rad,
-                              double *out_node, double *out_half, cudaStream_t st);
+                              double *out_node, double *out_half, int num_sms, cudaStream_t st);
 
 cudaError_t launch_stiffness(const Kerr &P, int variable, int Nr, int Ntheta, int NP,
                              const double *rad, const double *ang, unsigned long long *out,
@@ -197,10 +201,10 @@ cudaError_t launch_stiffness(const Kerr &P, int variable, int Nr, int Ntheta, in
 // ---- state import / export (tk_layout.cu) ----
 cudaError_t launch_import_state(int precision, int Nr, int Ntheta, int NP, double drs,
                                 const double *phi_re, const double *phi_im, const double *pi_re,
-                                const double *pi_im, const double *b_node, void *u,
+                                const double *pi_im, const double *b_node, void *u, int num_sms,
                                 cudaStream_t st);
 cudaError_t launch_export_state(int precision, int Nr, int Ntheta, int NP, const void *u,
-                                double *planes4, cudaStream_t st);
+                                double *planes4, int num_sms, cudaStream_t st);
 cudaError_t launch_gaussian(int Nr, int Ntheta, double rs_min, double drs, double amp,
                             double center, double width, double noise, unsigned long long seed,
                             double *re, double *im, cudaStream_t st);

@@ -192,10 +192,10 @@ gaussian_kernel(int Nr, int Nth, double rs_min, double drs, double dth, double a
 
 cudaError_t launch_import_state(int precision, int Nr, int Ntheta, int NP, double drs,
                                 const double *phi_re, const double *phi_im, const double *pi_re,
-                                const double *pi_im, const double *b_node, void *u,
+                                const double *pi_im, const double *b_node, void *u, int num_sms,
                                 cudaStream_t st)
 {
-    const int ti = tile_columns(Nr, NP);
+    const int ti = tile_columns(Nr, NP, num_sms);
     const dim3 grid(NP / 32, (Nr + ti - 1) / ti);
     const Divisor d = divisor(2.0 * drs);
     auto go = [&](auto kern, auto *w) {
@@ -207,9 +207,9 @@ cudaError_t launch_import_state(int precision, int Nr, int Ntheta, int NP, doubl
 }
 
 cudaError_t launch_export_state(int precision, int Nr, int Ntheta, int NP, const void *u,
-                                double *planes4, cudaStream_t st)
+                                double *planes4, int num_sms, cudaStream_t st)
 {
-    const int ti = tile_columns(Nr, NP);
+    const int ti = tile_columns(Nr, NP, num_sms);
     const dim3 grid(NP / 32, (Nr + ti - 1) / ti);
     auto go = [&](auto kern, auto *w) { kern<<<grid, kTileThreads, 0, st>>>(Nr, Ntheta, NP, w, planes4); };
     if (precision == 0) go(ti == 8 ? export_kernel<double, 8> : export_kernel<double, 32>, (const double *)u);
