@@ -74,8 +74,10 @@ struct RowExps {
             f = g = 0;
             return;
         }
-        // a lifted term is below 2^(top - 1)
-        auto lifted = [&](double k, int n) { return n == 0 || k == 0.0 ? k : scalbn(1.0, top - 1); };
+        // a lifted term is below 2^(top - 1) (assembled from bits: a product costs
+        // the FP64 pipe 64 cycles)
+        const double bound = __hiloint2double(max(top + 1022, 1) << 20, 0);
+        auto lifted = [&](double k, int n) { return n == 0 || k == 0.0 ? k : bound; };
         f = split_exponent(t.f + (lifted(t.ku, l.u) + lifted(t.kd, l.d)));
         if (g != kSplitAbsent) ++g;
     }
