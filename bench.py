@@ -58,8 +58,8 @@ ADJ_FLOP_PER_UPDATE = (2 + 2 * 14) + (6 + 2 * 12)                # = 60
 ADJ_INSTR_PER_UPDATE = 16 + 18
 STATE_BYTES_PER_UPDATE = {0: 64, 1: 32}                         # read u^n, write u^{n+1}
 # FP64: 9 doubles, 12 limb pairs, two exponents and the block's flags per point
-# (5648 bytes per column and 32 rows); FP32: 11 + 10 table entries
-TABLE_BYTES_PER_UPDATE = {0: 5648 / 32, 1: 21 * 4}
+# (5776 bytes per column and 32 rows); FP32: 11 + 10 table entries
+TABLE_BYTES_PER_UPDATE = {0: 5776 / 32, 1: 21 * 4}
 # the four-step FP32 sweep reads the compact FP32 tables: 16 of the 21 entries
 # per point (the other five are derived in the kernel)
 FP32_SWEEP_TABLE_BYTES = 16 * 4

@@ -94,6 +94,7 @@ constexpr int kStepExps = (kStepHalfF64 + kStepNodeF64 + 2 * kSplitEntries) * 25
 constexpr int kStepHead = kStepExps + 256 + 128;   // offset of the column's two flags
 constexpr int kStepBytes = kStepHead + 16;
 constexpr int kSplitAbsent = -14000;    // exponent of a class whose entries are all zero
+constexpr int kSplitFloor = -4;         // smallest exponent of a sum
 constexpr int kLiftAbsent = 14000;      // lift of a neighbour's coefficient that is zero
 constexpr int kLiftSpread = 6;          // largest difference of the lifts that two tables share
 constexpr int kSplitMaxClass = 20;      // largest class exponent; larger tables are cold

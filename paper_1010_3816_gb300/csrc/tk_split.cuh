@@ -49,7 +49,8 @@
 // rows per lane (three warps, 168 registers) the same arithmetic took 124 us.
 // 20 warps (96 registers, spills): 120 us.
 //
-// Subnormal values and couplings are taken and rounded like any other.  Columns
+// Subnormal values and couplings are taken and rounded like any other (sums are not
+// aligned below kSplitFloor, ten places under the smallest subnormal).  Columns
 // with a Phi above 1e263, infinite or NaN, and columns whose
 // tables are not finite or too large, take the FP64 instructions alone, so that
 // such values propagate as IEEE arithmetic has them; Pi only ever meets FP64
@@ -141,13 +142,21 @@ struct SplitSum {
     }
 };
 
-// T 2^(o - 1080) in FP64, rounded to the nearest (ties to even); subnormal ones
-// are rounded once more by a product with 2^-64.  In integers: the conversion
-// instruction holds the FP64 pipe as long as a DFMA does.
+// q, whose place 10 stands for 2^-1074, rounded to a subnormal number.
+__device__ __forceinline__ double split_subnormal(unsigned long long q, unsigned sign)
+{
+    q += 0x1ffu + (((unsigned)q >> 10) & 1u);
+    return __longlong_as_double((long long)((q >> 10) | ((unsigned long long)sign << 32)));
+}
+
+// T 2^(o - 1080) in FP64, rounded to the nearest (ties to even); o >= kSplitFloor.
+// In integers: the conversion instruction holds the FP64 pipe as long as a DFMA
+// does.  Where a pulse's tails underflow, whole columns take the branch: with a DFMA
+// in it (a normal number times 2^-64) 16001 x 128 took 127 us a step instead of 118.
 __device__ __forceinline__ double split_value(long long T, int o)
 {
     const long long s = T >> 63;
-    const unsigned long long m = (unsigned long long)((T ^ s) - s);
+    const unsigned long long m = (unsigned long long)((T ^ s) - s);   // < 2^62
     const unsigned mh = (unsigned)(m >> 32), ml = (unsigned)m;
     int n = __clz((int)mh);
     if (mh == 0) n = 32 + __clz((int)ml);
@@ -158,9 +167,7 @@ __device__ __forceinline__ double split_value(long long T, int o)
     const unsigned lo = __funnelshift_r(ql, qh, 10);
     const unsigned hi = ((qh >> 10) + ((unsigned)(e - 1) << 20)) | ((unsigned)s & 0x80000000u);
     if (e > 0 || m == 0) return __hiloint2double(m != 0 ? (int)hi : 0, (int)lo);
-    return e < -60 ? 0.0
-                   : __hiloint2double((int)(((qh >> 10) + ((unsigned)(e + 63) << 20)) | ((unsigned)s & 0x80000000u)),
-                                      (int)lo) * 0x1p-64;
+    return split_subnormal(m << (o - kSplitFloor), (unsigned)s & 0x80000000u);
 }
 
 // ---- teams ----
@@ -286,8 +293,8 @@ __device__ __forceinline__ bool split_coupling(const SplitInts &a, const SplitIn
     const int rx = tab.row_exp(), cf = (short)(rx & 0xffff), cg = (rx >> 16) - cf;
     const int lx = tab.lifts(), lu = (short)(lx & 0xffff), ld = lx >> 16;
     int f[2];
-    f[0] = max(max(eu2.x - lu, ed2.x - ld), e1[0]);
-    f[1] = max(max(eu2.y - lu, ed2.y - ld), e1[1]);
+    f[0] = max(max(eu2.x - lu, ed2.x - ld), max(e1[0], kSplitFloor - cf));
+    f[1] = max(max(eu2.y - lu, ed2.y - ld), max(e1[1], kSplitFloor - cf));
     if (imag) {
         f[0] = max(f[0], e1[1] + cg);
         f[1] = max(f[1], e1[0] + cg);

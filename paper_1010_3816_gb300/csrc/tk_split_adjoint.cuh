@@ -189,7 +189,7 @@ __device__ __forceinline__ AdjSums adj_add(const AdjSums &a, const AdjSums &b)
 __device__ __forceinline__ void adj_zero(AdjSums &a)
 {
     a.T[0] = a.T[1] = 0;
-    a.O[0] = a.O[1] = kSplitAbsent;
+    a.O[0] = a.O[1] = kSplitFloor;
 }
 
 // Both sums of the Pi values v[2], v[3] with the block of tab, whose head is
@@ -212,8 +212,8 @@ __device__ __forceinline__ bool adj_pair(const double (&v)[4], const AdjTab<HALF
     const int rx = tab.row_exp(), cf = (short)(rx & 0xffff), cg = (rx >> 16) - cf;
     const int lx = tab.lifts(), lu = (short)(lx & 0xffff), ld = lx >> 16;
     int f[2];
-    f[0] = max(max(eu2.x - lu, ed2.x - ld), p.e[0]);
-    f[1] = max(max(eu2.y - lu, ed2.y - ld), p.e[1]);
+    f[0] = max(max(eu2.x - lu, ed2.x - ld), max(p.e[0], kSplitFloor - cf));
+    f[1] = max(max(eu2.y - lu, ed2.y - ld), max(p.e[1], kSplitFloor - cf));
     if (imag) {
         f[0] = max(f[0], p.e[1] + cg);
         f[1] = max(f[1], p.e[0] + cg);
