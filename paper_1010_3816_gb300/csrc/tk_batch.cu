@@ -35,7 +35,6 @@ struct BatchMember {
     void *u0, *u1;            // the member's two time levels
     const void *half, *node;  // folded coefficient tables
     const unsigned char *step;   // FP64: the step's tables
-    size_t pitch;             // (StepLaunch)
     int *err;                 // raised where a copy of them did not come
     int Nr, K;
     int substeps, ratio;      // k_i and kmax / k_i
@@ -99,12 +98,13 @@ __device__ void sweep(const BatchMember &m, const T *__restrict__ u_in, T *__res
 
 // A member's unsplit tables and error word, looked up where they are used: six
 // registers less in the sweep, which spills otherwise.
+template <int K>
 struct MemberRare {
     const BatchMember *m;
     __device__ __forceinline__ const double *half() const { return (const double *)m->half; }
     __device__ __forceinline__ const double *node() const { return (const double *)m->node; }
     __device__ __forceinline__ int *err() const { return m->err; }
-    __device__ __forceinline__ size_t pitch() const { return m->pitch; }
+    __device__ __forceinline__ size_t pitch() const { return K * kStepBytes; }   // (members with tables: queue_fits)
 };
 
 // The block's share of an FP64 item: its teams take equal parts of the columns.
@@ -116,7 +116,7 @@ __device__ void sweep_teams(const BatchMember &m, SplitRing *ring, unsigned long
     constexpr int TEAMS = kBatchThreads / 32 / K, NP = 32 * K;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, t = wib / K;
     SplitTeam<K> team{rows + t * K, wib % K, lane, 1 + t};
-    const SplitSweep<K, MemberRare> sw{ring + wib, bar, m.step + team.h * kStepBytes, {&m}, m.Nr, m.en};
+    const SplitSweep<K, MemberRare<K>> sw{ring + wib, bar, m.step + team.h * kStepBytes, {&m}, m.Nr, m.en};
     const int a = i0 + t * (i1 - i0) / TEAMS, b = i0 + (t + 1) * (i1 - i0) / TEAMS;
     if (b <= a) return;
     sw.run(st, team, u_in, a, b, false, [] {}, [&](int i, const double (&o)[4]) {
@@ -368,7 +368,6 @@ tk_status upload_members(tk_batch *B)
         tkh::fill_launch(S, L);
         m.obs = L.obs;
         m.step = L.step;
-        m.pitch = L.pitch;
         m.err = L.err;
     }
     TKB_CUDA(B, cudaMemcpyAsync(B->d_mem, h.data(), B->n * sizeof(tk::BatchMember),
@@ -419,6 +418,16 @@ tk_status advance_members(tk_batch *B, int n)
         TKB_CUDA(B, tkh::mark_unchecked(S, B->stream));
     }
     return TK_OK;
+}
+
+// Whether the queue can step the members: FP64 ones with tables of their own for
+// every column (not those that had to give them up; a pitch from the member costs a
+// tick up to 5 %).  Otherwise they are stepped one after another.
+bool queue_fits(const tk_batch *B)
+{
+    for (tk_solver *S : B->mem)
+        if (B->precision == TK_PREC_F64 && S->step_pitch == 0) return false;
+    return true;
 }
 
 tk_status check_members(tk_batch *B)
@@ -517,16 +526,16 @@ tk_status tk_batch_step(tk_batch *B, int n)
     TKB_CUDA(B, cudaSetDevice(B->device));
     tk_status st = check_members(B);
     if (st != TK_OK || n == 0) return st;
-    if (B->per_member) {
+    for (tk_solver *S : B->mem) {
+        st = tkh::ensure_wave(S, S->count + n);   // (may give up tables)
+        if (st != TK_OK) return bfail(B, st, "tk_batch_step: %s", S->err);
+    }
+    if (B->per_member || !queue_fits(B)) {
         for (tk_solver *S : B->mem) {
             st = tk_step(S, n);
             if (st != TK_OK) return bfail(B, st, "tk_batch_step: %s", S->err);
         }
         return TK_OK;
-    }
-    for (tk_solver *S : B->mem) {
-        st = tkh::ensure_wave(S, S->count + n);
-        if (st != TK_OK) return bfail(B, st, "tk_batch_step: %s", S->err);
     }
     st = upload_members(B);
     if (st != TK_OK) return st;
@@ -593,6 +602,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
     TKB_CUDA(B, cudaStreamSynchronize(B->stream));
     const int old_chunk = B->graph_chunk;
     B->graph_chunk = 0;   // trials launch directly
+    const bool queue = queue_fits(B);
     // the search space: segment length (columns per work item) x grid size
     // (blocks per SM, up to the resident maximum; fewer blocks leave each
     // warp more items of the queue)
@@ -603,7 +613,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (int per_sm = max_per_sm; per_sm >= 1 && st == TK_OK; --per_sm)
+    for (int per_sm = queue ? max_per_sm : 0; per_sm >= 1 && st == TK_OK; --per_sm)
     for (int seg : candidates) {
         B->blocks = sms * per_sm;
         st = build_items(B, seg);
@@ -637,7 +647,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
     // cooperative launch and host synchronization), which a long
     // tk_batch_step amortizes, count for neither.
     double queue_ms = 1e300;
-    if (st == TK_OK) {
+    if (st == TK_OK && queue) {
         B->blocks = best_blocks;
         st = build_items(B, best);
         if (st == TK_OK) st = upload_members(B);
@@ -668,7 +678,7 @@ tk_status tk_batch_tune(tk_batch *B, int trial_steps, int *best_seg, double *bes
     // are what the work queue is for (24 members of 1601 x 32 run 1.18x
     // faster through it), and short trials of direct launches understate it.
     bool all_fill = true;
-    for (tk_solver *S : B->mem) all_fill = all_fill && S->persist && S->warps != tk::kNarrowWarps;
+    for (tk_solver *S : B->mem) all_fill = all_fill && (!queue || (S->persist && S->warps != tk::kNarrowWarps));
     bool per_member = false;
     if (st == TK_OK && all_fill) {
         std::vector<int> cur0(B->n);

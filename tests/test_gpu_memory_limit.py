@@ -89,3 +89,39 @@ def test_grids_that_fit_without_the_split_tables(left, mode):
     if adjoint:
         assert np.linalg.norm(got_grad - want_grad) <= TOL * np.linalg.norm(want_grad)
 
+
+
+def test_batch_with_a_member_without_the_split_tables():
+    """The queue needs them of every member; the members are then stepped one after
+    another, the second of these without its tables."""
+    import torch
+
+    import paper_1010_3816_gb300 as tk
+    dev = torch.device("cuda")
+    planes = [torch.from_numpy(x).to(dev) for x in initial_planes(W)]
+    state, grad = (torch.empty((4, W.Ntheta, W.Nr), dtype=torch.float64, device=dev) for _ in range(2))
+    g = _solver()
+    want = _run(g, planes, None, state, grad, 0).cpu().numpy()
+    g.close()
+    torch.cuda.synchronize()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (2 * BASE + SPLIT + SPLIT // 4 + 2 * STATE), dtype=torch.uint8, device=dev)
+    try:
+        gs = [_solver(), _solver()]
+        for g in gs:
+            g.set_initial(*planes)
+        b = tk.Batch(gs)
+        b.step(2)
+        seg, ms = b.tune(1)
+        assert seg == 0 and ms > 0.0
+        b.step(N - 2)
+        got = [g.state(out=state).cpu().numpy() for g in gs]
+        b.close()
+        for g in gs:
+            g.close()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert not np.array_equal(got[0], got[1])
+    for s in got:
+        for c in range(4):
+            assert np.linalg.norm(s[c] - want[c]) <= TOL * np.linalg.norm(want[c])
