@@ -402,9 +402,8 @@ struct AdjSweep {
 
     __device__ __forceinline__ void fetch(SplitRingState &st, int slot, int i, int lane) const
     {
-        if (st.lost) return;
         __syncwarp();
-        if (lane == 0) {
+        if (lane == 0 && !(st.wait & kLost)) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_expect(&bar[slot], kAdjBytes);
             bulk_fetch(ring->tab[slot], tab + (size_t)i * pitch, kAdjBytes, &bar[slot]);
@@ -414,9 +413,12 @@ struct AdjSweep {
     __device__ __forceinline__ void await(SplitRingState &st, int slot) const
     {
         const unsigned parity = (st.wait >> slot) & 1u;
-        if (!__all_sync(kFull, mbar_test(&bar[slot], parity))) {
-            if (!st.lost) st.lost = !warp_mbar_wait(&bar[slot], parity, ErrWord{err});
-            if (st.lost) return;
+        if (!mbar_test(&bar[slot], parity)) {
+            if (!(st.wait & kLost) && !mbar_wait(&bar[slot], parity, err)) {
+                st.wait |= kLost;
+                atomicExch(err, 1);
+            }
+            if (st.wait & kLost) return;
         }
         st.wait ^= 1u << slot;
     }
