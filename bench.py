@@ -57,7 +57,7 @@ ADJ_SCHEME_FLOP_PER_UPDATE = 108
 ADJ_FLOP_PER_UPDATE = (2 + 2 * 14) + (6 + 2 * 12)                # = 60
 ADJ_INSTR_PER_UPDATE = 16 + 18
 STATE_BYTES_PER_UPDATE = {0: 64, 1: 32}                         # read u^n, write u^{n+1}
-# FP64: 9 doubles, 12 limb pairs, two exponents and the block's flags per point
+# FP64: 9 doubles, 12 limb pairs, exponents, lifts and the block's flags per point
 # (5776 bytes per column and 32 rows); FP32: 11 + 10 table entries
 TABLE_BYTES_PER_UPDATE = {0: 5776 / 32, 1: 21 * 4}
 # the four-step FP32 sweep reads the compact FP32 tables: 16 of the 21 entries
@@ -74,8 +74,8 @@ FP32_FMA_PER_CLK_PER_SM = 128
 # keyed by (workload name, precision); the capture's command and figures are in the
 # named summary under profiles/.
 MEASURED_TRAFFIC = {
-    # one persistent launch of 100 steps: 34.491594 + 5.232270 GB, per step
-    ("kerr_a0.9_25601x64_38400steps", 0): ((34.491594e9 + 5.232270e9) / 100,
+    # one persistent launch of 100 steps: 35.152628 + 5.232659 GB, per step
+    ("kerr_a0.9_25601x64_38400steps", 0): ((35.152628e9 + 5.232659e9) / 100,
                                            "profiles/lw_persistent_f64_kerr_25601x64.md"),
     # one launch of 50 sweeps of four steps: 6.726055 + 1.280336 GB
     ("kerr_a0.9_25601x64_38400steps", 1): ((6.726055e9 + 1.280336e9) / 50,
@@ -757,7 +757,8 @@ def measure_solve(args, tk, torch, w, precision, steps, warmup, rank, world, loc
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "kernel": ("lw_step_kernel<double>" if not fp64_persistent else "lw_column_kernel"
-                           if w.Nr * (1 if w.Ntheta <= 32 else 2 if w.Ntheta <= 64 else 4) <= 1824
+                           if w.Nr * (1 if w.Ntheta <= 32 else 2 if w.Ntheta <= 64 else 4)
+                           <= (2128 if w.Ntheta <= 64 else 1824)
                            else "lw_persistent_kernel"),
                 "peak_source": "152 SMs x 2 DFMA/clk x 2 flop x median SM clock "
                                f"{f_clk / 1e6:.0f} MHz (GB300 FP64 FMA issue rate; "

@@ -646,8 +646,8 @@ lw_adjoint_team_persistent_kernel(double *a0, double *a1, const double *__restri
 // ends), and the one to the left goes to the left team through shared memory with
 // lam~; eta and its sum to the right go to the right team for mu.  Two block
 // barriers a step; tables and columns stay in the SM.  us per step, this launch
-// (lw_adjoint_team_persistent_kernel, one or two columns per team): 1601 x 32 6.5
-// (10.0), 1824 x 32 7.2 (10.0 at 1825), 912 x 64 7.6 (9.6), 456 x 128 8.3 (10.9).
+// (lw_adjoint_team_persistent_kernel, one or two columns per team): 1601 x 32 6.2
+// (10.0), 1824 x 32 6.2 (9.3 at 1825), 912 x 64 7.0 (9.6), 456 x 128 7.8 (10.9).
 // Bound by the chain pair - barrier - eta - pair - barrier - mu and by the FP64
 // pipe of the SMs with four blocks.  first: launch step s is the transposed step
 // first + s of the call; stride != 0: step s writes the whole level to a1 + s
@@ -1497,8 +1497,8 @@ extern "C" tk_status tk_param_gradient(tk_solver *S, int param, const double *dL
     // small grids: a segment's levels in one launch (lw_column_kernel writing a
     // trajectory), 4.3 us a step at 1601 x 32 where a launch per step takes 8.6
     const bool columns = S->persist && S->persist_columns && C * k <= 0x7fffffff;
-    // and the transposed steps that one tangent launch contracts (6.5 us a step
-    // there, 11 with a launch each; for fewer than four the launch costs more)
+    // and the transposed steps that one tangent launch contracts (6.2 us a step
+    // there, 10.6 with a launch each; for fewer than four the launch costs more)
     int cblocks = S->persist && Q >= 4 ? tk::adjoint_column_blocks(0, S->K, S->Nr, S->num_sms) : 0;
     const size_t nflags = (size_t)2 * S->K * std::max(columns ? S->persist_blocks : 0, cblocks);
 

@@ -251,8 +251,8 @@ constexpr double kAutoGrowthPerStep = 2.5e-5;
 // waits only for the warps it depends on, so that no launch boundary or block
 // barrier separates the steps.  Measured: FP32 25601 x 64, 15.7 us per step in
 // sweeps of four, 16.6 in pairs, 18.3 with a launch per pair; FP64 1601 x 32,
-// 6.2 against 8.6 us with a launch per step; FP64 25601 x 32 / 64 / 128, 44.3
-// / 89.3 / 185.2 against 49.4 / 93.9 / 189.9 us.  A grid whose blocks cannot
+// 4.3 against 8.6 us with a launch per step; FP64 25601 x 32 / 64 / 128, 43.7
+// / 87.6 / 179.5 against 49.0 / 92.4 / 185.6 us.  A grid whose blocks cannot
 // all be resident at once falls back to one launch per step (2 for FP32).
 static void set_launch_mode(tk_solver *S, int mode)
 {

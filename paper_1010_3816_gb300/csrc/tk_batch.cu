@@ -205,8 +205,9 @@ batch_step_kernel(const BatchMember *__restrict__ mem, int nmem, const BatchItem
 constexpr size_t kBatchSmem = kBatchThreads / 32 * sizeof(SplitRing);
 
 // The FP64 kernel for members that all have 32 kall rows (0: mixed).  With the
-// three sweeps in one kernel it spills 250 bytes, 20 loads and 12 stores per
-// column; alone none does: 6 x 1601 x 32 28.1 -> 25.8 us per tick.
+// three sweeps in one kernel it keeps 88 bytes on the stack (240 bytes of spills);
+// alone those of 32 and 128 rows keep nothing there and that of 64 rows four bytes:
+// 6 x 1601 x 32 24.5 us a tick, 28.1 in the mixed kernel when they were split.
 using BatchKernel = void (*)(const BatchMember *, int, const BatchItem *, int, int, int, int, unsigned int *);
 static BatchKernel batch_kernel_f64(int kall)
 {

@@ -393,7 +393,7 @@ __device__ __forceinline__ void table_entries(const Geo &P, int variable, int Nr
 // what depends on the angle alone is formed once per thread, which takes
 // columns in turns (with both formed at every point 372 us at 4001 x 64, now
 // 217; with the divisions by dr* and e as multiplications where these are powers
-// of two 193).
+// of two 193, 198 with the lifts of the step's tables).
 constexpr int kTableThreads = 256;
 
 template <typename T>

@@ -5,8 +5,10 @@
 //                           jp: theta row padded to NP = 32*K (rows >= Ntheta are 0)
 //   tables  half[i][q][jp]  q < kNCH: folded coefficients of Eq. (lw1) at r*_{i+1/2}
 //           node[i][q][jp]  q < kNCN: folded coefficients of Eq. (lw2) at r*_i
-// One warp owns every theta row of a column (lane l holds rows K*l .. K*l+K-1),
-// so a column of any plane or table is one contiguous, coalesced vector load.
+// One warp owns every theta row of a column (FP32: lane l holds rows K*l ..
+// K*l+K-1; the FP64 parameter gradient's tangent too), or a team of K warps does
+// (FP64: one row per lane), so a column of any plane or table is one contiguous,
+// coalesced load.
 #pragma once
 
 #include <math.h>
@@ -251,7 +253,7 @@ cudaError_t launch_lw_step(const StepLaunch &L, cudaStream_t st);
 int step_grid_shape(int precision, int K, int Nr, int num_sms, int *warps);
 // Many FP64 steps in one cooperative launch: the grid size for it, 0 if it
 // cannot run; the launch itself (L.u_in holds u^n, u_other is the
-// second level; flags: one zeroed unsigned int per block; *err set on a wait
+// second level; flags: 2 K zeroed unsigned ints per block; *err set on a wait
 // that timed out).
 // *columns: what L.columns has to be.
 int persistent_grid_blocks(int K, int Nr, int num_sms, int warps, int *columns);

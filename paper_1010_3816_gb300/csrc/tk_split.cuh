@@ -14,10 +14,10 @@
 //
 // Measured, 25601 x 64, per step of the persistent launch: 147.0 us with the 54
 // instructions, 100.2 with this coupling converted by the FP64 conversion
-// instruction (which costs as much as a DFMA), 88.8 with the conversion in
-// integers too; the FP64 pipe is then 83 % busy, the rest is latency of the
-// integer chains with four warps per sub-partition.  25601 x 32: 73.2 -> 44.3,
-// x 128: 287 -> 184 us.  More of the node in integers does not pay: with Pi + T
+// instruction (which costs as much as a DFMA), 87.6 with the conversion in
+// integers too; the FP64 pipe is then 84 % busy, the rest is latency of the
+// integer chains with four warps per sub-partition.  25601 x 32: 73.2 -> 43.7,
+// x 128: 287 -> 180 us.  More of the node in integers does not pay: with Pi + T
 // rounded once there (26 FP64 instructions) 90.0, with B (m - p) + Phi too (22)
 // 92.0 us: 37 integer instructions cost what a DFMA does.  All of the step in integers (8 FP64 instructions left)
 // took 147 us: its 1235 integer instructions per update are then the bound.
@@ -36,9 +36,12 @@
 // the values are shifted right to the largest of these, per row and component:
 // what is lost lies 2^-60 below a product of the sum's largest exponent.  The
 // sum, T = sum / 2^64, stands for T 2^(E - 1080) and is converted to FP64 once
-// (split_value).  The l l products, zero in the mean, are left out.  T's last
-// place is at most 2^-53 of the sum's largest product, typically 2^-55: an FMA
-// chain rounds to 2^-53 of its partial sum at every product.
+// (split_value).  The l l products, zero in the mean, are left out.  That, and T's
+// rounding to an integer, cost up to 2^-53 each of the largest product that the sum's
+// exponents allow, typically 2^-56, and the conversion half a unit: an FMA chain
+// rounds to 2^-53 of its partial sum at every product.  The row's own two coefficients
+// share an exponent, so one that cancels to far less than the other keeps fewer bits
+// (as many as its own rounding left it).
 // Every operation treats both signs alike, so that conjugate
 // data and a -> -a still give conjugate results to the bit.
 //
@@ -54,7 +57,7 @@
 // with a Phi above 1e263, infinite or NaN, and columns whose
 // tables are not finite or too large, take the FP64 instructions alone, so that
 // such values propagate as IEEE arithmetic has them; Pi only ever meets FP64
-// instructions (testing it too took 89.6 instead of 88.8 us on 25601 x 64).
+// instructions (testing it too took 1 % more on 25601 x 64).
 #pragma once
 
 #include "tk_split_tables.cuh"

@@ -13,7 +13,7 @@
 // left (26 where the coefficients are real).
 //
 // Measured, 16001 x 128, per step of the persistent launch: 225 us with 62 FP64
-// instructions, 151 us (x 32: 36 us); the FP64 pipe is 75 % busy, 1240
+// instructions, 147 us (x 32: 37 us); the FP64 pipe is 78 % busy, 1310
 // instructions per update and row of a warp are issued.
 #pragma once
 

@@ -601,9 +601,9 @@ __device__ __forceinline__ void observe(int i, int lane, const T (&o)[4][K], con
 }
 
 // Bulk copies (the TMA unit's cp.async.bulk) of a column's tables into a
-// warp's shared-memory ring: one thread issues the two copies of a column
-// (half-node and node tables, contiguous in global memory), which complete on
-// the mbarrier of their ring slot; the warp waits on that mbarrier's phase
+// warp's shared-memory ring: one thread issues the copies of a column (FP64: one
+// block; FP32: the half-node and node tables, or the compact table), which complete
+// on the mbarrier of their ring slot; the warp waits on that mbarrier's phase
 // before reading the slot.
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
